@@ -76,9 +76,9 @@ __global__ void __launch_bounds__(NT) k_adj_elas_coef(Geo G, DevParams P, AdjVie
     const int k0 = blockIdx.z * G.zc, k1 = min(G.nz, k0 + G.zc);
     for (int k = k0; k < k1; ++k) {
       const Nbr nb = make_nbr(G, i, j, k);
-      const long long c = nb.at(0, 0, 0);
-      const long long np[3] = {nb.at(1, 0, 0), nb.at(0, 1, 0), nb.at(0, 0, 1)};
-      const long long nm[3] = {nb.at(-1, 0, 0), nb.at(0, -1, 0), nb.at(0, 0, -1)};
+      const int c = nb.at(0, 0, 0);
+      const int np[3] = {nb.at(1, 0, 0), nb.at(0, 1, 0), nb.at(0, 0, 1)};
+      const int nm[3] = {nb.at(-1, 0, 0), nb.at(0, -1, 0), nb.at(0, 0, -1)};
       double lmu = 0.0, lla = 0.0, leta = 0.0;
       double Dpsi[3][3], Du[3][3];   // [component][direction], centred differences
 #pragma unroll
@@ -256,7 +256,7 @@ __global__ void __launch_bounds__(NT) k_adj_react(Geo G, DevParams P, double dt,
   if (i < G.nx && j < G.ny) {
     const int k0 = blockIdx.z * G.zc, k1 = min(G.nz, k0 + G.zc);
     for (int k = k0; k < k1; ++k) {
-      const long long c = ((long long)k * G.ny + j) * G.nx + i;
+      const int c = (k * G.ny + j) * G.nx + i;
       // ---- forward recomputation: fix-up, species Heun, oxygen and edema inputs
       const double id = T.idag[c], idd = T.iddag[c];
       const double g0 = T.gdag[c], w0 = T.wdag[c];
@@ -377,9 +377,9 @@ __global__ void __launch_bounds__(NT) k_adj_cn_post(Geo G, DevParams P, double h
     const double* out[3] = {T.iddag, T.odag, T.ldag};
     for (int k = k0; k < k1; ++k) {
       const Nbr nb = make_nbr(G, i, j, k);
-      const long long c = nb.at(0, 0, 0);
-      const long long np[3] = {nb.at(1, 0, 0), nb.at(0, 1, 0), nb.at(0, 0, 1)};
-      const long long nm[3] = {nb.at(-1, 0, 0), nb.at(0, -1, 0), nb.at(0, 0, -1)};
+      const int c = nb.at(0, 0, 0);
+      const int np[3] = {nb.at(1, 0, 0), nb.at(0, 1, 0), nb.at(0, 0, 1)};
+      const int nm[3] = {nb.at(-1, 0, 0), nb.at(0, -1, 0), nb.at(0, 0, -1)};
       auto K = [&](long long e) {
         const double kr = nodeK_raw(P, T.g[e], T.w[e], T.f[e]);
         return kr > 0.0 ? kr : 0.0;
@@ -441,7 +441,7 @@ __global__ void __launch_bounds__(NT) k_cn_init_rhs(Geo G, Cn3 C, AdjView A) {
   if (i < G.nx && j < G.ny) {
     const int k0 = blockIdx.z * G.zc, k1 = min(G.nz, k0 + G.zc);
     for (int k = k0; k < k1; ++k) {
-      const long long c = ((long long)k * G.ny + j) * G.nx + i;
+      const int c = (k * G.ny + j) * G.nx + i;
       const double di = C.dinv[c];
 #pragma unroll
       for (int r = 0; r < 3; ++r) {
@@ -564,7 +564,7 @@ __global__ void __launch_bounds__(NT) k_adj_sl(Geo G, double dt, double3 dt_h, A
   double* tv[3] = {A.LV[0], A.LV[1], A.LV[2]};
   const double dth[3] = {dt_h.x, dt_h.y, dt_h.z};
   for (int k = k0; k < k1; ++k) {
-    const long long c = ((long long)k * G.ny + j) * G.nx + i;
+    const int c = (k * G.ny + j) * G.nx + i;
     const double v0[3] = {T.v[0][c], T.v[1][c], T.v[2][c]};
     Cub Cs, Cx;
     cub_setup(Cs, G, i - v0[0] * dth[0], j - v0[1] * dth[1], k - v0[2] * dth[2]);
@@ -628,7 +628,7 @@ __global__ void __launch_bounds__(NT) k_adj_div(Geo G, AdjView A) {
   const int k0 = blockIdx.z * G.zc, k1 = min(G.nz, k0 + G.zc);
   for (int k = k0; k < k1; ++k) {
     const Nbr nb = make_nbr(G, i, j, k);
-    const long long c = nb.at(0, 0, 0);
+    const int c = nb.at(0, 0, 0);
     A.lam.v[0][c] = A.LV[0][c] - (A.LDEL[nb.at(1, 0, 0)] - A.LDEL[nb.at(-1, 0, 0)]) * G.inv2h[0];
     A.lam.v[1][c] = A.LV[1][c] - (A.LDEL[nb.at(0, 1, 0)] - A.LDEL[nb.at(0, -1, 0)]) * G.inv2h[1];
     A.lam.v[2][c] = A.LV[2][c] - (A.LDEL[nb.at(0, 0, 1)] - A.LDEL[nb.at(0, 0, -1)]) * G.inv2h[2];
@@ -643,7 +643,7 @@ int flat_blocks(long long n) {
 }  // namespace
 
 cudaError_t launch_adj_prep(const Geo& G, const AdjView& A, double inv_dt, cudaStream_t st) {
-  k_adj_prep<<<flat_blocks(G.nvox), NT, 0, st>>>(G.nvox, A, inv_dt);
+  launch(k_adj_prep, flat_blocks(G.nvox), NT, 0, st, G.nvox, A, inv_dt);
   return cudaGetLastError();
 }
 
@@ -651,37 +651,37 @@ cudaError_t launch_adj_elas_coef(const Geo& G, const DevParams& P, const AdjView
                                  const double* mu, const double* lam, const double* p,
                                  const double* n, double inv_Escale, bool species,
                                  cudaStream_t st) {
-  k_adj_elas_coef<<<G.grid, dim3(BX, BY), 0, st>>>(G, P, A, mu, lam, p, n, inv_Escale,
-                                                   species ? 1 : 0);
+  launch(k_adj_elas_coef, G.grid, dim3(BX, BY), 0, st, G, P, A, mu, lam, p, n, inv_Escale,
+         species ? 1 : 0);
   return cudaGetLastError();
 }
 
 cudaError_t launch_adj_react(const Geo& G, const DevParams& P, double dt, const AdjView& A,
                              const TapeView& T, const double* rho, cudaStream_t st) {
-  k_adj_react<<<G.grid, dim3(BX, BY), 0, st>>>(G, P, dt, A, T, rho);
+  launch(k_adj_react, G.grid, dim3(BX, BY), 0, st, G, P, dt, A, T, rho);
   return cudaGetLastError();
 }
 
 cudaError_t launch_cn_init_rhs(const Geo& G, const Cn3& C, const AdjView& A, cudaStream_t st) {
-  k_cn_init_rhs<<<G.grid, dim3(BX, BY), 0, st>>>(G, C, A);
+  launch(k_cn_init_rhs, G.grid, dim3(BX, BY), 0, st, G, C, A);
   return cudaGetLastError();
 }
 
 cudaError_t launch_adj_cn_post(const Geo& G, const DevParams& P, double dt, const AdjView& A,
                                const TapeView& T, cudaStream_t st) {
-  k_adj_cn_post<<<G.grid, dim3(BX, BY), 0, st>>>(G, P, 0.5 * dt, A, T);
+  launch(k_adj_cn_post, G.grid, dim3(BX, BY), 0, st, G, P, 0.5 * dt, A, T);
   return cudaGetLastError();
 }
 
 cudaError_t launch_adj_sl(const Geo& G, double dt, const AdjView& A, const TapeView& T,
                           const double* div, cudaStream_t st) {
   const double3 dth = make_double3(dt / G.h[0], dt / G.h[1], dt / G.h[2]);
-  k_adj_sl<<<G.grid, dim3(BX, BY), 0, st>>>(G, dt, dth, A, T, div);
+  launch(k_adj_sl, G.grid, dim3(BX, BY), 0, st, G, dt, dth, A, T, div);
   return cudaGetLastError();
 }
 
 cudaError_t launch_adj_div(const Geo& G, const AdjView& A, cudaStream_t st) {
-  k_adj_div<<<G.grid, dim3(BX, BY), 0, st>>>(G, A);
+  launch(k_adj_div, G.grid, dim3(BX, BY), 0, st, G, A);
   return cudaGetLastError();
 }
 

@@ -726,7 +726,7 @@ bool cn_df_ok(const tg_ctx* X) {
 // mask: bit r set for the fields this call solves (the others are left untouched)
 tg_status cn_solve3(tg_ctx* X, tg_stats* stats, int mask = 7) {
   const Cn3 C = cn_view(X);
-  k_cg_reset<<<1, 32, 0, X->stream>>>(X->scal, 3, X->prm.rtol_diff, X->prm.maxit_diff);
+  launch(k_cg_reset, 1, 32, 0, X->stream, X->scal, 3, X->prm.rtol_diff, X->prm.maxit_diff);
   CK(cudaGetLastError());
   CK(launch_cn_init(X->G, C, X->stream, mask));
   X->launches += 2;
@@ -794,7 +794,7 @@ tg_status cn_solve3_mixed(tg_ctx* X, tg_stats* stats, int mask) {
   if (nslot <= 2)
     for (int q = 0; q < nslot; ++q) I.z[slot[q]] = X->b32[B_PB0 + slot[q]];
   const long long cap = (long long)X->G.nblocks * MAX_NV;
-  k_cg_reset<<<1, 32, 0, X->stream>>>(X->scal, 3, X->prm.rtol_diff, X->prm.maxit_diff);
+  launch(k_cg_reset, 1, 32, 0, X->stream, X->scal, 3, X->prm.rtol_diff, X->prm.maxit_diff);
   CK(cudaGetLastError());
   X->launches += 1;
   int inner_total[3] = {0, 0, 0};
@@ -919,7 +919,7 @@ tg_status ox_begin(tg_ctx* X) {
   CK(cudaStreamWaitEvent(so, X->fork_ev, 0));
   if (X->host_in) CK(cudaStreamWaitEvent(so, X->up_ev[2], 0));   // o is up (tg_step_host)
   X->ox_running = true;
-  k_cg_reset<<<1, 32, 0, so>>>(P.dev, P.ns, X->prm.rtol_diff, X->prm.maxit_diff);
+  launch(k_cg_reset, 1, 32, 0, so, P.dev, P.ns, X->prm.rtol_diff, X->prm.maxit_diff);
   CK(cudaGetLastError());
   CK(P.df ? launch_ox_start(X->G, P.O, so) : launch_cn_init(X->G, P.C, so, MASK_O));
   X->ox_chunk = first_chunk(X->prev_it_diff);
@@ -1028,7 +1028,7 @@ tg_status elas_solve_mixed(tg_ctx* X, double* const u[3], double* const b_ext[3]
   } else {
     for (int d = 0; d < 3; ++d) CK(cudaMemsetAsync(E.du[d], 0, bytes, X->stream));
   }
-  k_cg_reset<<<1, 32, 0, X->stream>>>(Sout, 1, X->prm.rtol_elas, X->prm.maxit_elas);
+  launch(k_cg_reset, 1, 32, 0, X->stream, Sout, 1, X->prm.rtol_elas, X->prm.maxit_elas);
   CK(cudaGetLastError());
   // with the double-FP32 residual the node coefficients came with the faces, and the
   // extrapolation wrote the pairs of a step's starting u; otherwise u is packed here
@@ -1108,7 +1108,7 @@ tg_status elas_solve(tg_ctx* X, double* const u[3], double* const b_ext[3], bool
   if (X->prec == TG_MIXED) return elas_solve_mixed(X, u, b_ext, minus_b, inv_dt, stats);
   const Elas E = elas_view(X, u, b_ext);
   const bool spec = spectral_on(X);
-  k_cg_reset<<<1, 32, 0, X->stream>>>(X->scal + 3, 1, X->prm.rtol_elas, X->prm.maxit_elas);
+  launch(k_cg_reset, 1, 32, 0, X->stream, X->scal + 3, 1, X->prm.rtol_elas, X->prm.maxit_elas);
   CK(cudaGetLastError());
   const double* const r64[3] = {E.r[0], E.r[1], E.r[2]};
   if (inv_dt > 0.0) {   // a step's solve: start from u extrapolated in time
@@ -1484,7 +1484,7 @@ tg_status do_adjoint_step(tg_ctx* X, double dt, const void* tape, const tg_state
   {
     Cn3 C = cn_view(X);
     for (int r = 0; r < 3; ++r) C.x[r] = A.phi[r];
-    k_cg_reset<<<1, 32, 0, s>>>(X->scal, 3, X->prm.rtol_diff, X->prm.maxit_diff);
+    launch(k_cg_reset, 1, 32, 0, s, X->scal, 3, X->prm.rtol_diff, X->prm.maxit_diff);
     CK(cudaGetLastError());
     CK(launch_cn_init_rhs(G, C, A, s));
     X->launches += 2;

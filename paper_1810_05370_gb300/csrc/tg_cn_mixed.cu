@@ -25,7 +25,7 @@ __global__ void __launch_bounds__(NT) k_cn_ir_residual(Geo G, Cn3 C, Cn32 I, CgS
     const int k0 = blockIdx.z * G.zc, k1 = min(G.nz, k0 + G.zc);
     for (int k = k0; k < k1; ++k) {
       const Nbr nb = make_nbr(G, i, j, k);
-      const long long c = nb.at(0, 0, 0);
+      const int c = nb.at(0, 0, 0);
       const Faces F = load_faces(C, nb, c);
       const float di = I.dinv[c];
 #pragma unroll
@@ -82,8 +82,8 @@ __global__ void __launch_bounds__(NT) k_cn_ir_residual_df(Geo G, Cn3 C, Cn32 I, 
     const int k0 = blockIdx.z * G.zc, k1 = min(G.nz, k0 + G.zc);
     for (int k = k0; k < k1; ++k) {
       const Nbr nb = make_nbr(G, i, j, k);
-      const long long c = nb.at(0, 0, 0);
-      const long long nbr[6] = {nb.at(1, 0, 0), nb.at(-1, 0, 0), nb.at(0, 1, 0),
+      const int c = nb.at(0, 0, 0);
+      const int nbr[6] = {nb.at(1, 0, 0), nb.at(-1, 0, 0), nb.at(0, 1, 0),
                                 nb.at(0, -1, 0), nb.at(0, 0, 1), nb.at(0, 0, -1)};
       const Df f[6] = {df_of(C.Kfdf[0][c]), df_of(C.Kfdf[0][nbr[1]]), df_of(C.Kfdf[1][c]),
                        df_of(C.Kfdf[1][nbr[3]]), df_of(C.Kfdf[2][c]), df_of(C.Kfdf[2][nbr[5]])};
@@ -162,8 +162,8 @@ __global__ void __launch_bounds__(NT) k_cn32_matvec(Geo G, Cn32 I) {
     const int k0 = blockIdx.z * G.zc, k1 = min(G.nz, k0 + G.zc);
     for (int k = k0; k < k1; ++k) {
       const Nbr nb = make_nbr(G, i, j, k);
-      const long long c = nb.at(0, 0, 0);
-      const long long xp = nb.at(1, 0, 0), xm = nb.at(-1, 0, 0), yp = nb.at(0, 1, 0),
+      const int c = nb.at(0, 0, 0);
+      const int xp = nb.at(1, 0, 0), xm = nb.at(-1, 0, 0), yp = nb.at(0, 1, 0),
                       ym = nb.at(0, -1, 0), zp = nb.at(0, 0, 1), zm = nb.at(0, 0, -1);
       const float fxp = __ldg(I.Kf[0] + c), fxm = __ldg(I.Kf[0] + xm);
       const float fyp = __ldg(I.Kf[1] + c), fym = __ldg(I.Kf[1] + ym);
@@ -234,8 +234,6 @@ __global__ void __launch_bounds__(MV_CELLS, 2) k_cn32_matvec_neu(Geo G, Cn32 I, 
   }
   __shared__ float sp[2][2][MV_CELLS];   // p of the step's plane: [step parity][solve][cell]
   __shared__ float sfy[2][MV_CELLS];     // the y face above each cell, same planes
-  __shared__ double red[MV_CELLS / 32][2];
-  __shared__ bool last;
   const int tx = threadIdx.x, ty = threadIdx.y, cell = ty * MV_X + tx;
   const int iu = blockIdx.x * MV_OX - 1 + tx, ju = blockIdx.y * MV_OY - 1 + ty;   // unwrapped
   const int gx = ((iu % G.nx) + G.nx) % G.nx, gy = ((ju % G.ny) + G.ny) % G.ny;
@@ -319,52 +317,16 @@ __global__ void __launch_bounds__(MV_CELLS, 2) k_cn32_matvec_neu(Geo G, Cn32 I, 
     buf ^= 1;
   }
 
-  // <p, q> per solve: warps, then the block's warps in order, then the blocks in order by the
-  // last block to finish
-  const int lane = cell & 31, warp = cell >> 5, nb = gridDim.x * gridDim.y * gridDim.z;
+  double sums[2] = {(double)part[0], (double)part[1]}, tot[2];
+  const int nb = gridDim.x * gridDim.y * gridDim.z;
   const int b = (blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
+  if (reduce_items<2, MV_CELLS>(sums, I.partial, I.counter, cell, b, nb, tot) && cell == 0) {
 #pragma unroll
-  for (int q = 0; q < 2; ++q) {
-    const double v = warp_sum((double)part[q]);
-    if (lane == 0) red[warp][q] = v;
-  }
-  __syncthreads();
-  if (cell == 0) {
-#pragma unroll
-    for (int q = 0; q < 2; ++q) {
-      double v = 0.0;
-      for (int w = 0; w < MV_CELLS / 32; ++w) v += red[w][q];
-      I.partial[2 * (size_t)b + q] = v;
-    }
-    __threadfence();
-    last = atomicAdd(I.counter, 1u) == (unsigned int)(nb - 1);
-  }
-  __syncthreads();
-  if (!last) return;
-  __threadfence();
-  double tot[2] = {0.0, 0.0};
-  for (int k = cell; k < nb; k += MV_CELLS) {
-#pragma unroll
-    for (int q = 0; q < 2; ++q) tot[q] += __ldcg(I.partial + 2 * (size_t)k + q);
-  }
-  __syncthreads();
-#pragma unroll
-  for (int q = 0; q < 2; ++q) {
-    const double v = warp_sum(tot[q]);
-    if (lane == 0) red[warp][q] = v;
-  }
-  __syncthreads();
-  if (cell == 0) {
-#pragma unroll
-    for (int q = 0; q < 2; ++q) {
-      double v = 0.0;
-      for (int w = 0; w < MV_CELLS / 32; ++w) v += red[w][q];
+    for (int q = 0; q < 2; ++q)
       if (run[q]) {
-        I.S[ld[q]].pq = v;
-        I.S[ld[q]].alpha = I.S[ld[q]].rz / v;
+        I.S[ld[q]].pq = tot[q];
+        I.S[ld[q]].alpha = I.S[ld[q]].rz / tot[q];
       }
-    }
-    *I.counter = 0u;
   }
 }
 
@@ -520,8 +482,6 @@ constexpr int NM_CELLS = NM_X * NM_Y;
 struct NmTile {
   float2 y[3][2][NM_CELLS];     // terms 0..2 of the two solves: [term][plane parity][cell]
   float ay[4][NM_CELLS];        // y faces of the last four planes (index plane & 3)
-  double red[NM_CELLS / 32][2];
-  bool last;
 };
 
 __global__ void __launch_bounds__(NM_CELLS, 1) k_cn32_neumann(Geo G, Cn32 I, int r0, int r1,
@@ -694,49 +654,13 @@ __global__ void __launch_bounds__(NM_CELLS, 1) k_cn32_neumann(Geo G, Cn32 I, int
     }
   }
 
-  // <r, z> per solve: warps, then the block's warps in order, then the blocks in order by the
-  // last block to finish
-  const int lane = cell & 31, warp = cell >> 5, nb = gridDim.x * gridDim.y * gridDim.z;
+  double sums[2] = {(double)acc[0], (double)acc[1]}, tot[2];
+  const int nb = gridDim.x * gridDim.y * gridDim.z;
   const int b = (blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
+  if (reduce_items<2, NM_CELLS>(sums, I.partial, I.counter, cell, b, nb, tot) && cell == 0) {
 #pragma unroll
-  for (int q = 0; q < 2; ++q) {
-    const double v = warp_sum((double)acc[q]);
-    if (lane == 0) T.red[warp][q] = v;
-  }
-  __syncthreads();
-  if (cell == 0) {
-#pragma unroll
-    for (int q = 0; q < 2; ++q) {
-      double v = 0.0;
-      for (int w = 0; w < NM_CELLS / 32; ++w) v += T.red[w][q];
-      I.partial[2 * (size_t)b + q] = v;
-    }
-    __threadfence();
-    T.last = atomicAdd(I.counter, 1u) == (unsigned int)(nb - 1);
-  }
-  __syncthreads();
-  if (!T.last) return;
-  __threadfence();
-  double tot[2] = {0.0, 0.0};
-  for (int k = cell; k < nb; k += NM_CELLS) {
-#pragma unroll
-    for (int q = 0; q < 2; ++q) tot[q] += __ldcg(I.partial + 2 * (size_t)k + q);
-  }
-  __syncthreads();
-#pragma unroll
-  for (int q = 0; q < 2; ++q) {
-    const double v = warp_sum(tot[q]);
-    if (lane == 0) T.red[warp][q] = v;
-  }
-  __syncthreads();
-  if (cell == 0) {
-#pragma unroll
-    for (int q = 0; q < 2; ++q) {
-      double v = 0.0;
-      for (int w = 0; w < NM_CELLS / 32; ++w) v += T.red[w][q];
-      if (run[q]) cg_after_precond(I.S[ld[q]], v);
-    }
-    *I.counter = 0u;
+    for (int q = 0; q < 2; ++q)
+      if (run[q]) cg_after_precond(I.S[ld[q]], tot[q]);
   }
 }
 
@@ -768,12 +692,12 @@ cudaError_t launch_cn_ir_residual(const Geo& G, const Cn3& C, const Cn32& I, CgS
                                   cudaStream_t st) {
   if (C.df)
     TG_TIMED(K_CN_IR_RESIDUAL_DF, st,
-             k_cn_ir_residual_df<<<G.grid, dim3(BX, BY), 0, st>>>(G, C, I, Sout, init ? 1 : 0, tau_min,
-                                                                  max_sweeps, mask));
+             launch(k_cn_ir_residual_df, G.grid, dim3(BX, BY), 0, st, G, C, I, Sout, init ? 1 : 0,
+                    tau_min, max_sweeps, mask));
   else
     TG_TIMED(K_CN_IR_RESIDUAL, st,
-             k_cn_ir_residual<<<G.grid, dim3(BX, BY), 0, st>>>(G, C, I, Sout, init ? 1 : 0, tau_min,
-                                                               max_sweeps, mask));
+             launch(k_cn_ir_residual, G.grid, dim3(BX, BY), 0, st, G, C, I, Sout, init ? 1 : 0,
+                    tau_min, max_sweeps, mask));
   return cudaGetLastError();
 }
 
@@ -782,9 +706,10 @@ cudaError_t launch_cn_ir_residual(const Geo& G, const Cn3& C, const Cn32& I, CgS
 cudaError_t launch_cn32_iter(const Geo& G, const Cn32& I, cudaStream_t st, int r0, int r1,
                              long long partial_capacity) {
   if (I.z[0] == nullptr && I.z[1] == nullptr && I.z[2] == nullptr) {
-    TG_TIMED(K_CN32_PUPDATE, st, k_cn32_pupdate<false><<<flat_blocks(G), NT, 0, st>>>(G.nvox, I));
-    TG_TIMED(K_CN32_MATVEC, st, k_cn32_matvec<<<G.grid, dim3(BX, BY), 0, st>>>(G, I));
-    TG_TIMED(K_CN32_UPDATE, st, k_cn32_update<false><<<flat_blocks(G), NT, 0, st>>>(G.nvox, I));
+    TG_TIMED(K_CN32_PUPDATE, st, launch(k_cn32_pupdate<false>, flat_blocks(G), NT, 0, st, G.nvox,
+                                        I));
+    TG_TIMED(K_CN32_MATVEC, st, launch(k_cn32_matvec, G.grid, dim3(BX, BY), 0, st, G, I));
+    TG_TIMED(K_CN32_UPDATE, st, launch(k_cn32_update<false>, flat_blocks(G), NT, 0, st, G.nvox, I));
     return cudaGetLastError();
   }
   // z chunk: 32 planes, more while the blocks' two partial sums would not fit the buffer
@@ -796,8 +721,8 @@ cudaError_t launch_cn32_iter(const Geo& G, const Cn32& I, cudaStream_t st, int r
   if (gx * gy * gz * 2 > partial_capacity || r0 < 0) return cudaErrorInvalidValue;
   if (G.nvox >= (1LL << 31)) return cudaErrorInvalidValue;   // 32-bit offsets below
   TG_TIMED(K_CN32_NEUMANN, st,
-           k_cn32_neumann<<<dim3((unsigned)gx, (unsigned)gy, (unsigned)gz), dim3(NM_X, NM_Y), 0,
-                            st>>>(G, I, r0, r1, zc));
+           launch(k_cn32_neumann, dim3((unsigned)gx, (unsigned)gy, (unsigned)gz), dim3(NM_X, NM_Y),
+                  0, st, G, I, r0, r1, zc));
   // the operator's grid: about as many blocks as the standard one, each block's two sums in
   // the partial buffer
   const long long mgx = (G.nx + MV_OX - 1) / MV_OX, mgy = (G.ny + MV_OY - 1) / MV_OY;
@@ -809,15 +734,16 @@ cudaError_t launch_cn32_iter(const Geo& G, const Cn32& I, cudaStream_t st, int r
   mgz = (G.nz + mzc - 1) / mzc;
   if (mgx * mgy * mgz * 2 > partial_capacity) return cudaErrorInvalidValue;
   TG_TIMED(K_CN32_MATVEC, st,
-           k_cn32_matvec_neu<<<dim3((unsigned)mgx, (unsigned)mgy, (unsigned)mgz),
-                               dim3(MV_X, MV_Y), 0, st>>>(G, I, r0, r1, mzc));
-  TG_TIMED(K_CN32_UPDATE, st, k_cn32_update<true><<<flat_blocks(G), NT, 0, st>>>(G.nvox, I));
+           launch(k_cn32_matvec_neu, dim3((unsigned)mgx, (unsigned)mgy, (unsigned)mgz), dim3(MV_X,
+                  MV_Y), 0, st, G, I, r0, r1, mzc));
+  TG_TIMED(K_CN32_UPDATE, st, launch(k_cn32_update<true>, flat_blocks(G), NT, 0, st, G.nvox, I));
   return cudaGetLastError();
 }
 
 cudaError_t launch_cn_ir_correct(const Geo& G, const Cn3& C, const Cn32& I, int mask,
                                  cudaStream_t st) {
-  TG_TIMED(K_CN_IR_CORRECT, st, k_cn_ir_correct<<<flat_blocks(G), NT, 0, st>>>(G.nvox, C, I, mask));
+  TG_TIMED(K_CN_IR_CORRECT, st, launch(k_cn_ir_correct, flat_blocks(G), NT, 0, st, G.nvox, C, I,
+                                       mask));
   return cudaGetLastError();
 }
 

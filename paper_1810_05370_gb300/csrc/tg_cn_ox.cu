@@ -20,8 +20,8 @@
 namespace tg {
 namespace {
 
-__device__ __forceinline__ Df ld_df(const float2* a, long long i) { return df_of(a[i]); }
-__device__ __forceinline__ void st_df(float2* a, long long i, Df v) {
+__device__ __forceinline__ Df ld_df(const float2* a, int i) { return df_of(a[i]); }
+__device__ __forceinline__ void st_df(float2* a, int i, Df v) {
   a[i] = make_float2(v.hi, v.lo);
 }
 __device__ __forceinline__ Df df_scale2(Df x) { return {2.0f * x.hi, 2.0f * x.lo}; }   // exact
@@ -42,7 +42,7 @@ __device__ __forceinline__ void df_acc(Df (&acc)[NV], int q, Df v) { acc[q] = df
 struct FacesDf {
   Df xp, xm, yp, ym, zp, zm;
 };
-__device__ __forceinline__ FacesDf faces_df(const OxDf& O, const Nbr& nb, long long c) {
+__device__ __forceinline__ FacesDf faces_df(const OxDf& O, const Nbr& nb, int c) {
   FacesDf F;
   F.xp = ld_df(O.Kf[0], c);
   F.xm = ld_df(O.Kf[0], nb.at(-1, 0, 0));
@@ -69,7 +69,7 @@ __global__ void __launch_bounds__(NT) k_ox_prep(Geo G, OxDf O) {
   const int k0 = blockIdx.z * G.zc, k1 = min(G.nz, k0 + G.zc);
   for (int k = k0; k < k1; ++k) {
     const Nbr nb = make_nbr(G, i, j, k);
-    const long long c = nb.at(0, 0, 0);
+    const int c = nb.at(0, 0, 0);
     const FacesDf F = faces_df(O, nb, c);
     // d = 1 + (xp + xm) + (yp + ym) + (zp + zm), the FP64 diagonal's order
     Df d = df_add(df_add(df_add(Df{1.0f, 0.0f}, df_add(F.xp, F.xm)), df_add(F.yp, F.ym)),
@@ -90,7 +90,7 @@ __global__ void __launch_bounds__(NT) k_ox_init(Geo G, OxDf O) {
     const int k0 = blockIdx.z * G.zc, k1 = min(G.nz, k0 + G.zc);
     for (int k = k0; k < k1; ++k) {
       const Nbr nb = make_nbr(G, i, j, k);
-      const long long c = nb.at(0, 0, 0);
+      const int c = nb.at(0, 0, 0);
       const FacesDf F = faces_df(O, nb, c);
       const Df xc = ld_df(O.x, c);
       Df s = df_mul(F.xp, df_sub(ld_df(O.x, nb.at(1, 0, 0)), xc));
@@ -124,7 +124,7 @@ __global__ void __launch_bounds__(NT) k_ox_matvec(Geo G, OxDf O) {
     const int k0 = blockIdx.z * G.zc, k1 = min(G.nz, k0 + G.zc);
     for (int k = k0; k < k1; ++k) {
       const Nbr nb = make_nbr(G, i, j, k);
-      const long long c = nb.at(0, 0, 0);
+      const int c = nb.at(0, 0, 0);
       const FacesDf F = faces_df(O, nb, c);
       const Df pc = ld_df(O.p, c);
       Df off = df_mul(F.xp, ld_df(O.p, nb.at(1, 0, 0)));
@@ -155,7 +155,7 @@ __global__ void __launch_bounds__(NT) k_ox_update(Geo G, OxDf O) {
   if (i < G.nx && j < G.ny) {
     const int k0 = blockIdx.z * G.zc, k1 = min(G.nz, k0 + G.zc);
     for (int k = k0; k < k1; ++k) {
-      const long long c = ((long long)k * G.ny + j) * G.nx + i;
+      const int c = (k * G.ny + j) * G.nx + i;
       st_df(O.x, c, df_add(ld_df(O.x, c), df_mul(a, ld_df(O.p, c))));
       const Df r = df_sub(ld_df(O.r, c), df_mul(a, ld_df(O.q, c)));
       st_df(O.r, c, r);
@@ -177,7 +177,7 @@ __global__ void __launch_bounds__(NT) k_ox_pupdate(Geo G, OxDf O) {
   if (i >= G.nx || j >= G.ny) return;
   const int k0 = blockIdx.z * G.zc, k1 = min(G.nz, k0 + G.zc);
   for (int k = k0; k < k1; ++k) {
-    const long long c = ((long long)k * G.ny + j) * G.nx + i;
+    const int c = (k * G.ny + j) * G.nx + i;
     st_df(O.p, c, df_add(df_mul(ld_df(O.di, c), ld_df(O.r, c)), df_mul(b, ld_df(O.p, c))));
   }
 }
@@ -190,7 +190,7 @@ __global__ void __launch_bounds__(NT) k_ox_finish(Geo G, OxDf O) {
   if (i >= G.nx || j >= G.ny) return;
   const int k0 = blockIdx.z * G.zc, k1 = min(G.nz, k0 + G.zc);
   for (int k = k0; k < k1; ++k) {
-    const long long c = ((long long)k * G.ny + j) * G.nx + i;
+    const int c = (k * G.ny + j) * G.nx + i;
     O.o[c] = zero ? 0.0 : df_value(ld_df(O.x, c));
   }
 }
@@ -198,20 +198,20 @@ __global__ void __launch_bounds__(NT) k_ox_finish(Geo G, OxDf O) {
 }  // namespace
 
 cudaError_t launch_ox_start(const Geo& G, const OxDf& O, cudaStream_t st) {
-  TG_TIMED(K_OX_PREP, st, k_ox_prep<<<G.grid, dim3(BX, BY), 0, st>>>(G, O));
-  TG_TIMED(K_OX_INIT, st, k_ox_init<<<G.grid, dim3(BX, BY), 0, st>>>(G, O));
+  TG_TIMED(K_OX_PREP, st, launch(k_ox_prep, G.grid, dim3(BX, BY), 0, st, G, O));
+  TG_TIMED(K_OX_INIT, st, launch(k_ox_init, G.grid, dim3(BX, BY), 0, st, G, O));
   return cudaGetLastError();
 }
 
 cudaError_t launch_ox_iter(const Geo& G, const OxDf& O, cudaStream_t st) {
-  TG_TIMED(K_OX_MATVEC, st, k_ox_matvec<<<G.grid, dim3(BX, BY), 0, st>>>(G, O));
-  TG_TIMED(K_OX_UPDATE, st, k_ox_update<<<G.grid, dim3(BX, BY), 0, st>>>(G, O));
-  TG_TIMED(K_OX_PUPDATE, st, k_ox_pupdate<<<G.grid, dim3(BX, BY), 0, st>>>(G, O));
+  TG_TIMED(K_OX_MATVEC, st, launch(k_ox_matvec, G.grid, dim3(BX, BY), 0, st, G, O));
+  TG_TIMED(K_OX_UPDATE, st, launch(k_ox_update, G.grid, dim3(BX, BY), 0, st, G, O));
+  TG_TIMED(K_OX_PUPDATE, st, launch(k_ox_pupdate, G.grid, dim3(BX, BY), 0, st, G, O));
   return cudaGetLastError();
 }
 
 cudaError_t launch_ox_finish(const Geo& G, const OxDf& O, cudaStream_t st) {
-  TG_TIMED(K_OX_FINISH, st, k_ox_finish<<<G.grid, dim3(BX, BY), 0, st>>>(G, O));
+  TG_TIMED(K_OX_FINISH, st, launch(k_ox_finish, G.grid, dim3(BX, BY), 0, st, G, O));
   return cudaGetLastError();
 }
 

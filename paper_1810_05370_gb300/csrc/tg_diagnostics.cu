@@ -47,7 +47,7 @@ __global__ void __launch_bounds__(NT) k_diagnostics(Geo G, DiagArgs A) {
     const int k0 = blockIdx.z * G.zc, k1 = min(G.nz, k0 + G.zc);
     for (int k = k0; k < k1; ++k) {
       const Nbr nb = make_nbr(G, i, j, k);
-      const long long c = nb.at(0, 0, 0);
+      const int c = nb.at(0, 0, 0);
       double D[3][3];   // D[a][d] = d u_a / d x_d
 #pragma unroll
       for (int a = 0; a < 3; ++a) {
@@ -145,7 +145,7 @@ __global__ void __launch_bounds__(NT) k_diagnostics(Geo G, DiagArgs A) {
 }  // namespace
 
 cudaError_t launch_diagnostics(const Geo& G, const DiagArgs& A, cudaStream_t st) {
-  k_diagnostics<<<G.grid, dim3(BX, BY), 0, st>>>(G, A);
+  launch(k_diagnostics, G.grid, dim3(BX, BY), 0, st, G, A);
   return cudaGetLastError();
 }
 

@@ -7,6 +7,8 @@
 //   (A c)_j = c_j + sum_d [ a_d,j (c_j - c_{j+e_d}) + a_d,j-e_d (c_j - c_{j-e_d}) ].
 // The three right-hand sides share the coefficient reads: every kernel below streams the
 // six face values of a node once and applies them to all active solves.
+#include <algorithm>
+
 #include "tg_tiles.cuh"
 
 namespace tg {
@@ -39,7 +41,7 @@ __global__ void __launch_bounds__(NT) k_diff_faces(Geo G, DevParams P, double ha
   for (int k = k0; k < k1; ++k) {
     const Nbr nb = make_nbr(G, i, j, k);
     auto K = [&](long long e) { return node_K(P, g[e], w[e], f[e]); };
-    const long long c = nb.at(0, 0, 0);
+    const int c = nb.at(0, 0, 0);
     const double kc = K(c);
     const double fx = sx * harmonic(kc, K(nb.at(1, 0, 0)));
     const double fy = sy * harmonic(kc, K(nb.at(0, 1, 0)));
@@ -75,7 +77,7 @@ __global__ void __launch_bounds__(NT) k_diff_node_df(Geo G, DevParams P,
   const Df ks = df_split(P.k_scale), rg = df_split(P.rho_g), rw = df_split(P.rho_w);
   const int k0 = blockIdx.z * G.zc, k1 = min(G.nz, k0 + G.zc);
   for (int k = k0; k < k1; ++k) {
-    const long long c = ((long long)k * G.ny + j) * G.nx + i;
+    const int c = (k * G.ny + j) * G.nx + i;
     const Df gc = df_split(g[c]), wc = df_split(w[c]);
     // node_K's order: k_scale ((k_g g + k_w w) + k_f f), clamped at 0
     Df K = df_mul(ks, df_add(df_add(df_mul(kg, gc), df_mul(kw, wc)), df_mul(kf, df_split(f[c]))));
@@ -109,7 +111,7 @@ __global__ void __launch_bounds__(NT) k_diff_faces_df(Geo G, Df sx, Df sy, Df sz
   const int k0 = blockIdx.z * G.zc, k1 = on ? min(G.nz, k0 + G.zc) : k0;
   for (int k = k0; k < k1; ++k) {
     const Nbr nb = make_nbr(G, i, j, k);
-    const long long c = nb.at(0, 0, 0);
+    const int c = nb.at(0, 0, 0);
     auto K = [&](long long e) { return df_of(__ldg(Kn + e)); };
     const Df kc = K(c);
     const Df fxp = df_mul(sx, df_harmonic(kc, K(nb.at(1, 0, 0))));
@@ -154,7 +156,7 @@ __global__ void __launch_bounds__(NT) k_diff_diag(Geo G, const double* __restric
   const int k0 = blockIdx.z * G.zc, k1 = min(G.nz, k0 + G.zc);
   for (int k = k0; k < k1; ++k) {
     const Nbr nb = make_nbr(G, i, j, k);
-    const long long c = nb.at(0, 0, 0);
+    const int c = nb.at(0, 0, 0);
     const double d = 1.0 + (Kfx[c] + Kfx[nb.at(-1, 0, 0)]) + (Kfy[c] + Kfy[nb.at(0, -1, 0)]) +
                      (Kfz[c] + Kfz[nb.at(0, 0, -1)]);
     dsum[c] = d;
@@ -202,41 +204,70 @@ __global__ void __launch_bounds__(NT) k_cn_matvec(Geo G, Cn3 C) {
   }
 }
 
-__global__ void __launch_bounds__(NT) k_cn_update(Geo G, Cn3 C) {
-  bool act[3];
-  double alpha[3];
-  bool any = false;
-#pragma unroll
-  for (int r = 0; r < 3; ++r) {
-    act[r] = C.S[r].status == CG_RUNNING;
-    alpha[r] = C.S[r].alpha;
-    any |= act[r];
+// x += alpha p, r -= alpha q and the p-update, flat over voxel pairs; blockIdx.y is the solve.
+// Each solve's blocks reduce among themselves (its own counter and stretch of the partials) and
+// their last block takes its decision, so a finished solve's blocks leave at once.  Bound by
+// the FP64 pipe (5 operations per voxel and solve) and HBM alike.
+__global__ void __launch_bounds__(NT) k_cn_update(long long n, Cn3 C) {
+  const int s = blockIdx.y;
+  if (C.S[s].status != CG_RUNNING) return;
+  const double alpha = C.S[s].alpha;
+  double* __restrict__ x = C.x[s];
+  double* __restrict__ r = C.r[s];
+  const double* __restrict__ p = C.p[s];
+  const double* __restrict__ q = C.q[s];
+  const double* __restrict__ di = C.dinv;
+  double acc[2] = {0.0, 0.0};
+  auto one = [&](double& xv, double& res, double pv, double qv, double dv) {
+    xv = fma(alpha, pv, xv);
+    res = fma(-alpha, qv, res);
+    acc[0] = fma(res, dv * res, acc[0]);
+    acc[1] = fma(res, res, acc[1]);
+  };
+  const long long pairs = n / 2, gs = (long long)gridDim.x * NT;
+  for (long long v = (long long)blockIdx.x * NT + threadIdx.x; v < pairs; v += gs) {
+    double2 xv = reinterpret_cast<double2*>(x)[v], rv = reinterpret_cast<double2*>(r)[v];
+    const double2 pv = reinterpret_cast<const double2*>(p)[v];
+    const double2 qv = reinterpret_cast<const double2*>(q)[v];
+    const double2 dv = reinterpret_cast<const double2*>(di)[v];
+    one(xv.x, rv.x, pv.x, qv.x, dv.x);
+    one(xv.y, rv.y, pv.y, qv.y, dv.y);
+    reinterpret_cast<double2*>(x)[v] = xv;
+    reinterpret_cast<double2*>(r)[v] = rv;
   }
-  if (!any) return;
-  double acc[6];
-#pragma unroll
-  for (int q = 0; q < 6; ++q) acc[q] = 0.0;
-  cn_update_tile(G, C, act, alpha, blockIdx.x, blockIdx.y, blockIdx.z, acc);
-  double out[6];
-  if (reduce_last_block<6>(acc, C.partial, C.counter, out) && threadIdx.x == 0 && threadIdx.y == 0) {
-#pragma unroll
-    for (int r = 0; r < 3; ++r)
-      if (act[r]) cg_after_update(C.S[r], out[2 * r], out[2 * r + 1]);
-  }
+  if ((n & 1) && blockIdx.x == 0 && threadIdx.x == 0)
+    one(x[n - 1], r[n - 1], p[n - 1], q[n - 1], di[n - 1]);
+  double out[2];
+  if (reduce_indexed<2>(acc, C.partial + (size_t)s * gridDim.x * 2, C.counter + s, blockIdx.x,
+                        gridDim.x, out) &&
+      threadIdx.x == 0)
+    cg_after_update(C.S[s], out[0], out[1]);
 }
 
-__global__ void __launch_bounds__(NT) k_cn_pupdate(Geo G, Cn3 C) {
-  bool act[3];
-  double beta[3];
-  bool any = false;
-#pragma unroll
-  for (int r = 0; r < 3; ++r) {
-    act[r] = C.S[r].status == CG_RUNNING;
-    beta[r] = C.S[r].beta;
-    any |= act[r];
+__global__ void __launch_bounds__(NT) k_cn_pupdate(long long n, Cn3 C) {
+  const int s = blockIdx.y;
+  if (C.S[s].status != CG_RUNNING) return;
+  const double beta = C.S[s].beta;
+  double* __restrict__ p = C.p[s];
+  const double* __restrict__ r = C.r[s];
+  const double* __restrict__ di = C.dinv;
+  const long long pairs = n / 2, gs = (long long)gridDim.x * NT;
+  for (long long v = (long long)blockIdx.x * NT + threadIdx.x; v < pairs; v += gs) {
+    const double2 rv = reinterpret_cast<const double2*>(r)[v];
+    const double2 dv = reinterpret_cast<const double2*>(di)[v];
+    const double2 pv = reinterpret_cast<const double2*>(p)[v];
+    reinterpret_cast<double2*>(p)[v] =
+        double2{fma(beta, pv.x, dv.x * rv.x), fma(beta, pv.y, dv.y * rv.y)};
   }
-  if (!any) return;
-  cn_pupdate_tile(G, C, act, beta, blockIdx.x, blockIdx.y, blockIdx.z);
+  if ((n & 1) && blockIdx.x == 0 && threadIdx.x == 0)
+    p[n - 1] = fma(beta, p[n - 1], di[n - 1] * r[n - 1]);
+}
+
+// (blocks over voxel pairs, solves), as the elasticity's flat updates
+dim3 cn_flat3(const Geo& G) {
+  const long long want = (G.nvox / 2 + NT - 1) / NT;
+  const long long most = std::min(304LL, (long long)G.nblocks);
+  return dim3((unsigned)std::max(1LL, std::min(want, most)), 3);
 }
 
 }  // namespace
@@ -249,10 +280,10 @@ cudaError_t launch_diff_coef(const Geo& G, const DevParams& P, double dt, const 
   if (Kfdf)
     for (int d = 0; d < 3; ++d) df[d] = reinterpret_cast<float2*>(Kfdf[d]);
   TG_TIMED(K_DIFF_FACES, st,
-           k_diff_faces<<<G.grid, dim3(BX, BY), 0, st>>>(G, P, 0.5 * dt, g, w, f, Kf[0], Kf[1], Kf[2],
-                                                         rho, df[0], df[1], df[2]));
+           launch(k_diff_faces, G.grid, dim3(BX, BY), 0, st, G, P, 0.5 * dt, g, w, f, Kf[0], Kf[1],
+                  Kf[2], rho, df[0], df[1], df[2]));
   TG_TIMED(K_DIFF_DIAG, st,
-           k_diff_diag<<<G.grid, dim3(BX, BY), 0, st>>>(G, Kf[0], Kf[1], Kf[2], dsum, dinv));
+           launch(k_diff_diag, G.grid, dim3(BX, BY), 0, st, G, Kf[0], Kf[1], Kf[2], dsum, dinv));
   return cudaGetLastError();
 }
 
@@ -261,25 +292,24 @@ cudaError_t launch_diff_coef_df(const Geo& G, const DevParams& P, double dt, con
                                 float2* const Kfdf[3], float* const Kf32[3], float* dinv32,
                                 float* dmax, cudaStream_t st) {
   TG_TIMED(K_DIFF_NODE_DF, st,
-           k_diff_node_df<<<G.grid, dim3(BX, BY), 0, st>>>(G, P, g, w, f, Kn, rho));
+           launch(k_diff_node_df, G.grid, dim3(BX, BY), 0, st, G, P, g, w, f, Kn, rho));
   const Df sx = df_split_host(0.5 * dt * G.ih2[0]), sy = df_split_host(0.5 * dt * G.ih2[1]),
            sz = df_split_host(0.5 * dt * G.ih2[2]);
   TG_TIMED(K_DIFF_FACES_DF, st,
-           k_diff_faces_df<<<G.grid, dim3(BX, BY), 0, st>>>(G, sx, sy, sz, Kn, Kfdf[0], Kfdf[1],
-                                                            Kfdf[2], Kf32[0], Kf32[1], Kf32[2],
-                                                            dinv32, dmax));
+           launch(k_diff_faces_df, G.grid, dim3(BX, BY), 0, st, G, sx, sy, sz, Kn, Kfdf[0],
+                  Kfdf[1], Kfdf[2], Kf32[0], Kf32[1], Kf32[2], dinv32, dmax));
   return cudaGetLastError();
 }
 
 cudaError_t launch_cn_init(const Geo& G, const Cn3& C, cudaStream_t st, int mask) {
-  TG_TIMED(K_CN_INIT, st, k_cn_init<<<G.grid, dim3(BX, BY), 0, st>>>(G, C, mask));
+  TG_TIMED(K_CN_INIT, st, launch(k_cn_init, G.grid, dim3(BX, BY), 0, st, G, C, mask));
   return cudaGetLastError();
 }
 
 cudaError_t launch_cn_iter(const Geo& G, const Cn3& C, cudaStream_t st) {
-  TG_TIMED(K_CN_MATVEC, st, k_cn_matvec<<<G.grid, dim3(BX, BY), 0, st>>>(G, C));
-  TG_TIMED(K_CN_UPDATE, st, k_cn_update<<<G.grid, dim3(BX, BY), 0, st>>>(G, C));
-  TG_TIMED(K_CN_PUPDATE, st, k_cn_pupdate<<<G.grid, dim3(BX, BY), 0, st>>>(G, C));
+  TG_TIMED(K_CN_MATVEC, st, launch(k_cn_matvec, G.grid, dim3(BX, BY), 0, st, G, C));
+  TG_TIMED(K_CN_UPDATE, st, launch(k_cn_update, cn_flat3(G), NT, 0, st, G.nvox, C));
+  TG_TIMED(K_CN_PUPDATE, st, launch(k_cn_pupdate, cn_flat3(G), NT, 0, st, G.nvox, C));
   return cudaGetLastError();
 }
 

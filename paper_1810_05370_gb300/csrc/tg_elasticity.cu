@@ -10,6 +10,8 @@
 // Per-step precomputation trades bytes for FP64 arithmetic: face coefficients already
 // divided by h_d^2 and the Jacobi diagonal are stored, so a matrix-vector product needs
 // 1 multiply and 6 fused multiply-adds per component for the face part.
+#include <algorithm>
+
 #include "tg_internal.cuh"
 
 namespace tg {
@@ -24,11 +26,11 @@ __global__ void __launch_bounds__(NT) k_elas_coef(Geo G, DevParams P, Elas E,
   const int k0 = blockIdx.z * G.zc, k1 = min(G.nz, k0 + G.zc);
   for (int k = k0; k < k1; ++k) {
     const Nbr nb = make_nbr(G, i, j, k);
-    const long long c = nb.at(0, 0, 0);
+    const int c = nb.at(0, 0, 0);
     const double muc = E.mu[c], lac = E.lam[c];
     double mfp[3], mfm[3], lfp[3], lfm[3];
-    long long np[3] = {nb.at(1, 0, 0), nb.at(0, 1, 0), nb.at(0, 0, 1)};
-    long long nm[3] = {nb.at(-1, 0, 0), nb.at(0, -1, 0), nb.at(0, 0, -1)};
+    int np[3] = {nb.at(1, 0, 0), nb.at(0, 1, 0), nb.at(0, 0, 1)};
+    int nm[3] = {nb.at(-1, 0, 0), nb.at(0, -1, 0), nb.at(0, 0, -1)};
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
       mfp[d] = 0.5 * (muc + E.mu[np[d]]);
@@ -98,9 +100,9 @@ __global__ void __launch_bounds__(NT, 4) k_elas_coef_df(Geo G, DevParams P, Elas
   const int k0 = blockIdx.z * G.zc, k1 = min(G.nz, k0 + G.zc);
   for (int k = k0; k < k1; ++k) {
     const Nbr nb = make_nbr(G, i, j, k);
-    const long long c = nb.at(0, 0, 0);
-    const long long np[3] = {nb.at(1, 0, 0), nb.at(0, 1, 0), nb.at(0, 0, 1)};
-    const long long nm[3] = {nb.at(-1, 0, 0), nb.at(0, -1, 0), nb.at(0, 0, -1)};
+    const int c = nb.at(0, 0, 0);
+    const int np[3] = {nb.at(1, 0, 0), nb.at(0, 1, 0), nb.at(0, 0, 1)};
+    const int nm[3] = {nb.at(-1, 0, 0), nb.at(0, -1, 0), nb.at(0, 0, -1)};
     const Df muc = df_of(E.mudf[c]), lac = df_of(E.lamdf[c]);
     Df Fp[3], Fm[3], Gp[3], Gm[3];
 #pragma unroll
@@ -150,7 +152,7 @@ __global__ void __launch_bounds__(NT) k_elas_init(Geo G, Elas E, int minus_b) {
     const int k0 = blockIdx.z * G.zc, k1 = min(G.nz, k0 + G.zc);
     for (int k = k0; k < k1; ++k) {
       const Nbr nb = make_nbr(G, i, j, k);
-      const long long c = nb.at(0, 0, 0);
+      const int c = nb.at(0, 0, 0);
       double Au[3];
       Au[0] = elas_row64<0>(G, nb, c, E, u);
       Au[1] = elas_row64<1>(G, nb, c, E, u);
@@ -176,7 +178,7 @@ __global__ void __launch_bounds__(NT) k_elas_init(Geo G, Elas E, int minus_b) {
     cg_after_init(*E.S, out[0], out[1], out[2]);
 }
 
-__global__ void __launch_bounds__(NT) k_elas_matvec(Geo G, Elas E) {
+__global__ void __launch_bounds__(NT, 3) k_elas_matvec(Geo G, Elas E) {
   if (E.S->status != CG_RUNNING) return;
   const double* const p[3] = {E.p[0], E.p[1], E.p[2]};
   const int i = blockIdx.x * BX + threadIdx.x;
@@ -187,7 +189,7 @@ __global__ void __launch_bounds__(NT) k_elas_matvec(Geo G, Elas E) {
     const int k0 = blockIdx.z * G.zc, k1 = min(G.nz, k0 + G.zc);
     for (int k = k0; k < k1; ++k) {
       const Nbr nb = make_nbr(G, i, j, k);
-      const long long c = nb.at(0, 0, 0);
+      const int c = nb.at(0, 0, 0);
       const double q0 = elas_row64<0>(G, nb, c, E, p);
       const double q1 = elas_row64<1>(G, nb, c, E, p);
       const double q2 = elas_row64<2>(G, nb, c, E, p);
@@ -204,31 +206,43 @@ __global__ void __launch_bounds__(NT) k_elas_matvec(Geo G, Elas E) {
   }
 }
 
+// The CG vector updates run flat over the voxels, blockIdx.y the component, two voxels per
+// 16-byte access and a grid of a few blocks per SM.  They were bound by the blocks' reductions
+// and not by their arithmetic or traffic when every 32 x 8 tile of one z plane was a block of
+// its own (2160 blocks at 96 x 80 x 72).  Workspace arrays start on 256-byte boundaries.
 template <bool SPEC>
-__global__ void __launch_bounds__(NT) k_elas_update(Geo G, Elas E) {
+__global__ void __launch_bounds__(NT) k_elas_update(long long n, Elas E) {
   if (E.S->status != CG_RUNNING) return;
   const double alpha = E.S->alpha;
-  const int i = blockIdx.x * BX + threadIdx.x;
-  const int j = blockIdx.y * BY + threadIdx.y;
-  const bool on = (i < G.nx) && (j < G.ny);
+  const int a = blockIdx.y;
+  double* __restrict__ du = E.du[a];
+  double* __restrict__ r = E.r[a];
+  const double* __restrict__ p = E.p[a];
+  const double* __restrict__ q = E.q[a];
+  const double* __restrict__ di = E.dinv[a];
   double acc[2] = {0.0, 0.0};
-  if (on) {
-    const int k0 = blockIdx.z * G.zc, k1 = min(G.nz, k0 + G.zc);
-    for (int k = k0; k < k1; ++k) {
-      const long long c = ((long long)k * G.ny + j) * G.nx + i;
-#pragma unroll
-      for (int a = 0; a < 3; ++a) {
-        E.du[a][c] += alpha * E.p[a][c];
-        const double res = E.r[a][c] - alpha * E.q[a][c];
-        E.r[a][c] = res;
-        if (!SPEC) acc[0] += res * (E.dinv[a][c] * res);
-        acc[1] += res * res;
-      }
-    }
+  auto one = [&](double& d, double& res, double pv, double qv, double dv) {
+    d = fma(alpha, pv, d);
+    res = fma(-alpha, qv, res);
+    if (!SPEC) acc[0] = fma(res, dv * res, acc[0]);
+    acc[1] = fma(res, res, acc[1]);
+  };
+  const long long pairs = n / 2, gs = (long long)gridDim.x * NT;
+  for (long long v = (long long)blockIdx.x * NT + threadIdx.x; v < pairs; v += gs) {
+    double2 d = reinterpret_cast<double2*>(du)[v], x = reinterpret_cast<double2*>(r)[v];
+    const double2 pv = reinterpret_cast<const double2*>(p)[v];
+    const double2 qv = reinterpret_cast<const double2*>(q)[v];
+    const double2 dv = SPEC ? double2{0.0, 0.0} : reinterpret_cast<const double2*>(di)[v];
+    one(d.x, x.x, pv.x, qv.x, dv.x);
+    one(d.y, x.y, pv.y, qv.y, dv.y);
+    reinterpret_cast<double2*>(du)[v] = d;
+    reinterpret_cast<double2*>(r)[v] = x;
   }
+  if ((n & 1) && blockIdx.x == 0 && threadIdx.x == 0)
+    one(du[n - 1], r[n - 1], p[n - 1], q[n - 1], SPEC ? 0.0 : di[n - 1]);
   double out[2];
-  if (reduce_last_block<2>(acc, E.partial, E.counter, out) && threadIdx.x == 0 &&
-      threadIdx.y == 0) {
+  if (reduce_indexed<2>(acc, E.partial, E.counter, block_linear(), block_count(), out) &&
+      threadIdx.x == 0) {
     if (SPEC)
       cg_after_update_rr(*E.S, out[1]);
     else
@@ -236,34 +250,30 @@ __global__ void __launch_bounds__(NT) k_elas_update(Geo G, Elas E) {
   }
 }
 
-__global__ void __launch_bounds__(NT) k_elas_pupdate(Geo G, Elas E) {
+// p = z + beta p with z = D^{-1} r (Jacobi), or z from the spectral preconditioner (p = z on
+// the first iteration); flat as the update
+template <bool SPEC>
+__global__ void __launch_bounds__(NT) k_elas_pupdate(long long n, Elas E) {
   if (E.S->status != CG_RUNNING) return;
   const double beta = E.S->beta;
-  const int i = blockIdx.x * BX + threadIdx.x;
-  const int j = blockIdx.y * BY + threadIdx.y;
-  if (i >= G.nx || j >= G.ny) return;
-  const int k0 = blockIdx.z * G.zc, k1 = min(G.nz, k0 + G.zc);
-  for (int k = k0; k < k1; ++k) {
-    const long long c = ((long long)k * G.ny + j) * G.nx + i;
-#pragma unroll
-    for (int a = 0; a < 3; ++a) E.p[a][c] = E.dinv[a][c] * E.r[a][c] + beta * E.p[a][c];
+  const bool first = SPEC && E.S->it == 0;
+  const int a = blockIdx.y;
+  double* __restrict__ p = E.p[a];
+  const double* __restrict__ r = E.r[a];
+  const double* __restrict__ z = SPEC ? E.z[a] : E.dinv[a];
+  auto one = [&](double zv, double rv, double pv) {
+    const double zz = SPEC ? zv : zv * rv;
+    return first ? zz : fma(beta, pv, zz);
+  };
+  const long long pairs = n / 2, gs = (long long)gridDim.x * NT;
+  for (long long v = (long long)blockIdx.x * NT + threadIdx.x; v < pairs; v += gs) {
+    const double2 zv = reinterpret_cast<const double2*>(z)[v];
+    const double2 rv = SPEC ? zv : reinterpret_cast<const double2*>(r)[v];
+    const double2 pv = reinterpret_cast<const double2*>(p)[v];
+    reinterpret_cast<double2*>(p)[v] = double2{one(zv.x, rv.x, pv.x), one(zv.y, rv.y, pv.y)};
   }
-}
-
-// p = z + beta p with z from the spectral preconditioner (p = z on the first iteration)
-__global__ void __launch_bounds__(NT) k_elas_pupdate_spec(Geo G, Elas E) {
-  if (E.S->status != CG_RUNNING) return;
-  const double beta = E.S->beta;
-  const bool first = E.S->it == 0;
-  const int i = blockIdx.x * BX + threadIdx.x;
-  const int j = blockIdx.y * BY + threadIdx.y;
-  if (i >= G.nx || j >= G.ny) return;
-  const int k0 = blockIdx.z * G.zc, k1 = min(G.nz, k0 + G.zc);
-  for (int k = k0; k < k1; ++k) {
-    const long long c = ((long long)k * G.ny + j) * G.nx + i;
-#pragma unroll
-    for (int a = 0; a < 3; ++a) E.p[a][c] = first ? E.z[a][c] : E.z[a][c] + beta * E.p[a][c];
-  }
+  if ((n & 1) && blockIdx.x == 0 && threadIdx.x == 0)
+    p[n - 1] = one(z[n - 1], SPEC ? 0.0 : r[n - 1], p[n - 1]);
 }
 
 // u += du (du = -u when the right-hand side vanished, i.e. u = 0), v = vo + du / dt with vo
@@ -277,7 +287,7 @@ __global__ void __launch_bounds__(NT) k_elas_finish(Geo G, Elas E, double inv_dt
   if (i >= G.nx || j >= G.ny) return;
   const int k0 = blockIdx.z * G.zc, k1 = min(G.nz, k0 + G.zc);
   for (int k = k0; k < k1; ++k) {
-    const long long c = ((long long)k * G.ny + j) * G.nx + i;
+    const int c = (k * G.ny + j) * G.nx + i;
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
       const double uo = E.u[a][c];
@@ -293,60 +303,68 @@ __global__ void __launch_bounds__(NT) k_elas_finish(Geo G, Elas E, double inv_dt
   }
 }
 
+// (blocks over voxel pairs, components): two blocks per SM and component, never more than the
+// partial-sum buffer holds (nine doubles per block of the grid-shaped kernels)
+dim3 flat3(const Geo& G) {
+  const long long want = (G.nvox / 2 + NT - 1) / NT;
+  const long long most = std::min(304LL, (long long)G.nblocks);
+  return dim3((unsigned)std::max(1LL, std::min(want, most)), 3);
+}
+
 }  // namespace
 
 cudaError_t launch_elas_coef_df(const Geo& G, const DevParams& P, const Elas& E,
                                 const Elas32& I, const float2* sdf, bool force, cudaStream_t st) {
   TG_TIMED(K_ELAS_COEF_DF, st,
-           k_elas_coef_df<<<G.grid, dim3(BX, BY), 0, st>>>(G, P, E, I, sdf, force ? 1 : 0));
+           launch(k_elas_coef_df, G.grid, dim3(BX, BY), 0, st, G, P, E, I, sdf, force ? 1 : 0));
   return cudaGetLastError();
 }
 
 cudaError_t launch_elas_coef(const Geo& G, const DevParams& P, const Elas& E, const double* p,
                              const double* n, bool force, cudaStream_t st) {
   TG_TIMED(K_ELAS_COEF, st,
-           k_elas_coef<<<G.grid, dim3(BX, BY), 0, st>>>(G, P, E, p, n, force ? 1 : 0));
+           launch(k_elas_coef, G.grid, dim3(BX, BY), 0, st, G, P, E, p, n, force ? 1 : 0));
   return cudaGetLastError();
 }
 
 cudaError_t launch_elas_init(const Geo& G, const Elas& E, bool minus_b, cudaStream_t st) {
   TG_TIMED(K_ELAS_INIT, st,
-           k_elas_init<false><<<G.grid, dim3(BX, BY), 0, st>>>(G, E, minus_b ? 1 : 0));
+           launch(k_elas_init<false>, G.grid, dim3(BX, BY), 0, st, G, E, minus_b ? 1 : 0));
   return cudaGetLastError();
 }
 
 cudaError_t launch_elas_init_spec(const Geo& G, const Elas& E, bool minus_b, cudaStream_t st) {
   TG_TIMED(K_ELAS_INIT_SPEC, st,
-           k_elas_init<true><<<G.grid, dim3(BX, BY), 0, st>>>(G, E, minus_b ? 1 : 0));
+           launch(k_elas_init<true>, G.grid, dim3(BX, BY), 0, st, G, E, minus_b ? 1 : 0));
   return cudaGetLastError();
 }
 
 cudaError_t launch_elas_matvec(const Geo& G, const Elas& E, cudaStream_t st) {
-  TG_TIMED(K_ELAS_MATVEC, st, k_elas_matvec<<<G.grid, dim3(BX, BY), 0, st>>>(G, E));
+  TG_TIMED(K_ELAS_MATVEC, st, launch(k_elas_matvec, G.grid, dim3(BX, BY), 0, st, G, E));
   return cudaGetLastError();
 }
 
 cudaError_t launch_elas_update(const Geo& G, const Elas& E, cudaStream_t st) {
-  TG_TIMED(K_ELAS_UPDATE, st, k_elas_update<false><<<G.grid, dim3(BX, BY), 0, st>>>(G, E));
-  TG_TIMED(K_ELAS_PUPDATE, st, k_elas_pupdate<<<G.grid, dim3(BX, BY), 0, st>>>(G, E));
+  TG_TIMED(K_ELAS_UPDATE, st, launch(k_elas_update<false>, flat3(G), NT, 0, st, G.nvox, E));
+  TG_TIMED(K_ELAS_PUPDATE, st, launch(k_elas_pupdate<false>, flat3(G), NT, 0, st, G.nvox, E));
   return cudaGetLastError();
 }
 
 cudaError_t launch_elas_update_spec(const Geo& G, const Elas& E, cudaStream_t st) {
-  TG_TIMED(K_ELAS_UPDATE_SPEC, st, k_elas_update<true><<<G.grid, dim3(BX, BY), 0, st>>>(G, E));
+  TG_TIMED(K_ELAS_UPDATE_SPEC, st, launch(k_elas_update<true>, flat3(G), NT, 0, st, G.nvox, E));
   return cudaGetLastError();
 }
 
 cudaError_t launch_elas_pupdate_spec(const Geo& G, const Elas& E, cudaStream_t st) {
-  TG_TIMED(K_ELAS_PUPDATE_SPEC, st, k_elas_pupdate_spec<<<G.grid, dim3(BX, BY), 0, st>>>(G, E));
+  TG_TIMED(K_ELAS_PUPDATE_SPEC, st, launch(k_elas_pupdate<true>, flat3(G), NT, 0, st, G.nvox, E));
   return cudaGetLastError();
 }
 
 cudaError_t launch_elas_finish(const Geo& G, const Elas& E, double inv_dt, bool zero_rhs,
                                int extrap, cudaStream_t st) {
   TG_TIMED(K_ELAS_FINISH, st,
-           k_elas_finish<<<G.grid, dim3(BX, BY), 0, st>>>(G, E, inv_dt, zero_rhs ? 1 : 0,
-                                                          extrap));
+           launch(k_elas_finish, G.grid, dim3(BX, BY), 0, st, G, E, inv_dt, zero_rhs ? 1 : 0,
+                  extrap));
   return cudaGetLastError();
 }
 

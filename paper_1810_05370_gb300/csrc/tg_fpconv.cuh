@@ -333,4 +333,29 @@ TG_HD Df df_tanh(Df s) {
   return neg ? df_neg(t) : t;
 }
 
+// ------------------------------------------------- scalars of the CG solves
+// The power of two nearest 1 / sqrt(x) on the logarithmic scale, 2^-rint(log2(x) / 2), for a
+// finite x > 0, from its exponent e and significand m in [1, 2): log2(x) / 2 lies in
+// [e/2, e/2 + 1/2), so it rounds to e/2 for even e and to (e + 1)/2 for odd e, the tie at
+// m = 1 of an odd e going to the even integer.  One thread evaluates it on the critical path
+// of every residual; log2 and exp2 in FP64 took it about 3 us.
+TG_HD double pow2_inv_root(double x) {
+  const int e = ilogb(x);
+  int k = (e + (e & 1)) >> 1;
+  if ((e & 1) && (k & 1) && scalbn(x, -e) == 1.0) --k;
+  return scalbn(1.0, -k);
+}
+
+// sqrt(rr) <= rtol sqrt(bb), decided from the squares where they are clearly apart (the last
+// block's thread 0 evaluates it alone, and an FP64 square root takes it some 500 clocks); the
+// square roots only within 1e-12 of the threshold or where the squares leave FP64's range.
+TG_HD bool cg_norm_met(double rr, double rtol, double bb) {
+  const double t = rtol * rtol * bb;
+  if (t > 1e-280 && t < 1e280) {
+    if (rr < t * (1.0 - 1e-12)) return true;
+    if (rr > t * (1.0 + 1e-12)) return false;
+  }
+  return sqrt(rr) <= rtol * sqrt(bb);
+}
+
 }  // namespace tg

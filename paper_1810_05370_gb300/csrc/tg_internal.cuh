@@ -89,31 +89,34 @@ struct CgScal {
 };
 
 // Periodic neighbour offsets of node (i, j, k): X[o+1], Y[o+1], Z[o+1] for o in {-1, 0, 1};
-// the linear index of (i + ox, j + oy, k + oz) is Z[oz+1] + Y[oy+1] + X[ox+1].
+// the linear index of (i + ox, j + oy, k + oz) is Z[oz+1] + Y[oy+1] + X[ox+1].  32-bit: a grid
+// of 2^31 voxels would need a terabyte of workspace (tg_init refuses it), and nine 64-bit
+// offsets cost the operator kernels nine more registers and their adds twice the instructions.
 struct Nbr {
-  long long X[3], Y[3], Z[3];
-  __device__ __forceinline__ long long at(int ox, int oy, int oz) const {
+  int X[3], Y[3], Z[3];
+  __device__ __forceinline__ int at(int ox, int oy, int oz) const {
     return Z[oz + 1] + Y[oy + 1] + X[ox + 1];
   }
 };
 
 __device__ __forceinline__ Nbr make_nbr(const Geo& g, int i, int j, int k) {
   Nbr n;
+  const int nxy = g.nx * g.ny;
   n.X[0] = (i == 0) ? g.nx - 1 : i - 1;
   n.X[1] = i;
   n.X[2] = (i + 1 == g.nx) ? 0 : i + 1;
-  n.Y[0] = (long long)((j == 0) ? g.ny - 1 : j - 1) * g.nx;
-  n.Y[1] = (long long)j * g.nx;
-  n.Y[2] = (long long)((j + 1 == g.ny) ? 0 : j + 1) * g.nx;
-  n.Z[0] = (long long)((k == 0) ? g.nz - 1 : k - 1) * g.nxy;
-  n.Z[1] = (long long)k * g.nxy;
-  n.Z[2] = (long long)((k + 1 == g.nz) ? 0 : k + 1) * g.nxy;
+  n.Y[0] = ((j == 0) ? g.ny - 1 : j - 1) * g.nx;
+  n.Y[1] = j * g.nx;
+  n.Y[2] = ((j + 1 == g.ny) ? 0 : j + 1) * g.nx;
+  n.Z[0] = ((k == 0) ? g.nz - 1 : k - 1) * nxy;
+  n.Z[1] = k * nxy;
+  n.Z[2] = ((k + 1 == g.nz) ? 0 : k + 1) * nxy;
   return n;
 }
 
 // offset vector with s_a along axis A and s_d along axis D
 template <int A, int D>
-__device__ __forceinline__ long long at2(const Nbr& n, int sa, int sd) {
+__device__ __forceinline__ int at2(const Nbr& n, int sa, int sd) {
   int o[3] = {0, 0, 0};
   o[A] += sa;
   o[D] += sd;
@@ -121,7 +124,7 @@ __device__ __forceinline__ long long at2(const Nbr& n, int sa, int sd) {
 }
 
 template <int A>
-__device__ __forceinline__ long long at1(const Nbr& n, int s) {
+__device__ __forceinline__ int at1(const Nbr& n, int s) {
   int o[3] = {0, 0, 0};
   o[A] += s;
   return n.at(o[0], o[1], o[2]);
@@ -139,61 +142,95 @@ __device__ __forceinline__ int block_linear() {
 
 __device__ __forceinline__ int block_count() { return gridDim.x * gridDim.y * gridDim.z; }
 
-// Block-level sum of NV values, written to partial[b][NV] for work item b of nb; the last item
-// to finish sums all partials in item order (deterministic) and returns true in every thread
-// of that block, with the totals in out[] valid in thread 0.  counter is reset by the last.
+// ------------------------------------------------------------------ sums over a launch
+// Every CG scalar is a sum over all blocks of a launch, so the tail of each reducing kernel --
+// the block's sum, the ticket, the last block's sum of the partials -- is on the solver's
+// critical path once per kernel (three times an iteration).  What bounds it is latency and the
+// FP64 pipe (2 lanes per clock per SM: one warp addition takes 16 clocks):
+//  * a block sums through shared memory, one warp per value adding eight values per lane and
+//    then five shuffle rounds: 12 warp additions per value instead of the 40 of a shuffle tree
+//    in every warp plus a serial sum over the warps;
+//  * the ticket is one acquire-release atomic instead of a full fence and a relaxed one.
+// Deterministic: the order of the additions depends on the launch's shape only.
+__device__ __forceinline__ unsigned int ticket_acq_rel(unsigned int* counter) {
+  unsigned int t;
+  asm volatile("atom.add.acq_rel.gpu.global.u32 %0, [%1], 1;" : "=r"(t) : "l"(counter) : "memory");
+  return t;
+}
+
+// Sum of sh[0 .. n) (n a multiple of 32, at most 1024) by one whole warp; every lane calls it
+// and lane 0 holds the result.
+__device__ __forceinline__ double warp_sum_shared(const double* sh, int n, int lane) {
+  double s;
+  if (n == 256) {   // the usual block: eight values per lane as a tree
+    const double a = sh[lane] + sh[lane + 32], b = sh[lane + 64] + sh[lane + 96];
+    const double c = sh[lane + 128] + sh[lane + 160], d = sh[lane + 192] + sh[lane + 224];
+    s = (a + b) + (c + d);
+  } else {
+    s = sh[lane];
+    for (int k = lane + 32; k < n; k += 32) s += sh[k];
+  }
+  return warp_sum(s);
+}
+
+// Sum of part[0], part[ld], ..., part[(nb - 1) ld] over the threads tid, tid + nt, ... (this
+// thread's share, four loads in flight), read from L2: other blocks wrote them.
+__device__ __forceinline__ double strided_partials(const double* part, int ld, int nb, int tid,
+                                                   int nt) {
+  double s = 0.0;
+  int k = tid;
+  for (; k + 3 * nt < nb; k += 4 * nt) {
+    const double a = __ldcg(part + (size_t)k * ld), b = __ldcg(part + (size_t)(k + nt) * ld);
+    const double c = __ldcg(part + (size_t)(k + 2 * nt) * ld);
+    const double d = __ldcg(part + (size_t)(k + 3 * nt) * ld);
+    s += (a + b) + (c + d);
+  }
+  for (; k < nb; k += nt) s += __ldcg(part + (size_t)k * ld);
+  return s;
+}
+
+// Sum of NV values per thread over a block of NTH threads (a multiple of 32), written to
+// partial[b][NV] for work item b of nb; the last item to finish sums all partials and returns
+// true in every thread of that block, with the totals in out[] valid in thread 0.  counter is
+// reset by the last.
+template <int NV, int NTH>
+__device__ bool reduce_items(double (&v)[NV], double* partial, unsigned int* counter, int tid,
+                             int b, int nb, double (&out)[NV]) {
+  constexpr int NW = NTH / 32;
+  __shared__ double sh[NV][NTH];
+  __shared__ double tot[NV];
+  __shared__ bool am_last;
+  const int lane = tid & 31, warp = tid >> 5;
+#pragma unroll
+  for (int q = 0; q < NV; ++q) sh[q][tid] = v[q];
+  __syncthreads();
+  for (int q = warp; q < NV; q += NW) {
+    const double s = warp_sum_shared(sh[q], NTH, lane);
+    if (lane == 0) partial[(size_t)b * NV + q] = s;
+  }
+  if (NV > 1) __syncthreads();   // the other warps' partials precede thread 0's release
+  if (tid == 0) am_last = ticket_acq_rel(counter) == (unsigned int)(nb - 1);
+  __syncthreads();
+  if (!am_last) return false;
+#pragma unroll
+  for (int q = 0; q < NV; ++q) sh[q][tid] = strided_partials(partial + q, NV, nb, tid, NTH);
+  __syncthreads();
+  for (int q = warp; q < NV; q += NW) {
+    const double s = warp_sum_shared(sh[q], NTH, lane);
+    if (lane == 0) tot[q] = s;
+  }
+  if (tid == 0) *counter = 0u;
+  __syncthreads();
+#pragma unroll
+  for (int q = 0; q < NV; ++q) out[q] = tot[q];
+  return true;
+}
+
 template <int NV>
 __device__ bool reduce_indexed(double (&v)[NV], double* partial, unsigned int* counter, int b,
                                int nb, double (&out)[NV]) {
-  __shared__ double sh[NV][NWARP];
-  __shared__ bool am_last;
-  const int tid = threadIdx.y * blockDim.x + threadIdx.x;
-  const int lane = tid & 31, warp = tid >> 5;
-#pragma unroll
-  for (int q = 0; q < NV; ++q) {
-    double s = warp_sum(v[q]);
-    if (lane == 0) sh[q][warp] = s;
-  }
-  __syncthreads();
-  if (tid == 0) {
-#pragma unroll
-    for (int q = 0; q < NV; ++q) {
-      double s = 0.0;
-      for (int w = 0; w < NWARP; ++w) s += sh[q][w];
-      partial[(size_t)b * NV + q] = s;
-    }
-    __threadfence();
-    unsigned int ticket = atomicAdd(counter, 1u);
-    am_last = (ticket == (unsigned int)(nb - 1));
-  }
-  __syncthreads();
-  if (!am_last) return false;
-  __threadfence();
-  double acc[NV];
-#pragma unroll
-  for (int q = 0; q < NV; ++q) acc[q] = 0.0;
-  for (int k = tid; k < nb; k += NT) {
-#pragma unroll
-    for (int q = 0; q < NV; ++q) acc[q] += __ldcg(partial + (size_t)k * NV + q);
-  }
-  __syncthreads();
-#pragma unroll
-  for (int q = 0; q < NV; ++q) {
-    double s = warp_sum(acc[q]);
-    if (lane == 0) sh[q][warp] = s;
-  }
-  __syncthreads();
-  if (tid == 0) {
-#pragma unroll
-    for (int q = 0; q < NV; ++q) {
-      double s = 0.0;
-      for (int w = 0; w < NWARP; ++w) s += sh[q][w];
-      out[q] = s;
-    }
-    *counter = 0u;
-  }
-  __syncthreads();
-  return true;
+  return reduce_items<NV, NT>(v, partial, counter, threadIdx.y * blockDim.x + threadIdx.x, b, nb,
+                              out);
 }
 
 // the same over the blocks of a launch
@@ -210,7 +247,7 @@ __device__ __forceinline__ void cg_after_update(CgScal& S, double rz_new, double
   S.rr = rr;
   if (!isfinite(rr)) {
     S.status = CG_NONFINITE;
-  } else if (sqrt(rr) <= S.rtol * sqrt(S.bb)) {
+  } else if (cg_norm_met(rr, S.rtol, S.bb)) {
     S.status = CG_CONVERGED;
   } else if (S.it >= S.maxit) {
     S.status = CG_MAXIT;
@@ -227,7 +264,7 @@ __device__ __forceinline__ void cg_after_update_rr(CgScal& S, double rr) {
   S.rr = rr;
   if (!isfinite(rr)) {
     S.status = CG_NONFINITE;
-  } else if (sqrt(rr) <= S.rtol * sqrt(S.bb)) {
+  } else if (cg_norm_met(rr, S.rtol, S.bb)) {
     S.status = CG_CONVERGED;
   } else if (S.it >= S.maxit) {
     S.status = CG_MAXIT;
@@ -262,7 +299,7 @@ __device__ __forceinline__ void cg_after_init(CgScal& S, double bb, double rr, d
     S.status = CG_ZERO_RHS;
   } else if (!isfinite(rr)) {
     S.status = CG_NONFINITE;
-  } else if (sqrt(rr) <= S.rtol * sqrt(bb)) {
+  } else if (cg_norm_met(rr, S.rtol, bb)) {
     S.status = CG_CONVERGED;
   } else if (S.maxit <= 0) {
     S.status = CG_MAXIT;
@@ -390,6 +427,18 @@ template <typename R> size_t spec_smem_y(const Spec<R>& V) {
 }
 template <typename R> size_t spec_smem_z(const Spec<R>& V) {
   return (1 + 2 * (size_t)3 * V.tz) * V.nz * sizeof(typename CxOf<R>::T);
+}
+
+// ----------------------------------------------------------------------------- launch helper
+template <class... P, class... A>
+inline void launch(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                   const A&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
 }
 
 // ----------------------------------------------------------------------------- launches
@@ -540,7 +589,10 @@ cudaError_t launch_diff_coef_df(const Geo&, const DevParams&, double dt, const d
                                 float2* const Kfdf[3], float* const Kf32[3], float* dinv32,
                                 float* dmax, cudaStream_t st);
 
-// 4 h_A h_D [ d_D(mu d_A u_D) + d_A(lambda d_D u_D) ] at the centre node (centred differences)
+// m + 4 h_A h_D [ d_D(mu d_A u_D) + d_A(lambda d_D u_D) ] at the centre node (centred
+// differences).  Written as one chain of fused multiply-adds: the FP64 pipe (2 lanes per clock
+// per SM) bounds every kernel that applies this operator, and an operation counts the same
+// whether it is an addition, a product or both.
 template <int A, int D>
 __device__ __forceinline__ double elas_mixed64(const Nbr& nb, const double* __restrict__ xd,
                                               const double* __restrict__ mu,
@@ -549,13 +601,16 @@ __device__ __forceinline__ double elas_mixed64(const Nbr& nb, const double* __re
   const double epm = xd[at2<A, D>(nb, -1, +1)];  // c - e_A + e_D
   const double emp = xd[at2<A, D>(nb, +1, -1)];  // c + e_A - e_D
   const double emm = xd[at2<A, D>(nb, -1, -1)];  // c - e_A - e_D
-  return mu[at1<D>(nb, +1)] * (epp - epm) - mu[at1<D>(nb, -1)] * (emp - emm) +
-         lam[at1<A>(nb, +1)] * (epp - emp) - lam[at1<A>(nb, -1)] * (epm - emm);
+  double m = mu[at1<D>(nb, +1)] * (epp - epm);
+  m = fma(-mu[at1<D>(nb, -1)], emp - emm, m);
+  m = fma(lam[at1<A>(nb, +1)], epp - emp, m);
+  return fma(-lam[at1<A>(nb, -1)], epm - emm, m);
 }
 
-// component A of (eta I - L_h) x at node c, from the stored FP64 faces and diagonal
+// component A of (eta I - L_h) x at node c, from the stored FP64 faces and diagonal: 25 FP64
+// operations (7 for the diagonal and the faces, 9 for each mixed term)
 template <int A>
-__device__ __forceinline__ double elas_row64(const Geo& G, const Nbr& nb, long long c,
+__device__ __forceinline__ double elas_row64(const Geo& G, const Nbr& nb, int c,
                                              const Elas& E, const double* const x[3]) {
   constexpr int D1 = (A + 1) % 3, D2 = (A + 2) % 3;
   const double* __restrict__ xa = x[A];
@@ -563,12 +618,14 @@ __device__ __forceinline__ double elas_row64(const Geo& G, const Nbr& nb, long l
   const double* __restrict__ C1 = E.G[D1];
   const double* __restrict__ C2 = E.G[D2];
   double v = E.dsum[A][c] * xa[c];
-  v -= CA[c] * xa[at1<A>(nb, 1)] + CA[at1<A>(nb, -1)] * xa[at1<A>(nb, -1)];
-  v -= C1[c] * xa[at1<D1>(nb, 1)] + C1[at1<D1>(nb, -1)] * xa[at1<D1>(nb, -1)];
-  v -= C2[c] * xa[at1<D2>(nb, 1)] + C2[at1<D2>(nb, -1)] * xa[at1<D2>(nb, -1)];
-  v -= G.s_cross[A][D1] * elas_mixed64<A, D1>(nb, x[D1], E.mu, E.lam);
-  v -= G.s_cross[A][D2] * elas_mixed64<A, D2>(nb, x[D2], E.mu, E.lam);
-  return v;
+  v = fma(-CA[c], xa[at1<A>(nb, 1)], v);
+  v = fma(-CA[at1<A>(nb, -1)], xa[at1<A>(nb, -1)], v);
+  v = fma(-C1[c], xa[at1<D1>(nb, 1)], v);
+  v = fma(-C1[at1<D1>(nb, -1)], xa[at1<D1>(nb, -1)], v);
+  v = fma(-C2[c], xa[at1<D2>(nb, 1)], v);
+  v = fma(-C2[at1<D2>(nb, -1)], xa[at1<D2>(nb, -1)], v);
+  v = fma(-G.s_cross[A][D1], elas_mixed64<A, D1>(nb, x[D1], E.mu, E.lam), v);
+  return fma(-G.s_cross[A][D2], elas_mixed64<A, D2>(nb, x[D2], E.mu, E.lam), v);
 }
 
 cudaError_t launch_elas_coef(const Geo&, const DevParams&, const Elas&, const double* p,

@@ -134,7 +134,7 @@ __global__ void __launch_bounds__(NT) k_elas32_update_spec(long long n, Elas32 I
 
 // FP64 residual of the current iterate, outer stopping test and start of the inner solve
 template <bool DF>
-__global__ void __launch_bounds__(NT, DF ? 3 : 1) k_elas_ir_residual(Geo G, Elas E, Elas32 I, CgScal* Sout,
+__global__ void __launch_bounds__(NT, DF ? 3 : 2) k_elas_ir_residual(Geo G, Elas E, Elas32 I, CgScal* Sout,
                                                             int minus_b, double tau_min,
                                                             int max_sweeps, ScDf scd) {
   double acc[3] = {0.0, 0.0, 0.0};
@@ -325,7 +325,7 @@ __global__ void __launch_bounds__(NT) k_sl32_pack(Geo G, const double* __restric
   const int k0 = blockIdx.z * G.zc, k1 = min(G.nz, k0 + G.zc);
   for (int k = k0; k < k1; ++k) {
     const Nbr nb = make_nbr(G, i, j, k);
-    const long long c = nb.at(0, 0, 0);
+    const int c = nb.at(0, 0, 0);
     const float div = diff(vx[nb.at(1, 0, 0)], vx[nb.at(-1, 0, 0)]) * i2h[0] +
                       diff(vy[nb.at(0, 1, 0)], vy[nb.at(0, -1, 0)]) * i2h[1] +
                       diff(vz[nb.at(0, 0, 1)], vz[nb.at(0, 0, -1)]) * i2h[2];
@@ -379,22 +379,22 @@ int stream_blocks(long long n) {
 }  // namespace
 
 cudaError_t launch_to_f32(long long n, const F32Copy& c, cudaStream_t st) {
-  TG_TIMED(K_TO_F32, st, k_to_f32<<<stream_blocks(n), NT, 0, st>>>(n, c));
+  TG_TIMED(K_TO_F32, st, launch(k_to_f32, stream_blocks(n), NT, 0, st, n, c));
   return cudaGetLastError();
 }
 
 cudaError_t launch_elas32_coef(const Geo& G, const Elas& E, const Elas32& I, cudaStream_t st,
                               int parts) {
   TG_TIMED(K_ELAS32_COEF, st,
-           k_elas32_coef<<<stream_blocks(G.nvox), NT, 0, st>>>(G.nvox, E, I, parts));
+           launch(k_elas32_coef, stream_blocks(G.nvox), NT, 0, st, G.nvox, E, I, parts));
   return cudaGetLastError();
 }
 
 cudaError_t launch_df_pack3(const Geo& G, const double* const b[3], double* const out[3],
                             cudaStream_t st) {
   TG_TIMED(K_DF_PACK3, st,
-           k_df_pack3<<<stream_blocks(G.nvox), NT, 0, st>>>(G.nvox, b[0], b[1], b[2], out[0], out[1],
-                                                            out[2]));
+           launch(k_df_pack3, stream_blocks(G.nvox), NT, 0, st, G.nvox, b[0], b[1], b[2], out[0],
+                  out[1], out[2]));
   return cudaGetLastError();
 }
 
@@ -404,20 +404,18 @@ cudaError_t launch_elas_ir_residual(const Geo& G, const Elas& E, const Elas32& I
                                     bool minus_b, double tau_min, cudaStream_t st) {
   if (E.df)
     TG_TIMED(K_ELAS_IR_RESIDUAL_DF, st,
-             k_elas_ir_residual<true><<<G.grid, dim3(BX, BY), 0, st>>>(G, E, I, Sout, minus_b ? 1 : 0,
-                                                                       tau_min, 1 << 30,
-                                                                       sc_df_host(G)));
+             launch(k_elas_ir_residual<true>, G.grid, dim3(BX, BY), 0, st, G, E, I, Sout,
+                    minus_b ? 1 : 0, tau_min, 1 << 30, sc_df_host(G)));
   else
     TG_TIMED(K_ELAS_IR_RESIDUAL, st,
-             k_elas_ir_residual<false><<<G.grid, dim3(BX, BY), 0, st>>>(G, E, I, Sout, minus_b ? 1 : 0,
-                                                                        tau_min, 1 << 30,
-                                                                        ScDf{}));
+             launch(k_elas_ir_residual<false>, G.grid, dim3(BX, BY), 0, st, G, E, I, Sout,
+                    minus_b ? 1 : 0, tau_min, 1 << 30, ScDf{}));
   return cudaGetLastError();
 }
 
 cudaError_t launch_elas32_matvec(const Geo& G, const Elas32& I, cudaStream_t st) {
   TG_TIMED(K_ELAS32_MATVEC, st,
-           k_elas32_matvec<<<G.grid, dim3(BX, BY), 0, st>>>(G, make_consts32(G), I));
+           launch(k_elas32_matvec, G.grid, dim3(BX, BY), 0, st, G, make_consts32(G), I));
   return cudaGetLastError();
 }
 
@@ -431,45 +429,47 @@ static int reduce_blocks(const Geo& G, long long items) {
 
 cudaError_t launch_elas32_update(const Geo& G, const Elas32& I, cudaStream_t st) {
   TG_TIMED(K_ELAS32_UPDATE, st,
-           k_elas32_update<<<reduce_blocks(G, (G.nvox + 3) / 4), NT, 0, st>>>(G.nvox, I));
+           launch(k_elas32_update, reduce_blocks(G, (G.nvox + 3) / 4), NT, 0, st, G.nvox, I));
   return cudaGetLastError();
 }
 
 cudaError_t launch_elas32_scale_r(const Geo& G, const Elas32& I, cudaStream_t st) {
-  TG_TIMED(K_ELAS32_SCALE_R, st, k_elas32_scale_r<<<stream_blocks(G.nvox), NT, 0, st>>>(G.nvox, I));
+  TG_TIMED(K_ELAS32_SCALE_R, st, launch(k_elas32_scale_r, stream_blocks(G.nvox), NT, 0, st, G.nvox,
+                                        I));
   return cudaGetLastError();
 }
 
 cudaError_t launch_elas32_matvec_spec(const Geo& G, const Elas32& I, cudaStream_t st) {
   TG_TIMED(K_ELAS32_MATVEC_SPEC, st,
-           k_elas32_matvec_spec<<<G.grid, dim3(BX, BY), 0, st>>>(G, make_consts32(G), I));
+           launch(k_elas32_matvec_spec, G.grid, dim3(BX, BY), 0, st, G, make_consts32(G), I));
   return cudaGetLastError();
 }
 
 cudaError_t launch_elas32_update_spec(const Geo& G, const Elas32& I, cudaStream_t st) {
   TG_TIMED(K_ELAS32_UPDATE_SPEC, st,
-           k_elas32_update_spec<<<reduce_blocks(G, (G.nvox + 3) / 4), NT, 0, st>>>(G.nvox, I));
+           launch(k_elas32_update_spec, reduce_blocks(G, (G.nvox + 3) / 4), NT, 0, st, G.nvox, I));
   return cudaGetLastError();
 }
 
 cudaError_t launch_elas_ir_correct(const Geo& G, const Elas& E, const Elas32& I, cudaStream_t st) {
   TG_TIMED(K_ELAS_IR_CORRECT, st,
-           k_elas_ir_correct<<<stream_blocks(G.nvox), NT, 0, st>>>(G.nvox, E, I));
+           launch(k_elas_ir_correct, stream_blocks(G.nvox), NT, 0, st, G.nvox, E, I));
   return cudaGetLastError();
 }
 
 cudaError_t launch_elas_extrapolate(const Geo& G, const Elas& E, double dt, bool quadratic,
                                     cudaStream_t st) {
   TG_TIMED(K_ELAS_EXTRAPOLATE, st,
-           k_elas_extrapolate<<<stream_blocks(G.nvox), NT, 0, st>>>(G.nvox, E, dt,
-                                                                    quadratic ? 1 : 0));
+           launch(k_elas_extrapolate, stream_blocks(G.nvox), NT, 0, st, G.nvox, E, dt,
+                  quadratic ? 1 : 0));
   return cudaGetLastError();
 }
 
 cudaError_t launch_elas_ir_finish(const Geo& G, const Elas& E, double inv_dt, bool zero_rhs,
                                   cudaStream_t st) {
   TG_TIMED(K_ELAS_IR_FINISH, st,
-           k_elas_ir_finish<<<stream_blocks(G.nvox), NT, 0, st>>>(G.nvox, E, inv_dt, zero_rhs ? 1 : 0));
+           launch(k_elas_ir_finish, stream_blocks(G.nvox), NT, 0, st, G.nvox, E, inv_dt,
+                  zero_rhs ? 1 : 0));
   return cudaGetLastError();
 }
 
@@ -479,14 +479,14 @@ cudaError_t launch_sl32_pack(const Geo& G, const double* const v[3], const doubl
   Species6 qs;
   for (int s = 0; s < 6; ++s) qs.a[s] = q[s];
   TG_TIMED(K_SL32_PACK, st,
-           k_sl32_pack<<<G.grid, dim3(BX, BY), 0, st>>>(G, v[0], v[1], v[2], qs, S));
+           launch(k_sl32_pack, G.grid, dim3(BX, BY), 0, st, G, v[0], v[1], v[2], qs, S));
   return cudaGetLastError();
 }
 
 cudaError_t launch_sl32(const Geo& G, double dt, const Sl32& S, cudaStream_t st) {
   if (G.nvox >= (1LL << 31)) return cudaErrorInvalidValue;
   const float3 dth = make_float3((float)(dt / G.h[0]), (float)(dt / G.h[1]), (float)(dt / G.h[2]));
-  TG_TIMED(K_SL32, st, k_sl32<<<G.grid, dim3(BX, BY), 0, st>>>(G, (float)dt, dth, S));
+  TG_TIMED(K_SL32, st, launch(k_sl32, G.grid, dim3(BX, BY), 0, st, G, (float)dt, dth, S));
   return cudaGetLastError();
 }
 

@@ -88,7 +88,7 @@ __global__ void __launch_bounds__(NT) k_react(Geo G, DevParams P, double dt, int
   if (i >= G.nx || j >= G.ny) return;
   const int k0 = blockIdx.z * G.zc, k1 = min(G.nz, k0 + G.zc);
   for (int k = k0; k < k1; ++k) {
-    const long long c = ((long long)k * G.ny + j) * G.nx + i;
+    const int c = (k * G.ny + j) * G.nx + i;
     // S2 fix-up: the Crank-Nicolson increment of i comes out of g and w, in proportion (the
     // proportions in T: a relative error of ~1e-7 in them moves g and w by ~1e-7 of the small
     // increment)
@@ -169,7 +169,7 @@ __global__ void __launch_bounds__(NT, 4) k_react_f32(Geo G, DevParams P, float d
   const float hdt = 0.5f * dt;
   const RateParams32 Q(P);
   for (int k = k0; k < k1; ++k) {
-    const long long c = ((long long)k * G.ny + j) * G.nx + i;
+    const int c = (k * G.ny + j) * G.nx + i;
     const double y0 = p[c], y1 = ii[c], y2 = n[c], y3 = g[c], y4 = w[c];
     // S2 fix-up
     const float di = df_sub(df_split(single ? y0 : y1), df_split(i_dag[c])).hi;
@@ -241,7 +241,7 @@ __global__ void __launch_bounds__(NT) k_lame(Geo G, DevParams P, const double* _
   if (i >= G.nx || j >= G.ny) return;
   const int k0 = blockIdx.z * G.zc, k1 = min(G.nz, k0 + G.zc);
   for (int k = k0; k < k1; ++k) {
-    const long long c = ((long long)k * G.ny + j) * G.nx + i;
+    const int c = (k * G.ny + j) * G.nx + i;
     const double iota[5] = {p[c] + ii[c] + n[c], g[c], w[c], f[c], bg[c]};
     double smu = 0.0, slam = 0.0, seta = 0.0;
 #pragma unroll
@@ -284,7 +284,7 @@ __global__ void __launch_bounds__(NT) k_lame_df(Geo G, DevParams P, const double
   }
   const int k0 = blockIdx.z * G.zc, k1 = min(G.nz, k0 + G.zc);
   for (int k = k0; k < k1; ++k) {
-    const long long c = ((long long)k * G.ny + j) * G.nx + i;
+    const int c = (k * G.ny + j) * G.nx + i;
     const Df sp = df_split(p[c]), sn = df_split(n[c]);
     const Df iota[5] = {df_add_pos(df_add_pos(sp, df_split(ii[c])), sn), df_split(g[c]), df_split(w[c]),
                         df_split(f[c]), df_split(bg[c])};
@@ -317,12 +317,12 @@ cudaError_t launch_react(const Geo& G, const DevParams& P, double dt, const doub
   const int sg = single ? 1 : 0;
   if (fp32_rates)
     TG_TIMED(K_REACT, st,
-             k_react_f32<<<G.grid, dim3(BX, BY), 0, st>>>(G, P, (float)dt, sg, rho, i_dag, p, i, n,
-                                                          g, w, o, l));
+             launch(k_react_f32, G.grid, dim3(BX, BY), 0, st, G, P, (float)dt, sg, rho, i_dag, p,
+                    i, n, g, w, o, l));
   else
     TG_TIMED(K_REACT, st,
-             k_react<double><<<G.grid, dim3(BX, BY), 0, st>>>(G, P, dt, sg, rho, i_dag, p, i, n, g, w, o,
-                                                               l));
+             launch(k_react<double>, G.grid, dim3(BX, BY), 0, st, G, P, dt, sg, rho, i_dag, p, i,
+                    n, g, w, o, l));
   return cudaGetLastError();
 }
 
@@ -330,7 +330,7 @@ cudaError_t launch_lame(const Geo& G, const DevParams& P, const double* p, const
                         const double* n, const double* g, const double* w, const double* f,
                         const double* bg, double* mu, double* lam, double* eta, cudaStream_t st) {
   TG_TIMED(K_LAME, st,
-           k_lame<<<G.grid, dim3(BX, BY), 0, st>>>(G, P, p, i, n, g, w, f, bg, mu, lam, eta));
+           launch(k_lame, G.grid, dim3(BX, BY), 0, st, G, P, p, i, n, g, w, f, bg, mu, lam, eta));
   return cudaGetLastError();
 }
 
@@ -340,8 +340,8 @@ cudaError_t launch_lame_df(const Geo& G, const DevParams& P, const double* p, co
                            float* lam32, float* eta32, float2* mudf, float2* lamdf, float2* sdf,
                            cudaStream_t st) {
   TG_TIMED(K_LAME_DF, st,
-           k_lame_df<<<G.grid, dim3(BX, BY), 0, st>>>(G, P, p, i, n, g, w, f, bg, mu, lam, eta,
-                                                      mu32, lam32, eta32, mudf, lamdf, sdf));
+           launch(k_lame_df, G.grid, dim3(BX, BY), 0, st, G, P, p, i, n, g, w, f, bg, mu, lam, eta,
+                  mu32, lam32, eta32, mudf, lamdf, sdf));
   return cudaGetLastError();
 }
 

@@ -432,37 +432,38 @@ __device__ __forceinline__ bool spec_skip(const CgScal* S) {
   return S != nullptr && S->status != CG_RUNNING;
 }
 
-// Sum of one value per thread over a launch of any block size (a multiple of 32): warps,
-// then the block's warps in order into partial[b]; the last block to finish sums the
-// partials (each thread a fixed stride, then its warps in order: deterministic) and returns
-// true in thread 0 with the total.
-__device__ bool block_sum_last(double v, double* partial, unsigned int* counter, int b, int nb,
-                               double& total) {
-  __shared__ double sh[32];
-  __shared__ bool am_last;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  v = warp_sum(v);
-  if (lane == 0) sh[warp] = v;
+// Sum of one value per thread over a launch of any block size (a multiple of 32, at most NT),
+// as reduce_items of tg_internal.cuh but in two halves, so that the block's sum and its ticket
+// (an atomic's round trip to L2, some 700 clocks) run in warp 0 while the other warps go on
+// with the transform between the halves.  begin: one barrier; end: one barrier, true in thread
+// 0 of the last block, with the total.  The pass must not reuse B in between.
+struct BlockSum {
+  double sh[NT];
+  bool am_last;
+};
+__device__ __forceinline__ void block_sum_begin(BlockSum& B, double v, double* partial,
+                                                unsigned int* counter, int b, int nb) {
+  const int tid = threadIdx.x;
+  B.sh[tid] = v;
   __syncthreads();
-  if (threadIdx.x == 0) {
-    double s = 0.0;
-    for (int w = 0; w < nw; ++w) s += sh[w];
-    partial[b] = s;
-    __threadfence();
-    am_last = atomicAdd(counter, 1u) == (unsigned int)(nb - 1);
+  if (tid < 32) {
+    const double s = warp_sum_shared(B.sh, blockDim.x, tid);
+    if (tid == 0) {
+      partial[b] = s;
+      B.am_last = ticket_acq_rel(counter) == (unsigned int)(nb - 1);
+    }
   }
+}
+__device__ __forceinline__ bool block_sum_end(BlockSum& B, double* partial, unsigned int* counter,
+                                              int nb, double& total) {
+  const int tid = threadIdx.x, nt = blockDim.x;
   __syncthreads();
-  if (!am_last) return false;
-  __threadfence();
-  double s = 0.0;   // every thread a fixed stride of the partials, then warps in order
-  for (int k = threadIdx.x; k < nb; k += blockDim.x) s += __ldcg(partial + k);
-  s = warp_sum(s);
+  if (!B.am_last) return false;
+  B.sh[tid] = strided_partials(partial, 1, nb, tid, nt);
   __syncthreads();
-  if (lane == 0) sh[warp] = s;
-  __syncthreads();
-  if (threadIdx.x != 0) return false;
-  double t = 0.0;
-  for (int w = 0; w < nw; ++w) t += sh[w];
+  if (tid >= 32) return false;
+  const double t = warp_sum_shared(B.sh, nt, tid);
+  if (tid != 0) return false;
   total = t;
   *counter = 0u;
   return true;
@@ -608,14 +609,13 @@ __global__ void __launch_bounds__(NT, 4) k_spec_update_xfwd(Spec<float> V, Elas3
       }
     }
   }
-  double acc[1] = {(double)rr};
-  double out[1];
+  __shared__ BlockSum B;
   const int nb = gridDim.x * gridDim.y * gridDim.z;
   const int bl = (blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
-  if (reduce_indexed<1>(acc, V.partial, V.counter, bl, nb, out) && threadIdx.x == 0)
-    cg_after_update_rr(*I.S, out[0]);   // reduce_indexed's barriers also publish the staging
-  __syncthreads();
+  block_sum_begin(B, (double)rr, V.partial, V.counter, bl, nb);   // also publishes the staging
   x_fwd_finish<float, 0>(V, t, a, b, tw);   // two buffers (in place it ran slower)
+  double out;
+  if (block_sum_end(B, V.partial, V.counter, nb, out)) cg_after_update_rr(*I.S, out);
 }
 
 // ---------------------------------------------------------------------------- y pass
@@ -692,12 +692,15 @@ __global__ void __launch_bounds__(NT) k_spec_z(Spec<R> V, CgScal* S) {
       F[(size_t)kz * lw + q * tz + col] = zq;
     }
   }
+  __shared__ BlockSum B;
+  if (S != nullptr)
+    block_sum_begin(B, (double)rz_part, V.partial, V.counter,
+                    blockIdx.y * gridDim.x + blockIdx.x, gridDim.x * gridDim.y);
   __syncthreads();
   fft_to_global<+1>(F, other, io, 1, lw, ilog2(V.nz), ltz, 3, tw);
   if (S == nullptr) return;
   double out;
-  if (block_sum_last((double)rz_part, V.partial, V.counter, blockIdx.y * gridDim.x + blockIdx.x,
-                     gridDim.x * gridDim.y, out))
+  if (block_sum_end(B, V.partial, V.counter, gridDim.x * gridDim.y, out))
     cg_after_precond(*S, out);
 }
 
@@ -843,6 +846,10 @@ __global__ void __launch_bounds__(ZR_COLS * P, 512 / (ZR_COLS * P))
     }
   }
 
+  __shared__ BlockSum B;
+  if (S != nullptr)
+    block_sum_begin(B, (double)rz_part, V.partial, V.counter,
+                    blockIdx.y * gridDim.x + blockIdx.x, gridDim.x * gridDim.y);
   inverse(2);
 #pragma unroll
   for (int q = 0; q < 2; ++q) {
@@ -852,8 +859,7 @@ __global__ void __launch_bounds__(ZR_COLS * P, 512 / (ZR_COLS * P))
   }
   if (S == nullptr) return;
   double out;
-  if (block_sum_last((double)rz_part, V.partial, V.counter, blockIdx.y * gridDim.x + blockIdx.x,
-                     gridDim.x * gridDim.y, out))
+  if (block_sum_end(B, V.partial, V.counter, gridDim.x * gridDim.y, out))
     cg_after_precond(*S, out);
 }
 
@@ -1073,6 +1079,10 @@ __global__ void __launch_bounds__(ZR_COLS * P)
     }
   }
 
+  __shared__ BlockSum B;
+  if (S != nullptr)
+    block_sum_begin(B, (double)rz_part, V.partial, V.counter,
+                    blockIdx.y * gridDim.x + blockIdx.x, gridDim.x * gridDim.y);
 #pragma unroll 1
   for (int q = 0; q < 3; ++q) inverse(q);
   fence_proxy_async_smem();                    // the tile's writes, visible to the copies
@@ -1083,8 +1093,7 @@ __global__ void __launch_bounds__(ZR_COLS * P)
     bulk_commit_and_wait();
   }
   double out;
-  if (block_sum_last((double)rz_part, V.partial, V.counter, blockIdx.y * gridDim.x + blockIdx.x,
-                     gridDim.x * gridDim.y, out))
+  if (block_sum_end(B, V.partial, V.counter, gridDim.x * gridDim.y, out))
     cg_after_precond(*S, out);
 }
 
@@ -1266,7 +1275,7 @@ __global__ void __launch_bounds__(NT) k_spec_scale(long long n, Spec<R> V, Elas 
 
 }  // namespace
 
-// Every pass kernel may use up to the device's opt-in shared memory per block, less 1 KB for
+// Every pass kernel may use up to the device's opt-in shared memory per block, less 3 KB for
 // the kernels' static shared memory (the attribute is a limit, not a reservation), so
 // contexts of different grid sizes never lower it for one another; V's own needs must fit.
 template <typename R>
@@ -1275,7 +1284,7 @@ cudaError_t spec_prepare(const Spec<R>& V) {
   cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
   if (e != cudaSuccess) return e;
-  optin -= 1024;
+  optin -= 3072;
   if (spec_smem_x2(V) > (size_t)optin || spec_smem_y(V) > (size_t)optin ||
       spec_smem_z(V) > (size_t)optin)
     return cudaErrorInvalidValue;
@@ -1329,14 +1338,14 @@ cudaError_t launch_spec_scale(const Geo& G, const Spec<R>& V, const Elas& E, cud
   const long long want = (G.nvox + NT - 1) / NT;
   const int blocks = (int)(want < 4096 ? (want > 0 ? want : 1) : 4096);
   TG_TIMED(K_SPEC_SCALE, st,
-           k_spec_scale<R><<<blocks, NT, 0, st>>>(G.nvox, V, E, G.ih2[0], G.ih2[1], G.ih2[2]));
+           launch(k_spec_scale<R>, blocks, NT, 0, st, G.nvox, V, E, G.ih2[0], G.ih2[1], G.ih2[2]));
   return cudaGetLastError();
 }
 
 template <typename R>
 cudaError_t launch_spec_tables(const Spec<R>& V, const double h[3], cudaStream_t st) {
   const int nmax = max(V.nx, max(V.ny, V.nz));
-  k_spec_tables<R><<<dim3((nmax + 127) / 128, 3), 128, 0, st>>>(V, h[0], h[1], h[2]);
+  launch(k_spec_tables<R>, dim3((nmax + 127) / 128, 3), 128, 0, st, V, h[0], h[1], h[2]);
   return cudaGetLastError();
 }
 
@@ -1347,10 +1356,11 @@ cudaError_t launch_spec_mean(long long n, const double* mu, const double* lam,
   const int blocks = (int)(want < 1024 ? (want > 0 ? want : 1) : 1024);
   if (fp32_terms)
     TG_TIMED(K_SPEC_MEAN, st,
-             k_spec_mean<true><<<blocks, NT, 0, st>>>(n, mu, lam, eta, mean, partial, counter));
+             launch(k_spec_mean<true>, blocks, NT, 0, st, n, mu, lam, eta, mean, partial, counter));
   else
     TG_TIMED(K_SPEC_MEAN, st,
-             k_spec_mean<false><<<blocks, NT, 0, st>>>(n, mu, lam, eta, mean, partial, counter));
+             launch(k_spec_mean<false>, blocks, NT, 0, st, n, mu, lam, eta, mean, partial,
+                    counter));
   return cudaGetLastError();
 }
 
@@ -1365,23 +1375,23 @@ void launch_spec_z(const Spec<R>& V, CgScal* S, cudaStream_t st) {
       const CUtensorMap& map = *static_cast<const CUtensorMap*>(V.zmap);
       if (V.nz == 256)
         TG_TIMED(K_SPEC_ZR, st,
-                 k_spec_zr_tma<16><<<g, 16 * ZR_COLS, spec_smem_zr_tma<16>(), st>>>(map, V, S));
+                 launch(k_spec_zr_tma<16>, g, 16 * ZR_COLS, spec_smem_zr_tma<16>(), st, map, V, S));
       else
         TG_TIMED(K_SPEC_ZR, st,
-                 k_spec_zr_tma<8><<<g, 8 * ZR_COLS, spec_smem_zr_tma<8>(), st>>>(map, V, S));
+                 launch(k_spec_zr_tma<8>, g, 8 * ZR_COLS, spec_smem_zr_tma<8>(), st, map, V, S));
       return;
     }
     if (V.nz == 256) {
-      TG_TIMED(K_SPEC_ZR, st, k_spec_zr<16><<<g, 16 * ZR_COLS, spec_smem_zr<16>(), st>>>(V, S));
+      TG_TIMED(K_SPEC_ZR, st, launch(k_spec_zr<16>, g, 16 * ZR_COLS, spec_smem_zr<16>(), st, V, S));
       return;
     }
     if (V.nz == 128) {
-      TG_TIMED(K_SPEC_ZR, st, k_spec_zr<8><<<g, 8 * ZR_COLS, spec_smem_zr<8>(), st>>>(V, S));
+      TG_TIMED(K_SPEC_ZR, st, launch(k_spec_zr<8>, g, 8 * ZR_COLS, spec_smem_zr<8>(), st, V, S));
       return;
     }
   }
   const dim3 gz((V.nxh + V.tz - 1) / V.tz, V.ny);
-  TG_TIMED(K_SPEC_Z, st, k_spec_z<R><<<gz, V.nt_z, spec_smem_z(V), st>>>(V, S));
+  TG_TIMED(K_SPEC_Z, st, launch(k_spec_z<R>, gz, V.nt_z, spec_smem_z(V), st, V, S));
 }
 
 template <typename R>
@@ -1390,25 +1400,28 @@ cudaError_t launch_spectral(const Spec<R>& V, const R* const r[3], R* const z[3]
   const dim3 gx(V.ny / (2 * V.pb), V.nz, 3);
   const dim3 gy((V.nxh + V.tx - 1) / V.tx, V.nz, 3);
   TG_TIMED(K_SPEC_X_FWD, st,
-           k_spec_x_fwd<R><<<gx, NT, spec_smem_x(V), st>>>(V, r[0], r[1], r[2], S));
-  TG_TIMED(K_SPEC_Y_FWD, st, k_spec_y<R, -1><<<gy, NT, spec_smem_y(V), st>>>(V, S));
+           launch(k_spec_x_fwd<R>, gx, NT, spec_smem_x(V), st, V, r[0], r[1], r[2], S));
+  TG_TIMED(K_SPEC_Y_FWD, st, launch((k_spec_y<R, -1>), gy, NT, spec_smem_y(V), st, V, S));
   launch_spec_z(V, S, st);
-  TG_TIMED(K_SPEC_Y_INV, st, k_spec_y<R, +1><<<gy, NT, spec_smem_y(V), st>>>(V, S));
+  TG_TIMED(K_SPEC_Y_INV, st, launch((k_spec_y<R, +1>), gy, NT, spec_smem_y(V), st, V, S));
   PUpd<R> P = {};
   if constexpr (sizeof(R) == 4) {
     if (pu) {
       P = *pu;
       if (V.x_inpl)
         TG_TIMED(K_SPEC_X_INV_P, st,
-                 k_spec_x_inv<R, true, 1><<<gx, NT, spec_smem_x(V), st>>>(V, z[0], z[1], z[2], S, P));
+                 launch((k_spec_x_inv<R, true, 1>), gx, NT, spec_smem_x(V), st, V, z[0], z[1],
+                        z[2], S, P));
       else
         TG_TIMED(K_SPEC_X_INV_P, st,
-                 k_spec_x_inv<R, true, 0><<<gx, NT, spec_smem_x(V), st>>>(V, z[0], z[1], z[2], S, P));
+                 launch((k_spec_x_inv<R, true, 0>), gx, NT, spec_smem_x(V), st, V, z[0], z[1],
+                        z[2], S, P));
       return cudaGetLastError();
     }
   }
   TG_TIMED(K_SPEC_X_INV, st,
-           k_spec_x_inv<R, false, 2><<<gx, NT, spec_smem_x(V), st>>>(V, z[0], z[1], z[2], S, P));
+           launch((k_spec_x_inv<R, false, 2>), gx, NT, spec_smem_x(V), st, V, z[0], z[1], z[2], S,
+                  P));
   return cudaGetLastError();
 }
 
@@ -1418,19 +1431,21 @@ cudaError_t launch_spectral_update(const Spec<float>& V, const Elas32& I, float*
                                    cudaStream_t st) {
   const dim3 gx(V.ny / (2 * V.pb), V.nz, 3);
   const dim3 gy((V.nxh + V.tx - 1) / V.tx, V.nz, 3);
-  TG_TIMED(K_SPEC_UPDATE_XFWD, st, k_spec_update_xfwd<<<gx, NT, spec_smem_x2(V), st>>>(V, I));
-  TG_TIMED(K_SPEC_Y_FWD, st, k_spec_y<float, -1><<<gy, NT, spec_smem_y(V), st>>>(V, I.S));
+  TG_TIMED(K_SPEC_UPDATE_XFWD, st, launch(k_spec_update_xfwd, gx, NT, spec_smem_x2(V), st, V, I));
+  TG_TIMED(K_SPEC_Y_FWD, st, launch((k_spec_y<float, -1>), gy, NT, spec_smem_y(V), st, V, I.S));
   launch_spec_z(V, I.S, st);
-  TG_TIMED(K_SPEC_Y_INV, st, k_spec_y<float, +1><<<gy, NT, spec_smem_y(V), st>>>(V, I.S));
+  TG_TIMED(K_SPEC_Y_INV, st, launch((k_spec_y<float, +1>), gy, NT, spec_smem_y(V), st, V, I.S));
   PUpd<float> P;   // p = z + beta p_old straight from the last pass
   for (int b = 0; b < 2; ++b)
     for (int a = 0; a < 3; ++a) P.p[b][a] = I.p[b][a];
   if (V.x_inpl)
     TG_TIMED(K_SPEC_X_INV_P, st,
-             k_spec_x_inv<float, true, 1><<<gx, NT, spec_smem_x(V), st>>>(V, z[0], z[1], z[2], I.S, P));
+             launch((k_spec_x_inv<float, true, 1>), gx, NT, spec_smem_x(V), st, V, z[0], z[1],
+                    z[2], I.S, P));
   else
     TG_TIMED(K_SPEC_X_INV_P, st,
-             k_spec_x_inv<float, true, 0><<<gx, NT, spec_smem_x(V), st>>>(V, z[0], z[1], z[2], I.S, P));
+             launch((k_spec_x_inv<float, true, 0>), gx, NT, spec_smem_x(V), st, V, z[0], z[1],
+                    z[2], I.S, P));
   return cudaGetLastError();
 }
 

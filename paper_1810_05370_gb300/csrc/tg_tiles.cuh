@@ -487,7 +487,7 @@ __device__ __forceinline__ void elas_ir_residual_tile(const Geo& G, const Elas& 
     const int k0 = bz * G.zc, k1 = min(G.nz, k0 + G.zc);
     for (int k = k0; k < k1; ++k) {
       const Nbr nb = make_nbr(G, i, j, k);
-      const long long c = nb.at(0, 0, 0);
+      const int c = nb.at(0, 0, 0);
       double Au[3];
       Au[0] = elas_row64<0>(G, nb, c, E, u);
       Au[1] = elas_row64<1>(G, nb, c, E, u);
@@ -534,7 +534,7 @@ __device__ __forceinline__ Df elas_mixed_cs(const Nbr& nb, const float2* __restr
 
 // component A of rhs - (eta I - L_h) u at node c
 template <int A>
-__device__ __forceinline__ Df elas_res_row_cs(const Nbr& nb, long long c, const Elas& E,
+__device__ __forceinline__ Df elas_res_row_cs(const Nbr& nb, int c, const Elas& E,
                                               const Df (&sc)[3][3], Df rhs) {
   constexpr int D1 = (A + 1) % 3, D2 = (A + 2) % 3;
   const float2* __restrict__ xa = E.udf[A];
@@ -580,7 +580,7 @@ __device__ __forceinline__ void elas_ir_residual_tile_df(const Geo& G, const Ela
     const int k0 = bz * G.zc, k1 = min(G.nz, k0 + G.zc);
     for (int k = k0; k < k1; ++k) {
       const Nbr nb = make_nbr(G, i, j, k);
-      const long long c = nb.at(0, 0, 0);
+      const int c = nb.at(0, 0, 0);
       Df rhs[3];
 #pragma unroll
       for (int a = 0; a < 3; ++a) {
@@ -627,15 +627,14 @@ __device__ __forceinline__ void elas_ir_residual_finalize(CgScal& O, CgScal& S, 
     O.status = CG_ZERO_RHS;
   } else if (!isfinite(rr)) {
     O.status = CG_NONFINITE;
-  } else if (sqrt(rr) <= O.rtol * sqrt(bb)) {
+  } else if (cg_norm_met(rr, O.rtol, bb)) {
     O.status = CG_CONVERGED;
   } else if (O.it > max_sweeps || O.pad >= O.maxit) {
     O.status = CG_MAXIT;
   } else {
     O.status = CG_RUNNING;
   }
-  const double s =
-      (normalize && rr > 0.0 && isfinite(rr)) ? exp2(-rint(0.5 * log2(rr))) : 1.0;
+  const double s = (normalize && rr > 0.0 && isfinite(rr)) ? pow2_inv_root(rr) : 1.0;
   S.scale = s;
   S.bb = rr * s * s;
   S.rr = rr * s * s;
@@ -672,7 +671,7 @@ struct Faces {
   double xp, xm, yp, ym, zp, zm;
 };
 
-__device__ __forceinline__ Faces load_faces(const Cn3& C, const Nbr& nb, long long c) {
+__device__ __forceinline__ Faces load_faces(const Cn3& C, const Nbr& nb, int c) {
   Faces F;
   F.xp = C.Kf[0][c];
   F.xm = C.Kf[0][nb.at(-1, 0, 0)];
@@ -693,7 +692,7 @@ __device__ __forceinline__ void cn_init_tile(const Geo& G, const Cn3& C, int bx,
   const int k0 = bz * G.zc, k1 = min(G.nz, k0 + G.zc);
   for (int k = k0; k < k1; ++k) {
     const Nbr nb = make_nbr(G, i, j, k);
-    const long long c = nb.at(0, 0, 0);
+    const int c = nb.at(0, 0, 0);
     const Faces F = load_faces(C, nb, c);
     const double di = C.dinv[c];
 #pragma unroll
@@ -726,7 +725,7 @@ __device__ __forceinline__ void cn_matvec_tile(const Geo& G, const Cn3& C, const
   const int k0 = bz * G.zc, k1 = min(G.nz, k0 + G.zc);
   for (int k = k0; k < k1; ++k) {
     const Nbr nb = make_nbr(G, i, j, k);
-    const long long c = nb.at(0, 0, 0);
+    const int c = nb.at(0, 0, 0);
     const Faces F = load_faces(C, nb, c);
     const double d = C.dsum[c];
 #pragma unroll
@@ -752,7 +751,7 @@ __device__ __forceinline__ void cn_update_tile(const Geo& G, const Cn3& C, const
   if (i >= G.nx || j >= G.ny) return;
   const int k0 = bz * G.zc, k1 = min(G.nz, k0 + G.zc);
   for (int k = k0; k < k1; ++k) {
-    const long long c = ((long long)k * G.ny + j) * G.nx + i;
+    const int c = (k * G.ny + j) * G.nx + i;
     const double di = C.dinv[c];
 #pragma unroll
     for (int r = 0; r < 3; ++r) {
@@ -774,7 +773,7 @@ __device__ __forceinline__ void cn_pupdate_tile(const Geo& G, const Cn3& C, cons
   if (i >= G.nx || j >= G.ny) return;
   const int k0 = bz * G.zc, k1 = min(G.nz, k0 + G.zc);
   for (int k = k0; k < k1; ++k) {
-    const long long c = ((long long)k * G.ny + j) * G.nx + i;
+    const int c = (k * G.ny + j) * G.nx + i;
     const double di = C.dinv[c];
 #pragma unroll
     for (int r = 0; r < 3; ++r)

@@ -94,7 +94,7 @@ __global__ void __launch_bounds__(NT) k_sl(Geo G, double dt, double3 dt_h,
   if (i >= G.nx || j >= G.ny) return;
   const int k0 = blockIdx.z * G.zc, k1 = min(G.nz, k0 + G.zc);
   for (int k = k0; k < k1; ++k) {
-    const long long c = ((long long)k * G.ny + j) * G.nx + i;
+    const int c = (k * G.ny + j) * G.nx + i;
     const double v0x = vx[c], v0y = vy[c], v0z = vz[c];
     Tricubic T;
     setup(T, G, i - v0x * dt_h.x, j - v0y * dt_h.y, k - v0z * dt_h.z);
@@ -119,7 +119,7 @@ __global__ void __launch_bounds__(NT) k_sl(Geo G, double dt, double3 dt_h,
 
 cudaError_t launch_divergence(const Geo& G, const double* const v[3], double* div, cudaStream_t st) {
   TG_TIMED(K_DIVERGENCE, st,
-           k_divergence<<<G.grid, dim3(BX, BY), 0, st>>>(G, v[0], v[1], v[2], div));
+           launch(k_divergence, G.grid, dim3(BX, BY), 0, st, G, v[0], v[1], v[2], div));
   return cudaGetLastError();
 }
 
@@ -133,7 +133,7 @@ cudaError_t launch_sl_advect(const Geo& G, double dt, const double* const v[3], 
   }
   const double3 dth = make_double3(dt / G.h[0], dt / G.h[1], dt / G.h[2]);
   TG_TIMED(K_SL, st,
-           k_sl<<<G.grid, dim3(BX, BY), 0, st>>>(G, dt, dth, v[0], v[1], v[2], div, a, b));
+           launch(k_sl, G.grid, dim3(BX, BY), 0, st, G, dt, dth, v[0], v[1], v[2], div, a, b));
   return cudaGetLastError();
 }
 
