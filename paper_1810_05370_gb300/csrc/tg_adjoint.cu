@@ -35,6 +35,7 @@ __device__ void add_theta(double (&v)[NV], const int (&slot)[NV], const AdjView&
 // rhs = lambda_u + lambda_v / dt (for S6^T), lambda_u^n = -lambda_v / dt; copy the incoming
 // lambdas of the reacted species and of f+ to scratch.
 __global__ void __launch_bounds__(NT) k_adj_prep(long long n, AdjView A, double inv_dt) {
+  pdl_sync();
   const long long stride = (long long)gridDim.x * blockDim.x;
   for (long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x; c < n; c += stride) {
 #pragma unroll
@@ -69,6 +70,7 @@ __global__ void __launch_bounds__(NT) k_adj_elas_coef(Geo G, DevParams P, AdjVie
                                                       const double* __restrict__ p,
                                                       const double* __restrict__ nn,
                                                       double inv_Escale, int species) {
+  pdl_sync();
   const int i = blockIdx.x * BX + threadIdx.x;
   const int j = blockIdx.y * BY + threadIdx.y;
   double acc[1] = {0.0};
@@ -250,6 +252,7 @@ __device__ __forceinline__ void species_rates_f(const DevParams& P, double rho, 
 
 __global__ void __launch_bounds__(NT) k_adj_react(Geo G, DevParams P, double dt, AdjView A,
                                                   TapeView T, const double* __restrict__ rho) {
+  pdl_sync();
   const int i = blockIdx.x * BX + threadIdx.x;
   const int j = blockIdx.y * BY + threadIdx.y;
   double acc[3] = {0.0, 0.0, 0.0};   // rho, o_hyp, o_inv
@@ -368,6 +371,7 @@ __device__ __forceinline__ double nodeK_raw(const DevParams& P, double g, double
 // transport adjoint scatters into them.
 __global__ void __launch_bounds__(NT) k_adj_cn_post(Geo G, DevParams P, double half_dt, AdjView A,
                                                     TapeView T) {
+  pdl_sync();
   const int i = blockIdx.x * BX + threadIdx.x;
   const int j = blockIdx.y * BY + threadIdx.y;
   double acc[1] = {0.0};
@@ -433,6 +437,7 @@ __global__ void __launch_bounds__(NT) k_adj_cn_post(Geo G, DevParams P, double h
 
 // CN adjoint solve start: x = 0, r = rhs, p = D^{-1} r
 __global__ void __launch_bounds__(NT) k_cn_init_rhs(Geo G, Cn3 C, AdjView A) {
+  pdl_sync();
   const int i = blockIdx.x * BX + threadIdx.x;
   const int j = blockIdx.y * BY + threadIdx.y;
   double acc[9];
@@ -555,6 +560,7 @@ __device__ __forceinline__ void cub_scatter(const Cub& C, double* const* tgt, co
 
 __global__ void __launch_bounds__(NT) k_adj_sl(Geo G, double dt, double3 dt_h, AdjView A,
                                                TapeView T, const double* __restrict__ div) {
+  pdl_sync();
   const int i = blockIdx.x * BX + threadIdx.x;
   const int j = blockIdx.y * BY + threadIdx.y;
   if (i >= G.nx || j >= G.ny) return;
@@ -622,6 +628,7 @@ __global__ void __launch_bounds__(NT) k_adj_sl(Geo G, double dt, double3 dt_h, A
 
 // lambda_v^n = (scattered part) + div_h^T lambda_delta = LV - D lambda_delta
 __global__ void __launch_bounds__(NT) k_adj_div(Geo G, AdjView A) {
+  pdl_sync();
   const int i = blockIdx.x * BX + threadIdx.x;
   const int j = blockIdx.y * BY + threadIdx.y;
   if (i >= G.nx || j >= G.ny) return;

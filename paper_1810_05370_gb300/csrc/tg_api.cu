@@ -360,6 +360,7 @@ DevParams make_dev_params(const tg_params* p) {
 }
 
 __global__ void k_cg_reset(CgScal* S, int count, double rtol, int maxit) {
+  pdl_sync();
   const int t = threadIdx.x;
   if (t < count) {
     CgScal s = {};

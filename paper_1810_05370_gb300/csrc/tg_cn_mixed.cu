@@ -16,6 +16,7 @@ namespace {
 __global__ void __launch_bounds__(NT) k_cn_ir_residual(Geo G, Cn3 C, Cn32 I, CgScal* Sout,
                                                        int init, double tau_min,
                                                        int max_sweeps, int mask) {
+  pdl_sync();
   double acc[9];
 #pragma unroll
   for (int q = 0; q < 9; ++q) acc[q] = 0.0;
@@ -75,6 +76,7 @@ __global__ void __launch_bounds__(NT) k_cn_ir_residual(Geo G, Cn3 C, Cn32 I, CgS
 __global__ void __launch_bounds__(NT) k_cn_ir_residual_df(Geo G, Cn3 C, Cn32 I, CgScal* Sout,
                                                           int init, double tau_min,
                                                           int max_sweeps, int mask) {
+  pdl_sync();
   float sbb[3] = {0.0f, 0.0f, 0.0f}, srr[3] = {0.0f, 0.0f, 0.0f}, srz[3] = {0.0f, 0.0f, 0.0f};
   const int i = blockIdx.x * BX + threadIdx.x;
   const int j = blockIdx.y * BY + threadIdx.y;
@@ -153,6 +155,7 @@ __device__ __forceinline__ bool active3(const Cn32& I, bool (&act)[3]) {
 
 // q = A p (diagonal 1 + sum of the six faces), <p, q>
 __global__ void __launch_bounds__(NT) k_cn32_matvec(Geo G, Cn32 I) {
+  pdl_sync();
   bool act[3];
   if (!active3(I, act)) return;
   float part[3] = {0.0f, 0.0f, 0.0f};
@@ -210,6 +213,7 @@ constexpr int MV_CELLS = MV_X * MV_Y;
 
 __global__ void __launch_bounds__(MV_CELLS, 2) k_cn32_matvec_neu(Geo G, Cn32 I, int r0, int r1,
                                                                  int zc) {
+  pdl_sync();
   const bool run0 = r0 >= 0 && I.S[r0].status == CG_RUNNING;
   const bool run1 = r1 >= 0 && I.S[r1].status == CG_RUNNING;
   if (!run0 && !run1) return;
@@ -336,6 +340,7 @@ __global__ void __launch_bounds__(MV_CELLS, 2) k_cn32_matvec_neu(Geo G, Cn32 I, 
 // the next iteration's preconditioner kernel forms <r, z> and beta.
 template <bool NEU>
 __global__ void __launch_bounds__(NT) k_cn32_update(long long n, Cn32 I) {
+  pdl_sync();
   bool act[3];
   if (!active3(I, act)) return;
   float alpha[3];
@@ -400,6 +405,7 @@ __global__ void __launch_bounds__(NT) k_cn32_update(long long n, Cn32 I) {
 // (Jacobi) or the polynomial preconditioner's output I.z (NEU)
 template <bool NEU>
 __global__ void __launch_bounds__(NT) k_cn32_pupdate(long long n, Cn32 I) {
+  pdl_sync();
   bool act[3];
   if (!active3(I, act)) return;
   float beta[3];
@@ -486,6 +492,7 @@ struct NmTile {
 
 __global__ void __launch_bounds__(NM_CELLS, 1) k_cn32_neumann(Geo G, Cn32 I, int r0, int r1,
                                                               int zc) {
+  pdl_sync();
   const bool run0 = r0 >= 0 && I.S[r0].status == CG_RUNNING;
   const bool run1 = r1 >= 0 && I.S[r1].status == CG_RUNNING;
   if (!run0 && !run1) return;
@@ -666,6 +673,7 @@ __global__ void __launch_bounds__(NM_CELLS, 1) k_cn32_neumann(Geo G, Cn32 I, int
 
 // x += e in FP64 for the solves in the mask (e = 0 for those that did not run this sweep)
 __global__ void __launch_bounds__(NT) k_cn_ir_correct(long long n, Cn3 C, Cn32 I, int mask) {
+  pdl_sync();
   const long long stride = (long long)gridDim.x * blockDim.x;
   for (long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x; c < n; c += stride) {
 #pragma unroll

@@ -63,6 +63,7 @@ __device__ bool ox_reduce(const OxDf& O, const Df (&acc)[NV], double (&out)[NV])
 }
 
 __global__ void __launch_bounds__(NT) k_ox_prep(Geo G, OxDf O) {
+  pdl_sync();
   const int i = blockIdx.x * BX + threadIdx.x;
   const int j = blockIdx.y * BY + threadIdx.y;
   if (i >= G.nx || j >= G.ny) return;
@@ -83,6 +84,7 @@ __global__ void __launch_bounds__(NT) k_ox_prep(Geo G, OxDf O) {
 // rhs = x + s, r = 2 s (s = sum over faces of a (x_n - x_c)), p = D^{-1} r; (|rhs|^2, |r|^2,
 // <r, D^{-1} r>)
 __global__ void __launch_bounds__(NT) k_ox_init(Geo G, OxDf O) {
+  pdl_sync();
   Df acc[3] = {{0.0f, 0.0f}, {0.0f, 0.0f}, {0.0f, 0.0f}};
   const int i = blockIdx.x * BX + threadIdx.x;
   const int j = blockIdx.y * BY + threadIdx.y;
@@ -116,6 +118,7 @@ __global__ void __launch_bounds__(NT) k_ox_init(Geo G, OxDf O) {
 
 // q = d p - sum over faces of a p_n, <p, q>, alpha = rz / <p, q>
 __global__ void __launch_bounds__(NT) k_ox_matvec(Geo G, OxDf O) {
+  pdl_sync();
   if (O.S->status != CG_RUNNING) return;
   Df acc[1] = {{0.0f, 0.0f}};
   const int i = blockIdx.x * BX + threadIdx.x;
@@ -147,6 +150,7 @@ __global__ void __launch_bounds__(NT) k_ox_matvec(Geo G, OxDf O) {
 
 // x += alpha p, r -= alpha q; <r, D^{-1} r>, <r, r>; beta and the convergence test
 __global__ void __launch_bounds__(NT) k_ox_update(Geo G, OxDf O) {
+  pdl_sync();
   if (O.S->status != CG_RUNNING) return;
   const Df a = df_split(O.S->alpha);
   Df acc[2] = {{0.0f, 0.0f}, {0.0f, 0.0f}};
@@ -170,6 +174,7 @@ __global__ void __launch_bounds__(NT) k_ox_update(Geo G, OxDf O) {
 
 // p = D^{-1} r + beta p
 __global__ void __launch_bounds__(NT) k_ox_pupdate(Geo G, OxDf O) {
+  pdl_sync();
   if (O.S->status != CG_RUNNING) return;
   const Df b = df_split(O.S->beta);
   const int i = blockIdx.x * BX + threadIdx.x;
@@ -184,6 +189,7 @@ __global__ void __launch_bounds__(NT) k_ox_pupdate(Geo G, OxDf O) {
 
 // o = x (a vanishing right-hand side: o = 0)
 __global__ void __launch_bounds__(NT) k_ox_finish(Geo G, OxDf O) {
+  pdl_sync();
   const bool zero = O.S->status == CG_ZERO_RHS;
   const int i = blockIdx.x * BX + threadIdx.x;
   const int j = blockIdx.y * BY + threadIdx.y;

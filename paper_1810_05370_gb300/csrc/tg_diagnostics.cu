@@ -39,6 +39,7 @@ __device__ __forceinline__ void identity(double (&a)[NQ]) {
 }
 
 __global__ void __launch_bounds__(NT) k_diagnostics(Geo G, DiagArgs A) {
+  pdl_sync();
   double acc[NQ];
   identity(acc);
   const int i = blockIdx.x * BX + threadIdx.x;

@@ -33,6 +33,7 @@ __global__ void __launch_bounds__(NT) k_diff_faces(Geo G, DevParams P, double ha
                                                    const double* __restrict__ f, double* Kfx,
                                                    double* Kfy, double* Kfz, double* rho,
                                                    float2* dfx, float2* dfy, float2* dfz) {
+  pdl_sync();
   const int i = blockIdx.x * BX + threadIdx.x;
   const int j = blockIdx.y * BY + threadIdx.y;
   if (i >= G.nx || j >= G.ny) return;
@@ -70,6 +71,7 @@ __global__ void __launch_bounds__(NT) k_diff_node_df(Geo G, DevParams P,
                                                      const double* __restrict__ w,
                                                      const double* __restrict__ f, float2* Kn,
                                                      double* rho) {
+  pdl_sync();
   const int i = blockIdx.x * BX + threadIdx.x;
   const int j = blockIdx.y * BY + threadIdx.y;
   if (i >= G.nx || j >= G.ny) return;
@@ -104,6 +106,7 @@ __global__ void __launch_bounds__(NT) k_diff_faces_df(Geo G, Df sx, Df sy, Df sz
                                                       float2* dfx, float2* dfy, float2* dfz,
                                                       float* f32x, float* f32y, float* f32z,
                                                       float* dinv32, float* dmax) {
+  pdl_sync();
   const int i = blockIdx.x * BX + threadIdx.x;
   const int j = blockIdx.y * BY + threadIdx.y;
   float dm = 0.0f;   // the largest diagonal this thread formed
@@ -150,6 +153,7 @@ __global__ void __launch_bounds__(NT) k_diff_diag(Geo G, const double* __restric
                                                   const double* __restrict__ Kfy,
                                                   const double* __restrict__ Kfz, double* dsum,
                                                   double* dinv) {
+  pdl_sync();
   const int i = blockIdx.x * BX + threadIdx.x;
   const int j = blockIdx.y * BY + threadIdx.y;
   if (i >= G.nx || j >= G.ny) return;
@@ -166,6 +170,7 @@ __global__ void __launch_bounds__(NT) k_diff_diag(Geo G, const double* __restric
 
 // mask: bit r set for the solves to start; the others are marked finished
 __global__ void __launch_bounds__(NT) k_cn_init(Geo G, Cn3 C, int mask) {
+  pdl_sync();
   double acc[9];
 #pragma unroll
   for (int q = 0; q < 9; ++q) acc[q] = 0.0;
@@ -183,6 +188,7 @@ __global__ void __launch_bounds__(NT) k_cn_init(Geo G, Cn3 C, int mask) {
 }
 
 __global__ void __launch_bounds__(NT) k_cn_matvec(Geo G, Cn3 C) {
+  pdl_sync();
   bool act[3];
   bool any = false;
 #pragma unroll
@@ -209,6 +215,7 @@ __global__ void __launch_bounds__(NT) k_cn_matvec(Geo G, Cn3 C) {
 // their last block takes its decision, so a finished solve's blocks leave at once.  Bound by
 // the FP64 pipe (5 operations per voxel and solve) and HBM alike.
 __global__ void __launch_bounds__(NT) k_cn_update(long long n, Cn3 C) {
+  pdl_sync();
   const int s = blockIdx.y;
   if (C.S[s].status != CG_RUNNING) return;
   const double alpha = C.S[s].alpha;
@@ -245,6 +252,7 @@ __global__ void __launch_bounds__(NT) k_cn_update(long long n, Cn3 C) {
 }
 
 __global__ void __launch_bounds__(NT) k_cn_pupdate(long long n, Cn3 C) {
+  pdl_sync();
   const int s = blockIdx.y;
   if (C.S[s].status != CG_RUNNING) return;
   const double beta = C.S[s].beta;

@@ -20,6 +20,7 @@ namespace {
 __global__ void __launch_bounds__(NT) k_elas_coef(Geo G, DevParams P, Elas E,
                                                   const double* __restrict__ p,
                                                   const double* __restrict__ n, int force) {
+  pdl_sync();
   const int i = blockIdx.x * BX + threadIdx.x;
   const int j = blockIdx.y * BY + threadIdx.y;
   if (i >= G.nx || j >= G.ny) return;
@@ -85,6 +86,7 @@ __global__ void __launch_bounds__(NT) k_elas_coef(Geo G, DevParams P, Elas E,
 // FP32 inverse diagonal.
 __global__ void __launch_bounds__(NT, 4) k_elas_coef_df(Geo G, DevParams P, Elas E, Elas32 I,
                                                      const float2* __restrict__ sdf, int force) {
+  pdl_sync();
   const int i = blockIdx.x * BX + threadIdx.x;
   const int j = blockIdx.y * BY + threadIdx.y;
   if (i >= G.nx || j >= G.ny) return;
@@ -143,6 +145,7 @@ __global__ void __launch_bounds__(NT, 4) k_elas_coef_df(Geo G, DevParams P, Elas
 // preconditioner runs in separate kernels afterwards: only r, du and the norms here.
 template <bool SPEC>
 __global__ void __launch_bounds__(NT) k_elas_init(Geo G, Elas E, int minus_b) {
+  pdl_sync();
   const double* const u[3] = {E.u[0], E.u[1], E.u[2]};
   const int i = blockIdx.x * BX + threadIdx.x;
   const int j = blockIdx.y * BY + threadIdx.y;
@@ -179,6 +182,7 @@ __global__ void __launch_bounds__(NT) k_elas_init(Geo G, Elas E, int minus_b) {
 }
 
 __global__ void __launch_bounds__(NT, 3) k_elas_matvec(Geo G, Elas E) {
+  pdl_sync();
   if (E.S->status != CG_RUNNING) return;
   const double* const p[3] = {E.p[0], E.p[1], E.p[2]};
   const int i = blockIdx.x * BX + threadIdx.x;
@@ -212,6 +216,7 @@ __global__ void __launch_bounds__(NT, 3) k_elas_matvec(Geo G, Elas E) {
 // its own (2160 blocks at 96 x 80 x 72).  Workspace arrays start on 256-byte boundaries.
 template <bool SPEC>
 __global__ void __launch_bounds__(NT) k_elas_update(long long n, Elas E) {
+  pdl_sync();
   if (E.S->status != CG_RUNNING) return;
   const double alpha = E.S->alpha;
   const int a = blockIdx.y;
@@ -254,6 +259,7 @@ __global__ void __launch_bounds__(NT) k_elas_update(long long n, Elas E) {
 // the first iteration); flat as the update
 template <bool SPEC>
 __global__ void __launch_bounds__(NT) k_elas_pupdate(long long n, Elas E) {
+  pdl_sync();
   if (E.S->status != CG_RUNNING) return;
   const double beta = E.S->beta;
   const bool first = SPEC && E.S->it == 0;
@@ -282,6 +288,7 @@ __global__ void __launch_bounds__(NT) k_elas_pupdate(long long n, Elas E) {
 // keeps v^n in vp before writing v^{n+1}.
 __global__ void __launch_bounds__(NT) k_elas_finish(Geo G, Elas E, double inv_dt, int zero_rhs,
                                                     int extrap) {
+  pdl_sync();
   const int i = blockIdx.x * BX + threadIdx.x;
   const int j = blockIdx.y * BY + threadIdx.y;
   if (i >= G.nx || j >= G.ny) return;

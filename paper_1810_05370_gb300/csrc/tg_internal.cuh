@@ -4,6 +4,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <algorithm>
+
 #include "tg.h"
 #include "tg_fpconv.cuh"
 
@@ -430,14 +432,65 @@ template <typename R> size_t spec_smem_z(const Spec<R>& V) {
 }
 
 // ----------------------------------------------------------------------------- launch helper
+// Kernels of one stream follow each other with programmatic dependent launch on grids up to
+// PDL_MAX_VOXELS: a kernel's blocks may be scheduled once every block of the kernel before it
+// has started (pdl_sync's second half) and wait there for that kernel to finish and its writes
+// to be visible (its first half), so that one kernel's launch latency and ramp pass under the
+// tail of the one before it -- the last block's reduction above all.  A step is 200 to 700
+// kernels, of which those of grids up to 64^3 run 3 to 15 us each.
+//
+// Where the lines lie (us a pass, plain -> overlapped): 16^3 static solve 736 -> 592, FP64
+// 32^3 3266 -> 2700, mixed 64^3 15235 -> 12900, mixed 128^3 16390 -> 15380, 256x256x128
+// 32290 -> 32030, but 256^3 139200 -> 143100: there a launch is long against its latency, and
+// blocks that arrive while the previous kernel runs find an SM whose shared memory / L1 split
+// is the other kernel's and cannot change until the SM is idle.  For the same reason the
+// overlapped kernels of grids from PDL_CARVE_VOXELS on ask for one common split, 60 % shared
+// memory (128^3: default split 16400, 50 % 15610, 60 % 15380, 75 % 15610, 100 % 16800); on
+// smaller grids the occupancy does not matter and each kernel keeps its own (FP64 32^3: 2700
+// against 2790).
+constexpr long long PDL_MAX_VOXELS = 1LL << 23;
+constexpr long long PDL_CARVE_VOXELS = 1LL << 17;
+constexpr int PDL_CARVE_PERCENT = 60;
+
+__device__ __forceinline__ void pdl_sync() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+// the voxels a kernel works on, from its arguments: its grid, its spectral plan or the count it
+// is given (none of them: a kernel of one block, or of a few tables)
+inline long long launch_voxels(const Geo& g) { return g.nvox; }
+template <typename R>
+inline long long launch_voxels(const Spec<R>& v) {
+  return (long long)v.nx * v.ny * v.nz;
+}
+inline long long launch_voxels(long long n) { return n; }
+template <typename T>
+inline long long launch_voxels(const T&) {
+  return 0;
+}
+
+// Every kernel launched here calls pdl_sync first, on every path, so a kernel that has finished
+// implies that all before it on its stream have.
 template <class... P, class... A>
 inline void launch(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
                    const A&... args) {
   cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr[2];
   cfg.gridDim = grid;
   cfg.blockDim = block;
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
+  cfg.attrs = attr;
+  const long long n = std::max({0LL, launch_voxels(args)...});
+  if (n <= PDL_MAX_VOXELS) {
+    attr[cfg.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[cfg.numAttrs++].val.programmaticStreamSerializationAllowed = 1;
+    if (n >= PDL_CARVE_VOXELS) {
+      attr[cfg.numAttrs].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
+      attr[cfg.numAttrs++].val.sharedMemCarveout = PDL_CARVE_PERCENT;
+    }
+  }
   cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
 }
 

@@ -21,6 +21,7 @@ namespace {
 // ------------------------------------------------------------------------------ conversions
 
 __global__ void __launch_bounds__(NT) k_to_f32(long long n, F32Copy c) {
+  pdl_sync();
   const long long stride = (long long)gridDim.x * blockDim.x;
   for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < n; e += stride) {
 #pragma unroll 1
@@ -32,6 +33,7 @@ __global__ void __launch_bounds__(NT) k_to_f32(long long n, F32Copy c) {
 // residual also the (hi, lo) pairs of mu, lambda and the starting u.  parts selects
 // ELAS32_NODES (mu, lambda, eta and their pairs), ELAS32_DINV, ELAS32_U.
 __global__ void __launch_bounds__(NT) k_elas32_coef(long long n, Elas E, Elas32 I, int parts) {
+  pdl_sync();
   const long long stride = (long long)gridDim.x * blockDim.x;
   for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < n; e += stride) {
     if (parts & ELAS32_NODES) {
@@ -60,6 +62,7 @@ __global__ void __launch_bounds__(NT) k_elas32_coef(long long n, Elas E, Elas32 
 __global__ void __launch_bounds__(NT) k_df_pack3(long long n, const double* b0, const double* b1,
                                                  const double* b2, double* o0, double* o1,
                                                  double* o2) {
+  pdl_sync();
   const long long stride = (long long)gridDim.x * blockDim.x;
   for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < n; e += stride) {
     reinterpret_cast<float2*>(o0)[e] = df_pack(b0[e]);
@@ -73,6 +76,7 @@ __global__ void __launch_bounds__(NT) k_df_pack3(long long n, const double* b0, 
 // ------------------------------------------------------------------------------ FP32 inner CG
 
 __global__ void __launch_bounds__(NT) k_elas32_matvec(Geo G, Consts32 K, Elas32 I) {
+  pdl_sync();
   if (!running(I.S)) return;
   __shared__ Tile32 T;
   const float part = elas32_matvec_tile<false>(G, K, I, I.S->it, I.S->beta, blockIdx.x, blockIdx.y,
@@ -86,6 +90,7 @@ __global__ void __launch_bounds__(NT) k_elas32_matvec(Geo G, Consts32 K, Elas32 
 }
 
 __global__ void __launch_bounds__(NT) k_elas32_update(long long n, Elas32 I) {
+  pdl_sync();
   if (!running(I.S)) return;
   const float alpha = (float)I.S->alpha;
   const int pb = (I.S->it & 1) ^ 1;
@@ -103,6 +108,7 @@ __global__ void __launch_bounds__(NT) k_elas32_update(long long n, Elas32 I) {
 // p = z + beta p_old, so the operator only stages p; the update decides convergence from
 // <r, r>
 __global__ void __launch_bounds__(NT) k_elas32_matvec_spec(Geo G, Consts32 K, Elas32 I) {
+  pdl_sync();
   if (!running(I.S)) return;
   __shared__ Tile32 T;
   const float part = elas32_matvec_tile_spec(G, K, I, I.S->it, blockIdx.x, blockIdx.y,
@@ -116,6 +122,7 @@ __global__ void __launch_bounds__(NT) k_elas32_matvec_spec(Geo G, Consts32 K, El
 }
 
 __global__ void __launch_bounds__(NT) k_elas32_update_spec(long long n, Elas32 I) {
+  pdl_sync();
   if (!running(I.S)) return;
   const float alpha = (float)I.S->alpha;
   const int pb = (I.S->it & 1) ^ 1;
@@ -137,6 +144,7 @@ template <bool DF>
 __global__ void __launch_bounds__(NT, DF ? 3 : 2) k_elas_ir_residual(Geo G, Elas E, Elas32 I, CgScal* Sout,
                                                             int minus_b, double tau_min,
                                                             int max_sweeps, ScDf scd) {
+  pdl_sync();
   double acc[3] = {0.0, 0.0, 0.0};
   if (DF)
     elas_ir_residual_tile_df(G, E, I, minus_b, blockIdx.x, blockIdx.y, blockIdx.z, scd, acc);
@@ -149,6 +157,7 @@ __global__ void __launch_bounds__(NT, DF ? 3 : 2) k_elas_ir_residual(Geo G, Elas
 
 // r *= scale (the inner solve's right-hand side normalisation, a power of two: exact)
 __global__ void __launch_bounds__(NT) k_elas32_scale_r(long long n, Elas32 I) {
+  pdl_sync();
   if (!running(I.S)) return;
   const float s = (float)I.S->scale;
   if (s == 1.0f) return;
@@ -161,6 +170,7 @@ __global__ void __launch_bounds__(NT) k_elas32_scale_r(long long n, Elas32 I) {
 
 // u += e, du += e (FP64 accumulation of the FP32 correction)
 __global__ void __launch_bounds__(NT) k_elas_ir_correct(long long n, Elas E, Elas32 I) {
+  pdl_sync();
   const long long stride = (long long)gridDim.x * blockDim.x;
   elas_ir_correct_range(E, I, (long long)blockIdx.x * blockDim.x + threadIdx.x, n, stride,
                         1.0 / I.S->scale);
@@ -173,6 +183,7 @@ __global__ void __launch_bounds__(NT) k_elas_ir_correct(long long n, Elas E, Ela
 // on its own (no contraction), in the oracle's order.
 __global__ void __launch_bounds__(NT) k_elas_extrapolate(long long n, Elas E, double dt,
                                                          int quadratic) {
+  pdl_sync();
   const long long stride = (long long)gridDim.x * blockDim.x;
   if (E.df) {   // mixed precision: s in double-FP32, two FP64 additions per component
     const Df dtd = df_split(dt);
@@ -205,6 +216,7 @@ __global__ void __launch_bounds__(NT) k_elas_extrapolate(long long n, Elas E, do
 // v = du / dt (a step: v^n is kept in vp first); a vanishing right-hand side means u = 0
 __global__ void __launch_bounds__(NT) k_elas_ir_finish(long long n, Elas E, double inv_dt,
                                                        int zero_rhs) {
+  pdl_sync();
   const long long stride = (long long)gridDim.x * blockDim.x;
   for (long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x; c < n; c += stride) {
 #pragma unroll
@@ -314,6 +326,7 @@ __device__ __forceinline__ float3 eval32x3(const Cubic32& T, const float4* __res
 __global__ void __launch_bounds__(NT) k_sl32_pack(Geo G, const double* __restrict__ vx,
                                                   const double* __restrict__ vy,
                                                   const double* __restrict__ vz, Species6 q, Sl32 S) {
+  pdl_sync();
   const int i = blockIdx.x * BX + threadIdx.x;
   const int j = blockIdx.y * BY + threadIdx.y;
   if (i >= G.nx || j >= G.ny) return;
@@ -339,6 +352,7 @@ __global__ void __launch_bounds__(NT) k_sl32_pack(Geo G, const double* __restric
 // two-stage rule of the FP64 path, tricubic interpolation of the species and div_h v there,
 // and the compression source -q div v by Heun's rule along the characteristic.
 __global__ void __launch_bounds__(NT, 3) k_sl32(Geo G, float dt, float3 dt_h, Sl32 S) {
+  pdl_sync();
   const int i = blockIdx.x * BX + threadIdx.x;
   const int j = blockIdx.y * BY + threadIdx.y;
   if (i >= G.nx || j >= G.ny) return;

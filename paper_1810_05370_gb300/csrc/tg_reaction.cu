@@ -83,6 +83,7 @@ __global__ void __launch_bounds__(NT) k_react(Geo G, DevParams P, double dt, int
                                               const double* __restrict__ i_dag, double* p,
                                               double* ii, double* n, double* g, double* w,
                                               double* o, double* l) {
+  pdl_sync();
   const int i = blockIdx.x * BX + threadIdx.x;
   const int j = blockIdx.y * BY + threadIdx.y;
   if (i >= G.nx || j >= G.ny) return;
@@ -162,6 +163,7 @@ __global__ void __launch_bounds__(NT, 4) k_react_f32(Geo G, DevParams P, float d
                                                   const double* __restrict__ i_dag, double* p,
                                                   double* ii, double* n, double* g, double* w,
                                                   double* o, double* l) {
+  pdl_sync();
   const int i = blockIdx.x * BX + threadIdx.x;
   const int j = blockIdx.y * BY + threadIdx.y;
   if (i >= G.nx || j >= G.ny) return;
@@ -236,6 +238,7 @@ __global__ void __launch_bounds__(NT) k_lame(Geo G, DevParams P, const double* _
                                              const double* __restrict__ f,
                                              const double* __restrict__ bg, double* mu,
                                              double* lam, double* eta) {
+  pdl_sync();
   const int i = blockIdx.x * BX + threadIdx.x;
   const int j = blockIdx.y * BY + threadIdx.y;
   if (i >= G.nx || j >= G.ny) return;
@@ -272,6 +275,7 @@ __global__ void __launch_bounds__(NT) k_lame_df(Geo G, DevParams P, const double
                                                 double* lam, double* eta, float* mu32,
                                                 float* lam32, float* eta32, float2* mudf,
                                                 float2* lamdf, float2* sdf) {
+  pdl_sync();
   const int i = blockIdx.x * BX + threadIdx.x;
   const int j = blockIdx.y * BY + threadIdx.y;
   if (i >= G.nx || j >= G.ny) return;

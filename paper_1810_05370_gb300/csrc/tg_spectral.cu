@@ -516,6 +516,7 @@ template <typename R>
 __global__ void __launch_bounds__(NT) k_spec_x_fwd(Spec<R> V, const R* __restrict__ r0,
                                                    const R* __restrict__ r1,
                                                    const R* __restrict__ r2, const CgScal* S) {
+  pdl_sync();
   using C = typename CxOf<R>::T;
   if (spec_skip<R>(S)) return;
   const XTile<R> t = x_tile(V);
@@ -557,6 +558,7 @@ __global__ void __launch_bounds__(NT) k_spec_x_fwd(Spec<R> V, const R* __restric
 // staged straight into the transform, and <r, r> reduced over the launch; the last block
 // takes the convergence decision.  Saves the pass that re-read r.
 __global__ void __launch_bounds__(NT, 4) k_spec_update_xfwd(Spec<float> V, Elas32 I) {
+  pdl_sync();
   using C = float2;
   if (!running(I.S)) return;
   const float alpha = (float)I.S->alpha;
@@ -622,6 +624,7 @@ __global__ void __launch_bounds__(NT, 4) k_spec_update_xfwd(Spec<float> V, Elas3
 // block (mode-column tile, z, component), in place; the FP32 pass at four blocks per SM
 template <typename R, int SGN>
 __global__ void __launch_bounds__(NT, sizeof(R) == 4 ? 4 : 0) k_spec_y(Spec<R> V, const CgScal* S) {
+  pdl_sync();
   using C = typename CxOf<R>::T;
   if (spec_skip<R>(S)) return;
   const int tx = V.tx, ltx = ilog2(tx);
@@ -640,6 +643,7 @@ __global__ void __launch_bounds__(NT, sizeof(R) == 4 ? 4 : 0) k_spec_y(Spec<R> V
 // constant-coefficient inverse per mode, inverse transform; in place
 template <typename R>
 __global__ void __launch_bounds__(NT) k_spec_z(Spec<R> V, CgScal* S) {
+  pdl_sync();
   using C = typename CxOf<R>::T;
   if (spec_skip<R>(S)) return;
   const int tz = V.tz, ltz = ilog2(tz), lw = 3 * tz;   // lines: (component, column)
@@ -734,6 +738,7 @@ constexpr size_t spec_smem_zr() {   // twiddles, the exchange buffer, two compon
 template <int P>
 __global__ void __launch_bounds__(ZR_COLS * P, 512 / (ZR_COLS * P))
     k_spec_zr(Spec<float> V, CgScal* S) {
+  pdl_sync();
   using C = float2;
   constexpr int N = 16 * P, J = 16 / P, LP = P == 16 ? 4 : (P == 8 ? 3 : 2);
   constexpr int NTH = ZR_COLS * P;
@@ -945,6 +950,7 @@ constexpr size_t spec_smem_zr_tma() {   // tile (3 components), twiddles, S_z an
 template <int P>
 __global__ void __launch_bounds__(ZR_COLS * P)
     k_spec_zr_tma(const __grid_constant__ CUtensorMap map, Spec<float> V, CgScal* S) {
+  pdl_sync();
   using C = float2;
   constexpr int N = 16 * P, J = 16 / P, LP = P == 16 ? 4 : (P == 8 ? 3 : 2);
   constexpr int TILE = N * ZR_COLS;            // elements of one component
@@ -1105,6 +1111,7 @@ __global__ void __launch_bounds__(ZR_COLS * P)
 template <typename R, bool PUP, int FORM>
 __global__ void __launch_bounds__(NT, PUP ? 4 : 2) k_spec_x_inv(Spec<R> V, R* z0, R* z1, R* z2,
                                                                 const CgScal* S, PUpd<R> PU) {
+  pdl_sync();
   using C = typename CxOf<R>::T;
   if (spec_skip<R>(S)) return;
   const int n = V.nx, ln = ilog2(n), half = n / 2, pb = V.pb, es = pb + 1;
@@ -1191,6 +1198,7 @@ __global__ void __launch_bounds__(NT, PUP ? 4 : 2) k_spec_x_inv(Spec<R> V, R* z0
 // ---------------------------------------------------------------------------- tables, means
 template <typename R>
 __global__ void k_spec_tables(Spec<R> V, double h0, double h1, double h2) {
+  pdl_sync();
   using C = typename CxOf<R>::T;
   const int d = blockIdx.y;
   const int n = d == 0 ? V.nx : (d == 1 ? V.ny : V.nz);
@@ -1210,6 +1218,7 @@ __global__ void __launch_bounds__(NT) k_spec_mean(long long n, const double* __r
                                                   const double* __restrict__ lam,
                                                   const double* __restrict__ eta, double* mean,
                                                   double* partial, unsigned int* counter) {
+  pdl_sync();
   // F32 (the mixed precision): a thread's terms summed in FP32 from FP32 values converted on
   // the integer pipes (the means only shape the preconditioner), threads and blocks in FP64;
   // otherwise every term in FP64, as the oracle forms the means
@@ -1247,6 +1256,7 @@ __global__ void __launch_bounds__(NT) k_spec_mean(long long n, const double* __r
 template <typename R>
 __global__ void __launch_bounds__(NT) k_spec_scale(long long n, Spec<R> V, Elas E, double ih20,
                                                    double ih21, double ih22) {
+  pdl_sync();
   const double mu0 = V.mean[0], lam0 = V.mean[1], eta0 = V.mean[2];
   const double ih2[3] = {ih20, ih21, ih22};
   R d0[3];

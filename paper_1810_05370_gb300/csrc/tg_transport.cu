@@ -15,6 +15,7 @@ namespace {
 __global__ void __launch_bounds__(NT) k_divergence(Geo G, const double* __restrict__ vx,
                                                    const double* __restrict__ vy,
                                                    const double* __restrict__ vz, double* div) {
+  pdl_sync();
   const int i = blockIdx.x * BX + threadIdx.x;
   const int j = blockIdx.y * BY + threadIdx.y;
   if (i >= G.nx || j >= G.ny) return;
@@ -89,6 +90,7 @@ __global__ void __launch_bounds__(NT) k_sl(Geo G, double dt, double3 dt_h,
                                            const double* __restrict__ vy,
                                            const double* __restrict__ vz,
                                            const double* __restrict__ div, Six qin, Six_out qout) {
+  pdl_sync();
   const int i = blockIdx.x * BX + threadIdx.x;
   const int j = blockIdx.y * BY + threadIdx.y;
   if (i >= G.nx || j >= G.ny) return;
