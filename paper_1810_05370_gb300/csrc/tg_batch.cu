@@ -259,8 +259,7 @@ __global__ void __launch_bounds__(NT, 4) k_batch_elas_inner(BatchDev B) {
       tile_coords(S, local, bx, by, bz);
       const int it = *(volatile const int*)&S.I.S->it;
       const double beta = *(volatile const double*)&S.I.S->beta;
-      const float part = elas32_matvec_tile<true>(S.G, S.K, S.I, it, beta, bx, by, bz, T);
-      double acc[1] = {(double)part};
+      double acc[1] = {elas32_matvec_tile<true>(S.G, S.K, S.I, it, beta, bx, by, bz, S.G.zc, T)};
       double out[1];
       if (reduce_indexed<1>(acc, S.I.partial, S.I.counter, local, S.ntiles, out) &&
           threadIdx.x == 0 && threadIdx.y == 0) {

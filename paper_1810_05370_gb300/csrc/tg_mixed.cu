@@ -75,13 +75,12 @@ __global__ void __launch_bounds__(NT) k_df_pack3(long long n, const double* b0, 
 
 // ------------------------------------------------------------------------------ FP32 inner CG
 
-__global__ void __launch_bounds__(NT) k_elas32_matvec(Geo G, Consts32 K, Elas32 I) {
+__global__ void __launch_bounds__(NT) k_elas32_matvec(Geo G, Consts32 K, Elas32 I, int zb) {
   pdl_sync();
   if (!running(I.S)) return;
   __shared__ Tile32 T;
-  const float part = elas32_matvec_tile<false>(G, K, I, I.S->it, I.S->beta, blockIdx.x, blockIdx.y,
-                                        blockIdx.z, T);
-  double acc[1] = {(double)part};
+  double acc[1] = {elas32_matvec_tile<false>(G, K, I, I.S->it, I.S->beta, blockIdx.x, blockIdx.y,
+                                             blockIdx.z, zb, T)};
   double out[1];
   if (reduce_last_block<1>(acc, I.partial, I.counter, out) && threadIdx.x == 0 && threadIdx.y == 0) {
     I.S->pq = out[0];
@@ -107,13 +106,12 @@ __global__ void __launch_bounds__(NT) k_elas32_update(long long n, Elas32 I) {
 // the same with the spectral preconditioner: the preconditioner's last pass already wrote
 // p = z + beta p_old, so the operator only stages p; the update decides convergence from
 // <r, r>
-__global__ void __launch_bounds__(NT) k_elas32_matvec_spec(Geo G, Consts32 K, Elas32 I) {
+__global__ void __launch_bounds__(NT) k_elas32_matvec_spec(Geo G, Consts32 K, Elas32 I, int zb) {
   pdl_sync();
   if (!running(I.S)) return;
   __shared__ Tile32 T;
-  const float part = elas32_matvec_tile_spec(G, K, I, I.S->it, blockIdx.x, blockIdx.y,
-                                             blockIdx.z, T);
-  double acc[1] = {(double)part};
+  double acc[1] = {elas32_matvec_tile_spec(G, K, I, I.S->it, blockIdx.x, blockIdx.y, blockIdx.z,
+                                           zb, T)};
   double out[1];
   if (reduce_last_block<1>(acc, I.partial, I.counter, out) && threadIdx.x == 0 && threadIdx.y == 0) {
     I.S->pq = out[0];
@@ -390,6 +388,20 @@ int stream_blocks(long long n) {
   return (int)(b < 4096 ? (b > 0 ? b : 1) : 4096);
 }
 
+// Planes a block of the FP32 operator marches.  A block stages two planes more than it
+// computes, so at one or a few planes per block (grids of 64^3 to 128^3, where 16 blocks per SM
+// leave no more) a third to two thirds of the staging is halo: two chunks of planes per block
+// where the launch still has four blocks per SM.  us a pass, one -> two chunks: mixed 64^3
+// 12937 -> 12352, 96^3 Jacobi 10136 -> 9257, 100x84x60 7455 -> 7211, 128^3 15503 -> 15217; three
+// or four chunks, or one wave of blocks, gain no more (128^3: 15325, 15466; 100x84x60: 7260).
+// From nine planes a chunk on (256^3: 27) the halo is small and the blocks' number counts:
+// 70741 -> 70856.
+int op_planes(const Geo& G) { return G.zc <= 8 && G.nblocks >= 4 * 152 ? 2 * G.zc : G.zc; }
+
+dim3 op_grid(const Geo& G, int zb) {
+  return dim3(G.grid.x, G.grid.y, (unsigned)((G.nz + zb - 1) / zb));
+}
+
 }  // namespace
 
 cudaError_t launch_to_f32(long long n, const F32Copy& c, cudaStream_t st) {
@@ -428,8 +440,9 @@ cudaError_t launch_elas_ir_residual(const Geo& G, const Elas& E, const Elas32& I
 }
 
 cudaError_t launch_elas32_matvec(const Geo& G, const Elas32& I, cudaStream_t st) {
+  const int zb = op_planes(G);
   TG_TIMED(K_ELAS32_MATVEC, st,
-           launch(k_elas32_matvec, G.grid, dim3(BX, BY), 0, st, G, make_consts32(G), I));
+           launch(k_elas32_matvec, op_grid(G, zb), dim3(BX, BY), 0, st, G, make_consts32(G), I, zb));
   return cudaGetLastError();
 }
 
@@ -454,8 +467,10 @@ cudaError_t launch_elas32_scale_r(const Geo& G, const Elas32& I, cudaStream_t st
 }
 
 cudaError_t launch_elas32_matvec_spec(const Geo& G, const Elas32& I, cudaStream_t st) {
+  const int zb = op_planes(G);
   TG_TIMED(K_ELAS32_MATVEC_SPEC, st,
-           launch(k_elas32_matvec_spec, G.grid, dim3(BX, BY), 0, st, G, make_consts32(G), I));
+           launch(k_elas32_matvec_spec, op_grid(G, zb), dim3(BX, BY), 0, st, G, make_consts32(G), I,
+                  zb));
   return cudaGetLastError();
 }
 

@@ -166,10 +166,13 @@ __device__ __forceinline__ float row_tile(const Tile32& T, const Cell& t, const 
 // block's shared staging area.  With Jacobi the tile forms p_new = D^{-1} r + beta p_old
 // while staging and writes it; with SPEC the spectral preconditioner's last pass already
 // wrote p_new (into the buffer p[(it & 1) ^ 1]), which the tile only reads.
+//
+// The block marches zb planes; <p, A p> is summed in FP32 over chunks of G.zc planes and the
+// chunks in FP64 (zb: a multiple of G.zc, so a thread's FP32 sums do not depend on it).
 template <bool COH, bool SPEC = false>
-__device__ __forceinline__ float elas32_matvec_tile(const Geo& G, const Consts32& K,
-                                                    const Elas32& I, int it, double beta_d,
-                                                    int bx, int by, int bz, Tile32& T) {
+__device__ __forceinline__ double elas32_matvec_tile(const Geo& G, const Consts32& K,
+                                                     const Elas32& I, int it, double beta_d,
+                                                     int bx, int by, int bz, int zb, Tile32& T) {
   const bool first = it == 0;                 // p = D^{-1} r (the old p is undefined)
   const float beta = first ? 0.0f : (float)beta_d;
   const float* __restrict__ po[3] = {I.p[it & 1][0], I.p[it & 1][1], I.p[it & 1][2]};
@@ -179,7 +182,7 @@ __device__ __forceinline__ float elas32_matvec_tile(const Geo& G, const Consts32
   const int i0 = bx * BX, j0 = by * BY;
   const int i = i0 + tx, j = j0 + ty;
   const bool on = (i < G.nx) && (j < G.ny);
-  const int k0 = bz * G.zc, k1 = min(G.nz, k0 + G.zc);
+  const int k0 = bz * zb, k1 = min(G.nz, k0 + zb);
 
   // the (at most two) halo-tile nodes this thread stages: tile slot tid and tid + NT; their
   // wrapped (x, y) offsets (full modulo: a tile may be wider than the grid)
@@ -233,6 +236,8 @@ __device__ __forceinline__ float elas32_matvec_tile(const Geo& G, const Consts32
   }
 
   float part = 0.0f;
+  double sum = 0.0;
+  int left = G.zc;                       // planes left of the current chunk
   const int ci = (ty + 1) * HX + (tx + 1);
   int s0 = 0, s1 = 1, s2 = 2, s3 = 3;    // slots of planes k-1, k, k+1 and the free one
   // eta of the thread's own node, loaded one plane ahead
@@ -275,6 +280,11 @@ __device__ __forceinline__ float elas32_matvec_tile(const Geo& G, const Consts32
       I.q[2][c] = q2;
       part += p0 * q0 + p1 * q1 + p2 * q2;
     }
+    if (--left == 0) {
+      sum += f64_of(part);
+      part = 0.0f;
+      left = G.zc;
+    }
     if (more) {                         // plane k+2 goes to the free slot
       put(r0, s3, tid);
       if (two) put(r1, s3, hs1);
@@ -286,7 +296,7 @@ __device__ __forceinline__ float elas32_matvec_tile(const Geo& G, const Consts32
     s3 = sf;
   }
   __syncthreads();                      // the tile may be restaged by the caller's next item
-  return part;
+  return sum + f64_of(part);
 }
 
 // The FP32 operator on the spectral path (p_new already written by the preconditioner), with
@@ -373,9 +383,9 @@ __device__ __forceinline__ void spec_step(const Geo& G, const Consts32& K, const
   }
 }
 
-__device__ __forceinline__ float elas32_matvec_tile_spec(const Geo& G, const Consts32& K,
-                                                         const Elas32& I, int it, int bx, int by,
-                                                         int bz, Tile32& T) {
+__device__ __forceinline__ double elas32_matvec_tile_spec(const Geo& G, const Consts32& K,
+                                                          const Elas32& I, int it, int bx, int by,
+                                                          int bz, int zb, Tile32& T) {
   SpecTileCtx X;
 #pragma unroll
   for (int a = 0; a < 3; ++a) X.pn[a] = I.p[(it & 1) ^ 1][a];
@@ -384,8 +394,8 @@ __device__ __forceinline__ float elas32_matvec_tile_spec(const Geo& G, const Con
   const int i0 = bx * BX, j0 = by * BY;
   const int i = i0 + tx, j = j0 + ty;
   X.on = (i < G.nx) && (j < G.ny);
-  const int k0 = bz * G.zc;
-  X.k1 = min(G.nz, k0 + G.zc);
+  const int k0 = bz * zb;
+  X.k1 = min(G.nz, k0 + zb);
   auto wrapped = [&](int s) {   // full modulo: a tile may be wider than the grid
     int gi = (i0 - 1 + s % HX) % G.nx, gj = (j0 - 1 + s / HX) % G.ny;
     gi = gi < 0 ? gi + G.nx : gi;
@@ -417,15 +427,34 @@ __device__ __forceinline__ float elas32_matvec_tile_spec(const Geo& G, const Con
     }
   }
   float part = 0.0f;
+  double sum = 0.0;
+  int left = G.zc;   // planes left of the current chunk
+  auto chunk = [&]() {
+    if (--left == 0) {
+      sum += f64_of(part);
+      part = 0.0f;
+      left = G.zc;
+    }
+  };
   float eta_next = (X.on && k0 < X.k1) ? __ldg(I.eta + (long long)k0 * G.nxy + X.col) : 0.0f;
   for (int k = k0; k < X.k1; k += 4) {
     spec_step<0, 1, 2, 3>(G, K, I, X, T, k, eta_next, r0, r1, part);
-    if (k + 1 < X.k1) spec_step<1, 2, 3, 0>(G, K, I, X, T, k + 1, eta_next, r0, r1, part);
-    if (k + 2 < X.k1) spec_step<2, 3, 0, 1>(G, K, I, X, T, k + 2, eta_next, r0, r1, part);
-    if (k + 3 < X.k1) spec_step<3, 0, 1, 2>(G, K, I, X, T, k + 3, eta_next, r0, r1, part);
+    chunk();
+    if (k + 1 < X.k1) {
+      spec_step<1, 2, 3, 0>(G, K, I, X, T, k + 1, eta_next, r0, r1, part);
+      chunk();
+    }
+    if (k + 2 < X.k1) {
+      spec_step<2, 3, 0, 1>(G, K, I, X, T, k + 2, eta_next, r0, r1, part);
+      chunk();
+    }
+    if (k + 3 < X.k1) {
+      spec_step<3, 0, 1, 2>(G, K, I, X, T, k + 3, eta_next, r0, r1, part);
+      chunk();
+    }
   }
   __syncthreads();
-  return part;
+  return sum + f64_of(part);
 }
 
 // e += alpha p, r -= alpha q (p as written by this iteration's operator kernel, buffer pb),

@@ -74,6 +74,16 @@ def test_convergence_test_from_the_squares(lib):
 @pytest.mark.parametrize("n", [(5, 5, 5), (9, 7, 5), (33, 9, 7), (35, 17, 13)])
 @pytest.mark.parametrize("precision", ["fp64", "mixed"])
 def test_remainders_against_the_oracle(oracle, n, precision):
+    against_the_oracle(oracle, n, precision)
+
+
+@pytest.mark.gpu
+def test_operator_blocks_of_two_chunks(oracle):
+    """666 blocks of one plane: the FP32 operator takes two planes a block, the last block one."""
+    against_the_oracle(oracle, (64, 72, 37), "mixed")
+
+
+def against_the_oracle(oracle, n, precision):
     torch = pytest.importorskip("torch")
     if not torch.cuda.is_available():
         pytest.skip("no CUDA device")
