@@ -71,6 +71,7 @@ constexpr int MAX_NV = 9;    // largest number of values reduced by one kernel
 // 3 diffusion solves (outer in the mixed precision), elasticity (outer), elasticity inner
 // FP32, 3 inner FP32 diffusion solves
 constexpr int N_SCAL = 11;   // 3 CN, 2 elasticity, 3 inner CN, 3 concurrent CN
+constexpr int SMALL_COUNTERS = 16;    // first counter word of the small grids' solves
 constexpr int MAX_SWEEPS = 64;        // refinement sweeps of one mixed-precision solve
 constexpr double TAU_INNER = 1e-4;    // smallest relative reduction asked of an inner solve
 // ... of a spectrally preconditioned inner elasticity solve: its few, well-conditioned FP32
@@ -407,7 +408,7 @@ const char* const kKernelNames[K_COUNT] = {
     "k_spec_update_xfwd", "k_elas_ir_correct", "k_elas_ir_finish", "k_elas_init",
     "k_elas_init_spec", "k_elas_matvec", "k_elas_update", "k_elas_pupdate", "k_elas_update_spec",
     "k_elas_pupdate_spec", "k_elas_finish", "k_ox_prep", "k_ox_init", "k_ox_matvec",
-    "k_ox_update", "k_ox_pupdate", "k_ox_finish", "k_sl32_pack", "k_lame_df"};
+    "k_ox_update", "k_ox_pupdate", "k_ox_finish", "k_sl32_pack", "k_lame_df", "k_elas_cg"};
 
 }  // namespace
 
@@ -429,8 +430,10 @@ struct tg_ctx {
   double* grad;          // 5 device accumulators of dJ/dtheta
   double* tape[T_COUNT]; // tape being recorded by the current step, or null
   double* partial;
-  unsigned int* counter;
+  unsigned int* counter;   // ALIGN bytes: words 0 .. 2 the reductions' tickets, words
+                           // SMALL_COUNTERS and the next those of the small grids' solves
   CgScal* scal;
+  int sms;               // SMs of the device
   // TG_MIXED: the FP64 oxygen solve of S2 runs on a side stream (created on first use),
   // forked from and joined to the context's stream by events, with its own reductions
   double* partial2;
@@ -1134,16 +1137,24 @@ tg_status elas_solve(tg_ctx* X, double* const u[3], double* const b_ext[3], bool
     X->launches += 2;
   }
   CgScal host[1];
-  tg_status s = drive_cg(X, [&](int) {
-    X->launches += spec ? 8 : 3;
-    cudaError_t e = launch_elas_matvec(X->G, E, X->stream);
-    if (e != cudaSuccess) return e;
-    if (!spec) return launch_elas_update(X->G, E, X->stream);
-    e = launch_elas_update_spec(X->G, E, X->stream);
-    if (e == cudaSuccess) e = launch_spectral(V, r64, X->z64, E.S, X->stream);
-    if (e == cudaSuccess) e = launch_elas_pupdate_spec(X->G, E, X->stream);
-    return e;
-  }, E.S, 1, X->prm.maxit_elas, X->prev_it_elas, host);
+  tg_status s = TG_OK;
+  if (!spec && cg_small_ok(X->G, X->sms)) {   // one launch runs every iteration
+    CK(launch_elas_cg_small(X->G, E, X->sms, X->counter + SMALL_COUNTERS, X->stream));
+    X->launches += 1;
+    CK(cudaMemcpyAsync(host, E.S, sizeof(CgScal), cudaMemcpyDeviceToHost, X->stream));
+    CK(cudaStreamSynchronize(X->stream));
+  } else {
+    s = drive_cg(X, [&](int) {
+      X->launches += spec ? 8 : 3;
+      cudaError_t e = launch_elas_matvec(X->G, E, X->stream);
+      if (e != cudaSuccess) return e;
+      if (!spec) return launch_elas_update(X->G, E, X->stream);
+      e = launch_elas_update_spec(X->G, E, X->stream);
+      if (e == cudaSuccess) e = launch_spectral(V, r64, X->z64, E.S, X->stream);
+      if (e == cudaSuccess) e = launch_elas_pupdate_spec(X->G, E, X->stream);
+      return e;
+    }, E.S, 1, X->prm.maxit_elas, X->prev_it_elas, host);
+  }
   if (s != TG_OK) return s;
   X->prev_it_elas = host[0].it;
   if (stats) {
@@ -1605,6 +1616,7 @@ tg_status tg_init(const tg_grid* grid, const tg_params* params, tg_precision pre
   X->prec = prec;
   X->st = *state;
   X->stream = (cudaStream_t)cuda_stream;
+  X->sms = sm_count();
   cudaGetDevice(&X->device);
   X->ws = (char*)workspace;
   for (int a = 0; a < A_COUNT; ++a) X->a[a] = (double*)(X->ws + L.arr[a]);
@@ -1967,6 +1979,7 @@ extern "C" tg_status tg_solve_elasticity_static(const tg_grid* grid, const tg_pa
   X.prm = *params;
   X.dp = make_dev_params(params);
   X.prec = TG_FP64;
+  X.sms = sm_count();
   X.st = *state;
   X.stream = (cudaStream_t)cuda_stream;
   X.device = dev;
