@@ -408,7 +408,8 @@ const char* const kKernelNames[K_COUNT] = {
     "k_spec_update_xfwd", "k_elas_ir_correct", "k_elas_ir_finish", "k_elas_init",
     "k_elas_init_spec", "k_elas_matvec", "k_elas_update", "k_elas_pupdate", "k_elas_update_spec",
     "k_elas_pupdate_spec", "k_elas_finish", "k_ox_prep", "k_ox_init", "k_ox_matvec",
-    "k_ox_update", "k_ox_pupdate", "k_ox_finish", "k_sl32_pack", "k_lame_df", "k_elas_cg"};
+    "k_ox_update", "k_ox_pupdate", "k_ox_finish", "k_sl32_pack", "k_lame_df", "k_elas_cg",
+    "k_cn_cg"};
 
 }  // namespace
 
@@ -726,6 +727,22 @@ bool cn_df_ok(const tg_ctx* X) {
          X->prm.rtol_diff >= DF_RTOL_MIN;
 }
 
+// The iterations of the FP64 Crank-Nicolson solves started on C: one launch on a small grid,
+// else queued three kernels at a time.
+tg_status cn_iterate(tg_ctx* X, const Cn3& C, CgScal host[3]) {
+  if (cg_small_ok(X->G, X->sms)) {
+    CK(launch_cn_cg_small(X->G, C, X->sms, X->counter + SMALL_COUNTERS, X->stream));
+    X->launches += 1;
+    CK(cudaMemcpyAsync(host, C.S, 3 * sizeof(CgScal), cudaMemcpyDeviceToHost, X->stream));
+    CK(cudaStreamSynchronize(X->stream));
+    return TG_OK;
+  }
+  return drive_cg(X, [&](int) {
+    X->launches += 3;
+    return launch_cn_iter(X->G, C, X->stream);
+  }, C.S, 3, X->prm.maxit_diff, X->prev_it_diff, host);
+}
+
 // S2: the three Crank-Nicolson solves (i, o, l) on the faces built by S0.
 // mask: bit r set for the fields this call solves (the others are left untouched)
 tg_status cn_solve3(tg_ctx* X, tg_stats* stats, int mask = 7) {
@@ -735,10 +752,7 @@ tg_status cn_solve3(tg_ctx* X, tg_stats* stats, int mask = 7) {
   CK(launch_cn_init(X->G, C, X->stream, mask));
   X->launches += 2;
   CgScal host[3];
-  tg_status s = drive_cg(X, [&](int) {
-    X->launches += 3;
-    return launch_cn_iter(X->G, C, X->stream);
-  }, X->scal, 3, X->prm.maxit_diff, X->prev_it_diff, host);
+  const tg_status s = cn_iterate(X, C, host);
   if (s != TG_OK) return s;
   int itmax = 0;
   for (int r = 0; r < 3; ++r) {
@@ -1501,10 +1515,7 @@ tg_status do_adjoint_step(tg_ctx* X, double dt, const void* tape, const tg_state
     CK(launch_cn_init_rhs(G, C, A, s));
     X->launches += 2;
     CgScal host[3];
-    tg_status e = drive_cg(X, [&](int) {
-      X->launches += 3;
-      return launch_cn_iter(G, C, s);
-    }, X->scal, 3, X->prm.maxit_diff, X->prev_it_diff, host);
+    const tg_status e = cn_iterate(X, C, host);
     if (e != TG_OK) return e;
     for (int r = 0; r < 3; ++r) {
       tg_status e2 = status_of(host[r]);

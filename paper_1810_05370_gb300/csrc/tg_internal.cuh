@@ -34,7 +34,7 @@ enum KernelId : int {
   K_ELAS32_UPDATE_SPEC, K_SPEC_UPDATE_XFWD, K_ELAS_IR_CORRECT, K_ELAS_IR_FINISH,
   K_ELAS_INIT, K_ELAS_INIT_SPEC, K_ELAS_MATVEC, K_ELAS_UPDATE, K_ELAS_PUPDATE, K_ELAS_UPDATE_SPEC,
   K_ELAS_PUPDATE_SPEC, K_ELAS_FINISH, K_OX_PREP, K_OX_INIT, K_OX_MATVEC, K_OX_UPDATE,
-  K_OX_PUPDATE, K_OX_FINISH, K_SL32_PACK, K_LAME_DF, K_ELAS_CG,
+  K_OX_PUPDATE, K_OX_FINISH, K_SL32_PACK, K_LAME_DF, K_ELAS_CG, K_CN_CG,
   K_COUNT
 };
 
@@ -696,8 +696,10 @@ cudaError_t launch_elas_pupdate_spec(const Geo&, const Elas&, cudaStream_t st);
 cudaError_t launch_elas_finish(const Geo&, const Elas&, double inv_dt, bool zero_rhs,
                                int extrap, cudaStream_t st);
 
-// the whole Jacobi-CG solve of a small grid in one cooperative launch (tg_cg_small.cu)
+// the whole Jacobi-CG solves of a small grid in one cooperative launch each (tg_cg_small.cu)
 bool cg_small_ok(const Geo&, int sms);
+cudaError_t launch_cn_cg_small(const Geo&, const Cn3&, int sms, unsigned int* counters,
+                               cudaStream_t st);
 cudaError_t launch_elas_cg_small(const Geo&, const Elas&, int sms, unsigned int* counters,
                                  cudaStream_t st);
 
