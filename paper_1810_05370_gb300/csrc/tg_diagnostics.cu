@@ -28,6 +28,12 @@ __device__ __forceinline__ void combine(double (&a)[NQ], const double (&b)[NQ]) 
   a[6] = fmax(a[6], b[6]);
 }
 
+// the same for one of the seven
+__device__ __forceinline__ double combine_one(int q, double a, double b) {
+  if (q == 2) return a + b;
+  return q == 0 || q == 3 ? fmin(a, b) : fmax(a, b);
+}
+
 __device__ __forceinline__ void identity(double (&a)[NQ]) {
   a[0] = INFINITY;
   a[1] = -INFINITY;
@@ -90,48 +96,43 @@ __global__ void __launch_bounds__(NT) k_diagnostics(Geo G, DiagArgs A) {
       combine(acc, v);
     }
   }
-  // block: warp shuffles, then warps in order
-  __shared__ double sh[NQ][NWARP];
+  // one warp per value combines the block's 256, eight per lane and then across the lanes; the
+  // last block does the same with the blocks' results, every thread its share of them (one
+  // thread walking them in order took 400 of the kernel's 510 us at 64^3)
+  __shared__ double sh[NQ][NT];
+  __shared__ double tot[NQ];
   __shared__ bool am_last;
   const int tid = threadIdx.y * blockDim.x + threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int b = block_linear(), nb = block_count();
+  auto block_combine = [&](double* to) {
 #pragma unroll
-  for (int off = 16; off > 0; off >>= 1) {
-    double o[NQ];
+    for (int q = 0; q < NQ; ++q) sh[q][tid] = acc[q];
+    __syncthreads();
+    for (int q = warp; q < NQ; q += NWARP) {
+      double v = sh[q][lane];
 #pragma unroll
-    for (int q = 0; q < NQ; ++q) o[q] = __shfl_down_sync(0xffffffffu, acc[q], off);
-    combine(acc, o);
-  }
-  if (lane == 0)
+      for (int m = 1; m < NWARP; ++m) v = combine_one(q, v, sh[q][lane + 32 * m]);
 #pragma unroll
-    for (int q = 0; q < NQ; ++q) sh[q][warp] = acc[q];
-  __syncthreads();
-  const int b = (blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
-  const int nb = gridDim.x * gridDim.y * gridDim.z;
-  if (tid == 0) {
-    double s[NQ];
-    identity(s);
-    for (int w = 0; w < NWARP; ++w) {
-      double t[NQ];
-#pragma unroll
-      for (int q = 0; q < NQ; ++q) t[q] = sh[q][w];
-      combine(s, t);
+      for (int o = 16; o > 0; o >>= 1)
+        v = combine_one(q, v, __shfl_down_sync(0xffffffffu, v, o));
+      if (lane == 0) to[q] = v;
     }
-#pragma unroll
-    for (int q = 0; q < NQ; ++q) A.partial[(size_t)b * NQ + q] = s[q];
-    __threadfence();
-    am_last = atomicAdd(A.counter, 1u) == (unsigned int)(nb - 1);
-  }
+    __syncthreads();
+  };
+  block_combine(A.partial + (size_t)b * NQ);
+  if (tid == 0) am_last = ticket_acq_rel(A.counter) == (unsigned int)(nb - 1);
   __syncthreads();
-  if (!am_last || tid != 0) return;
-  __threadfence();
-  double s[NQ];
-  identity(s);
-  for (int k = 0; k < nb; ++k) {
+  if (!am_last) return;
+  identity(acc);
+  for (int k = tid; k < nb; k += NT) {
     double t[NQ];
 #pragma unroll
     for (int q = 0; q < NQ; ++q) t[q] = __ldcg(A.partial + (size_t)k * NQ + q);
-    combine(s, t);
+    combine(acc, t);
   }
+  block_combine(tot);
+  if (tid != 0) return;
+  const double(&s)[NQ] = tot;
   const double vol = G.h[0] * G.h[1] * G.h[2];
   A.result[0] = s[0];
   A.result[1] = s[1];
