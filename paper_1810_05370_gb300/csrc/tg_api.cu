@@ -1083,8 +1083,10 @@ tg_status elas_solve_mixed(tg_ctx* X, double* const u[3], double* const b_ext[3]
     X->launches += 1;
     if (spec) {   // p = P r and <r, P r> for the inner solve's first direction
       PUpd<float> pu;
-      for (int b = 0; b < 2; ++b)
-        for (int a = 0; a < 3; ++a) pu.p[b][a] = I.p[b][a];
+      for (int a = 0; a < 3; ++a) {
+        pu.e[a] = I.e[a];
+        for (int b = 0; b < 2; ++b) pu.p[b][a] = I.p[b][a];
+      }
       CK(launch_spectral(V, r32, X->z32, I.S, X->stream, &pu));
       X->launches += 5;
     }
@@ -1102,7 +1104,7 @@ tg_status elas_solve_mixed(tg_ctx* X, double* const u[3], double* const b_ext[3]
     X->prev_it_inner[slot] = host[0].it;
     inner_total += host[0].it;
     if (host[0].status == CG_NONFINITE) return fail(X, TG_ERR_NONFINITE);
-    CK(launch_elas_ir_correct(X->G, E, I, X->stream));
+    CK(launch_elas_ir_correct(X->G, E, I, spec, X->stream));
     X->launches += 1;
     ++sweeps;
   }

@@ -406,9 +406,13 @@ struct Spec {
 // The CG p-update fused into the x inverse pass (mixed precision): the pass writes the new
 // search direction p = z + beta p_old instead of z, into the buffer of the two that the
 // iteration's operator kernel reads (they alternate with the iteration count S->it).
+// From the solve's first iteration on it also writes the iterate, e += alpha p_old; the last
+// iteration of a solve, which ends before this pass, is added with the correction (launch_elas_ir_correct's
+// pending).
 template <typename R>
 struct PUpd {
   R* p[2][3];
+  R* e[3];
 };
 
 // shared memory of each pass (bytes): the line length's twiddles and two line buffers
@@ -714,7 +718,9 @@ cudaError_t launch_elas_ir_residual(const Geo&, const Elas&, const Elas32&, CgSc
                                     bool minus_b, double tau_min, cudaStream_t st);
 cudaError_t launch_elas32_matvec(const Geo&, const Elas32&, cudaStream_t st);
 cudaError_t launch_elas32_update(const Geo&, const Elas32&, cudaStream_t st);
-cudaError_t launch_elas_ir_correct(const Geo&, const Elas&, const Elas32&, cudaStream_t st);
+// u += e / scale; pending: the spectral solve's e lacks its last iteration's alpha p
+cudaError_t launch_elas_ir_correct(const Geo&, const Elas&, const Elas32&, bool pending,
+                                   cudaStream_t st);
 cudaError_t launch_elas_extrapolate(const Geo&, const Elas&, double dt, bool quadratic,
                                     cudaStream_t st);
 cudaError_t launch_elas_ir_finish(const Geo&, const Elas&, double inv_dt, bool zero_rhs,

@@ -166,12 +166,22 @@ __global__ void __launch_bounds__(NT) k_elas32_scale_r(long long n, Elas32 I) {
   }
 }
 
-// u += e, du += e (FP64 accumulation of the FP32 correction)
-__global__ void __launch_bounds__(NT) k_elas_ir_correct(long long n, Elas E, Elas32 I) {
+// u += e, du += e (FP64 accumulation of the FP32 correction).  pending: the spectral inner
+// solve leaves its last iteration's e += alpha p to this pass (the others are done where p is
+// read anyway, in the preconditioner's last pass)
+__global__ void __launch_bounds__(NT) k_elas_ir_correct(long long n, Elas E, Elas32 I,
+                                                        int pending) {
   pdl_sync();
   const long long stride = (long long)gridDim.x * blockDim.x;
-  elas_ir_correct_range(E, I, (long long)blockIdx.x * blockDim.x + threadIdx.x, n, stride,
-                        1.0 / I.S->scale);
+  const long long c0 = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  const double inv_scale = 1.0 / I.S->scale;
+  if (pending && I.S->it > 0) {
+    const int b = I.S->it & 1;   // the buffer of the last iteration's direction
+    const float* const p[3] = {I.p[b][0], I.p[b][1], I.p[b][2]};
+    elas_ir_correct_range(E, I, c0, n, stride, inv_scale, p, (float)I.S->alpha);
+  } else {
+    elas_ir_correct_range(E, I, c0, n, stride, inv_scale);
+  }
 }
 
 // Starting guess of a step's solve, extrapolation in time.  Linear: the increment
@@ -480,9 +490,11 @@ cudaError_t launch_elas32_update_spec(const Geo& G, const Elas32& I, cudaStream_
   return cudaGetLastError();
 }
 
-cudaError_t launch_elas_ir_correct(const Geo& G, const Elas& E, const Elas32& I, cudaStream_t st) {
+cudaError_t launch_elas_ir_correct(const Geo& G, const Elas& E, const Elas32& I, bool pending,
+                                   cudaStream_t st) {
   TG_TIMED(K_ELAS_IR_CORRECT, st,
-           launch(k_elas_ir_correct, stream_blocks(G.nvox), NT, 0, st, G.nvox, E, I));
+           launch(k_elas_ir_correct, stream_blocks(G.nvox), NT, 0, st, G.nvox, E, I,
+                  pending ? 1 : 0));
   return cudaGetLastError();
 }
 

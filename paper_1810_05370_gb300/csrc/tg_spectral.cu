@@ -553,43 +553,37 @@ __global__ void __launch_bounds__(NT) k_spec_x_fwd(Spec<R> V, const R* __restric
   x_fwd_finish<R, 2>(V, t, a, b, tw);
 }
 
-// The mixed precision's CG update fused into the x forward pass: for the block's rows
-// e += alpha p, r -= alpha q (p as written by this iteration's operator kernel), the new r
-// staged straight into the transform, and <r, r> reduced over the launch; the last block
-// takes the convergence decision.  Saves the pass that re-read r.
+// The mixed precision's residual update fused into the x forward pass: for the block's rows
+// r -= alpha q, the new r staged straight into the transform, and <r, r> reduced over the
+// launch; the last block takes the convergence decision.  Saves the pass that re-read r.  The
+// iterate's half of the update, e += alpha p, is left to the x inverse pass, which reads p
+// anyway (k_spec_x_inv): 12 of the 253 bytes per voxel that an iteration moves.
 __global__ void __launch_bounds__(NT, 4) k_spec_update_xfwd(Spec<float> V, Elas32 I) {
   pdl_sync();
   using C = float2;
   if (!running(I.S)) return;
   const float alpha = (float)I.S->alpha;
-  const int pbuf = (I.S->it & 1) ^ 1;
   const XTile<float> t = x_tile(V);
   const int n = t.n, ln = t.ln, es = t.es;
   C* tw = smem_cx<C>();
   C* a = tw + n;
   C* b = a + (size_t)es * n;
   load_roots(tw, V.tw[0], n);
-  float* e = I.e[t.comp];
   float* r = I.r[t.comp];
-  const float* p = I.p[pbuf][t.comp];
   const float* q = I.q[t.comp];
   const float* sc = V.s[t.comp];   // the transform takes s r with the scaled preconditioner
   constexpr int UB = 4;
   float rr = 0.0f;
   const int total = t.pb * n;
   for (int i0 = threadIdx.x; i0 < total; i0 += UB * blockDim.x) {
-    float ea[UB], eb[UB], ra[UB], rb[UB], pa[UB], pbv[UB], qa[UB], qb[UB], sa[UB], sb[UB];
+    float ra[UB], rb[UB], qa[UB], qb[UB], sa[UB], sb[UB];
 #pragma unroll
     for (int u = 0; u < UB; ++u) {
       const int idx = i0 + u * blockDim.x;
       if (idx < total) {
         const size_t o = t.row0 + (size_t)(2 * (idx >> ln)) * n + (idx & (n - 1));
-        ea[u] = e[o];
-        eb[u] = e[o + n];
         ra[u] = r[o];
         rb[u] = r[o + n];
-        pa[u] = p[o];
-        pbv[u] = p[o + n];
         qa[u] = q[o];
         qb[u] = q[o + n];
         sa[u] = sc ? __ldg(sc + o) : 1.0f;
@@ -602,8 +596,6 @@ __global__ void __launch_bounds__(NT, 4) k_spec_update_xfwd(Spec<float> V, Elas3
       if (idx < total) {
         const size_t o = t.row0 + (size_t)(2 * (idx >> ln)) * n + (idx & (n - 1));
         const float xa = ra[u] - alpha * qa[u], xb = rb[u] - alpha * qb[u];
-        e[o] = ea[u] + alpha * pa[u];
-        e[o + n] = eb[u] + alpha * pbv[u];
         r[o] = xa;
         r[o + n] = xb;
         rr += xa * xa + xb * xb;
@@ -1107,7 +1099,9 @@ __global__ void __launch_bounds__(ZR_COLS * P)
 // block (pair tile, z, component): the half spectra of rows y0 + 2l, y0 + 2l + 1 form
 // C[k] = A[k] + i B[k] over all k (Hermitian extension); the inverse transform is
 // a + i b.  Writes z = s (inverse transform) (s = 1 unscaled), or with PU the new search
-// direction p = z + beta p_old (beta = 0 on a solve's first iteration).
+// direction p = z + beta p_old (beta = 0 on a solve's first iteration) and, from the p_old in
+// hand, the iterate of the iteration that ends here, e += alpha p_old.  An iteration that
+// converged does not get here: the refinement's correction adds its alpha p (PUpd::e).
 template <typename R, bool PUP, int FORM>
 __global__ void __launch_bounds__(NT, PUP ? 4 : 2) k_spec_x_inv(Spec<R> V, R* z0, R* z1, R* z2,
                                                                 const CgScal* S, PUpd<R> PU) {
@@ -1155,7 +1149,8 @@ __global__ void __launch_bounds__(NT, PUP ? 4 : 2) k_spec_x_inv(Spec<R> V, R* z0
   const C* F = fft_x<+1, FORM>(V.x_inpl != 0, a, b, ln, ilog2(pb), es, tw);
   R* out = comp == 0 ? z0 : (comp == 1 ? z1 : z2);
   const R* pold = nullptr;
-  R beta = (R)0;
+  R* e = nullptr;
+  R beta = (R)0, alpha = (R)0;
   if (PUP) {   // selects written out: no indexed copy of the parameter arrays
     const int it = S->it;
     R* const p0 = comp == 0 ? PU.p[0][0] : (comp == 1 ? PU.p[0][1] : PU.p[0][2]);
@@ -1164,14 +1159,17 @@ __global__ void __launch_bounds__(NT, PUP ? 4 : 2) k_spec_x_inv(Spec<R> V, R* z0
     if (it > 0) {
       pold = (it & 1) ? p1 : p0;
       beta = (R)S->beta;
+      e = comp == 0 ? PU.e[0] : (comp == 1 ? PU.e[1] : PU.e[2]);
+      alpha = (R)S->alpha;
     }
   }
   const R* sc = V.s[comp];   // z = s A0^{-1} (s r) with the scaled preconditioner
   const size_t row0 = ((size_t)z * V.ny + y0) * n;
-  for (int i0 = threadIdx.x; i0 < total; i0 += LB * blockDim.x) {   // LB loads in flight
-    R sa[LB], sb[LB], pa[LB], pbv[LB];
+  constexpr int OB = PUP ? 4 : LB;   // loads in flight: 6 or 2 times this many
+  for (int i0 = threadIdx.x; i0 < total; i0 += OB * blockDim.x) {
+    R sa[OB], sb[OB], pa[OB], pbv[OB], ea[OB], eb[OB];
 #pragma unroll
-    for (int u = 0; u < LB; ++u) {
+    for (int u = 0; u < OB; ++u) {
       const int idx = i0 + u * blockDim.x;
       if (idx < total) {
         const size_t o = row0 + (size_t)(2 * (idx >> ln)) * n + (idx & (n - 1));
@@ -1179,10 +1177,12 @@ __global__ void __launch_bounds__(NT, PUP ? 4 : 2) k_spec_x_inv(Spec<R> V, R* z0
         sb[u] = sc ? __ldg(sc + o + n) : (R)1;
         pa[u] = (PUP && pold) ? pold[o] : (R)0;
         pbv[u] = (PUP && pold) ? pold[o + n] : (R)0;
+        ea[u] = (PUP && pold) ? e[o] : (R)0;
+        eb[u] = (PUP && pold) ? e[o + n] : (R)0;
       }
     }
 #pragma unroll
-    for (int u = 0; u < LB; ++u) {
+    for (int u = 0; u < OB; ++u) {
       const int idx = i0 + u * blockDim.x;
       if (idx < total) {
         const int l = idx >> ln, x = idx & (n - 1);
@@ -1190,6 +1190,10 @@ __global__ void __launch_bounds__(NT, PUP ? 4 : 2) k_spec_x_inv(Spec<R> V, R* z0
         const C f = F[x * es + l];
         out[o] = PUP ? f.x * sa[u] + beta * pa[u] : f.x * sa[u];
         out[o + n] = PUP ? f.y * sb[u] + beta * pbv[u] : f.y * sb[u];
+        if (PUP && pold) {
+          e[o] = ea[u] + alpha * pa[u];
+          e[o + n] = eb[u] + alpha * pbv[u];
+        }
       }
     }
   }
@@ -1446,8 +1450,10 @@ cudaError_t launch_spectral_update(const Spec<float>& V, const Elas32& I, float*
   launch_spec_z(V, I.S, st);
   TG_TIMED(K_SPEC_Y_INV, st, launch((k_spec_y<float, +1>), gy, NT, spec_smem_y(V), st, V, I.S));
   PUpd<float> P;   // p = z + beta p_old straight from the last pass
-  for (int b = 0; b < 2; ++b)
-    for (int a = 0; a < 3; ++a) P.p[b][a] = I.p[b][a];
+  for (int a = 0; a < 3; ++a) {
+    P.e[a] = I.e[a];
+    for (int b = 0; b < 2; ++b) P.p[b][a] = I.p[b][a];
+  }
   if (V.x_inpl)
     TG_TIMED(K_SPEC_X_INV_P, st,
              launch((k_spec_x_inv<float, true, 1>), gx, NT, spec_smem_x(V), st, V, z[0], z[1],

@@ -677,14 +677,18 @@ __device__ __forceinline__ void elas_ir_residual_finalize(CgScal& O, CgScal& S, 
 }
 
 // u += e / scale, du += e / scale over voxels c = c0, c0 + cs, ... < c1 (scale: the inner
-// right-hand side's factor, a power of two)
+// right-hand side's factor, a power of two); with pend, e + alpha pend in e's place
 __device__ __forceinline__ void elas_ir_correct_range(const Elas& E, const Elas32& I, long long c0,
                                                       long long c1, long long cs,
-                                                      double inv_scale = 1.0) {
+                                                      double inv_scale = 1.0,
+                                                      const float* const* pend = nullptr,
+                                                      float alpha = 0.0f) {
   for (long long c = c0; c < c1; c += cs) {
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-      const double e = f64_of_scaled(I.e[a][c], inv_scale);   // exact; no FP64 operation
+      float e32 = I.e[a][c];
+      if (pend) e32 += alpha * pend[a][c];
+      const double e = f64_of_scaled(e32, inv_scale);   // exact; no FP64 operation
       const double un = E.u[a][c] + e;
       E.u[a][c] = un;
       E.du[a][c] += e;
