@@ -558,6 +558,12 @@ __global__ void __launch_bounds__(NT) k_spec_x_fwd(Spec<R> V, const R* __restric
 // launch; the last block takes the convergence decision.  Saves the pass that re-read r.  The
 // iterate's half of the update, e += alpha p, is left to the x inverse pass, which reads p
 // anyway (k_spec_x_inv): 12 of the 253 bytes per voxel that an iteration moves.
+//
+// FORM: the transform in two line buffers (0) or in place (1).  In place a stage costs two
+// barriers instead of one but half the shared memory, which pays where two buffers leave the
+// SM fewer than four blocks (lines of 256: 72 KB a block); us a pass, 0 -> 1: mixed 256^3 131950
+// -> 128600, but 128^3 14763 -> 14874 and 64^3 11730 -> 11950, where both fit four times.
+template <int FORM>
 __global__ void __launch_bounds__(NT, 4) k_spec_update_xfwd(Spec<float> V, Elas32 I) {
   pdl_sync();
   using C = float2;
@@ -607,7 +613,7 @@ __global__ void __launch_bounds__(NT, 4) k_spec_update_xfwd(Spec<float> V, Elas3
   const int nb = gridDim.x * gridDim.y * gridDim.z;
   const int bl = (blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
   block_sum_begin(B, (double)rr, V.partial, V.counter, bl, nb);   // also publishes the staging
-  x_fwd_finish<float, 0>(V, t, a, b, tw);   // two buffers (in place it ran slower)
+  x_fwd_finish<float, FORM>(V, t, a, b, tw);
   double out;
   if (block_sum_end(B, V.partial, V.counter, nb, out)) cg_after_update_rr(*I.S, out);
 }
@@ -1304,7 +1310,8 @@ cudaError_t spec_prepare(const Spec<R>& V) {
     return cudaErrorInvalidValue;
   const cudaFuncAttribute A = cudaFuncAttributeMaxDynamicSharedMemorySize;
   e = cudaFuncSetAttribute(k_spec_x_fwd<R>, A, optin);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_spec_update_xfwd, A, optin);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_spec_update_xfwd<0>, A, optin);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_spec_update_xfwd<1>, A, optin);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(k_spec_x_inv<R, false, 2>, A, optin);
   if constexpr (sizeof(R) == 4) {
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k_spec_x_inv<R, true, 0>, A, optin);
@@ -1445,7 +1452,12 @@ cudaError_t launch_spectral_update(const Spec<float>& V, const Elas32& I, float*
                                    cudaStream_t st) {
   const dim3 gx(V.ny / (2 * V.pb), V.nz, 3);
   const dim3 gy((V.nxh + V.tx - 1) / V.tx, V.nz, 3);
-  TG_TIMED(K_SPEC_UPDATE_XFWD, st, launch(k_spec_update_xfwd, gx, NT, spec_smem_x2(V), st, V, I));
+  if (V.x_inpl && 4 * spec_smem_x2(V) > 224 * 1024)
+    TG_TIMED(K_SPEC_UPDATE_XFWD, st,
+             launch(k_spec_update_xfwd<1>, gx, NT, spec_smem_x(V), st, V, I));
+  else
+    TG_TIMED(K_SPEC_UPDATE_XFWD, st,
+             launch(k_spec_update_xfwd<0>, gx, NT, spec_smem_x2(V), st, V, I));
   TG_TIMED(K_SPEC_Y_FWD, st, launch((k_spec_y<float, -1>), gy, NT, spec_smem_y(V), st, V, I.S));
   launch_spec_z(V, I.S, st);
   TG_TIMED(K_SPEC_Y_INV, st, launch((k_spec_y<float, +1>), gy, NT, spec_smem_y(V), st, V, I.S));
