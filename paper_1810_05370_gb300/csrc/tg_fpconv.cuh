@@ -334,6 +334,11 @@ TG_HD Df df_tanh(Df s) {
 }
 
 // ------------------------------------------------- scalars of the CG solves
+// 1 / x for a normal power of two x whose reciprocal is normal too: exact, no division
+TG_HD double pow2_recip(double x) {
+  return fpc::from_bits64((unsigned)(0x7fe00000u - (unsigned)(fpc::bits64(x) >> 32)), 0u);
+}
+
 // The power of two nearest 1 / sqrt(x) on the logarithmic scale, 2^-rint(log2(x) / 2), for a
 // finite x > 0, from its exponent e and significand m in [1, 2): log2(x) / 2 lies in
 // [e/2, e/2 + 1/2), so it rounds to e/2 for even e and to (e + 1)/2 for odd e, the tie at

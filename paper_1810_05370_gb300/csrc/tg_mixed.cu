@@ -174,7 +174,7 @@ __global__ void __launch_bounds__(NT) k_elas_ir_correct(long long n, Elas E, Ela
   pdl_sync();
   const long long stride = (long long)gridDim.x * blockDim.x;
   const long long c0 = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  const double inv_scale = 1.0 / I.S->scale;
+  const double inv_scale = pow2_recip(I.S->scale);
   if (pending && I.S->it > 0) {
     const int b = I.S->it & 1;   // the buffer of the last iteration's direction
     const float* const p[3] = {I.p[b][0], I.p[b][1], I.p[b][2]};

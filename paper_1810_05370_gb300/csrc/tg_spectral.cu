@@ -638,13 +638,25 @@ __global__ void __launch_bounds__(NT, sizeof(R) == 4 ? 4 : 0) k_spec_y(Spec<R> V
 
 // ---------------------------------------------------------------------------- z pass
 // block (mode-column tile, ky): the three components' z columns; forward transform, the
-// constant-coefficient inverse per mode, inverse transform; in place
-template <typename R>
-__global__ void __launch_bounds__(NT) k_spec_z(Spec<R> V, CgScal* S) {
+// constant-coefficient inverse per mode, inverse transform; in place.
+//
+// NARROW: tiles of Z_NARROW columns instead of V.tz = 16, for FP32 grids whose wide tiles leave
+// the chip idle (64^3: 192 blocks of 192 threads).  The kernel is a chain of latencies there --
+// a thread's radix-4 butterflies and modes one after the other, 13.5 us for 4.7 MB -- and a
+// thread of a narrow tile has half of them.  The terms of <r, z> are summed as a wide tile's
+// threads sum them -- a column's modes kz = g, g + groups, ... in FP32, one thread per
+// (column, g) -- so the sum does not depend on the tile.  us a pass, 16 -> 8 -> 4 columns: mixed
+// 64^3 study 11815 -> 10825 -> 10626, 32^3 1218 -> 1124 -> 1112, but four columns cost the concurrent
+// batch, whose members fill each other's gaps, 1.8 % (16583 -> 16600 -> 16880): eight.
+constexpr int Z_NARROW = 8;
+constexpr int Z_NARROW_MAX = 64;        // largest nz
+constexpr int Z_NARROW_THREADS = 192;
+template <typename R, bool NARROW>
+__global__ void __launch_bounds__(NARROW ? Z_NARROW_THREADS : NT) k_spec_z(Spec<R> V, CgScal* S) {
   pdl_sync();
   using C = typename CxOf<R>::T;
   if (spec_skip<R>(S)) return;
-  const int tz = V.tz, ltz = ilog2(tz), lw = 3 * tz;   // lines: (component, column)
+  const int tz = NARROW ? Z_NARROW : V.tz, ltz = ilog2(tz), lw = 3 * tz;   // lines: (component, column)
   C* tw = smem_cx<C>();
   C* a = tw + V.nz;
   C* b = a + (size_t)lw * V.nz;
@@ -655,13 +667,17 @@ __global__ void __launch_bounds__(NT) k_spec_z(Spec<R> V, CgScal* S) {
   const ZIO<C> io{V.W + (size_t)ky * V.nxp + kx0, plane, comp_stride, tz, ltz, ncol};
   C* F = fft_from_global<-1>(io, a, b, 1, lw, ilog2(V.nz), ltz, 3, tw);
   C* other = F == a ? b : a;
-  const R mu0 = (R)V.mean[0], lam0 = (R)V.mean[1], eta0 = (R)V.mean[2];
+  // FP32: no FP64 operation (the volume is a power of two, so both forms are exact)
+  const R mu0 = sizeof(R) == 4 ? f32_of(V.mean[0]) : (R)V.mean[0];
+  const R lam0 = sizeof(R) == 4 ? f32_of(V.mean[1]) : (R)V.mean[1];
+  const R eta0 = sizeof(R) == 4 ? f32_of(V.mean[2]) : (R)V.mean[2];
   const R c = lam0 + mu0;
-  const R inv_vol = (R)(1.0 / ((double)V.nx * V.ny * V.nz));
+  const R inv_vol = (R)1 / ((R)V.nx * (R)V.ny * (R)V.nz);
   const R Sy = V.S[1][ky], Ty = V.T[1][ky];
   // <r, z> by Parseval: sum over modes of conj(r^) z^ (z^ already carries 1/V), each stored
   // mode with 0 < kx < nx/2 standing for its conjugate as well; every term is >= 0
   R rz_part = (R)0;
+  __shared__ R term[NARROW ? 3 * Z_NARROW * Z_NARROW_MAX : 1];   // [mode][component]
   for (int idx = threadIdx.x; idx < tz * V.nz; idx += blockDim.x) {
     const int kz = idx >> ltz, col = idx & (tz - 1);
     if (col >= ncol) continue;
@@ -690,11 +706,25 @@ __global__ void __launch_bounds__(NT) k_spec_z(Spec<R> V, CgScal* S) {
       const R g = f * Tv[q] * dinv[q];
       const C rq = F[(size_t)kz * lw + q * tz + col];
       const C zq = C{(y[q].x - g * s.x) * inv_vol, (y[q].y - g * s.y) * inv_vol};
-      rz_part += wgt * (rq.x * zq.x + rq.y * zq.y);
+      if constexpr (NARROW)
+        term[3 * idx + q] = rq.x * zq.x + rq.y * zq.y;
+      else
+        rz_part += wgt * (rq.x * zq.x + rq.y * zq.y);
       F[(size_t)kz * lw + q * tz + col] = zq;
     }
   }
   __shared__ BlockSum B;
+  if constexpr (NARROW) {
+    __syncthreads();
+    const int groups = V.nt_z >> 4, col = threadIdx.x & (tz - 1), g = threadIdx.x >> ltz;
+    if (g < groups && col < ncol) {
+      const int kx = kx0 + col;
+      const R wgt = (kx == 0 || kx == V.nx / 2) ? (R)1 : (R)2;
+      for (int kz = g; kz < V.nz; kz += groups)
+#pragma unroll
+        for (int q = 0; q < 3; ++q) rz_part += wgt * term[3 * (kz * tz + col) + q];
+    }
+  }
   if (S != nullptr)
     block_sum_begin(B, (double)rz_part, V.partial, V.counter,
                     blockIdx.y * gridDim.x + blockIdx.x, gridDim.x * gridDim.y);
@@ -1319,7 +1349,7 @@ cudaError_t spec_prepare(const Spec<R>& V) {
   }
   if (e == cudaSuccess) e = cudaFuncSetAttribute(k_spec_y<R, -1>, A, optin);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(k_spec_y<R, +1>, A, optin);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_spec_z<R>, A, optin);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_spec_z<R, false>, A, optin);
   if constexpr (sizeof(R) == 4) {
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k_spec_zr<16>, A, optin);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k_spec_zr<8>, A, optin);
@@ -1385,6 +1415,14 @@ cudaError_t launch_spec_mean(long long n, const double* mu, const double* lam,
   return cudaGetLastError();
 }
 
+// Narrow tiles while wide ones (16 columns at these nz) leave the SMs fewer than four blocks
+// each; their blocks' partial sums were counted in V.nb_partial.
+bool spec_z_narrow(const Spec<float>& V) {
+  const long long wide = (long long)((V.nxh + V.tz - 1) / V.tz) * V.ny;
+  const long long narrow = (long long)((V.nxh + Z_NARROW - 1) / Z_NARROW) * V.ny;
+  return V.nz <= Z_NARROW_MAX && V.tz == 16 && wide < 4 * 152 && narrow <= V.nb_partial;
+}
+
 // the z pass: for FP32 and nz = 128 or 256 in registers, from tiles staged by TMA when the
 // context made the tensor map (and the pass updates a solve's scalars), else from global
 // memory; staged through shared memory otherwise
@@ -1412,7 +1450,15 @@ void launch_spec_z(const Spec<R>& V, CgScal* S, cudaStream_t st) {
     }
   }
   const dim3 gz((V.nxh + V.tz - 1) / V.tz, V.ny);
-  TG_TIMED(K_SPEC_Z, st, launch(k_spec_z<R>, gz, V.nt_z, spec_smem_z(V), st, V, S));
+  if constexpr (sizeof(R) == 4) {
+    if (spec_z_narrow(V)) {
+      const dim3 gn((V.nxh + Z_NARROW - 1) / Z_NARROW, V.ny);
+      const size_t smem = (1 + 2 * (size_t)3 * Z_NARROW) * V.nz * sizeof(float2);
+      TG_TIMED(K_SPEC_Z, st, launch((k_spec_z<R, true>), gn, Z_NARROW_THREADS, smem, st, V, S));
+      return;
+    }
+  }
+  TG_TIMED(K_SPEC_Z, st, launch((k_spec_z<R, false>), gz, V.nt_z, spec_smem_z(V), st, V, S));
 }
 
 template <typename R>

@@ -12,4 +12,8 @@ void tgr_norm_met(const double* rr, const double* rtol, const double* bb, int* o
   for (long q = 0; q < n; ++q) out[q] = tg::cg_norm_met(rr[q], rtol[q], bb[q]) ? 1 : 0;
 }
 
+void tgr_pow2_recip(const double* x, double* out, long n) {
+  for (long q = 0; q < n; ++q) out[q] = tg::pow2_recip(x[q]);
+}
+
 }  // extern "C"
