@@ -106,10 +106,10 @@ __global__ void __launch_bounds__(NT) k_elas32_update(long long n, Elas32 I) {
 // the same with the spectral preconditioner: the preconditioner's last pass already wrote
 // p = z + beta p_old, so the operator only stages p; the update decides convergence from
 // <r, r>
-__global__ void __launch_bounds__(NT) k_elas32_matvec_spec(Geo G, Consts32 K, Elas32 I, int zb) {
+__global__ void __launch_bounds__(NT, 4) k_elas32_matvec_spec(Geo G, Consts32 K, Elas32 I, int zb) {
   pdl_sync();
   if (!running(I.S)) return;
-  __shared__ Tile32 T;
+  __shared__ TileSpec T;
   double acc[1] = {elas32_matvec_tile_spec(G, K, I, I.S->it, blockIdx.x, blockIdx.y, blockIdx.z,
                                            zb, T)};
   double out[1];

@@ -109,7 +109,8 @@ struct Fac32 {
   float eta;
 };
 
-__device__ __forceinline__ void tile_fac(const Tile32& T, const Cell& t, const float ih2[3],
+template <class Tile, class At>
+__device__ __forceinline__ void tile_fac(const Tile& T, const At& t, const float ih2[3],
                                          float eta, Fac32& f) {
   const float muc = tmu(T, t, 0, 0, 0), lac = tla(T, t, 0, 0, 0);
   f.eta = eta;
@@ -130,8 +131,8 @@ __device__ __forceinline__ void tile_fac(const Tile32& T, const Cell& t, const f
 }
 
 // component A of (eta I - L_h) p at the centre node, all operands from the tile
-template <int A>
-__device__ __forceinline__ float row_tile(const Tile32& T, const Cell& t, const Fac32& f,
+template <int A, class Tile, class At>
+__device__ __forceinline__ float row_tile(const Tile& T, const At& t, const Fac32& f,
                                           const float sc[3][3]) {
   constexpr int D1 = (A + 1) % 3, D2 = (A + 2) % 3;
   float diag = f.eta, off = 0.0f;
@@ -299,74 +300,137 @@ __device__ __forceinline__ double elas32_matvec_tile(const Geo& G, const Consts3
   return sum + f64_of(part);
 }
 
-// The FP32 operator on the spectral path (p_new already written by the preconditioner), with
-// the tile layout of elas32_matvec_tile and its arithmetic.  The z loop is unrolled by the
-// four plane slots, so the slots of planes k-1, k, k+1 and of the plane being staged are
-// compile-time constants and every shared address is the thread's base plus a constant (the
-// rotating slots of elas32_matvec_tile cost ~40 integer instructions per node).
+// The FP32 operator on the spectral path (p_new already written by the preconditioner): the
+// tiling and the arithmetic of elas32_matvec_tile with two thirds of its instructions around
+// it.  What bounds it is instruction issue and shared-memory reads (349 instructions and 59
+// reads per node in that form, 90 us of HBM at 256^3 against 185), so
+//  * a thread keeps what it reads of plane k + 1 in registers while the planes move down: its
+//    own column (p, mu, lambda), u_x and u_z of its x neighbours, u_y and u_z of its y
+//    neighbours -- 13 reads a plane; of plane k itself 20 more (the four corners, u_y and u_x
+//    of the x and y neighbours, their mu and lambda) -- 33 instead of 59;
+//  * planes go from global to shared memory by asynchronous copies issued one step ahead, with
+//    no registers and no store instructions in between;
+//  * the planes' slots are compile-time constants (the z loop is unrolled by the three), so
+//    every register index and shared address is.
+// us per launch at 256^3: 203 -> 182 (four blocks of 64 registers per SM; 197 at three of 80).
+constexpr int SSLOT = 3;   // planes k, k + 1 being read, k + 2 arriving
+struct TileSpec {
+  float p[SSLOT][3][HXY];   // [plane slot][component][node]
+  float mu[SSLOT][HXY];
+  float la[SSLOT][HXY];
+};
+
+// one thread's view of planes k - 1, k, k + 1 in registers, by slot
+struct SpecRing {
+  float own[SSLOT][3], mu[SSLOT], la[SSLOT];
+  float xp[SSLOT][2], xm[SSLOT][2];   // u_x, u_z at x + 1, x - 1
+  float yp[SSLOT][2], ym[SSLOT][2];   // u_y, u_z at y + 1, y - 1
+};
+
+// the operator's operands at the centre node: registers, or plane k in shared memory
 template <int S0, int S1, int S2>
-__device__ __forceinline__ Cell cell_of(Tile32& T, int ci) {
-  Cell t;
-  constexpr int sl[3] = {S0, S1, S2};
-#pragma unroll
-  for (int o = 0; o < 3; ++o) {
-#pragma unroll
-    for (int a = 0; a < 3; ++a) t.p[o][a] = &T.p[sl[o]][a][ci];
-    t.mu[o] = &T.mu[sl[o]][ci];
-    t.la[o] = &T.la[sl[o]][ci];
+struct SpecCell {
+  const SpecRing& R;
+  const TileSpec& T;
+  int ci;
+  static constexpr int slot(int oz) { return oz < 0 ? S0 : (oz == 0 ? S1 : S2); }
+  __device__ __forceinline__ float p(int a, int ox, int oy, int oz) const {
+    const int s = slot(oz);
+    if (ox == 0 && oy == 0) return R.own[s][a];
+    if (oy == 0 && a != 1) return ox > 0 ? R.xp[s][a >> 1] : R.xm[s][a >> 1];
+    if (ox == 0 && a != 0) return oy > 0 ? R.yp[s][a - 1] : R.ym[s][a - 1];
+    return T.p[S1][a][ci + ox + oy * HX];   // plane k: oz == 0 in every case left
   }
-  return t;
+  __device__ __forceinline__ float mu(int ox, int oy, int oz) const {
+    return ox == 0 && oy == 0 ? R.mu[slot(oz)] : T.mu[S1][ci + ox + oy * HX];
+  }
+  __device__ __forceinline__ float la(int ox, int oy, int oz) const {
+    return ox == 0 && oy == 0 ? R.la[slot(oz)] : T.la[S1][ci + ox + oy * HX];
+  }
+};
+template <int S0, int S1, int S2>
+__device__ __forceinline__ float tp(const TileSpec&, const SpecCell<S0, S1, S2>& t, int a, int ox,
+                                    int oy, int oz) {
+  return t.p(a, ox, oy, oz);
+}
+template <int S0, int S1, int S2>
+__device__ __forceinline__ float tmu(const TileSpec&, const SpecCell<S0, S1, S2>& t, int ox, int oy,
+                                     int oz) {
+  return t.mu(ox, oy, oz);
+}
+template <int S0, int S1, int S2>
+__device__ __forceinline__ float tla(const TileSpec&, const SpecCell<S0, S1, S2>& t, int ox, int oy,
+                                     int oz) {
+  return t.la(ox, oy, oz);
 }
 
 struct SpecTileCtx {
-  const float* __restrict__ pn[3];
-  long long ho0, ho1, col;
-  int tid, hs1, ci, k1;
+  const float* src[5];       // p_new (3 components), mu, lambda
+  unsigned dst;              // shared address of the thread's first staged node, slot 0
+  int ho0, ho1, col;         // (x, y) offsets of its staged nodes and of its own column
+  int ci, k1;
   bool two, on;
 };
 
-struct StagedNode {
-  float p[3], mu, la;
-};
-
-__device__ __forceinline__ long long spec_plane_offset(const Geo& G, int kk) {
-  const int kw = kk < 0 ? kk + G.nz : (kk >= G.nz ? kk - G.nz : kk);
-  return (long long)kw * G.nxy;
+__device__ __forceinline__ void copy4_async(unsigned dst, const float* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst), "l"(src) : "memory");
+}
+__device__ __forceinline__ void copies_commit() {
+  asm volatile("cp.async.commit_group;" ::: "memory");
+}
+__device__ __forceinline__ void copies_wait() {
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
 }
 
-__device__ __forceinline__ void spec_fetch(const SpecTileCtx& X, const Elas32& I, long long g,
-                                           StagedNode& v) {
-#pragma unroll
-  for (int a = 0; a < 3; ++a) v.p[a] = __ldg(X.pn[a] + g);
-  v.mu = __ldg(I.mu + g);
-  v.la = __ldg(I.lam + g);
-}
-
+// stage plane kk (wrapped) into slot S: at most two nodes per thread, five values each
 template <int S>
-__device__ __forceinline__ void spec_put(Tile32& T, const StagedNode& v, int s) {
+__device__ __forceinline__ void spec_stage(const Geo& G, const SpecTileCtx& X, int kk) {
+  const int kw = kk < 0 ? kk + G.nz : (kk >= G.nz ? kk - G.nz : kk);
+  const int zo = kw * (G.nx * G.ny);
+  // TileSpec in floats: p[S][a] at (3 S + a) HXY, mu[S] at (9 + S) HXY, la[S] at (12 + S) HXY
+  constexpr unsigned at[5] = {(3 * S) * HXY * 4, (3 * S + 1) * HXY * 4, (3 * S + 2) * HXY * 4,
+                              (9 + S) * HXY * 4, (12 + S) * HXY * 4};
 #pragma unroll
-  for (int a = 0; a < 3; ++a) T.p[S][a][s] = v.p[a];
-  T.mu[S][s] = v.mu;
-  T.la[S][s] = v.la;
+  for (int v = 0; v < 5; ++v) copy4_async(X.dst + at[v], X.src[v] + zo + X.ho0);
+  if (X.two) {
+#pragma unroll
+    for (int v = 0; v < 5; ++v) copy4_async(X.dst + at[v] + NT * 4, X.src[v] + zo + X.ho1);
+  }
+  copies_commit();
 }
 
-// plane k from slots (S0, S1, S2); plane k + 2 is staged into slot S3
-template <int S0, int S1, int S2, int S3>
+// what the thread keeps of the plane in slot S
+template <int S>
+__device__ __forceinline__ void spec_keep(const TileSpec& T, SpecRing& R, int ci) {
+#pragma unroll
+  for (int a = 0; a < 3; ++a) R.own[S][a] = T.p[S][a][ci];
+  R.mu[S] = T.mu[S][ci];
+  R.la[S] = T.la[S][ci];
+#pragma unroll
+  for (int q = 0; q < 2; ++q) {
+    R.xp[S][q] = T.p[S][2 * q][ci + 1];
+    R.xm[S][q] = T.p[S][2 * q][ci - 1];
+    R.yp[S][q] = T.p[S][1 + q][ci + HX];
+    R.ym[S][q] = T.p[S][1 + q][ci - HX];
+  }
+}
+
+// plane k: planes k - 1, k, k + 1 in slots S0, S1, S2; plane k + 2 arrives in S0's shared slot
+template <int S0, int S1, int S2>
 __device__ __forceinline__ void spec_step(const Geo& G, const Consts32& K, const Elas32& I,
-                                          const SpecTileCtx& X, Tile32& T, int k, float& eta_next,
-                                          StagedNode& r0, StagedNode& r1, float& part) {
+                                          const SpecTileCtx& X, TileSpec& T, SpecRing& R, int k,
+                                          float& eta_next, float& part) {
   const float eta_k = eta_next;
   const bool more = k + 1 < X.k1;
-  if (X.on && more) eta_next = __ldg(I.eta + (long long)(k + 1) * G.nxy + X.col);
-  if (more) {
-    const long long zo = spec_plane_offset(G, k + 2);
-    spec_fetch(X, I, zo + X.ho0, r0);
-    if (X.two) spec_fetch(X, I, zo + X.ho1, r1);
-  }
-  __syncthreads();   // plane k + 1 (staged by the previous step) is visible
+  const int nxy = G.nx * G.ny;
+  if (X.on && more) eta_next = __ldg(I.eta + (k + 1) * nxy + X.col);
+  copies_wait();
+  __syncthreads();   // plane k + 1 is visible, and plane k - 1's shared slot no longer read
+  if (more) spec_stage<S0>(G, X, k + 2);
   if (X.on) {
-    const Cell t = cell_of<S0, S1, S2>(T, X.ci);
-    const long long c = (long long)k * G.nxy + X.col;
+    spec_keep<S2>(T, R, X.ci);
+    const SpecCell<S0, S1, S2> t{R, T, X.ci};
+    const int c = k * nxy + X.col;
     Fac32 f;
     tile_fac(T, t, K.ih2, eta_k, f);
     const float q0 = row_tile<0>(T, t, f, K.sc);
@@ -377,20 +441,17 @@ __device__ __forceinline__ void spec_step(const Geo& G, const Consts32& K, const
     I.q[2][c] = q2;
     part += tp(T, t, 0, 0, 0, 0) * q0 + tp(T, t, 1, 0, 0, 0) * q1 + tp(T, t, 2, 0, 0, 0) * q2;
   }
-  if (more) {
-    spec_put<S3>(T, r0, X.tid);
-    if (X.two) spec_put<S3>(T, r1, X.hs1);
-  }
 }
 
 __device__ __forceinline__ double elas32_matvec_tile_spec(const Geo& G, const Consts32& K,
                                                           const Elas32& I, int it, int bx, int by,
-                                                          int bz, int zb, Tile32& T) {
+                                                          int bz, int zb, TileSpec& T) {
   SpecTileCtx X;
 #pragma unroll
-  for (int a = 0; a < 3; ++a) X.pn[a] = I.p[(it & 1) ^ 1][a];
-  const int tx = threadIdx.x, ty = threadIdx.y;
-  X.tid = ty * BX + tx;
+  for (int a = 0; a < 3; ++a) X.src[a] = I.p[(it & 1) ^ 1][a];
+  X.src[3] = I.mu;
+  X.src[4] = I.lam;
+  const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * BX + tx;
   const int i0 = bx * BX, j0 = by * BY;
   const int i = i0 + tx, j = j0 + ty;
   X.on = (i < G.nx) && (j < G.ny);
@@ -400,32 +461,17 @@ __device__ __forceinline__ double elas32_matvec_tile_spec(const Geo& G, const Co
     int gi = (i0 - 1 + s % HX) % G.nx, gj = (j0 - 1 + s / HX) % G.ny;
     gi = gi < 0 ? gi + G.nx : gi;
     gj = gj < 0 ? gj + G.ny : gj;
-    return (long long)gj * G.nx + gi;
+    return gj * G.nx + gi;
   };
-  X.hs1 = X.tid + NT;
-  X.two = X.hs1 < HXY;
-  X.ho0 = wrapped(X.tid);
-  X.ho1 = X.two ? wrapped(X.hs1) : 0;
+  X.two = tid + NT < HXY;
+  X.ho0 = wrapped(tid);
+  X.ho1 = X.two ? wrapped(tid + NT) : 0;
+  X.dst = (unsigned)__cvta_generic_to_shared(&T.p[0][0][0]) + tid * 4;
   X.ci = (ty + 1) * HX + (tx + 1);
-  X.col = (long long)j * G.nx + i;
-  StagedNode r0, r1;
-#pragma unroll
-  for (int o = 0; o < 3; ++o) {
-    const long long zo = spec_plane_offset(G, k0 - 1 + o);
-    spec_fetch(X, I, zo + X.ho0, r0);
-    if (X.two) spec_fetch(X, I, zo + X.ho1, r1);
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-      T.p[o][a][X.tid] = r0.p[a];
-      if (X.two) T.p[o][a][X.hs1] = r1.p[a];
-    }
-    T.mu[o][X.tid] = r0.mu;
-    T.la[o][X.tid] = r0.la;
-    if (X.two) {
-      T.mu[o][X.hs1] = r1.mu;
-      T.la[o][X.hs1] = r1.la;
-    }
-  }
+  X.col = j * G.nx + i;
+  spec_stage<0>(G, X, k0 - 1);
+  spec_stage<1>(G, X, k0);
+  spec_stage<2>(G, X, k0 + 1);
   float part = 0.0f;
   double sum = 0.0;
   int left = G.zc;   // planes left of the current chunk
@@ -436,24 +482,24 @@ __device__ __forceinline__ double elas32_matvec_tile_spec(const Geo& G, const Co
       left = G.zc;
     }
   };
-  float eta_next = (X.on && k0 < X.k1) ? __ldg(I.eta + (long long)k0 * G.nxy + X.col) : 0.0f;
-  for (int k = k0; k < X.k1; k += 4) {
-    spec_step<0, 1, 2, 3>(G, K, I, X, T, k, eta_next, r0, r1, part);
+  float eta_next = (X.on && k0 < X.k1) ? __ldg(I.eta + k0 * (G.nx * G.ny) + X.col) : 0.0f;
+  copies_wait();
+  __syncthreads();
+  SpecRing R;
+  spec_keep<0>(T, R, X.ci);
+  spec_keep<1>(T, R, X.ci);
+  for (int k = k0; k < X.k1; k += 3) {
+    spec_step<0, 1, 2>(G, K, I, X, T, R, k, eta_next, part);
     chunk();
     if (k + 1 < X.k1) {
-      spec_step<1, 2, 3, 0>(G, K, I, X, T, k + 1, eta_next, r0, r1, part);
+      spec_step<1, 2, 0>(G, K, I, X, T, R, k + 1, eta_next, part);
       chunk();
     }
     if (k + 2 < X.k1) {
-      spec_step<2, 3, 0, 1>(G, K, I, X, T, k + 2, eta_next, r0, r1, part);
-      chunk();
-    }
-    if (k + 3 < X.k1) {
-      spec_step<3, 0, 1, 2>(G, K, I, X, T, k + 3, eta_next, r0, r1, part);
+      spec_step<2, 0, 1>(G, K, I, X, T, R, k + 2, eta_next, part);
       chunk();
     }
   }
-  __syncthreads();
   return sum + f64_of(part);
 }
 
