@@ -132,14 +132,20 @@ template <int LR, int SGN, typename C> __device__ __forceinline__ void dft(C (&v
 // (ll, j, lh) with ll fastest, so consecutive threads take consecutive interleaved lines
 // (es > 1) or consecutive butterflies of one line (lo = 1, es = 1).  tw[k] =
 // exp(-2 pi i k / n) (the inverse transform conjugates it).
+// nt: the block's threads.  Where a caller's sizes are compile-time constants the trip counts
+// and every index but the thread's own become constants too.
+__device__ __forceinline__ int trips(int total, int nt) { return (total + nt - 1) / nt; }
+
 template <int LR, int SGN, typename C>
 __device__ __forceinline__ void fft_stage(const C* a, C* b, int ln, int lNs, int llo, int hi,
-                                          int ls, int es, const C* tw) {
+                                          int ls, int es, const C* tw, int nt) {
   constexpr int R = 1 << LR;
   const int lnb = ln - LR, nb = 1 << lnb, Ns = 1 << lNs, lts = ln - lNs - LR;
   const int lo_mask = (1 << llo) - 1;
   const int total = hi << (llo + lnb);
-  for (int it = threadIdx.x; it < total; it += blockDim.x) {
+  for (int m = 0; m < trips(total, nt); ++m) {
+    const int it = threadIdx.x + m * nt;
+    if (total % nt != 0 && it >= total) break;
     const int ll = it & lo_mask;
     const int rest = it >> llo;
     const int j = rest & (nb - 1);
@@ -166,11 +172,12 @@ __device__ __forceinline__ void fft_stage(const C* a, C* b, int ln, int lNs, int
 // each.  Entry: a and tw loaded and visible to the block.  Returns the buffer holding the
 // result (visible to the block).
 template <int SGN, typename C>
-__device__ C* fft_lines(C* a, C* b, int ln, int llo, int hi, int ls, int es, const C* tw) {
+__device__ __forceinline__ C* fft_lines(C* a, C* b, int ln, int llo, int hi, int ls, int es,
+                                        const C* tw, int nt) {
   int lNs = ln & 3;
-  if (lNs == 1) fft_stage<1, SGN>(a, b, ln, 0, llo, hi, ls, es, tw);
-  if (lNs == 2) fft_stage<2, SGN>(a, b, ln, 0, llo, hi, ls, es, tw);
-  if (lNs == 3) fft_stage<3, SGN>(a, b, ln, 0, llo, hi, ls, es, tw);
+  if (lNs == 1) fft_stage<1, SGN>(a, b, ln, 0, llo, hi, ls, es, tw, nt);
+  if (lNs == 2) fft_stage<2, SGN>(a, b, ln, 0, llo, hi, ls, es, tw, nt);
+  if (lNs == 3) fft_stage<3, SGN>(a, b, ln, 0, llo, hi, ls, es, tw, nt);
   if (lNs != 0) {
     __syncthreads();
     C* t = a;
@@ -178,7 +185,7 @@ __device__ C* fft_lines(C* a, C* b, int ln, int llo, int hi, int ls, int es, con
     b = t;
   }
   for (; lNs < ln; lNs += 4) {
-    fft_stage<4, SGN>(a, b, ln, lNs, llo, hi, ls, es, tw);
+    fft_stage<4, SGN>(a, b, ln, lNs, llo, hi, ls, es, tw, nt);
     __syncthreads();
     C* t = a;
     a = b;
@@ -194,13 +201,13 @@ __device__ C* fft_lines(C* a, C* b, int ln, int llo, int hi, int ls, int es, con
 // bit.  Two barriers per stage, half the shared memory.
 template <int LR, int SGN, typename C>
 __device__ __forceinline__ void fft_stage_inplace(C* a, int ln, int lNs, int llo, int hi, int ls,
-                                                  int es, const C* tw) {
+                                                  int es, const C* tw, int nt) {
   constexpr int R = 1 << LR;
   const int lnb = ln - LR, nb = 1 << lnb, Ns = 1 << lNs, lts = ln - lNs - LR;
   const int lo_mask = (1 << llo) - 1;
   const int total = hi << (llo + lnb);
   const int it = threadIdx.x;
-  const bool act = it < total;
+  const bool act = total >= nt || it < total;   // at most one butterfly per thread
   C v[R];
   int base = 0, d = 0;
   if (act) {
@@ -227,14 +234,15 @@ __device__ __forceinline__ void fft_stage_inplace(C* a, int ln, int lNs, int llo
 }
 
 template <int SGN, typename C>
-__device__ C* fft_lines_inplace(C* a, int ln, int llo, int hi, int ls, int es, const C* tw) {
+__device__ __forceinline__ C* fft_lines_inplace(C* a, int ln, int llo, int hi, int ls, int es,
+                                                const C* tw, int nt) {
   int lNs = ln & 3;
-  if (lNs == 1) fft_stage_inplace<1, SGN>(a, ln, 0, llo, hi, ls, es, tw);
-  if (lNs == 2) fft_stage_inplace<2, SGN>(a, ln, 0, llo, hi, ls, es, tw);
-  if (lNs == 3) fft_stage_inplace<3, SGN>(a, ln, 0, llo, hi, ls, es, tw);
+  if (lNs == 1) fft_stage_inplace<1, SGN>(a, ln, 0, llo, hi, ls, es, tw, nt);
+  if (lNs == 2) fft_stage_inplace<2, SGN>(a, ln, 0, llo, hi, ls, es, tw, nt);
+  if (lNs == 3) fft_stage_inplace<3, SGN>(a, ln, 0, llo, hi, ls, es, tw, nt);
   if (lNs != 0) __syncthreads();
   for (; lNs < ln; lNs += 4) {
-    fft_stage_inplace<4, SGN>(a, ln, lNs, llo, hi, ls, es, tw);
+    fft_stage_inplace<4, SGN>(a, ln, lNs, llo, hi, ls, es, tw, nt);
     __syncthreads();
   }
   return a;
@@ -246,9 +254,10 @@ __device__ __forceinline__ int ilog2(int v) { return 31 - __clz(v); }
 // shape's x_inpl says (the hot kernels are instantiated per form, so each holds one path)
 template <int SGN, int FORM, typename C>
 __device__ __forceinline__ const C* fft_x(bool inpl, C* a, C* b, int ln, int llo, int es,
-                                          const C* tw) {
-  if (FORM == 1 || (FORM == 2 && inpl)) return fft_lines_inplace<SGN>(a, ln, llo, 1, 1, es, tw);
-  return fft_lines<SGN>(a, b, ln, llo, 1, 1, es, tw);
+                                          const C* tw, int nt = NT) {
+  if (FORM == 1 || (FORM == 2 && inpl))
+    return fft_lines_inplace<SGN>(a, ln, llo, 1, 1, es, tw, nt);
+  return fft_lines<SGN>(a, b, ln, llo, 1, 1, es, tw, nt);
 }
 
 // --------------------------------------------------- stages that read or write global memory
@@ -276,6 +285,14 @@ template <typename C> struct ColIO {
   }
 };
 
+// the same for a full tile
+template <typename C> struct ColFullIO {
+  C* W;
+  int nxp;
+  __device__ __forceinline__ C ld(int l, int e) const { return W[e * nxp + l]; }
+  __device__ __forceinline__ void st(int l, int e, C v) const { W[e * nxp + l] = v; }
+};
+
 // z pass: line l = (component l >> ltz, column l & (tz - 1)); element e = plane kz
 template <typename C> struct ZIO {
   C* W;     // &W[0][0][ky][kx0]
@@ -295,12 +312,14 @@ template <typename C> struct ZIO {
 // fft_stage with accessors for its source and destination (same work mapping)
 template <int LR, int SGN, typename C, class SRC, class DST>
 __device__ __forceinline__ void fft_stage_io(const SRC& src, const DST& dst, int ln, int lNs,
-                                             int llo, int hi, const C* tw) {
+                                             int llo, int hi, const C* tw, int nt) {
   constexpr int R = 1 << LR;
   const int lnb = ln - LR, nb = 1 << lnb, Ns = 1 << lNs, lts = ln - lNs - LR;
   const int lo_mask = (1 << llo) - 1;
   const int total = hi << (llo + lnb);
-  for (int it = threadIdx.x; it < total; it += blockDim.x) {
+  for (int m = 0; m < trips(total, nt); ++m) {
+    const int it = threadIdx.x + m * nt;
+    if (total % nt != 0 && it >= total) break;
     const int ll = it & lo_mask;
     const int rest = it >> llo;
     const int j = rest & (nb - 1);
@@ -322,11 +341,11 @@ __device__ __forceinline__ void fft_stage_io(const SRC& src, const DST& dst, int
 
 template <int SGN, typename C, class SRC, class DST>
 __device__ __forceinline__ void stage_any(int LR, const SRC& src, const DST& dst, int ln, int lNs,
-                                          int llo, int hi, const C* tw) {
-  if (LR == 1) fft_stage_io<1, SGN>(src, dst, ln, lNs, llo, hi, tw);
-  else if (LR == 2) fft_stage_io<2, SGN>(src, dst, ln, lNs, llo, hi, tw);
-  else if (LR == 3) fft_stage_io<3, SGN>(src, dst, ln, lNs, llo, hi, tw);
-  else fft_stage_io<4, SGN>(src, dst, ln, lNs, llo, hi, tw);
+                                          int llo, int hi, const C* tw, int nt) {
+  if (LR == 1) fft_stage_io<1, SGN>(src, dst, ln, lNs, llo, hi, tw, nt);
+  else if (LR == 2) fft_stage_io<2, SGN>(src, dst, ln, lNs, llo, hi, tw, nt);
+  else if (LR == 3) fft_stage_io<3, SGN>(src, dst, ln, lNs, llo, hi, tw, nt);
+  else fft_stage_io<4, SGN>(src, dst, ln, lNs, llo, hi, tw, nt);
 }
 
 // Transforms of length 2^ln (plan as in fft_lines) whose first stage reads global memory
@@ -335,7 +354,7 @@ __device__ __forceinline__ void stage_any(int LR, const SRC& src, const DST& dst
 // visible by the second stage: a barrier follows every stage but the last.
 template <int SGN, typename C, class SRC>
 __device__ C* fft_from_global(const SRC& first, C* a, C* b, int ls, int es, int ln, int llo,
-                              int hi, const C* tw) {
+                              int hi, const C* tw, int nt) {
   const int rem = ln & 3, nst = (rem ? 1 : 0) + (ln >> 2);
   int lNs = 0;
   C* cur = b;
@@ -343,9 +362,9 @@ __device__ C* fft_from_global(const SRC& first, C* a, C* b, int ls, int es, int 
   for (int s = 0; s < nst; ++s) {
     const int LR = (s == 0 && rem) ? rem : 4;
     if (s == 0)
-      stage_any<SGN>(LR, first, SmemIO<C>{cur, ls, es}, ln, lNs, llo, hi, tw);
+      stage_any<SGN>(LR, first, SmemIO<C>{cur, ls, es}, ln, lNs, llo, hi, tw, nt);
     else
-      stage_any<SGN>(LR, SmemIO<C>{oth, ls, es}, SmemIO<C>{cur, ls, es}, ln, lNs, llo, hi, tw);
+      stage_any<SGN>(LR, SmemIO<C>{oth, ls, es}, SmemIO<C>{cur, ls, es}, ln, lNs, llo, hi, tw, nt);
     __syncthreads();
     lNs += LR;
     C* t = cur;   // the result of this stage becomes the next input
@@ -358,15 +377,15 @@ __device__ C* fft_from_global(const SRC& first, C* a, C* b, int ls, int es, int 
 // input in `in` (visible to the block), scratch `oth`; the last stage writes through `last`
 template <int SGN, typename C, class DST>
 __device__ void fft_to_global(C* in, C* oth, const DST& last, int ls, int es, int ln, int llo,
-                              int hi, const C* tw) {
+                              int hi, const C* tw, int nt) {
   const int rem = ln & 3, nst = (rem ? 1 : 0) + (ln >> 2);
   int lNs = 0;
   for (int s = 0; s < nst; ++s) {
     const int LR = (s == 0 && rem) ? rem : 4;
     if (s == nst - 1) {
-      stage_any<SGN>(LR, SmemIO<C>{in, ls, es}, last, ln, lNs, llo, hi, tw);
+      stage_any<SGN>(LR, SmemIO<C>{in, ls, es}, last, ln, lNs, llo, hi, tw, nt);
     } else {
-      stage_any<SGN>(LR, SmemIO<C>{in, ls, es}, SmemIO<C>{oth, ls, es}, ln, lNs, llo, hi, tw);
+      stage_any<SGN>(LR, SmemIO<C>{in, ls, es}, SmemIO<C>{oth, ls, es}, ln, lNs, llo, hi, tw, nt);
       __syncthreads();
       C* t = in;
       in = oth;
@@ -378,13 +397,13 @@ __device__ void fft_to_global(C* in, C* oth, const DST& last, int ls, int es, in
 
 // global lines in place: through shared memory, both ends direct
 template <int SGN, typename C, class IO>
-__device__ void fft_global_inplace(const IO& io, C* a, C* b, int ls, int es, int ln, int llo,
-                                   int hi, const C* tw) {
+__device__ __forceinline__ void fft_global_inplace(const IO& io, C* a, C* b, int ls, int es, int ln, int llo,
+                                   int hi, const C* tw, int nt) {
   const int rem = ln & 3, nst = (rem ? 1 : 0) + (ln >> 2);
   if (nst == 1) {   // one stage: stage into shared memory first (its reads and writes overlap)
-    C* r = fft_from_global<SGN>(io, a, b, ls, es, ln, llo, hi, tw);
+    C* r = fft_from_global<SGN>(io, a, b, ls, es, ln, llo, hi, tw, nt);
     const int nl = hi << llo, n = 1 << ln;
-    for (int q = threadIdx.x; q < nl * n; q += blockDim.x) {
+    for (int q = threadIdx.x; q < nl * n; q += nt) {
       const int l = q % nl, e = q / nl;
       io.st(l, e, r[l * ls + e * es]);
     }
@@ -392,7 +411,7 @@ __device__ void fft_global_inplace(const IO& io, C* a, C* b, int ls, int es, int
   }
   // first stage: global -> b; middle stages ping-pong; last stage -> global
   const int LR0 = rem ? rem : 4;
-  stage_any<SGN>(LR0, io, SmemIO<C>{b, ls, es}, ln, 0, llo, hi, tw);
+  stage_any<SGN>(LR0, io, SmemIO<C>{b, ls, es}, ln, 0, llo, hi, tw, nt);
   __syncthreads();
   const int rest_ln = ln;   // the remaining stages continue from Ns = 2^LR0
   int lNs = LR0;
@@ -400,9 +419,9 @@ __device__ void fft_global_inplace(const IO& io, C* a, C* b, int ls, int es, int
   C* oth = a;
   for (int s = 1; s < nst; ++s) {
     if (s == nst - 1) {
-      stage_any<SGN>(4, SmemIO<C>{in, ls, es}, io, rest_ln, lNs, llo, hi, tw);
+      stage_any<SGN>(4, SmemIO<C>{in, ls, es}, io, rest_ln, lNs, llo, hi, tw, nt);
     } else {
-      stage_any<SGN>(4, SmemIO<C>{in, ls, es}, SmemIO<C>{oth, ls, es}, rest_ln, lNs, llo, hi, tw);
+      stage_any<SGN>(4, SmemIO<C>{in, ls, es}, SmemIO<C>{oth, ls, es}, rest_ln, lNs, llo, hi, tw, nt);
       __syncthreads();
       C* t = in;
       in = oth;
@@ -469,6 +488,24 @@ __device__ __forceinline__ bool block_sum_end(BlockSum& B, double* partial, unsi
   return true;
 }
 
+// Compile-time line lengths (FP32).  The passes below are bound by instruction issue where their
+// data is in L2 (128^3: 252 instructions per voxel in the forward x pass, 295 in the inverse,
+// 132 in a y pass, of which the transforms' arithmetic is 40), most of them index arithmetic,
+// bounds checks and loop control of the general line length and tile.  LN > 0 instantiates a
+// pass for lines of 2^LN and its usual tile, 16 lines or columns; LN = 0 is the general form.
+// The arithmetic is the same.  us a pass, general -> compile-time: mixed 64^3 study 10870 -> 9960,
+// 128^3 14494 -> 13640, 256^3 126490 -> 122140 (per launch, update + forward 185 -> 161, inverse 197
+// -> 175).  The x passes take 64, 128 and 256; the y pass 64 and 128 (at 256 its four blocks per
+// SM leave 64 registers, which the unrolled form spills: 72 -> 88 us).  The FP64 passes stay
+// general: the FP64 pipe bounds them (128^3 50370 -> 50640).
+constexpr int XPB = 16, XLPB = 4;   // lines per block of the compile-time forms
+int x_lines(const Spec<float>& V) {
+  return V.pb == XPB && (V.nx == 64 || V.nx == 128 || V.nx == 256) ? 31 - __builtin_clz(V.nx) : 0;
+}
+int y_lines(const Spec<float>& V) {
+  return V.tx == XPB && (V.ny == 64 || V.ny == 128) ? 31 - __builtin_clz(V.ny) : 0;
+}
+
 // ---------------------------------------------------------------------------- x forward
 // block (pair tile, z, component): rows y0 .. y0 + 2 pb - 1 of plane z.  The staged lines
 // are interleaved, element e of line l at e * es + l; es = pb + 1 keeps the row-wise staging
@@ -495,14 +532,34 @@ __device__ __forceinline__ XTile<R> x_tile(const Spec<R>& V) {
 }
 
 // transform the staged rows (in a) and write both half spectra to W
-template <typename R, int FORM>
+template <typename R, int FORM, int LN>
 __device__ __forceinline__ void x_fwd_finish(const Spec<R>& V, const XTile<R>& t,
                                              typename CxOf<R>::T* a, typename CxOf<R>::T* b,
                                              const typename CxOf<R>::T* tw) {
   using C = typename CxOf<R>::T;
+  C* W = V.W + (((size_t)t.comp * V.nz + t.z) * V.ny + t.y0) * V.nxp;
+  if constexpr (LN > 0) {
+    constexpr int n = 1 << LN, es = XPB + 1, half = n / 2;
+    const C* F = fft_x<-1, FORM>(false, a, b, LN, XLPB, es, tw);
+    auto out = [&](int l, int k, C f, C g) {
+      C* w = W + (2 * l) * V.nxp + k;
+      w[0] = C{(R)0.5 * (f.x + g.x), (R)0.5 * (f.y - g.y)};
+      w[V.nxp] = C{(R)0.5 * (f.y + g.y), (R)-0.5 * (f.x - g.x)};
+    };
+    const int k = threadIdx.x & (half - 1), l0 = threadIdx.x >> (LN - 1), kk = (n - k) & (n - 1);
+#pragma unroll 4
+    for (int m = 0; m < XPB * half / NT; ++m) {
+      const int l = l0 + m * (NT / half);
+      out(l, k, F[k * es + l], F[kk * es + l]);
+    }
+    if (threadIdx.x < XPB) {
+      const C f = F[half * es + threadIdx.x];
+      out(threadIdx.x, half, f, f);
+    }
+    return;
+  }
   const int n = t.n, es = t.es;
   const C* F = fft_x<-1, FORM>(V.x_inpl != 0, a, b, t.ln, ilog2(t.pb), es, tw);
-  C* W = V.W + (((size_t)t.comp * V.nz + t.z) * V.ny + t.y0) * V.nxp;
   for (int idx = threadIdx.x; idx < t.pb * V.nxh; idx += blockDim.x) {
     const int l = idx / V.nxh, k = idx - l * V.nxh;
     const C f = F[k * es + l], g = F[((n - k) & (n - 1)) * es + l];
@@ -550,7 +607,7 @@ __global__ void __launch_bounds__(NT) k_spec_x_fwd(Spec<R> V, const R* __restric
     }
   }
   __syncthreads();
-  x_fwd_finish<R, 2>(V, t, a, b, tw);
+  x_fwd_finish<R, 2, 0>(V, t, a, b, tw);
 }
 
 // The mixed precision's residual update fused into the x forward pass: for the block's rows
@@ -563,7 +620,7 @@ __global__ void __launch_bounds__(NT) k_spec_x_fwd(Spec<R> V, const R* __restric
 // barriers instead of one but half the shared memory, which pays where two buffers leave the
 // SM fewer than four blocks (lines of 256: 72 KB a block); us a pass, 0 -> 1: mixed 256^3 131950
 // -> 128600, but 128^3 14763 -> 14874 and 64^3 11730 -> 11950, where both fit four times.
-template <int FORM>
+template <int FORM, int LN>
 __global__ void __launch_bounds__(NT, 4) k_spec_update_xfwd(Spec<float> V, Elas32 I) {
   pdl_sync();
   using C = float2;
@@ -580,32 +637,66 @@ __global__ void __launch_bounds__(NT, 4) k_spec_update_xfwd(Spec<float> V, Elas3
   const float* sc = V.s[t.comp];   // the transform takes s r with the scaled preconditioner
   constexpr int UB = 4;
   float rr = 0.0f;
-  const int total = t.pb * n;
-  for (int i0 = threadIdx.x; i0 < total; i0 += UB * blockDim.x) {
-    float ra[UB], rb[UB], qa[UB], qb[UB], sa[UB], sb[UB];
+  if constexpr (LN > 0) {
+    // thread's element m: line (tid >> LN) + m NT / n, position tid & (n - 1): a step of m is
+    // two rows times NT / n lines, 2 NT values whatever n
+    constexpr int N = 1 << LN;
+    const size_t o0 = t.row0 + (threadIdx.x >> LN) * (2 * N) + (threadIdx.x & (N - 1));
+    float* const rt = r + o0;
+    const float* const qt = q + o0;
+    const float* const st = sc ? sc + o0 : nullptr;
+    C* const at = a + (threadIdx.x & (N - 1)) * (XPB + 1) + (threadIdx.x >> LN);
+#pragma unroll 1
+    for (int m0 = 0; m0 < XPB * N / NT; m0 += UB) {
+      float ra[UB], rb[UB], qa[UB], qb[UB], sa[UB], sb[UB];
 #pragma unroll
-    for (int u = 0; u < UB; ++u) {
-      const int idx = i0 + u * blockDim.x;
-      if (idx < total) {
-        const size_t o = t.row0 + (size_t)(2 * (idx >> ln)) * n + (idx & (n - 1));
-        ra[u] = r[o];
-        rb[u] = r[o + n];
-        qa[u] = q[o];
-        qb[u] = q[o + n];
-        sa[u] = sc ? __ldg(sc + o) : 1.0f;
-        sb[u] = sc ? __ldg(sc + o + n) : 1.0f;
+      for (int u = 0; u < UB; ++u) {
+        const int o = (m0 + u) * (2 * NT);
+        ra[u] = rt[o];
+        rb[u] = rt[o + N];
+        qa[u] = qt[o];
+        qb[u] = qt[o + N];
+        sa[u] = st ? __ldg(st + o) : 1.0f;
+        sb[u] = st ? __ldg(st + o + N) : 1.0f;
+      }
+#pragma unroll
+      for (int u = 0; u < UB; ++u) {
+        const int o = (m0 + u) * (2 * NT);
+        const float xa = ra[u] - alpha * qa[u], xb = rb[u] - alpha * qb[u];
+        rt[o] = xa;
+        rt[o + N] = xb;
+        rr += xa * xa + xb * xb;
+        at[(m0 + u) * (NT / N)] = C{xa * sa[u], xb * sb[u]};
       }
     }
+  } else {
+    const int total = t.pb * n;
+    for (int i0 = threadIdx.x; i0 < total; i0 += UB * blockDim.x) {
+      float ra[UB], rb[UB], qa[UB], qb[UB], sa[UB], sb[UB];
 #pragma unroll
-    for (int u = 0; u < UB; ++u) {
-      const int idx = i0 + u * blockDim.x;
-      if (idx < total) {
-        const size_t o = t.row0 + (size_t)(2 * (idx >> ln)) * n + (idx & (n - 1));
-        const float xa = ra[u] - alpha * qa[u], xb = rb[u] - alpha * qb[u];
-        r[o] = xa;
-        r[o + n] = xb;
-        rr += xa * xa + xb * xb;
-        a[(idx & (n - 1)) * es + (idx >> ln)] = C{xa * sa[u], xb * sb[u]};
+      for (int u = 0; u < UB; ++u) {
+        const int idx = i0 + u * blockDim.x;
+        if (idx < total) {
+          const size_t o = t.row0 + (size_t)(2 * (idx >> ln)) * n + (idx & (n - 1));
+          ra[u] = r[o];
+          rb[u] = r[o + n];
+          qa[u] = q[o];
+          qb[u] = q[o + n];
+          sa[u] = sc ? __ldg(sc + o) : 1.0f;
+          sb[u] = sc ? __ldg(sc + o + n) : 1.0f;
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < UB; ++u) {
+        const int idx = i0 + u * blockDim.x;
+        if (idx < total) {
+          const size_t o = t.row0 + (size_t)(2 * (idx >> ln)) * n + (idx & (n - 1));
+          const float xa = ra[u] - alpha * qa[u], xb = rb[u] - alpha * qb[u];
+          r[o] = xa;
+          r[o + n] = xb;
+          rr += xa * xa + xb * xb;
+          a[(idx & (n - 1)) * es + (idx >> ln)] = C{xa * sa[u], xb * sb[u]};
+        }
       }
     }
   }
@@ -613,27 +704,33 @@ __global__ void __launch_bounds__(NT, 4) k_spec_update_xfwd(Spec<float> V, Elas3
   const int nb = gridDim.x * gridDim.y * gridDim.z;
   const int bl = (blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
   block_sum_begin(B, (double)rr, V.partial, V.counter, bl, nb);   // also publishes the staging
-  x_fwd_finish<float, FORM>(V, t, a, b, tw);
+  x_fwd_finish<float, FORM, LN>(V, t, a, b, tw);
   double out;
   if (block_sum_end(B, V.partial, V.counter, nb, out)) cg_after_update_rr(*I.S, out);
 }
 
 // ---------------------------------------------------------------------------- y pass
 // block (mode-column tile, z, component), in place; the FP32 pass at four blocks per SM
-template <typename R, int SGN>
+template <typename R, int SGN, int LN>
 __global__ void __launch_bounds__(NT, sizeof(R) == 4 ? 4 : 0) k_spec_y(Spec<R> V, const CgScal* S) {
   pdl_sync();
   using C = typename CxOf<R>::T;
   if (spec_skip<R>(S)) return;
-  const int tx = V.tx, ltx = ilog2(tx);
+  const int tx = LN > 0 ? XPB : V.tx, ny = LN > 0 ? 1 << LN : V.ny;
   C* tw = smem_cx<C>();
-  C* a = tw + V.ny;
-  C* b = spec_y_buffers(V.ny) == 1 ? a : a + (size_t)tx * V.ny;   // one or two stages: b only
-  load_roots(tw, V.tw[1], V.ny);
+  C* a = tw + ny;
+  C* b = spec_y_buffers(ny) == 1 ? a : a + (size_t)tx * ny;   // one or two stages: b only
+  load_roots(tw, V.tw[1], ny);
   const int kx0 = blockIdx.x * tx, z = blockIdx.y, comp = blockIdx.z;
-  const ColIO<C> io{V.W + ((size_t)comp * V.nz + z) * V.ny * V.nxp + kx0, V.nxp,
-                    min(tx, V.nxh - kx0)};
-  fft_global_inplace<SGN>(io, a, b, 1, tx, ilog2(V.ny), ltx, 1, tw);
+  C* const W = V.W + ((size_t)comp * V.nz + z) * V.ny * V.nxp + kx0;
+  const int ncol = min(tx, V.nxh - kx0);
+  if (LN > 0 && ncol == XPB) {
+    const ColFullIO<C> io{W, V.nxp};
+    fft_global_inplace<SGN>(io, a, b, 1, XPB, LN, XLPB, 1, tw, NT);
+    return;
+  }
+  const ColIO<C> io{W, V.nxp, ncol};
+  fft_global_inplace<SGN>(io, a, b, 1, tx, ilog2(ny), ilog2(tx), 1, tw, NT);
 }
 
 // ---------------------------------------------------------------------------- z pass
@@ -665,7 +762,8 @@ __global__ void __launch_bounds__(NARROW ? Z_NARROW_THREADS : NT) k_spec_z(Spec<
   const int ncol = min(tz, V.nxh - kx0);
   const size_t plane = (size_t)V.ny * V.nxp, comp_stride = (size_t)V.nz * plane;
   const ZIO<C> io{V.W + (size_t)ky * V.nxp + kx0, plane, comp_stride, tz, ltz, ncol};
-  C* F = fft_from_global<-1>(io, a, b, 1, lw, ilog2(V.nz), ltz, 3, tw);
+  C* F = fft_from_global<-1>(io, a, b, 1, lw, ilog2(V.nz), ltz, 3, tw,
+                                NARROW ? Z_NARROW_THREADS : (int)blockDim.x);
   C* other = F == a ? b : a;
   // FP32: no FP64 operation (the volume is a power of two, so both forms are exact)
   const R mu0 = sizeof(R) == 4 ? f32_of(V.mean[0]) : (R)V.mean[0];
@@ -729,7 +827,8 @@ __global__ void __launch_bounds__(NARROW ? Z_NARROW_THREADS : NT) k_spec_z(Spec<
     block_sum_begin(B, (double)rz_part, V.partial, V.counter,
                     blockIdx.y * gridDim.x + blockIdx.x, gridDim.x * gridDim.y);
   __syncthreads();
-  fft_to_global<+1>(F, other, io, 1, lw, ilog2(V.nz), ltz, 3, tw);
+  fft_to_global<+1>(F, other, io, 1, lw, ilog2(V.nz), ltz, 3, tw,
+                    NARROW ? Z_NARROW_THREADS : (int)blockDim.x);
   if (S == nullptr) return;
   double out;
   if (block_sum_end(B, V.partial, V.counter, gridDim.x * gridDim.y, out))
@@ -1138,13 +1237,14 @@ __global__ void __launch_bounds__(ZR_COLS * P)
 // direction p = z + beta p_old (beta = 0 on a solve's first iteration) and, from the p_old in
 // hand, the iterate of the iteration that ends here, e += alpha p_old.  An iteration that
 // converged does not get here: the refinement's correction adds its alpha p (PUpd::e).
-template <typename R, bool PUP, int FORM>
+template <typename R, bool PUP, int FORM, int LN>
 __global__ void __launch_bounds__(NT, PUP ? 4 : 2) k_spec_x_inv(Spec<R> V, R* z0, R* z1, R* z2,
                                                                 const CgScal* S, PUpd<R> PU) {
   pdl_sync();
   using C = typename CxOf<R>::T;
   if (spec_skip<R>(S)) return;
-  const int n = V.nx, ln = ilog2(n), half = n / 2, pb = V.pb, es = pb + 1;
+  const int n = LN > 0 ? 1 << LN : V.nx, ln = LN > 0 ? LN : ilog2(n), half = n / 2;
+  const int pb = LN > 0 ? XPB : V.pb, es = pb + 1;
   C* tw = smem_cx<C>();
   C* a = tw + n;
   C* b = a + (size_t)es * n;
@@ -1152,32 +1252,67 @@ __global__ void __launch_bounds__(NT, PUP ? 4 : 2) k_spec_x_inv(Spec<R> V, R* z0
   const int comp = blockIdx.z, z = blockIdx.y, y0 = 2 * V.pb * blockIdx.x;
   const C* W = V.W + (((size_t)comp * V.nz + z) * V.ny + y0) * V.nxp;
   const int total = pb * n;
-  for (int i0 = threadIdx.x; i0 < total; i0 += LB * blockDim.x) {
-    C A[LB], B[LB];
+  if constexpr (LN > 0) {
+    // a thread takes modes k < n / 2 and writes both C[k] and its mirror C[n - k]; k = 0 and
+    // n / 2 (real in each row) have none
+    constexpr int H = 1 << (LN - 1), N = 2 * H, IB = PUP ? 4 : 2;
+    const int k = threadIdx.x & (H - 1), l0 = threadIdx.x >> (LN - 1);
+    const C* const w0 = W + (2 * l0) * V.nxp + k;
+    const int step = 2 * (NT / H) * V.nxp;
+    C* const ak = a + k * es + l0;
+    C* const am = a + ((N - k) & (N - 1)) * es + l0;
+#pragma unroll 1
+    for (int m0 = 0; m0 < XPB * H / NT; m0 += IB < XPB * H / NT ? IB : XPB * H / NT) {
+      constexpr int U = IB < XPB * H / NT ? IB : XPB * H / NT;
+      C A[U], B[U];
 #pragma unroll
-    for (int u = 0; u < LB; ++u) {
-      const int idx = i0 + u * blockDim.x;
-      if (idx < total) {
-        const int l = idx >> ln, k = idx & (n - 1);
-        const int kk = k <= half ? k : n - k;
-        A[u] = __ldg(W + (size_t)(2 * l) * V.nxp + kk);
-        B[u] = __ldg(W + (size_t)(2 * l + 1) * V.nxp + kk);
+      for (int u = 0; u < U; ++u) {
+        A[u] = __ldg(w0 + (m0 + u) * step);
+        B[u] = __ldg(w0 + (m0 + u) * step + V.nxp);
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int d = (m0 + u) * (NT / H);
+        if (k == 0) {
+          ak[d] = C{A[u].x, B[u].x};
+        } else {
+          ak[d] = C{A[u].x - B[u].y, A[u].y + B[u].x};
+          am[d] = C{A[u].x + B[u].y, B[u].x - A[u].y};
+        }
       }
     }
+    if (threadIdx.x < XPB) {
+      const C* const wh = W + (2 * threadIdx.x) * V.nxp + H;
+      a[H * es + threadIdx.x] = C{__ldg(wh).x, __ldg(wh + V.nxp).x};
+    }
+  } else {
+    for (int i0 = threadIdx.x; i0 < total; i0 += LB * blockDim.x) {
+      C A[LB], B[LB];
 #pragma unroll
-    for (int u = 0; u < LB; ++u) {
-      const int idx = i0 + u * blockDim.x;
-      if (idx < total) {
-        const int l = idx >> ln, k = idx & (n - 1);
-        C a_ = A[u], b_ = B[u];
-        if (k == 0 || k == half) {
-          a_.y = (R)0;
-          b_.y = (R)0;
-        } else if (k > half) {
-          a_.y = -a_.y;
-          b_.y = -b_.y;
+      for (int u = 0; u < LB; ++u) {
+        const int idx = i0 + u * blockDim.x;
+        if (idx < total) {
+          const int l = idx >> ln, k = idx & (n - 1);
+          const int kk = k <= half ? k : n - k;
+          A[u] = __ldg(W + (size_t)(2 * l) * V.nxp + kk);
+          B[u] = __ldg(W + (size_t)(2 * l + 1) * V.nxp + kk);
         }
-        a[k * es + l] = C{a_.x - b_.y, a_.y + b_.x};
+      }
+#pragma unroll
+      for (int u = 0; u < LB; ++u) {
+        const int idx = i0 + u * blockDim.x;
+        if (idx < total) {
+          const int l = idx >> ln, k = idx & (n - 1);
+          C a_ = A[u], b_ = B[u];
+          if (k == 0 || k == half) {
+            a_.y = (R)0;
+            b_.y = (R)0;
+          } else if (k > half) {
+            a_.y = -a_.y;
+            b_.y = -b_.y;
+          }
+          a[k * es + l] = C{a_.x - b_.y, a_.y + b_.x};
+        }
       }
     }
   }
@@ -1202,6 +1337,41 @@ __global__ void __launch_bounds__(NT, PUP ? 4 : 2) k_spec_x_inv(Spec<R> V, R* z0
   const R* sc = V.s[comp];   // z = s A0^{-1} (s r) with the scaled preconditioner
   const size_t row0 = ((size_t)z * V.ny + y0) * n;
   constexpr int OB = PUP ? 4 : LB;   // loads in flight: 6 or 2 times this many
+  if constexpr (LN > 0) {
+    constexpr int N = 1 << LN, M = XPB * N / NT, U = OB < M ? OB : M;
+    const size_t o0 = row0 + (threadIdx.x >> LN) * (2 * N) + (threadIdx.x & (N - 1));
+    R* const outp = out + o0;
+    const R* const st = sc ? sc + o0 : nullptr;
+    const R* const pt = PUP && pold ? pold + o0 : nullptr;
+    R* const et = PUP && pold ? e + o0 : nullptr;
+    const C* const Ft = F + (threadIdx.x & (N - 1)) * es + (threadIdx.x >> LN);
+#pragma unroll 1
+    for (int m0 = 0; m0 < M; m0 += U) {
+      R sa[U], sb[U], pa[U], pbv[U], ea[U], eb[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int o = (m0 + u) * (2 * NT);
+        sa[u] = st ? __ldg(st + o) : (R)1;
+        sb[u] = st ? __ldg(st + o + N) : (R)1;
+        pa[u] = pt ? pt[o] : (R)0;
+        pbv[u] = pt ? pt[o + N] : (R)0;
+        ea[u] = pt ? et[o] : (R)0;
+        eb[u] = pt ? et[o + N] : (R)0;
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int o = (m0 + u) * (2 * NT);
+        const C f = Ft[(m0 + u) * (NT / N)];
+        outp[o] = PUP ? f.x * sa[u] + beta * pa[u] : f.x * sa[u];
+        outp[o + N] = PUP ? f.y * sb[u] + beta * pbv[u] : f.y * sb[u];
+        if (PUP && pt) {
+          et[o] = ea[u] + alpha * pa[u];
+          et[o + N] = eb[u] + alpha * pbv[u];
+        }
+      }
+    }
+    return;
+  }
   for (int i0 = threadIdx.x; i0 < total; i0 += OB * blockDim.x) {
     R sa[OB], sb[OB], pa[OB], pbv[OB], ea[OB], eb[OB];
 #pragma unroll
@@ -1327,7 +1497,8 @@ __global__ void __launch_bounds__(NT) k_spec_scale(long long n, Spec<R> V, Elas 
 
 // Every pass kernel may use up to the device's opt-in shared memory per block, less 3 KB for
 // the kernels' static shared memory (the attribute is a limit, not a reservation), so
-// contexts of different grid sizes never lower it for one another; V's own needs must fit.
+// contexts of different grid sizes never lower it for one another; V's own needs must fit.  The
+// compile-time forms take less than the default 48 KB.
 template <typename R>
 cudaError_t spec_prepare(const Spec<R>& V) {
   int dev = 0, optin = 0;
@@ -1340,15 +1511,15 @@ cudaError_t spec_prepare(const Spec<R>& V) {
     return cudaErrorInvalidValue;
   const cudaFuncAttribute A = cudaFuncAttributeMaxDynamicSharedMemorySize;
   e = cudaFuncSetAttribute(k_spec_x_fwd<R>, A, optin);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_spec_update_xfwd<0>, A, optin);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_spec_update_xfwd<1>, A, optin);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_spec_x_inv<R, false, 2>, A, optin);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_spec_update_xfwd<0, 0>, A, optin);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_spec_update_xfwd<1, 0>, A, optin);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_spec_x_inv<R, false, 2, 0>, A, optin);
   if constexpr (sizeof(R) == 4) {
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_spec_x_inv<R, true, 0>, A, optin);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_spec_x_inv<R, true, 1>, A, optin);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_spec_x_inv<R, true, 0, 0>, A, optin);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_spec_x_inv<R, true, 1, 0>, A, optin);
   }
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_spec_y<R, -1>, A, optin);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_spec_y<R, +1>, A, optin);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_spec_y<R, -1, 0>, A, optin);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_spec_y<R, +1, 0>, A, optin);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(k_spec_z<R, false>, A, optin);
   if constexpr (sizeof(R) == 4) {
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k_spec_zr<16>, A, optin);
@@ -1461,34 +1632,56 @@ void launch_spec_z(const Spec<R>& V, CgScal* S, cudaStream_t st) {
   TG_TIMED(K_SPEC_Z, st, launch((k_spec_z<R, false>), gz, V.nt_z, spec_smem_z(V), st, V, S));
 }
 
+// A pass in its compile-time form for the plan's line length, else the general one.
+template <int SGN, typename R>
+void launch_spec_y(const Spec<R>& V, const CgScal* S, cudaStream_t st) {
+  const dim3 g((V.nxh + V.tx - 1) / V.tx, V.nz, 3);
+  const size_t smem = spec_smem_y(V);
+  auto go = [&](auto kernel) {
+    TG_TIMED(SGN < 0 ? K_SPEC_Y_FWD : K_SPEC_Y_INV, st, launch(kernel, g, NT, smem, st, V, S));
+  };
+  if constexpr (sizeof(R) == 4) {
+    if (y_lines(V) == 6) return go(k_spec_y<R, SGN, 6>);
+    if (y_lines(V) == 7) return go(k_spec_y<R, SGN, 7>);
+  }
+  return go(k_spec_y<R, SGN, 0>);
+}
+
+// the x inverse pass with the p-update, P the buffers (mixed precision)
+void launch_spec_x_inv_p(const Spec<float>& V, float* const z[3], const CgScal* S,
+                         const PUpd<float>& P, cudaStream_t st) {
+  const dim3 g(V.ny / (2 * V.pb), V.nz, 3);
+  const size_t smem = spec_smem_x(V);
+  auto go = [&](auto kernel) {
+    TG_TIMED(K_SPEC_X_INV_P, st, launch(kernel, g, NT, smem, st, V, z[0], z[1], z[2], S, P));
+  };
+  switch (V.x_inpl ? x_lines(V) : 0) {
+    case 6: return go(k_spec_x_inv<float, true, 1, 6>);
+    case 7: return go(k_spec_x_inv<float, true, 1, 7>);
+    case 8: return go(k_spec_x_inv<float, true, 1, 8>);
+    default: break;
+  }
+  return V.x_inpl ? go(k_spec_x_inv<float, true, 1, 0>) : go(k_spec_x_inv<float, true, 0, 0>);
+}
+
 template <typename R>
 cudaError_t launch_spectral(const Spec<R>& V, const R* const r[3], R* const z[3], CgScal* S,
                             cudaStream_t st, const PUpd<R>* pu) {
   const dim3 gx(V.ny / (2 * V.pb), V.nz, 3);
-  const dim3 gy((V.nxh + V.tx - 1) / V.tx, V.nz, 3);
   TG_TIMED(K_SPEC_X_FWD, st,
            launch(k_spec_x_fwd<R>, gx, NT, spec_smem_x(V), st, V, r[0], r[1], r[2], S));
-  TG_TIMED(K_SPEC_Y_FWD, st, launch((k_spec_y<R, -1>), gy, NT, spec_smem_y(V), st, V, S));
+  launch_spec_y<-1>(V, S, st);
   launch_spec_z(V, S, st);
-  TG_TIMED(K_SPEC_Y_INV, st, launch((k_spec_y<R, +1>), gy, NT, spec_smem_y(V), st, V, S));
-  PUpd<R> P = {};
+  launch_spec_y<+1>(V, S, st);
   if constexpr (sizeof(R) == 4) {
     if (pu) {
-      P = *pu;
-      if (V.x_inpl)
-        TG_TIMED(K_SPEC_X_INV_P, st,
-                 launch((k_spec_x_inv<R, true, 1>), gx, NT, spec_smem_x(V), st, V, z[0], z[1],
-                        z[2], S, P));
-      else
-        TG_TIMED(K_SPEC_X_INV_P, st,
-                 launch((k_spec_x_inv<R, true, 0>), gx, NT, spec_smem_x(V), st, V, z[0], z[1],
-                        z[2], S, P));
+      launch_spec_x_inv_p(V, z, S, *pu, st);
       return cudaGetLastError();
     }
   }
   TG_TIMED(K_SPEC_X_INV, st,
-           launch((k_spec_x_inv<R, false, 2>), gx, NT, spec_smem_x(V), st, V, z[0], z[1], z[2], S,
-                  P));
+           launch((k_spec_x_inv<R, false, 2, 0>), gx, NT, spec_smem_x(V), st, V, z[0], z[1], z[2],
+                  S, PUpd<R>{}));
   return cudaGetLastError();
 }
 
@@ -1497,29 +1690,33 @@ cudaError_t launch_spectral(const Spec<R>& V, const R* const r[3], R* const z[3]
 cudaError_t launch_spectral_update(const Spec<float>& V, const Elas32& I, float* const z[3],
                                    cudaStream_t st) {
   const dim3 gx(V.ny / (2 * V.pb), V.nz, 3);
-  const dim3 gy((V.nxh + V.tx - 1) / V.tx, V.nz, 3);
-  if (V.x_inpl && 4 * spec_smem_x2(V) > 224 * 1024)
-    TG_TIMED(K_SPEC_UPDATE_XFWD, st,
-             launch(k_spec_update_xfwd<1>, gx, NT, spec_smem_x(V), st, V, I));
-  else
-    TG_TIMED(K_SPEC_UPDATE_XFWD, st,
-             launch(k_spec_update_xfwd<0>, gx, NT, spec_smem_x2(V), st, V, I));
-  TG_TIMED(K_SPEC_Y_FWD, st, launch((k_spec_y<float, -1>), gy, NT, spec_smem_y(V), st, V, I.S));
+  const int ln = x_lines(V);
+  const bool inplace = V.x_inpl && 4 * spec_smem_x2(V) > 224 * 1024;   // lines of 256
+  const size_t smem = inplace ? spec_smem_x(V) : spec_smem_x2(V);
+  auto go = [&](auto kernel) {
+    TG_TIMED(K_SPEC_UPDATE_XFWD, st, launch(kernel, gx, NT, smem, st, V, I));
+  };
+  if (inplace) {
+    if (ln == 8)
+      go(k_spec_update_xfwd<1, 8>);
+    else
+      go(k_spec_update_xfwd<1, 0>);
+  } else if (ln == 6) {
+    go(k_spec_update_xfwd<0, 6>);
+  } else if (ln == 7) {
+    go(k_spec_update_xfwd<0, 7>);
+  } else {
+    go(k_spec_update_xfwd<0, 0>);
+  }
+  launch_spec_y<-1>(V, I.S, st);
   launch_spec_z(V, I.S, st);
-  TG_TIMED(K_SPEC_Y_INV, st, launch((k_spec_y<float, +1>), gy, NT, spec_smem_y(V), st, V, I.S));
+  launch_spec_y<+1>(V, I.S, st);
   PUpd<float> P;   // p = z + beta p_old straight from the last pass
   for (int a = 0; a < 3; ++a) {
     P.e[a] = I.e[a];
     for (int b = 0; b < 2; ++b) P.p[b][a] = I.p[b][a];
   }
-  if (V.x_inpl)
-    TG_TIMED(K_SPEC_X_INV_P, st,
-             launch((k_spec_x_inv<float, true, 1>), gx, NT, spec_smem_x(V), st, V, z[0], z[1],
-                    z[2], I.S, P));
-  else
-    TG_TIMED(K_SPEC_X_INV_P, st,
-             launch((k_spec_x_inv<float, true, 0>), gx, NT, spec_smem_x(V), st, V, z[0], z[1],
-                    z[2], I.S, P));
+  launch_spec_x_inv_p(V, z, I.S, P, st);
   return cudaGetLastError();
 }
 
