@@ -454,6 +454,7 @@ template <typename R> size_t spec_smem_z(const Spec<R>& V) {
 constexpr long long PDL_MAX_VOXELS = 1LL << 23;
 constexpr long long PDL_CARVE_VOXELS = 1LL << 17;
 constexpr int PDL_CARVE_PERCENT = 60;
+constexpr int PDL_CARVE_ALL = 100;   // for a kernel whose blocks per SM its shared memory limits
 
 __device__ __forceinline__ void pdl_sync() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -476,8 +477,8 @@ inline long long launch_voxels(const T&) {
 // Every kernel launched here calls pdl_sync first, on every path, so a kernel that has finished
 // implies that all before it on its stream have.
 template <class... P, class... A>
-inline void launch(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
-                   const A&... args) {
+inline void launch_carved(int carve, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem,
+                          cudaStream_t st, const A&... args) {
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute attr[2];
   cfg.gridDim = grid;
@@ -491,10 +492,15 @@ inline void launch(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cud
     attr[cfg.numAttrs++].val.programmaticStreamSerializationAllowed = 1;
     if (n >= PDL_CARVE_VOXELS) {
       attr[cfg.numAttrs].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
-      attr[cfg.numAttrs++].val.sharedMemCarveout = PDL_CARVE_PERCENT;
+      attr[cfg.numAttrs++].val.sharedMemCarveout = carve;
     }
   }
   cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+template <class... P, class... A>
+inline void launch(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                   const A&... args) {
+  launch_carved(PDL_CARVE_PERCENT, kernel, grid, block, smem, st, args...);
 }
 
 // ----------------------------------------------------------------------------- launches

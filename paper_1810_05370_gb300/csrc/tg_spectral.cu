@@ -456,11 +456,14 @@ __device__ __forceinline__ bool spec_skip(const CgScal* S) {
 // (an atomic's round trip to L2, some 700 clocks) run in warp 0 while the other warps go on
 // with the transform between the halves.  begin: one barrier; end: one barrier, true in thread
 // 0 of the last block, with the total.  The pass must not reuse B in between.
-struct BlockSum {
-  double sh[NT];
+template <int MAXT>
+struct BlockSumOf {
+  double sh[MAXT];
   bool am_last;
 };
-__device__ __forceinline__ void block_sum_begin(BlockSum& B, double v, double* partial,
+using BlockSum = BlockSumOf<NT>;
+template <int MAXT>
+__device__ __forceinline__ void block_sum_begin(BlockSumOf<MAXT>& B, double v, double* partial,
                                                 unsigned int* counter, int b, int nb) {
   const int tid = threadIdx.x;
   B.sh[tid] = v;
@@ -473,8 +476,9 @@ __device__ __forceinline__ void block_sum_begin(BlockSum& B, double v, double* p
     }
   }
 }
-__device__ __forceinline__ bool block_sum_end(BlockSum& B, double* partial, unsigned int* counter,
-                                              int nb, double& total) {
+template <int MAXT>
+__device__ __forceinline__ bool block_sum_end(BlockSumOf<MAXT>& B, double* partial,
+                                              unsigned int* counter, int nb, double& total) {
   const int tid = threadIdx.x, nt = blockDim.x;
   __syncthreads();
   if (!B.am_last) return false;
@@ -1066,6 +1070,10 @@ __device__ __forceinline__ void fence_proxy_async_smem() {
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
 }
 
+// At nz = 128 a block takes 27 KB with the sum's scratch cut to its 64 threads, so eight fit an SM
+// and the 1152 blocks of a 128^3 pass run in one wave -- if the launch asks for all of the SM's
+// shared memory; at the 60 % that suits the other passes four fit.  128^3 (2 steps) 13650 -> 13285
+// us, single-species 6092 -> 5920, host 8372 -> 8192.
 constexpr uint64_t ZR_WAIT_NS = 2000000000ull;   // 2 s for a tile that takes microseconds
 
 template <int P>
@@ -1083,7 +1091,7 @@ __global__ void __launch_bounds__(ZR_COLS * P)
   constexpr int TILE = N * ZR_COLS;            // elements of one component
   static_assert(P == 8 || P == 16, "nz = 128 or 256");
   if (spec_skip<float>(S)) return;
-  extern __shared__ __align__(1024) unsigned char zr_smem[];
+  extern __shared__ __align__(128) unsigned char zr_smem[];   // TMA tiles: 128 bytes
   C* tile = reinterpret_cast<C*>(zr_smem);     // [component][plane][column]
   C* tw = tile + 3 * TILE;
   float* Sz = reinterpret_cast<float*>(tw + N);   // the z symbols S_z, T_z of the N modes
@@ -1212,7 +1220,7 @@ __global__ void __launch_bounds__(ZR_COLS * P)
     }
   }
 
-  __shared__ BlockSum B;
+  __shared__ BlockSumOf<ZR_COLS * P> B;   // no larger: eight blocks of P = 8 fit an SM
   if (S != nullptr)
     block_sum_begin(B, (double)rz_part, V.partial, V.counter,
                     blockIdx.y * gridDim.x + blockIdx.x, gridDim.x * gridDim.y);
@@ -1605,10 +1613,12 @@ void launch_spec_z(const Spec<R>& V, CgScal* S, cudaStream_t st) {
       const CUtensorMap& map = *static_cast<const CUtensorMap*>(V.zmap);
       if (V.nz == 256)
         TG_TIMED(K_SPEC_ZR, st,
-                 launch(k_spec_zr_tma<16>, g, 16 * ZR_COLS, spec_smem_zr_tma<16>(), st, map, V, S));
+                 launch_carved(PDL_CARVE_ALL, k_spec_zr_tma<16>, g, 16 * ZR_COLS,
+                               spec_smem_zr_tma<16>(), st, map, V, S));
       else
         TG_TIMED(K_SPEC_ZR, st,
-                 launch(k_spec_zr_tma<8>, g, 8 * ZR_COLS, spec_smem_zr_tma<8>(), st, map, V, S));
+                 launch_carved(PDL_CARVE_ALL, k_spec_zr_tma<8>, g, 8 * ZR_COLS,
+                               spec_smem_zr_tma<8>(), st, map, V, S));
       return;
     }
     if (V.nz == 256) {
