@@ -293,6 +293,19 @@ template <typename C> struct ColFullIO {
   __device__ __forceinline__ void st(int l, int e, C v) const { W[e * nxp + l] = v; }
 };
 
+// one mode column of consecutive planes: line l = plane z0 + l
+template <typename C> struct PlaneIO {
+  C* W;     // &W[comp][z0][0][kx]
+  size_t plane;
+  int nxp, nz;
+  __device__ __forceinline__ C ld(int l, int e) const {
+    return l < nz ? W[l * plane + e * nxp] : C{0, 0};
+  }
+  __device__ __forceinline__ void st(int l, int e, C v) const {
+    if (l < nz) W[l * plane + e * nxp] = v;
+  }
+};
+
 // z pass: line l = (component l >> ltz, column l & (tz - 1)); element e = plane kz
 template <typename C> struct ZIO {
   C* W;     // &W[0][0][ky][kx0]
@@ -714,7 +727,17 @@ __global__ void __launch_bounds__(NT, 4) k_spec_update_xfwd(Spec<float> V, Elas3
 }
 
 // ---------------------------------------------------------------------------- y pass
-// block (mode-column tile, z, component), in place; the FP32 pass at four blocks per SM
+// block (mode-column tile, z, component), in place; the FP32 pass at four blocks per SM.  The
+// nx/2 + 1 modes of a row leave one column over from whole tiles.  In FP64 the first rows of
+// blocks take that column of a tile's width of planes each, instead of one block per plane
+// transforming one column and tx - 1 of zeros: a fifth of the pass's work at 128^3, and the FP64
+// pipe bounds it (a pass of the case 50440 -> 49175 us).  In FP32 the mostly empty blocks cost
+// less than the strided loads of the gathered column (64^3 study 9950 -> 10530, 256^3 122100 ->
+// 123460).
+template <typename R>
+__host__ __device__ constexpr bool y_column_left(int nxh, int tx) {
+  return sizeof(R) == 8 && nxh > tx && nxh % tx == 1;
+}
 template <typename R, int SGN, int LN>
 __global__ void __launch_bounds__(NT, sizeof(R) == 4 ? 4 : 0) k_spec_y(Spec<R> V, const CgScal* S) {
   pdl_sync();
@@ -725,7 +748,17 @@ __global__ void __launch_bounds__(NT, sizeof(R) == 4 ? 4 : 0) k_spec_y(Spec<R> V
   C* a = tw + ny;
   C* b = spec_y_buffers(ny) == 1 ? a : a + (size_t)tx * ny;   // one or two stages: b only
   load_roots(tw, V.tw[1], ny);
-  const int kx0 = blockIdx.x * tx, z = blockIdx.y, comp = blockIdx.z;
+  const int rows = gridDim.y - V.nz;   // the first rows of blocks: the column left over
+  const int kx0 = blockIdx.x * tx, z = (int)blockIdx.y - rows, comp = blockIdx.z;
+  if (sizeof(R) == 8 && z < 0) {
+    if (blockIdx.x != 0) return;
+    const int z0 = blockIdx.y * tx;
+    const size_t plane = (size_t)V.ny * V.nxp;
+    const PlaneIO<C> io{V.W + ((size_t)comp * V.nz + z0) * plane + V.nxh - 1, plane, V.nxp,
+                        min(tx, V.nz - z0)};
+    fft_global_inplace<SGN>(io, a, b, 1, tx, ilog2(ny), ilog2(tx), 1, tw, NT);
+    return;
+  }
   C* const W = V.W + ((size_t)comp * V.nz + z) * V.ny * V.nxp + kx0;
   const int ncol = min(tx, V.nxh - kx0);
   if (LN > 0 && ncol == XPB) {
@@ -1645,7 +1678,9 @@ void launch_spec_z(const Spec<R>& V, CgScal* S, cudaStream_t st) {
 // A pass in its compile-time form for the plan's line length, else the general one.
 template <int SGN, typename R>
 void launch_spec_y(const Spec<R>& V, const CgScal* S, cudaStream_t st) {
-  const dim3 g((V.nxh + V.tx - 1) / V.tx, V.nz, 3);
+  const bool left = y_column_left<R>(V.nxh, V.tx);
+  const dim3 g(left ? V.nxh / V.tx : (V.nxh + V.tx - 1) / V.tx,
+               V.nz + (left ? (V.nz + V.tx - 1) / V.tx : 0), 3);
   const size_t smem = spec_smem_y(V);
   auto go = [&](auto kernel) {
     TG_TIMED(SGN < 0 ? K_SPEC_Y_FWD : K_SPEC_Y_INV, st, launch(kernel, g, NT, smem, st, V, S));
