@@ -512,15 +512,16 @@ __device__ __forceinline__ bool block_sum_end(BlockSumOf<MAXT>& B, double* parti
 // pass for lines of 2^LN and its usual tile, 16 lines or columns; LN = 0 is the general form.
 // The arithmetic is the same.  us a pass, general -> compile-time: mixed 64^3 study 10870 -> 9960,
 // 128^3 14494 -> 13640, 256^3 126490 -> 122140 (per launch, update + forward 185 -> 161, inverse 197
-// -> 175).  The x passes take 64, 128 and 256; the y pass 64 and 128 (at 256 its four blocks per
+// -> 175).  The x passes take 32 to 256, the y pass 32 to 128 (32^3 1118 -> 1080 us a pass; at 256 its four blocks per
 // SM leave 64 registers, which the unrolled form spills: 72 -> 88 us).  The FP64 passes stay
 // general: the FP64 pipe bounds them (128^3 50370 -> 50640).
 constexpr int XPB = 16, XLPB = 4;   // lines per block of the compile-time forms
 int x_lines(const Spec<float>& V) {
-  return V.pb == XPB && (V.nx == 64 || V.nx == 128 || V.nx == 256) ? 31 - __builtin_clz(V.nx) : 0;
+  const bool ok = V.pb == XPB && V.nx >= 32 && V.nx <= 256;   // powers of two
+  return ok ? 31 - __builtin_clz(V.nx) : 0;
 }
 int y_lines(const Spec<float>& V) {
-  return V.tx == XPB && (V.ny == 64 || V.ny == 128) ? 31 - __builtin_clz(V.ny) : 0;
+  return V.tx == XPB && V.ny >= 32 && V.ny <= 128 ? 31 - __builtin_clz(V.ny) : 0;
 }
 
 // ---------------------------------------------------------------------------- x forward
@@ -663,11 +664,12 @@ __global__ void __launch_bounds__(NT, 4) k_spec_update_xfwd(Spec<float> V, Elas3
     const float* const qt = q + o0;
     const float* const st = sc ? sc + o0 : nullptr;
     C* const at = a + (threadIdx.x & (N - 1)) * (XPB + 1) + (threadIdx.x >> LN);
+    constexpr int M = XPB * N / NT, U = UB < M ? UB : M;
 #pragma unroll 1
-    for (int m0 = 0; m0 < XPB * N / NT; m0 += UB) {
-      float ra[UB], rb[UB], qa[UB], qb[UB], sa[UB], sb[UB];
+    for (int m0 = 0; m0 < M; m0 += U) {
+      float ra[U], rb[U], qa[U], qb[U], sa[U], sb[U];
 #pragma unroll
-      for (int u = 0; u < UB; ++u) {
+      for (int u = 0; u < U; ++u) {
         const int o = (m0 + u) * (2 * NT);
         ra[u] = rt[o];
         rb[u] = rt[o + N];
@@ -677,7 +679,7 @@ __global__ void __launch_bounds__(NT, 4) k_spec_update_xfwd(Spec<float> V, Elas3
         sb[u] = st ? __ldg(st + o + N) : 1.0f;
       }
 #pragma unroll
-      for (int u = 0; u < UB; ++u) {
+      for (int u = 0; u < U; ++u) {
         const int o = (m0 + u) * (2 * NT);
         const float xa = ra[u] - alpha * qa[u], xb = rb[u] - alpha * qb[u];
         rt[o] = xa;
@@ -782,25 +784,28 @@ __global__ void __launch_bounds__(NT, sizeof(R) == 4 ? 4 : 0) k_spec_y(Spec<R> V
 // (column, g) -- so the sum does not depend on the tile.  us a pass, 16 -> 8 -> 4 columns: mixed
 // 64^3 study 11815 -> 10825 -> 10626, 32^3 1218 -> 1124 -> 1112, but four columns cost the concurrent
 // batch, whose members fill each other's gaps, 1.8 % (16583 -> 16600 -> 16880): eight.
-constexpr int Z_NARROW = 8;
+constexpr int Z_NARROW = 8, Z_LNARROW = 3;
 constexpr int Z_NARROW_MAX = 64;        // largest nz
 constexpr int Z_NARROW_THREADS = 192;
-template <typename R, bool NARROW>
+// LN > 0: columns of 2^LN at compile time (narrow tiles; 64: study 9960 -> 9730 us.  The form for
+// 32 was left out: the compiler contracts its radix-2 stage otherwise, so its roundings differ).
+template <typename R, bool NARROW, int LN>
 __global__ void __launch_bounds__(NARROW ? Z_NARROW_THREADS : NT) k_spec_z(Spec<R> V, CgScal* S) {
   pdl_sync();
   using C = typename CxOf<R>::T;
   if (spec_skip<R>(S)) return;
-  const int tz = NARROW ? Z_NARROW : V.tz, ltz = ilog2(tz), lw = 3 * tz;   // lines: (component, column)
+  const int nz = LN > 0 ? 1 << LN : V.nz, nt = NARROW ? Z_NARROW_THREADS : (int)blockDim.x;
+  const int tz = NARROW ? Z_NARROW : V.tz, ltz = NARROW ? Z_LNARROW : ilog2(tz);
+  const int lw = 3 * tz;   // lines: (component, column)
   C* tw = smem_cx<C>();
-  C* a = tw + V.nz;
-  C* b = a + (size_t)lw * V.nz;
-  load_roots(tw, V.tw[2], V.nz);
+  C* a = tw + nz;
+  C* b = a + (size_t)lw * nz;
+  load_roots(tw, V.tw[2], nz);
   const int kx0 = blockIdx.x * tz, ky = blockIdx.y;
   const int ncol = min(tz, V.nxh - kx0);
   const size_t plane = (size_t)V.ny * V.nxp, comp_stride = (size_t)V.nz * plane;
   const ZIO<C> io{V.W + (size_t)ky * V.nxp + kx0, plane, comp_stride, tz, ltz, ncol};
-  C* F = fft_from_global<-1>(io, a, b, 1, lw, ilog2(V.nz), ltz, 3, tw,
-                                NARROW ? Z_NARROW_THREADS : (int)blockDim.x);
+  C* F = fft_from_global<-1>(io, a, b, 1, lw, LN > 0 ? LN : ilog2(nz), ltz, 3, tw, nt);
   C* other = F == a ? b : a;
   // FP32: no FP64 operation (the volume is a power of two, so both forms are exact)
   const R mu0 = sizeof(R) == 4 ? f32_of(V.mean[0]) : (R)V.mean[0];
@@ -813,7 +818,7 @@ __global__ void __launch_bounds__(NARROW ? Z_NARROW_THREADS : NT) k_spec_z(Spec<
   // mode with 0 < kx < nx/2 standing for its conjugate as well; every term is >= 0
   R rz_part = (R)0;
   __shared__ R term[NARROW ? 3 * Z_NARROW * Z_NARROW_MAX : 1];   // [mode][component]
-  for (int idx = threadIdx.x; idx < tz * V.nz; idx += blockDim.x) {
+  for (int idx = threadIdx.x; idx < tz * nz; idx += nt) {
     const int kz = idx >> ltz, col = idx & (tz - 1);
     if (col >= ncol) continue;
     const int kx = kx0 + col;
@@ -855,7 +860,7 @@ __global__ void __launch_bounds__(NARROW ? Z_NARROW_THREADS : NT) k_spec_z(Spec<
     if (g < groups && col < ncol) {
       const int kx = kx0 + col;
       const R wgt = (kx == 0 || kx == V.nx / 2) ? (R)1 : (R)2;
-      for (int kz = g; kz < V.nz; kz += groups)
+      for (int kz = g; kz < nz; kz += groups)
 #pragma unroll
         for (int q = 0; q < 3; ++q) rz_part += wgt * term[3 * (kz * tz + col) + q];
     }
@@ -864,8 +869,7 @@ __global__ void __launch_bounds__(NARROW ? Z_NARROW_THREADS : NT) k_spec_z(Spec<
     block_sum_begin(B, (double)rz_part, V.partial, V.counter,
                     blockIdx.y * gridDim.x + blockIdx.x, gridDim.x * gridDim.y);
   __syncthreads();
-  fft_to_global<+1>(F, other, io, 1, lw, ilog2(V.nz), ltz, 3, tw,
-                    NARROW ? Z_NARROW_THREADS : (int)blockDim.x);
+  fft_to_global<+1>(F, other, io, 1, lw, LN > 0 ? LN : ilog2(nz), ltz, 3, tw, nt);
   if (S == nullptr) return;
   double out;
   if (block_sum_end(B, V.partial, V.counter, gridDim.x * gridDim.y, out))
@@ -1561,7 +1565,7 @@ cudaError_t spec_prepare(const Spec<R>& V) {
   }
   if (e == cudaSuccess) e = cudaFuncSetAttribute(k_spec_y<R, -1, 0>, A, optin);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(k_spec_y<R, +1, 0>, A, optin);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_spec_z<R, false>, A, optin);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_spec_z<R, false, 0>, A, optin);
   if constexpr (sizeof(R) == 4) {
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k_spec_zr<16>, A, optin);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k_spec_zr<8>, A, optin);
@@ -1668,11 +1672,14 @@ void launch_spec_z(const Spec<R>& V, CgScal* S, cudaStream_t st) {
     if (spec_z_narrow(V)) {
       const dim3 gn((V.nxh + Z_NARROW - 1) / Z_NARROW, V.ny);
       const size_t smem = (1 + 2 * (size_t)3 * Z_NARROW) * V.nz * sizeof(float2);
-      TG_TIMED(K_SPEC_Z, st, launch((k_spec_z<R, true>), gn, Z_NARROW_THREADS, smem, st, V, S));
-      return;
+      auto go = [&](auto kernel) {
+        TG_TIMED(K_SPEC_Z, st, launch(kernel, gn, Z_NARROW_THREADS, smem, st, V, S));
+      };
+      if (V.nz == 64) return go(k_spec_z<R, true, 6>);
+      return go(k_spec_z<R, true, 0>);
     }
   }
-  TG_TIMED(K_SPEC_Z, st, launch((k_spec_z<R, false>), gz, V.nt_z, spec_smem_z(V), st, V, S));
+  TG_TIMED(K_SPEC_Z, st, launch((k_spec_z<R, false, 0>), gz, V.nt_z, spec_smem_z(V), st, V, S));
 }
 
 // A pass in its compile-time form for the plan's line length, else the general one.
@@ -1686,6 +1693,7 @@ void launch_spec_y(const Spec<R>& V, const CgScal* S, cudaStream_t st) {
     TG_TIMED(SGN < 0 ? K_SPEC_Y_FWD : K_SPEC_Y_INV, st, launch(kernel, g, NT, smem, st, V, S));
   };
   if constexpr (sizeof(R) == 4) {
+    if (y_lines(V) == 5) return go(k_spec_y<R, SGN, 5>);
     if (y_lines(V) == 6) return go(k_spec_y<R, SGN, 6>);
     if (y_lines(V) == 7) return go(k_spec_y<R, SGN, 7>);
   }
@@ -1701,6 +1709,7 @@ void launch_spec_x_inv_p(const Spec<float>& V, float* const z[3], const CgScal* 
     TG_TIMED(K_SPEC_X_INV_P, st, launch(kernel, g, NT, smem, st, V, z[0], z[1], z[2], S, P));
   };
   switch (V.x_inpl ? x_lines(V) : 0) {
+    case 5: return go(k_spec_x_inv<float, true, 1, 5>);
     case 6: return go(k_spec_x_inv<float, true, 1, 6>);
     case 7: return go(k_spec_x_inv<float, true, 1, 7>);
     case 8: return go(k_spec_x_inv<float, true, 1, 8>);
@@ -1746,6 +1755,8 @@ cudaError_t launch_spectral_update(const Spec<float>& V, const Elas32& I, float*
       go(k_spec_update_xfwd<1, 8>);
     else
       go(k_spec_update_xfwd<1, 0>);
+  } else if (ln == 5) {
+    go(k_spec_update_xfwd<0, 5>);
   } else if (ln == 6) {
     go(k_spec_update_xfwd<0, 6>);
   } else if (ln == 7) {

@@ -98,6 +98,14 @@ def test_narrow_z_tiles(oracle, n):
     against_the_oracle(oracle, n, "mixed", workload_params(precond_elas=2))
 
 
+@pytest.mark.gpu
+@pytest.mark.parametrize("n", [(32, 32, 8), (64, 128, 4), (128, 64, 32), (256, 32, 4)])
+def test_compile_time_lines(oracle, n):
+    """The FP32 x and y passes' compile-time line lengths, 32 to 256 and 32 to 128, each beside
+    another length on the other axis."""
+    against_the_oracle(oracle, n, "mixed", workload_params(precond_elas=2))
+
+
 def against_the_oracle(oracle, n, precision, P=None):
     torch = pytest.importorskip("torch")
     if not torch.cuda.is_available():
