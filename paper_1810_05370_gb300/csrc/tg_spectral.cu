@@ -311,8 +311,9 @@ template <typename C> struct ZIO {
   C* W;     // &W[0][0][ky][kx0]
   size_t plane, comp_stride;
   int tz, ltz, ncol;
+  int col;  // from one column to the next: 1, or a row for one kx at consecutive ky
   __device__ __forceinline__ size_t at(int l, int e) const {
-    return (size_t)(l >> ltz) * comp_stride + (size_t)e * plane + (l & (tz - 1));
+    return (size_t)(l >> ltz) * comp_stride + (size_t)e * plane + (l & (tz - 1)) * col;
   }
   __device__ __forceinline__ C ld(int l, int e) const {
     return (l & (tz - 1)) < ncol ? W[at(l, e)] : C{0, 0};
@@ -789,6 +790,12 @@ constexpr int Z_NARROW_MAX = 64;        // largest nz
 constexpr int Z_NARROW_THREADS = 192;
 // LN > 0: columns of 2^LN at compile time (narrow tiles; 64: study 9960 -> 9730 us.  The form for
 // 32 was left out: the compiler contracts its radix-2 stage otherwise, so its roundings differ).
+//
+// blocks of the FP64 pass for the column left over from whole tiles (0: none)
+template <typename R>
+__host__ __device__ constexpr int z_left_blocks(int nxh, int tz, int ny) {
+  return y_column_left<R>(nxh, tz) ? (ny + tz - 1) / tz : 0;
+}
 template <typename R, bool NARROW, int LN>
 __global__ void __launch_bounds__(NARROW ? Z_NARROW_THREADS : NT) k_spec_z(Spec<R> V, CgScal* S) {
   pdl_sync();
@@ -801,10 +808,24 @@ __global__ void __launch_bounds__(NARROW ? Z_NARROW_THREADS : NT) k_spec_z(Spec<
   C* a = tw + nz;
   C* b = a + (size_t)lw * nz;
   load_roots(tw, V.tw[2], nz);
-  const int kx0 = blockIdx.x * tz, ky = blockIdx.y;
-  const int ncol = min(tz, V.nxh - kx0);
+  // FP32: block (tile, ky).  FP64: blocks in one row, the first of them the column left over
+  // from whole tiles at tz consecutive ky each (as in the y pass), then (tile, ky)
+  int kx0 = blockIdx.x * tz, ky = blockIdx.y, nb = gridDim.x * gridDim.y;
+  int bl = blockIdx.y * gridDim.x + blockIdx.x;
+  bool left = false;
+  if constexpr (sizeof(R) == 8) {
+    const int nleft = z_left_blocks<R>(V.nxh, tz, V.ny);
+    const int tiles = nleft > 0 ? V.nxh / tz : (V.nxh + tz - 1) / tz;
+    nb = gridDim.x;
+    bl = blockIdx.x;
+    left = bl < nleft;
+    ky = left ? bl * tz : (bl - nleft) / tiles;
+    kx0 = left ? V.nxh - 1 : (bl - nleft - ky * tiles) * tz;
+  }
+  const int ncol = left ? min(tz, V.ny - ky) : min(tz, V.nxh - kx0);
   const size_t plane = (size_t)V.ny * V.nxp, comp_stride = (size_t)V.nz * plane;
-  const ZIO<C> io{V.W + (size_t)ky * V.nxp + kx0, plane, comp_stride, tz, ltz, ncol};
+  const ZIO<C> io{V.W + (size_t)ky * V.nxp + kx0, plane, comp_stride, tz, ltz, ncol,
+                    left ? V.nxp : 1};
   C* F = fft_from_global<-1>(io, a, b, 1, lw, LN > 0 ? LN : ilog2(nz), ltz, 3, tw, nt);
   C* other = F == a ? b : a;
   // FP32: no FP64 operation (the volume is a power of two, so both forms are exact)
@@ -813,7 +834,7 @@ __global__ void __launch_bounds__(NARROW ? Z_NARROW_THREADS : NT) k_spec_z(Spec<
   const R eta0 = sizeof(R) == 4 ? f32_of(V.mean[2]) : (R)V.mean[2];
   const R c = lam0 + mu0;
   const R inv_vol = (R)1 / ((R)V.nx * (R)V.ny * (R)V.nz);
-  const R Sy = V.S[1][ky], Ty = V.T[1][ky];
+  const R Sy0 = V.S[1][ky], Ty0 = V.T[1][ky];
   // <r, z> by Parseval: sum over modes of conj(r^) z^ (z^ already carries 1/V), each stored
   // mode with 0 < kx < nx/2 standing for its conjugate as well; every term is >= 0
   R rz_part = (R)0;
@@ -821,7 +842,8 @@ __global__ void __launch_bounds__(NARROW ? Z_NARROW_THREADS : NT) k_spec_z(Spec<
   for (int idx = threadIdx.x; idx < tz * nz; idx += nt) {
     const int kz = idx >> ltz, col = idx & (tz - 1);
     if (col >= ncol) continue;
-    const int kx = kx0 + col;
+    const int kx = left ? kx0 : kx0 + col;
+    const R Sy = left ? V.S[1][ky + col] : Sy0, Ty = left ? V.T[1][ky + col] : Ty0;
     const R Sv[3] = {V.S[0][kx], Sy, V.S[2][kz]};
     const R Tv[3] = {V.T[0][kx], Ty, V.T[2][kz]};
     const R base = eta0 + mu0 * (Sv[0] + Sv[1] + Sv[2]);
@@ -866,13 +888,12 @@ __global__ void __launch_bounds__(NARROW ? Z_NARROW_THREADS : NT) k_spec_z(Spec<
     }
   }
   if (S != nullptr)
-    block_sum_begin(B, (double)rz_part, V.partial, V.counter,
-                    blockIdx.y * gridDim.x + blockIdx.x, gridDim.x * gridDim.y);
+    block_sum_begin(B, (double)rz_part, V.partial, V.counter, bl, nb);
   __syncthreads();
   fft_to_global<+1>(F, other, io, 1, lw, LN > 0 ? LN : ilog2(nz), ltz, 3, tw, nt);
   if (S == nullptr) return;
   double out;
-  if (block_sum_end(B, V.partial, V.counter, gridDim.x * gridDim.y, out))
+  if (block_sum_end(B, V.partial, V.counter, nb, out))
     cg_after_precond(*S, out);
 }
 
@@ -1678,6 +1699,13 @@ void launch_spec_z(const Spec<R>& V, CgScal* S, cudaStream_t st) {
       if (V.nz == 64) return go(k_spec_z<R, true, 6>);
       return go(k_spec_z<R, true, 0>);
     }
+  }
+  if constexpr (sizeof(R) == 8) {
+    const int left = z_left_blocks<R>(V.nxh, V.tz, V.ny);
+    const int blocks = left > 0 ? (V.nxh / V.tz) * V.ny + left : (int)(gz.x * gz.y);
+    TG_TIMED(K_SPEC_Z, st,
+             launch((k_spec_z<R, false, 0>), blocks, V.nt_z, spec_smem_z(V), st, V, S));
+    return;
   }
   TG_TIMED(K_SPEC_Z, st, launch((k_spec_z<R, false, 0>), gz, V.nt_z, spec_smem_z(V), st, V, S));
 }
