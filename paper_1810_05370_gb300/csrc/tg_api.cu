@@ -405,7 +405,7 @@ const char* const kKernelNames[K_COUNT] = {
     "k_elas32_coef", "k_df_pack3", "k_elas_extrapolate", "k_spec_mean", "k_spec_scale",
     "k_elas_ir_residual", "k_elas_ir_residual_df", "k_elas32_scale_r", "k_spec_x_fwd",
     "k_spec_y_fwd", "k_spec_z", "k_spec_zr", "k_spec_y_inv", "k_spec_x_inv", "k_spec_x_inv_p",
-    "k_elas32_matvec", "k_elas32_update", "k_elas32_matvec_spec", "k_elas32_update_spec",
+    "k_elas32_matvec", "k_elas32_update", "k_elas32_matvec_spec",
     "k_spec_update_xfwd", "k_elas_ir_correct", "k_elas_ir_finish", "k_elas_init",
     "k_elas_init_spec", "k_elas_matvec", "k_elas_update", "k_elas_pupdate", "k_elas_update_spec",
     "k_elas_pupdate_spec", "k_elas_finish", "k_ox_prep", "k_ox_init", "k_ox_matvec",

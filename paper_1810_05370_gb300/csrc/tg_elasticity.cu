@@ -213,7 +213,8 @@ __global__ void __launch_bounds__(NT, 3) k_elas_matvec(Geo G, Elas E) {
 // The CG vector updates run flat over the voxels, blockIdx.y the component, two voxels per
 // 16-byte access and a grid of a few blocks per SM.  They were bound by the blocks' reductions
 // and not by their arithmetic or traffic when every 32 x 8 tile of one z plane was a block of
-// its own (2160 blocks at 96 x 80 x 72).  Workspace arrays start on 256-byte boundaries.
+// its own (2160 blocks at 96 x 80 x 72, 38 us a launch against 10 to 15 of traffic; measured
+// with the reductions, tg_internal.cuh).  Workspace arrays start on 256-byte boundaries.
 template <bool SPEC>
 __global__ void __launch_bounds__(NT) k_elas_update(long long n, Elas E) {
   pdl_sync();

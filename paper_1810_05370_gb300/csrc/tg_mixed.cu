@@ -71,8 +71,6 @@ __global__ void __launch_bounds__(NT) k_df_pack3(long long n, const double* b0, 
   }
 }
 
-// ------------------------------------------------------------------------------ FP32 operator
-
 // ------------------------------------------------------------------------------ FP32 inner CG
 
 __global__ void __launch_bounds__(NT) k_elas32_matvec(Geo G, Consts32 K, Elas32 I, int zb) {
@@ -117,22 +115,6 @@ __global__ void __launch_bounds__(NT, 4) k_elas32_matvec_spec(Geo G, Consts32 K,
     I.S->pq = out[0];
     I.S->alpha = I.S->rz / out[0];
   }
-}
-
-__global__ void __launch_bounds__(NT) k_elas32_update_spec(long long n, Elas32 I) {
-  pdl_sync();
-  if (!running(I.S)) return;
-  const float alpha = (float)I.S->alpha;
-  const int pb = (I.S->it & 1) ^ 1;
-  const long long stride = (long long)gridDim.x * blockDim.x;
-  const long long t0 = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  double drz = 0.0, drr = 0.0;
-  elas32_update_range<false, true>(I, n, t0, n / 4, stride, alpha, pb, blockIdx.x == 0, drz,
-                                   drr);
-  double acc[1] = {drr};
-  double out[1];
-  if (reduce_last_block<1>(acc, I.partial, I.counter, out) && threadIdx.x == 0 && threadIdx.y == 0)
-    cg_after_update_rr(*I.S, out[0]);
 }
 
 // ------------------------------------------------------------------------------ refinement
@@ -481,12 +463,6 @@ cudaError_t launch_elas32_matvec_spec(const Geo& G, const Elas32& I, cudaStream_
   TG_TIMED(K_ELAS32_MATVEC_SPEC, st,
            launch(k_elas32_matvec_spec, op_grid(G, zb), dim3(BX, BY), 0, st, G, make_consts32(G), I,
                   zb));
-  return cudaGetLastError();
-}
-
-cudaError_t launch_elas32_update_spec(const Geo& G, const Elas32& I, cudaStream_t st) {
-  TG_TIMED(K_ELAS32_UPDATE_SPEC, st,
-           launch(k_elas32_update_spec, reduce_blocks(G, (G.nvox + 3) / 4), NT, 0, st, G.nvox, I));
   return cudaGetLastError();
 }
 

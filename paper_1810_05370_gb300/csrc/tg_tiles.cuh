@@ -164,13 +164,12 @@ __device__ __forceinline__ float row_tile(const Tile& T, const At& t, const Fac3
 
 // One tile (bx, by, bz) of the FP32 operator with the fused p-update, for CG iteration `it`
 // with coefficient beta; returns this thread's FP32 part of <p_new, A p_new>.  T is the
-// block's shared staging area.  With Jacobi the tile forms p_new = D^{-1} r + beta p_old
-// while staging and writes it; with SPEC the spectral preconditioner's last pass already
-// wrote p_new (into the buffer p[(it & 1) ^ 1]), which the tile only reads.
+// block's shared staging area.  The tile forms p_new = D^{-1} r + beta p_old while staging
+// and writes it (into the buffer p[(it & 1) ^ 1]).
 //
 // The block marches zb planes; <p, A p> is summed in FP32 over chunks of G.zc planes and the
 // chunks in FP64 (zb: a multiple of G.zc, so a thread's FP32 sums do not depend on it).
-template <bool COH, bool SPEC = false>
+template <bool COH>
 __device__ __forceinline__ double elas32_matvec_tile(const Geo& G, const Consts32& K,
                                                      const Elas32& I, int it, double beta_d,
                                                      int bx, int by, int bz, int zb, Tile32& T) {
@@ -205,12 +204,8 @@ __device__ __forceinline__ double elas32_matvec_tile(const Geo& G, const Consts3
   auto fetch = [&](long long g, Staged& v) {
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-      if (SPEC) {   // the preconditioner's last pass wrote p_new = z + beta p_old
-        v.p[a] = ldf<COH>(pn[a] + g);
-      } else {
-        const float z = __ldg(I.dinv[a] + g) * ldf<COH>(I.r[a] + g);
-        v.p[a] = first ? z : z + beta * ldf<COH>(po[a] + g);
-      }
+      const float z = __ldg(I.dinv[a] + g) * ldf<COH>(I.r[a] + g);
+      v.p[a] = first ? z : z + beta * ldf<COH>(po[a] + g);
     }
     v.mu = __ldg(I.mu + g);
     v.la = __ldg(I.lam + g);
@@ -271,11 +266,9 @@ __device__ __forceinline__ double elas32_matvec_tile(const Geo& G, const Consts3
       const float q1 = row_tile<1>(T, t, f, K.sc);
       const float q2 = row_tile<2>(T, t, f, K.sc);
       const float p0 = tp(T, t, 0, 0, 0, 0), p1 = tp(T, t, 1, 0, 0, 0), p2 = tp(T, t, 2, 0, 0, 0);
-      if (!SPEC) {
-        pn[0][c] = p0;
-        pn[1][c] = p1;
-        pn[2][c] = p2;
-      }
+      pn[0][c] = p0;
+      pn[1][c] = p1;
+      pn[2][c] = p2;
       I.q[0][c] = q0;
       I.q[1][c] = q1;
       I.q[2][c] = q2;
@@ -507,7 +500,7 @@ __device__ __forceinline__ double elas32_matvec_tile_spec(const Geo& G, const Co
 // over float4 groups g = g0, g0 + gs, ... < g1 of an n-voxel system, plus the scalar tail
 // n - n % 4 .. n when `tail` is set; accumulates <r, D^{-1} r> and <r, r>: the twelve products
 // of one group summed in FP32, the groups in FP64.
-template <bool COH, bool SPEC = false>
+template <bool COH>
 __device__ __forceinline__ void elas32_update_range(const Elas32& I, long long n, long long g0,
                                                     long long g1, long long gs, float alpha,
                                                     int pb, bool tail, double& drz,
@@ -525,10 +518,8 @@ __device__ __forceinline__ void elas32_update_range(const Elas32& I, long long n
       r.x -= alpha * q.x; r.y -= alpha * q.y; r.z -= alpha * q.z; r.w -= alpha * q.w;
       *e4 = e;
       *r4 = r;
-      if (!SPEC) {
-        const float4 d = __ldg(reinterpret_cast<const float4*>(I.dinv[a]) + v);
-        prz += r.x * (d.x * r.x) + r.y * (d.y * r.y) + r.z * (d.z * r.z) + r.w * (d.w * r.w);
-      }
+      const float4 d = __ldg(reinterpret_cast<const float4*>(I.dinv[a]) + v);
+      prz += r.x * (d.x * r.x) + r.y * (d.y * r.y) + r.z * (d.z * r.z) + r.w * (d.w * r.w);
       prr += r.x * r.x + r.y * r.y + r.z * r.z + r.w * r.w;
     }
     drz += (double)prz;
@@ -542,7 +533,7 @@ __device__ __forceinline__ void elas32_update_range(const Elas32& I, long long n
         I.e[a][c] += alpha * ldf<COH>(I.p[pb][a] + c);
         const float res = I.r[a][c] - alpha * ldf<COH>(I.q[a] + c);
         I.r[a][c] = res;
-        if (!SPEC) drz += (double)(res * (I.dinv[a][c] * res));
+        drz += (double)(res * (I.dinv[a][c] * res));
         drr += (double)(res * res);
       }
     }
