@@ -106,6 +106,14 @@ def test_compile_time_lines(oracle, n):
     against_the_oracle(oracle, n, "mixed", workload_params(precond_elas=2))
 
 
+@pytest.mark.gpu
+@pytest.mark.parametrize("n", [(64, 64, 19), (64, 64, 20), (47, 33, 50)])
+def test_cooperative_solve_size_limit(oracle, n):
+    """512 voxels on each of 152 SMs: the largest FP64 Jacobi solve of one launch, the smallest
+    above it, and a last block of part of its threads."""
+    against_the_oracle(oracle, n, "fp64")
+
+
 def against_the_oracle(oracle, n, precision, P=None):
     torch = pytest.importorskip("torch")
     if not torch.cuda.is_available():
