@@ -93,10 +93,10 @@ def mixed_kernel_bytes(n, precond):
         "k_spec_y_inv": 2 * W,
         "k_spec_zr": 2 * W,
         "k_spec_z": 2 * W,
-        "k_spec_x_inv_p": W + s + 24,  # half spectrum (and s), p_old in; p out
+        "k_spec_x_inv_p": W + s + 48,  # half spectrum (and s), p_old, e in; p, e out
         "k_elas32_matvec_spec": 36,  # p (3), mu, lambda, eta in; q (3) out
-        "k_spec_update_xfwd": 72 + s + W,  # e, p, r, q in; e, r out (3 each); spectrum out
-        "k_elas_ir_correct": 132,    # u, du, e in; u, du, u pairs out
+        "k_spec_update_xfwd": 36 + s + W,  # r, q (and s) in; r out (3 each); spectrum out
+        "k_elas_ir_correct": 144,    # u, du, e, p in; u, du, u pairs out
         "k_elas_ir_finish": 96,      # du, v in; v, v^{n-1} out
     }
 
