@@ -107,6 +107,15 @@ def test_compile_time_lines(oracle, n):
 
 
 @pytest.mark.gpu
+@pytest.mark.parametrize("n", [(4, 8, 16), (16, 4, 128), (32, 128, 8), (64, 16, 64),
+                               (256, 32, 4)])
+def test_fp64_transform_lengths(oracle, n):
+    """The FP64 transforms' folded twiddles and the z pass's one quotient per mode: first stages
+    of radix 2, 4, 8 and 16, a radix-16 stage after each, on every axis."""
+    against_the_oracle(oracle, n, "fp64", workload_params(precond_elas=2))
+
+
+@pytest.mark.gpu
 @pytest.mark.parametrize("n", [(64, 64, 19), (64, 64, 20), (47, 33, 50)])
 def test_cooperative_solve_size_limit(oracle, n):
     """512 voxels on each of 152 SMs: the largest FP64 Jacobi solve of one launch, the smallest
