@@ -351,10 +351,10 @@ tg_status tg_batch_autotune(tg_batch* batch, double dt, tg_batch_tune* result);
  * up to 256 bytes: tg_batch_concurrent_workspace_bytes gives the total, 0 if any member is
  * invalid.  The states are read after the work already queued on cuda_stream; each
  * tg_batch_step returns with every member's step complete.  tg_batch_autotune has nothing to
- * tune (result zeroed) and tg_batch_set_timeout nothing to limit; tg_batch_stats report the
- * summed iteration counts and launches (graph, tile_depth, coop_blocks are 0).  The first
- * member that fails stops the others at their next simulation and its status is returned;
- * the batch then refuses further steps (TG_ERR_STATE). */
+ * tune (result zeroed); tg_batch_set_timeout limits the waits of the members' small FP64 solves
+ * (TG_ERR_TIMEOUT); tg_batch_stats report the summed iteration counts and launches (graph,
+ * tile_depth, coop_blocks are 0).  The first member that fails stops the others at their next
+ * simulation and its status is returned; the batch then refuses further steps (TG_ERR_STATE). */
 size_t tg_batch_concurrent_workspace_bytes(int32_t nsims, const tg_grid* grids,
                                            const tg_params* params, tg_precision prec);
 tg_status tg_batch_concurrent_init(int32_t nsims, const tg_grid* grids, const tg_params* params,
@@ -365,7 +365,7 @@ tg_status tg_batch_concurrent_init(int32_t nsims, const tg_grid* grids, const tg
 /* Advance every simulation by nsteps steps of dt (the split of tg_step). */
 tg_status tg_batch_step(tg_batch* batch, double dt, int32_t nsteps, tg_batch_stats* stats);
 
-/* Time limit of one grid-wide wait in the persistent kernels (default 20 s). */
+/* Time limit of one grid-wide wait in the kernels that run a whole solve (default 20 s). */
 tg_status tg_batch_set_timeout(tg_batch* batch, uint64_t timeout_ns);
 
 void tg_batch_free(tg_batch* batch);

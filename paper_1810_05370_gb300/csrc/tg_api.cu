@@ -73,6 +73,7 @@ constexpr int MAX_NV = 9;    // largest number of values reduced by one kernel
 // FP32, 3 inner FP32 diffusion solves
 constexpr int N_SCAL = 11;   // 3 CN, 2 elasticity, 3 inner CN, 3 concurrent CN
 constexpr int SMALL_COUNTERS = 16;    // first counter word of the small grids' solves
+constexpr unsigned long long WAIT_NS = 20ULL * 1000 * 1000 * 1000;   // default limit of a wait
 constexpr int MAX_SWEEPS = 64;        // refinement sweeps of one mixed-precision solve
 constexpr double TAU_INNER = 1e-4;    // smallest relative reduction asked of an inner solve
 // ... of a spectrally preconditioned inner elasticity solve: its few, well-conditioned FP32
@@ -436,6 +437,7 @@ struct tg_ctx {
                            // SMALL_COUNTERS and the next those of the small grids' solves
   CgScal* scal;
   int sms;               // SMs of the device
+  unsigned long long wait_ns;   // limit of one grid-wide wait (the small grids' solves)
   // TG_MIXED: the FP64 oxygen solve of S2 runs on a side stream (created on first use),
   // forked from and joined to the context's stream by events, with its own reductions
   double* partial2;
@@ -750,7 +752,8 @@ bool cn_df_ok(const tg_ctx* X) {
 // else queued three kernels at a time.
 tg_status cn_iterate(tg_ctx* X, const Cn3& C, CgScal host[3]) {
   if (cg_small_ok(X->G, X->sms)) {
-    CK(launch_cn_cg_small(X->G, C, X->sms, X->counter + SMALL_COUNTERS, X->stream));
+    CK(launch_cn_cg_small(X->G, C, X->sms, X->counter + SMALL_COUNTERS, X->wait_ns,
+                            X->stream));
     X->launches += 1;
     CK(cudaMemcpyAsync(host, C.S, 3 * sizeof(CgScal), cudaMemcpyDeviceToHost, X->stream));
     CK(cudaStreamSynchronize(X->stream));
@@ -1174,7 +1177,8 @@ tg_status elas_solve(tg_ctx* X, double* const u[3], double* const b_ext[3], bool
   CgScal host[1];
   tg_status s = TG_OK;
   if (!spec && cg_small_ok(X->G, X->sms)) {   // one launch runs every iteration
-    CK(launch_elas_cg_small(X->G, E, X->sms, X->counter + SMALL_COUNTERS, X->stream));
+    CK(launch_elas_cg_small(X->G, E, X->sms, X->counter + SMALL_COUNTERS, X->wait_ns,
+                            X->stream));
     X->launches += 1;
     CK(cudaMemcpyAsync(host, E.S, sizeof(CgScal), cudaMemcpyDeviceToHost, X->stream));
     CK(cudaStreamSynchronize(X->stream));
@@ -1649,6 +1653,7 @@ tg_status tg_init(const tg_grid* grid, const tg_params* params, tg_precision pre
   X->st = *state;
   X->stream = (cudaStream_t)cuda_stream;
   X->sms = sm_count();
+  X->wait_ns = WAIT_NS;
   cudaGetDevice(&X->device);
   X->ws = (char*)workspace;
   for (int a = 0; a < A_COUNT; ++a) X->a[a] = (double*)(X->ws + L.arr[a]);
@@ -2012,6 +2017,7 @@ extern "C" tg_status tg_solve_elasticity_static(const tg_grid* grid, const tg_pa
   X.dp = make_dev_params(params);
   X.prec = TG_FP64;
   X.sms = sm_count();
+  X.wait_ns = WAIT_NS;
   X.st = *state;
   X.stream = (cudaStream_t)cuda_stream;
   X.device = dev;
@@ -2041,7 +2047,6 @@ namespace {
 constexpr int BATCH_GRAPH_SWEEPS = 6;   // refinement sweeps inside the step graph
 constexpr int BATCH_MAX_SWEEPS = 64;    // total, including sweeps run after the graph
 const int kZcCandidates[] = {8, 16, 32, 64};
-constexpr unsigned long long kDefaultTimeoutNs = 20ULL * 1000 * 1000 * 1000;   // 20 s
 
 struct BatchArea {
   size_t sims, tile_sim, item_sim, partial, counters, bar, stat, total;
@@ -2405,7 +2410,7 @@ tg_status tg_batch_init(int32_t nsims, const tg_grid* grids, const tg_params* pa
   B->nsims = nsims;
   B->stream = (cudaStream_t)cuda_stream;
   cudaGetDevice(&B->device);
-  B->timeout_ns = kDefaultTimeoutNs;
+  B->timeout_ns = WAIT_NS;
   B->use_graph = true;
   char* base = (char*)workspace;
   size_t off = 0;
@@ -2667,6 +2672,7 @@ tg_status tg_batch_autotune(tg_batch* B, double dt, tg_batch_tune* result) {
 tg_status tg_batch_set_timeout(tg_batch* B, uint64_t timeout_ns) {
   if (!B || timeout_ns == 0) return TG_ERR_ARG;
   B->timeout_ns = timeout_ns;
+  for (tg_ctx* X : B->ctx) X->wait_ns = timeout_ns;
   if (B->graph_ready) {
     cudaGraphExecDestroy(B->graph);
     B->graph_ready = false;

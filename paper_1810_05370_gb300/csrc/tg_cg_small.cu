@@ -23,10 +23,11 @@
 // 25200.  Near the size limit (69120 voxels) an iteration takes 20.4 us, 11.5 of them on the
 // FP64 pipe; the rest is the two waits and the neighbours' z from L2.
 //
-// The waits are bounded in time: a block that gives up marks the solve CG_TIMEOUT and returns,
-// and so do the others in their turn.  Launched cooperatively, so all blocks are resident; the
-// limit is far above the microseconds of a wait for programs that keep other kernels, or other
-// processes' time slices, on the same GPU.
+// The waits are bounded in time (tg_wait.cuh; the context's limit, 20 s unless it is set): a
+// block that gives up marks the solve CG_TIMEOUT and returns, the others give up in their turn
+// or, if all arrived late, finish, and the solve stays marked either way.  Launched
+// cooperatively, so all blocks are resident; the default limit is far above the microseconds of a
+// wait for programs that keep other kernels, or other processes' time slices, on the same GPU.
 #include <type_traits>
 
 #include "tg_internal.cuh"
@@ -35,44 +36,22 @@ namespace tg {
 namespace {
 
 constexpr int CGS_MAX_THREADS = 512;
-constexpr unsigned long long CGS_WAIT_NS = 20000000000ull;   // 20 s
-
-__device__ __forceinline__ unsigned long long timer_ns() {
-  unsigned long long t;
-  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-  return t;
-}
 
 // Waits until all blocks of the launch have arrived for the round-th time (round = 1, 2, ...);
 // everything any thread wrote before its block's arrival is visible after it (the barrier and
 // the release of thread 0 order the block's writes before the arrival, its acquire and the
 // second barrier order the others' before what follows).  False in every thread of the block if
 // the wait ran out.
-__device__ __forceinline__ bool grid_wait(unsigned int* arrived, unsigned int round) {
-  __shared__ int ok;
+__device__ __forceinline__ bool grid_wait(unsigned int* words, unsigned int round,
+                                          unsigned long long limit_ns) {
+  __shared__ bool ok;
   __syncthreads();
   if (threadIdx.x == 0) {
-    const unsigned int want = round * gridDim.x;
-    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(arrived) : "memory");
-    int good = 1;
-    unsigned long long t0 = 0;
-    for (unsigned int spin = 0;; ++spin) {
-      unsigned int seen;
-      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(arrived) : "memory");
-      if ((int)(seen - want) >= 0) break;   // rounds may wrap
-      if ((spin & 255u) == 0u) {
-        const unsigned long long t = timer_ns();
-        if (t0 == 0) t0 = t;
-        if (t - t0 > CGS_WAIT_NS) {
-          good = 0;
-          break;
-        }
-      }
-    }
-    ok = good;
+    wait_arrive(words);
+    ok = wait_for_arrivals(words, round, gridDim.x, limit_ns);
   }
   __syncthreads();
-  return ok != 0;
+  return ok;
 }
 
 // NV sums over the block's threads into partial[q * gridDim.x + block], one warp per value
@@ -95,14 +74,6 @@ __device__ __forceinline__ double all_partials(const double* partial) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
   return s;
-}
-
-// Leaves the launch's two counters at zero for the next one: the last block out resets them.
-__device__ __forceinline__ void leave_counters(unsigned int* counters) {
-  if (threadIdx.x == 0 && ticket_acq_rel(counters + 1) == gridDim.x - 1) {
-    counters[0] = 0u;
-    counters[1] = 0u;
-  }
 }
 
 // The operator's coefficients of one voxel, in shared memory: coefficient q of thread t at
@@ -145,7 +116,8 @@ __device__ __forceinline__ double row_small(const Geo& G, const Nbr& nb, int c, 
 // The elasticity solve A du = r (E.r, E.p = D^{-1} r and the scalars E.S from k_elas_init):
 // the increments in E.du, the scalars as the many-kernel form leaves them.  E.p carries z.
 __global__ void __launch_bounds__(CGS_MAX_THREADS, 1) k_elas_cg(Geo G, Elas E,
-                                                                unsigned int* counters) {
+                                                                unsigned int* words,
+                                                                unsigned long long wait_ns) {
   extern __shared__ double coef[];
   __shared__ double sc[2];   // alpha, beta
   __shared__ CgScal sS;
@@ -202,7 +174,7 @@ __global__ void __launch_bounds__(CGS_MAX_THREADS, 1) k_elas_cg(Geo G, Elas E,
       }
     }
     leave_partials<1>(acc1, part_pq);
-    if (!(waited = grid_wait(counters, ++round))) break;
+    if (!(waited = grid_wait(words, ++round, wait_ns))) break;
     if (threadIdx.x < 32) {
       const double pq = all_partials(part_pq);
       if (threadIdx.x == 0) {
@@ -224,7 +196,7 @@ __global__ void __launch_bounds__(CGS_MAX_THREADS, 1) k_elas_cg(Geo G, Elas E,
       acc2[1] = fma(r[a], r[a], acc2[1]);
     }
     leave_partials<2>(acc2, part_r);
-    if (!(waited = grid_wait(counters, ++round))) break;
+    if (!(waited = grid_wait(words, ++round, wait_ns))) break;
     if (threadIdx.x < 32) {
       const double rz = all_partials(part_r), rr = all_partials(part_r + gridDim.x);
       if (threadIdx.x == 0) {
@@ -236,7 +208,7 @@ __global__ void __launch_bounds__(CGS_MAX_THREADS, 1) k_elas_cg(Geo G, Elas E,
     if (sS.status != CG_RUNNING) break;   // decided alike in every block
     beta = sc[1];
   }
-  if (!waited) {   // the counters stay as they are: the context is unusable after a timeout
+  if (!waited) {
     if (threadIdx.x == 0) E.S->status = CG_TIMEOUT;
     return;
   }
@@ -244,15 +216,15 @@ __global__ void __launch_bounds__(CGS_MAX_THREADS, 1) k_elas_cg(Geo G, Elas E,
 #pragma unroll
     for (int a = 0; a < 3; ++a) E.du[a][c] = du[a];
   }
-  if (blockIdx.x == 0 && threadIdx.x == 0) *E.S = sS;
-  leave_counters(counters);
+  if (threadIdx.x == 0 && leave_last(words, gridDim.x)) *E.S = sS;
 }
 
 // The three Crank-Nicolson solves (C.r, C.p = D^{-1} r and the scalars C.S from k_cn_init) the
 // same way: the fields C.x updated in place, C.p carrying z.  A finished solve's vectors stand
 // still while the others go on.
 __global__ void __launch_bounds__(CGS_MAX_THREADS, 1) k_cn_cg(Geo G, Cn3 C,
-                                                              unsigned int* counters) {
+                                                              unsigned int* words,
+                                                              unsigned long long wait_ns) {
   __shared__ double sa[3], sb[3];
   __shared__ CgScal sS[3];
   if (threadIdx.x < 3) sS[threadIdx.x] = C.S[threadIdx.x];
@@ -302,7 +274,7 @@ __global__ void __launch_bounds__(CGS_MAX_THREADS, 1) k_cn_cg(Geo G, Cn3 C,
       }
     }
     leave_partials<3>(acc1, part_pq);
-    if (!(waited = grid_wait(counters, ++round))) break;
+    if (!(waited = grid_wait(words, ++round, wait_ns))) break;
     if (threadIdx.x < 32) {
 #pragma unroll
       for (int s = 0; s < 3; ++s) {
@@ -329,7 +301,7 @@ __global__ void __launch_bounds__(CGS_MAX_THREADS, 1) k_cn_cg(Geo G, Cn3 C,
       acc2[2 * s + 1] = r[s] * r[s];
     }
     leave_partials<6>(acc2, part_r);
-    if (!(waited = grid_wait(counters, ++round))) break;
+    if (!(waited = grid_wait(words, ++round, wait_ns))) break;
     if (threadIdx.x < 32) {
 #pragma unroll
       for (int s = 0; s < 3; ++s) {
@@ -358,14 +330,16 @@ __global__ void __launch_bounds__(CGS_MAX_THREADS, 1) k_cn_cg(Geo G, Cn3 C,
     if (threadIdx.x < 3) C.S[threadIdx.x].status = CG_TIMEOUT;
     return;
   }
-  if (blockIdx.x == 0 && threadIdx.x < 3) C.S[threadIdx.x] = sS[threadIdx.x];
-  leave_counters(counters);
+  if (threadIdx.x == 0 && leave_last(words, gridDim.x)) {
+#pragma unroll
+    for (int s = 0; s < 3; ++s) C.S[s] = sS[s];
+  }
 }
 
 template <class View>
-cudaError_t launch_small(void (*kernel)(Geo, View, unsigned int*), const Geo& G, const View& V,
-                         int doubles_per_thread, int sms, unsigned int* counters,
-                         cudaStream_t st) {
+cudaError_t launch_small(void (*kernel)(Geo, View, unsigned int*, unsigned long long), const Geo& G,
+                         const View& V, int doubles_per_thread, int sms, unsigned int* words,
+                         unsigned long long wait_ns, cudaStream_t st) {
   const long long warps = (G.nvox + 31) / 32;
   const int threads = (int)(32 * ((warps + sms - 1) / sms));
   const int blocks = (int)((G.nvox + threads - 1) / threads);
@@ -389,7 +363,7 @@ cudaError_t launch_small(void (*kernel)(Geo, View, unsigned int*), const Geo& G,
   cfg.stream = st;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kernel, G, V, counters);
+  return cudaLaunchKernelEx(&cfg, kernel, G, V, words, wait_ns);
 }
 
 }  // namespace
@@ -398,18 +372,18 @@ bool cg_small_ok(const Geo& G, int sms) {
   return G.nvox <= (long long)CGS_MAX_THREADS * sms && sms > 0;
 }
 
-// counters: two zeroed words, left at zero
-cudaError_t launch_elas_cg_small(const Geo& G, const Elas& E, int sms, unsigned int* counters,
-                                 cudaStream_t st) {
+// words: two zeroed words (tg_wait.cuh), left at zero by a launch that ended well
+cudaError_t launch_elas_cg_small(const Geo& G, const Elas& E, int sms, unsigned int* words,
+                                 unsigned long long wait_ns, cudaStream_t st) {
   cudaError_t e = cudaSuccess;
-  TG_TIMED(K_ELAS_CG, st, e = launch_small(k_elas_cg, G, E, EC_COUNT, sms, counters, st));
+  TG_TIMED(K_ELAS_CG, st, e = launch_small(k_elas_cg, G, E, EC_COUNT, sms, words, wait_ns, st));
   return e;
 }
 
-cudaError_t launch_cn_cg_small(const Geo& G, const Cn3& C, int sms, unsigned int* counters,
-                               cudaStream_t st) {
+cudaError_t launch_cn_cg_small(const Geo& G, const Cn3& C, int sms, unsigned int* words,
+                               unsigned long long wait_ns, cudaStream_t st) {
   cudaError_t e = cudaSuccess;
-  TG_TIMED(K_CN_CG, st, e = launch_small(k_cn_cg, G, C, 0, sms, counters, st));
+  TG_TIMED(K_CN_CG, st, e = launch_small(k_cn_cg, G, C, 0, sms, words, wait_ns, st));
   return e;
 }
 

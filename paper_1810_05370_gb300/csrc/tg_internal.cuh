@@ -8,6 +8,7 @@
 
 #include "tg.h"
 #include "tg_fpconv.cuh"
+#include "tg_wait.cuh"
 
 namespace tg {
 
@@ -152,18 +153,13 @@ __device__ __forceinline__ int block_count() { return gridDim.x * gridDim.y * gr
 //  * a block sums through shared memory, one warp per value adding eight values per lane and
 //    then five shuffle rounds: 12 warp additions per value instead of the 40 of a shuffle tree
 //    in every warp plus a serial sum over the warps;
-//  * the ticket is one acquire-release atomic instead of a full fence and a relaxed one.
+//  * the ticket is one acquire-release atomic (tg_wait.cuh) instead of a full fence and a relaxed
+//    one.
 // Deterministic: the order of the additions depends on the launch's shape only.
 // Measured with the flat vector updates and the fused operator rows (us a pass, before ->
 // after): FP64 solve at 96 x 80 x 72 35100 -> 30100, 16^3 static solve 820 -> 736, FP64 step at
 // 32^3 3590 -> 3260 and at 128^3 53300 -> 51000, mixed step at 100 x 84 x 60 9380 -> 8280; at
 // 256^3, where a launch is long, nothing.
-__device__ __forceinline__ unsigned int ticket_acq_rel(unsigned int* counter) {
-  unsigned int t;
-  asm volatile("atom.add.acq_rel.gpu.global.u32 %0, [%1], 1;" : "=r"(t) : "l"(counter) : "memory");
-  return t;
-}
-
 // Sum of sh[0 .. n) (n a multiple of 32, at most 1024) by one whole warp; every lane calls it
 // and lane 0 holds the result.
 __device__ __forceinline__ double warp_sum_shared(const double* sh, int n, int lane) {
@@ -712,9 +708,9 @@ cudaError_t launch_elas_finish(const Geo&, const Elas&, double inv_dt, bool zero
 // the whole Jacobi-CG solves of a small grid in one cooperative launch each (tg_cg_small.cu)
 bool cg_small_ok(const Geo&, int sms);
 cudaError_t launch_cn_cg_small(const Geo&, const Cn3&, int sms, unsigned int* counters,
-                               cudaStream_t st);
+                               unsigned long long wait_ns, cudaStream_t st);
 cudaError_t launch_elas_cg_small(const Geo&, const Elas&, int sms, unsigned int* counters,
-                                 cudaStream_t st);
+                                 unsigned long long wait_ns, cudaStream_t st);
 
 // mixed precision (tg_mixed.cu)
 cudaError_t launch_to_f32(long long n, const F32Copy& c, cudaStream_t st);
