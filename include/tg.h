@@ -345,7 +345,10 @@ tg_status tg_batch_autotune(tg_batch* batch, double dt, tg_batch_tune* result);
  * grid allows it), the double-FP32 refinements, the Neumann inner CN solves, the extrapolated
  * elasticity starts -- on a CUDA stream of its own.  A pool of nthreads host threads (0: up to
  * 8) drives them: each thread takes the largest simulation not yet stepped and advances it by
- * all nsteps of a tg_batch_step call, so several simulations' kernels share the GPU.  Members
+ * all nsteps of a tg_batch_step call, so several simulations' kernels share the GPU.  A
+ * member's results are those of a simulation of its own: bit for bit in TG_MIXED; in TG_FP64
+ * to rounding, because the threads decide whether a small grid's Jacobi solves run as one
+ * launch each or as queued kernels, which add in another order.  Members
  * may mix grids, preconditioners, models and precisions' solvers (prec applies to all).  The
  * workspace holds one tg_workspace_bytes(grid, params, prec) region per member, each rounded
  * up to 256 bytes: tg_batch_concurrent_workspace_bytes gives the total, 0 if any member is

@@ -437,6 +437,7 @@ struct tg_ctx {
                            // SMALL_COUNTERS and the next those of the small grids' solves
   CgScal* scal;
   int sms;               // SMs of the device
+  int sharers;           // host threads stepping simulations side by side (a concurrent batch)
   unsigned long long wait_ns;   // limit of one grid-wide wait (the small grids' solves)
   // TG_MIXED: the FP64 oxygen solve of S2 runs on a side stream (created on first use),
   // forked from and joined to the context's stream by events, with its own reductions
@@ -751,7 +752,7 @@ bool cn_df_ok(const tg_ctx* X) {
 // The iterations of the FP64 Crank-Nicolson solves started on C: one launch on a small grid,
 // else queued three kernels at a time.
 tg_status cn_iterate(tg_ctx* X, const Cn3& C, CgScal host[3]) {
-  if (cg_small_ok(X->G, X->sms)) {
+  if (cg_small_fits(X->G.nvox, X->sms, X->sharers)) {
     CK(launch_cn_cg_small(X->G, C, X->sms, X->counter + SMALL_COUNTERS, X->wait_ns,
                             X->stream));
     X->launches += 1;
@@ -1176,7 +1177,7 @@ tg_status elas_solve(tg_ctx* X, double* const u[3], double* const b_ext[3], bool
   }
   CgScal host[1];
   tg_status s = TG_OK;
-  if (!spec && cg_small_ok(X->G, X->sms)) {   // one launch runs every iteration
+  if (!spec && cg_small_fits(X->G.nvox, X->sms, X->sharers)) {   // one launch runs every iteration
     CK(launch_elas_cg_small(X->G, E, X->sms, X->counter + SMALL_COUNTERS, X->wait_ns,
                             X->stream));
     X->launches += 1;
@@ -1653,6 +1654,7 @@ tg_status tg_init(const tg_grid* grid, const tg_params* params, tg_precision pre
   X->st = *state;
   X->stream = (cudaStream_t)cuda_stream;
   X->sms = sm_count();
+  X->sharers = 1;
   X->wait_ns = WAIT_NS;
   cudaGetDevice(&X->device);
   X->ws = (char*)workspace;
@@ -2017,6 +2019,7 @@ extern "C" tg_status tg_solve_elasticity_static(const tg_grid* grid, const tg_pa
   X.dp = make_dev_params(params);
   X.prec = TG_FP64;
   X.sms = sm_count();
+  X.sharers = 1;
   X.wait_ns = WAIT_NS;
   X.st = *state;
   X.stream = (cudaStream_t)cuda_stream;
@@ -2505,6 +2508,7 @@ tg_status tg_batch_concurrent_init(int32_t nsims, const tg_grid* grids, const tg
       tg_batch_free(B);
       return e;
     }
+    X->sharers = B->nthreads;
     B->streams.push_back(st);
     B->ctx.push_back(X);
     off += round_up(b);

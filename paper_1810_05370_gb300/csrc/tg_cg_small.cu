@@ -35,8 +35,6 @@
 namespace tg {
 namespace {
 
-constexpr int CGS_MAX_THREADS = 512;
-
 // Waits until all blocks of the launch have arrived for the round-th time (round = 1, 2, ...);
 // everything any thread wrote before its block's arrival is visible after it (the barrier and
 // the release of thread 0 order the block's writes before the arrival, its acquire and the
@@ -367,10 +365,6 @@ cudaError_t launch_small(void (*kernel)(Geo, View, unsigned int*, unsigned long 
 }
 
 }  // namespace
-
-bool cg_small_ok(const Geo& G, int sms) {
-  return G.nvox <= (long long)CGS_MAX_THREADS * sms && sms > 0;
-}
 
 // words: two zeroed words (tg_wait.cuh), left at zero by a launch that ended well
 cudaError_t launch_elas_cg_small(const Geo& G, const Elas& E, int sms, unsigned int* words,

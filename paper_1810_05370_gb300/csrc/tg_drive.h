@@ -1,0 +1,21 @@
+// tg_drive.h -- host-side decisions of the CG solves, free of CUDA so that the CPU tests build
+// them too.
+#pragma once
+
+namespace tg {
+
+constexpr int CGS_MAX_THREADS = 512;   // voxels per SM of a solve that is one launch (tg_cg_small.cu)
+
+// Whether an FP64 Jacobi solve on nvox voxels runs as one cooperative launch.  It needs every SM's
+// registers for at most 512 voxels each.  sharers: the host threads that step simulations side
+// by side (a concurrent batch), 1 alone.  The launch spends its waits idle, which the other
+// members' solves fill only while several fit an SM; the queued kernels interleave at any size.
+// So with sharers the solves in flight may take twice the chip's 512 voxels per SM.  ms for two
+// steps of every member, queued -> one launch: 8 x 24^3 4.2 -> 4.0, 8 x 28^3 6.2 -> 6.9, 8 x 32^3
+// 8.5 -> 11.3, 4 x 32^3 5.6 -> 5.6, 4 x 40^3 13.8 -> 14.6, 2 x 42^3 10.5 -> 8.6.
+inline bool cg_small_fits(long long nvox, int sms, int sharers) {
+  const long long most = (long long)CGS_MAX_THREADS * sms;
+  return nvox <= most && (sharers <= 1 || nvox * sharers <= 2 * most);
+}
+
+}  // namespace tg

@@ -7,6 +7,7 @@
 #include <algorithm>
 
 #include "tg.h"
+#include "tg_drive.h"
 #include "tg_fpconv.cuh"
 #include "tg_wait.cuh"
 
@@ -705,8 +706,8 @@ cudaError_t launch_elas_pupdate_spec(const Geo&, const Elas&, cudaStream_t st);
 cudaError_t launch_elas_finish(const Geo&, const Elas&, double inv_dt, bool zero_rhs,
                                int extrap, cudaStream_t st);
 
-// the whole Jacobi-CG solves of a small grid in one cooperative launch each (tg_cg_small.cu)
-bool cg_small_ok(const Geo&, int sms);
+// the whole Jacobi-CG solves of a small grid (tg_drive.h's cg_small_fits) in one cooperative
+// launch each (tg_cg_small.cu)
 cudaError_t launch_cn_cg_small(const Geo&, const Cn3&, int sms, unsigned int* counters,
                                unsigned long long wait_ns, cudaStream_t st);
 cudaError_t launch_elas_cg_small(const Geo&, const Elas&, int sms, unsigned int* counters,
