@@ -438,6 +438,7 @@ struct tg_ctx {
   CgScal* scal;
   int sms;               // SMs of the device
   int sharers;           // host threads stepping simulations side by side (a concurrent batch)
+  bool coop_refused;     // the driver took no cooperative launch of a small solve
   unsigned long long wait_ns;   // limit of one grid-wide wait (the small grids' solves)
   // TG_MIXED: the FP64 oxygen solve of S2 runs on a side stream (created on first use),
   // forked from and joined to the context's stream by events, with its own reductions
@@ -749,21 +750,37 @@ bool cn_df_ok(const tg_ctx* X) {
          X->prm.rtol_diff >= DF_RTOL_MIN;
 }
 
+// A solve of a small grid as one launch (tg_cg_small.cu), where it fits and the driver takes it.
+static_assert(COOP_REFUSED[0] == (int)cudaErrorCooperativeLaunchTooLarge &&
+                  COOP_REFUSED[1] == (int)cudaErrorNotSupported,
+              "tg_drive.h's error codes");
+template <class Launch>
+SmallRun small_solve(tg_ctx* X, Launch launch) {
+  const SmallRun r = run_small(cg_small_fits(X->G.nvox, X->sms, X->sharers), X->coop_refused,
+                               [&]() -> int {
+    const cudaError_t e = launch();
+    if (e != cudaSuccess) cudaGetLastError();   // a refusal leaves nothing behind
+    return (int)e;
+  });
+  if (r == SMALL_TAKEN) X->launches += 1;
+  return r;
+}
+
 // The iterations of the FP64 Crank-Nicolson solves started on C: one launch on a small grid,
 // else queued three kernels at a time.
 tg_status cn_iterate(tg_ctx* X, const Cn3& C, CgScal host[3]) {
-  if (cg_small_fits(X->G.nvox, X->sms, X->sharers)) {
-    CK(launch_cn_cg_small(X->G, C, X->sms, X->counter + SMALL_COUNTERS, X->wait_ns,
-                            X->stream));
-    X->launches += 1;
-    CK(cudaMemcpyAsync(host, C.S, 3 * sizeof(CgScal), cudaMemcpyDeviceToHost, X->stream));
-    CK(cudaStreamSynchronize(X->stream));
-    return TG_OK;
-  }
-  return drive_cg(X, [&](int) {
-    X->launches += 3;
-    return launch_cn_iter(X->G, C, X->stream);
-  }, C.S, 3, X->prm.maxit_diff, X->prev_it_diff, host);
+  const SmallRun small = small_solve(X, [&] {
+    return launch_cn_cg_small(X->G, C, X->sms, X->counter + SMALL_COUNTERS, X->wait_ns, X->stream);
+  });
+  if (small == SMALL_QUEUE)
+    return drive_cg(X, [&](int) {
+      X->launches += 3;
+      return launch_cn_iter(X->G, C, X->stream);
+    }, C.S, 3, X->prm.maxit_diff, X->prev_it_diff, host);
+  if (small == SMALL_FAILED) return fail(X, TG_ERR_CUDA);
+  CK(cudaMemcpyAsync(host, C.S, 3 * sizeof(CgScal), cudaMemcpyDeviceToHost, X->stream));
+  CK(cudaStreamSynchronize(X->stream));
+  return TG_OK;
 }
 
 // S2: the three Crank-Nicolson solves (i, o, l) on the faces built by S0.
@@ -1177,10 +1194,11 @@ tg_status elas_solve(tg_ctx* X, double* const u[3], double* const b_ext[3], bool
   }
   CgScal host[1];
   tg_status s = TG_OK;
-  if (!spec && cg_small_fits(X->G.nvox, X->sms, X->sharers)) {   // one launch runs every iteration
-    CK(launch_elas_cg_small(X->G, E, X->sms, X->counter + SMALL_COUNTERS, X->wait_ns,
-                            X->stream));
-    X->launches += 1;
+  const SmallRun small = spec ? SMALL_QUEUE : small_solve(X, [&] {
+    return launch_elas_cg_small(X->G, E, X->sms, X->counter + SMALL_COUNTERS, X->wait_ns, X->stream);
+  });
+  if (small == SMALL_FAILED) return fail(X, TG_ERR_CUDA);
+  if (small == SMALL_TAKEN) {   // one launch ran every iteration
     CK(cudaMemcpyAsync(host, E.S, sizeof(CgScal), cudaMemcpyDeviceToHost, X->stream));
     CK(cudaStreamSynchronize(X->stream));
   } else {
@@ -1655,6 +1673,7 @@ tg_status tg_init(const tg_grid* grid, const tg_params* params, tg_precision pre
   X->stream = (cudaStream_t)cuda_stream;
   X->sms = sm_count();
   X->sharers = 1;
+  X->coop_refused = false;
   X->wait_ns = WAIT_NS;
   cudaGetDevice(&X->device);
   X->ws = (char*)workspace;
@@ -2020,6 +2039,7 @@ extern "C" tg_status tg_solve_elasticity_static(const tg_grid* grid, const tg_pa
   X.prec = TG_FP64;
   X.sms = sm_count();
   X.sharers = 1;
+  X.coop_refused = false;
   X.wait_ns = WAIT_NS;
   X.st = *state;
   X.stream = (cudaStream_t)cuda_stream;

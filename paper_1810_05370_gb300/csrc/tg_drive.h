@@ -18,4 +18,23 @@ inline bool cg_small_fits(long long nvox, int sms, int sharers) {
   return nvox <= most && (sharers <= 1 || nvox * sharers <= 2 * most);
 }
 
+// The CUDA runtime's errors for a cooperative launch that it does not take, before anything ran:
+// its blocks cannot all be resident (a process or partition that may use fewer SMs than the
+// device has), or the device has no such launches.  cudaErrorCooperativeLaunchTooLarge and
+// cudaErrorNotSupported; tg_api.cu asserts the values.
+constexpr int COOP_REFUSED[2] = {720, 801};
+
+enum SmallRun { SMALL_TAKEN, SMALL_QUEUE, SMALL_FAILED };
+
+// Runs launch() (0 or the CUDA error) for a solve that fits one launch.  SMALL_QUEUE: the solve
+// goes to the queued kernels, now and, with `refused` set, for the context's later solves.
+template <class Launch>
+SmallRun run_small(bool fits, bool& refused, Launch launch) {
+  if (!fits || refused) return SMALL_QUEUE;
+  const int e = launch();
+  if (e == 0) return SMALL_TAKEN;
+  refused = e == COOP_REFUSED[0] || e == COOP_REFUSED[1];
+  return refused ? SMALL_QUEUE : SMALL_FAILED;
+}
+
 }  // namespace tg

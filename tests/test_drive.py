@@ -48,6 +48,26 @@ def test_small_solve_rule(lib):
     assert not fits(1, 0, 1)
 
 
+TAKEN, QUEUE, FAILED = 0, 1, 2
+
+
+@pytest.mark.parametrize("error,outcome", [(0, TAKEN), (720, QUEUE), (801, QUEUE), (1, FAILED),
+                                           (700, FAILED), (719, FAILED)])
+def test_refused_cooperative_launch_goes_to_the_queued_kernels(lib, error, outcome):
+    """A fake launch that returns a CUDA error: only the two refusals that come before anything
+    ran send the solve to the queued kernels, and then the context's later solves too."""
+    refused, launched = ctypes.c_int(0), ctypes.c_int(0)
+
+    def run(fits):
+        return lib.tgd_run_small(fits, ctypes.byref(refused), error, ctypes.byref(launched))
+
+    assert run(0) == QUEUE and launched.value == 0 and not refused.value
+    assert run(1) == outcome and launched.value == 1
+    assert bool(refused.value) == (outcome == QUEUE)
+    assert run(1) == outcome
+    assert launched.value == (1 if outcome == QUEUE else 2)
+
+
 @pytest.mark.gpu
 @pytest.mark.parametrize("n,one_launch", [(16, True), (30, False)])
 def test_concurrent_fp64_members(n, one_launch):
