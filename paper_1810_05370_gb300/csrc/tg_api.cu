@@ -611,34 +611,17 @@ struct HookScope {
   ~HookScope() { tg_khook = saved; }
 };
 
-// Queue iterations in chunks and read the device-side flags back between chunks.  Kernels of
-// a finished solve return at once, so overshooting a chunk only costs empty launches.
+// Queue iterations in chunks (tg_drive.h) and read the device-side flags back between chunks.
+// Kernels of a finished solve return at once, so overshooting a chunk only costs empty launches.
 // On stream st; `queued` iterations may already be in flight (then the loop reads the flags
 // first).
-int first_chunk(int prev) { return prev > 0 ? std::max(1, prev - prev / 8) : 4; }
-
-// Iterations the running solves still need, if their residuals keep falling at the mean rate
-// from |rhs| (the first residual of a solve that starts from zero, as the refined solves do; a
-// better start makes the estimate too small, which costs another read).  Each read of the flags
-// leaves the GPU idle for some 10 us, so the queue is filled by the estimate and not by a
-// growing guess: a solve of 50 iterations takes two or three reads instead of four or five.
-int next_chunk(const CgScal* host, int nsolves, int grown) {
-  double need = 0.0;
-  for (int r = 0; r < nsolves; ++r) {
-    const CgScal& s = host[r];
-    if (s.status != CG_RUNNING) continue;
-    const double target = s.rtol * s.rtol * s.bb;
-    if (!(s.it > 0 && target > 0.0 && s.rr > target && s.rr < s.bb)) return grown;
-    need = std::max(need, s.it * log(s.rr / target) / log(s.bb / s.rr));
-  }
-  return (int)std::max(1.0, std::min(std::ceil(need), 64.0));
-}
-
 template <class IterFn>
 tg_status drive_cg_loop(tg_ctx* X, cudaStream_t st, IterFn iter, const CgScal* dev, int nsolves,
                         int maxit, int prev, CgScal* host, long long queued, int slot) {
   int chunk = queued > 0 ? 0 : first_chunk(prev);
   int grown = 2;
+  CgScal seen[3];   // the solves' scalars at the first read
+  bool looked = false;
   for (;;) {
     for (int c = 0; c < chunk; ++c) {
       prof_iter(X, slot, (int)(queued + c));
@@ -651,7 +634,9 @@ tg_status drive_cg_loop(tg_ctx* X, cudaStream_t st, IterFn iter, const CgScal* d
     for (int r = 0; r < nsolves; ++r) running |= host[r].status == CG_RUNNING;
     if (!running) return TG_OK;
     if (queued > (long long)maxit + 64) return fail(X, TG_ERR_CUDA);  // flags never settled
-    chunk = next_chunk(host, nsolves, grown);
+    chunk = next_chunk(host, looked ? seen : nullptr, nsolves, CG_RUNNING, grown);
+    if (!looked) std::copy(host, host + nsolves, seen);
+    looked = true;
     grown = std::min(grown * 2, 32);
   }
 }

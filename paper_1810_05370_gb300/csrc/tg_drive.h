@@ -2,6 +2,9 @@
 // them too.
 #pragma once
 
+#include <algorithm>
+#include <cmath>
+
 namespace tg {
 
 constexpr int CGS_MAX_THREADS = 512;   // voxels per SM of a solve that is one launch (tg_cg_small.cu)
@@ -16,6 +19,35 @@ constexpr int CGS_MAX_THREADS = 512;   // voxels per SM of a solve that is one l
 inline bool cg_small_fits(long long nvox, int sms, int sharers) {
   const long long most = (long long)CGS_MAX_THREADS * sms;
   return nvox <= most && (sharers <= 1 || nvox * sharers <= 2 * most);
+}
+
+// Iterations queued before the first look at a solve's flags, prev those of the last such solve.
+inline int first_chunk(int prev) { return prev > 0 ? std::max(1, prev - prev / 8) : 4; }
+
+// Iterations the running solves still need (S: the solves' scalars; `running` their status while
+// they iterate; `grown` where a residual shows no rate).  Each read of the flags leaves the GPU
+// idle for some 10 us, so the queue is filled by an estimate and not by a growing guess: a solve
+// of 50 iterations takes two or three reads instead of four or five.  The residual is taken to
+// keep falling at its mean rate from |rhs|, which is where a refined solve starts.  A solve that
+// starts from a good guess starts lower, and that rate comes out too high: from the second read on
+// the rate since the first (first: the scalars read then, or null) counts too, for at most twice
+// the iterations that it was seen over, as a few iterations' rate may be off.
+template <class S>
+int next_chunk(const S* host, const S* first, int nsolves, int running, int grown) {
+  double need = 0.0;
+  for (int r = 0; r < nsolves; ++r) {
+    const S& s = host[r];
+    if (s.status != running) continue;
+    const double target = s.rtol * s.rtol * s.bb;
+    if (!(s.it > 0 && target > 0.0 && s.rr > target && s.rr < s.bb)) return grown;
+    const double left = std::log(s.rr / target);
+    need = std::max(need, s.it * left / std::log(s.bb / s.rr));
+    if (first && s.it > first[r].it && s.rr < first[r].rr) {
+      const double seen = s.it - first[r].it;
+      need = std::max(need, seen * std::min(left / std::log(first[r].rr / s.rr), 2.0));
+    }
+  }
+  return (int)std::max(1.0, std::min(std::ceil(need), 64.0));
 }
 
 // The CUDA runtime's errors for a cooperative launch that it does not take, before anything ran:

@@ -48,6 +48,25 @@ def test_small_solve_rule(lib):
     assert not fits(1, 0, 1)
 
 
+@pytest.mark.parametrize("rr0", [1.0, 1e-4, 1e-8, 1e-12])
+@pytest.mark.parametrize("prev,total", [(0, 50), (20, 80), (60, 62), (80, 20), (10, 120), (12, 14)])
+def test_flags_are_read_few_times(lib, rr0, prev, total):
+    """A residual that falls evenly, from |rhs| or from the much smaller one of a good starting
+    guess.  From |rhs|: the first look, one for every 64 iterations then left (the most queued at
+    once), and one more where the estimate rounds.  From any start no more than with a guess that
+    doubles from two iterations to 32."""
+    reads = lib.tgd_reads(total, prev, ctypes.c_double(1.0), ctypes.c_double(rr0),
+                          ctypes.c_double(1e-8))
+    first = prev - prev // 8 if prev else 4
+    left = max(0, total - first)
+    if rr0 == 1.0:
+        assert reads <= 1 + -(-left // 64) + (left > 0)
+    queued, guess, most = first, 2, 1
+    while queued < total:
+        queued, guess, most = queued + guess, min(2 * guess, 32), most + 1
+    assert reads <= most
+
+
 TAKEN, QUEUE, FAILED = 0, 1, 2
 
 
