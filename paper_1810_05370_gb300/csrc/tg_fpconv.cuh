@@ -339,6 +339,15 @@ TG_HD double pow2_recip(double x) {
   return fpc::from_bits64((unsigned)(0x7fe00000u - (unsigned)(fpc::bits64(x) >> 32)), 0u);
 }
 
+// 2^-e for a normal x = m 2^e, 1 <= m < 2, with e taken into [-880, 880]; 1 for zero and
+// subnormals.  A product of six factors up to 2^20 apart around x stays in FP64's range once each
+// is scaled by it.  Integer operations only.
+TG_HD double pow2_scale(double x) {
+  const int e = (int)(fpc::bits64(x) >> 52 & 0x7ff);
+  const int k = e == 0 ? 1023 : 2046 - e;   // the exponent field of 2^-e
+  return fpc::from_bits64((unsigned)(k < 143 ? 143 : (k > 1903 ? 1903 : k)) << 20, 0u);
+}
+
 // The power of two nearest 1 / sqrt(x) on the logarithmic scale, 2^-rint(log2(x) / 2), for a
 // finite x > 0, from its exponent e and significand m in [1, 2): log2(x) / 2 lies in
 // [e/2, e/2 + 1/2), so it rounds to e/2 for even e and to (e + 1)/2 for odd e, the tie at

@@ -870,11 +870,17 @@ __global__ void __launch_bounds__(NT, sizeof(R) == 4 ? 4 : 0) k_spec_y(Spec<R> V
 // D_q = base + c (S_q - T_q^2) and Sherman-Morrison, z = D^{-1} (r - f T (T^T D^{-1} r)), f = c /
 // (1 + c T^T D^{-1} T).  On the FP64 pipe, which bounds the pass, a quotient is nine operations,
 // so one serves all four: P = D_0 D_1 D_2, N = P T^T D^{-1} T, 1 / (P (P + c N)).
-// D_q = 0 (the mean mode when eta0 = 0) stands for a zero inverse.
+// D_q = 0 (the mean mode when eta0 = 0) stands for a zero inverse.  P (P + c N) is of degree six in
+// D: D and c are first scaled by the power of two that brings base, which no D_q is below, to
+// [1, 2), so any normal base will do, as with a quotient for each D_q, and the bits stay.
 // FP64 step at 128^3 46385 -> 45753 us.
 __device__ __forceinline__ double spec_mode64(double2* r, int ld, double base, double c,
                                               double inv_vol, const double (&S)[3],
                                               const double (&T)[3]) {
+  const double scale = pow2_scale(base);
+  base *= scale;
+  c *= scale;
+  inv_vol *= scale;
   double D[3], T2[3];
   bool on[3];
 #pragma unroll
