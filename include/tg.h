@@ -70,7 +70,8 @@ typedef enum {
 } tg_precision;
 
 /* Periodic box [0, L[0]) x [0, L[1]) x [0, L[2]) with n[d] nodes per axis, spacing
- * h_d = L[d] / n[d] (Section 3 uses a uniform grid on a fictitious box).  n[d] >= 4. */
+ * h_d = L[d] / n[d] (Section 3 uses a uniform grid on a fictitious box).  n[d] >= 4,
+ * n[0] * n[1] * n[2] < 2^31. */
 typedef struct {
   int32_t n[3];
   double L[3];

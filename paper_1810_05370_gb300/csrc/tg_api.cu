@@ -89,13 +89,17 @@ constexpr int CN_MIXED_MASK = 0b101;
 
 size_t round_up(size_t x) { return (x + ALIGN - 1) / ALIGN * ALIGN; }
 
+// the kernels' voxel offsets are 32-bit (tg_internal.cuh); the state and workspace of 2^31 voxels
+// would take more than a terabyte
+constexpr long long MAX_VOXELS = 1LL << 31;
+
 bool grid_ok(const tg_grid* g) {
   if (!g) return false;
   for (int d = 0; d < 3; ++d) {
     if (g->n[d] < 4 || g->n[d] > (1 << 20)) return false;
     if (!(g->L[d] > 0.0) || !isfinite(g->L[d])) return false;
   }
-  return true;
+  return (long long)g->n[0] * g->n[1] * g->n[2] < MAX_VOXELS;
 }
 
 Geo make_geo(const tg_grid* g, int sms) {

@@ -94,7 +94,7 @@ struct CgScal {
 
 // Periodic neighbour offsets of node (i, j, k): X[o+1], Y[o+1], Z[o+1] for o in {-1, 0, 1};
 // the linear index of (i + ox, j + oy, k + oz) is Z[oz+1] + Y[oy+1] + X[ox+1].  32-bit: a grid
-// of 2^31 voxels would need a terabyte of workspace (tg_init refuses it), and nine 64-bit
+// of 2^31 voxels would need a terabyte of workspace (grid_ok refuses it), and nine 64-bit
 // offsets cost the operator kernels nine more registers and their adds twice the instructions.
 struct Nbr {
   int X[3], Y[3], Z[3];
