@@ -619,9 +619,13 @@ struct HookScope {
 // Kernels of a finished solve return at once, so overshooting a chunk only costs empty launches.
 // On stream st; `queued` iterations may already be in flight (then the loop reads the flags
 // first).
+// what a solve starts from: the residual is then |rhs|, or may be far below
+enum CgStart { CG_FROM_ZERO, CG_FROM_GUESS };
+
 template <class IterFn>
 tg_status drive_cg_loop(tg_ctx* X, cudaStream_t st, IterFn iter, const CgScal* dev, int nsolves,
-                        int maxit, int prev, CgScal* host, long long queued, int slot) {
+                        int maxit, int prev, CgStart start, CgScal* host, long long queued,
+                        int slot) {
   int chunk = queued > 0 ? 0 : first_chunk(prev);
   int grown = 2;
   CgScal seen[3];   // the solves' scalars at the first read
@@ -638,7 +642,7 @@ tg_status drive_cg_loop(tg_ctx* X, cudaStream_t st, IterFn iter, const CgScal* d
     for (int r = 0; r < nsolves; ++r) running |= host[r].status == CG_RUNNING;
     if (!running) return TG_OK;
     if (queued > (long long)maxit + 64) return fail(X, TG_ERR_CUDA);  // flags never settled
-    chunk = next_chunk(host, looked ? seen : nullptr, nsolves, CG_RUNNING, grown);
+    chunk = next_chunk(host, looked && start == CG_FROM_GUESS ? seen : nullptr, nsolves, CG_RUNNING, grown);
     if (!looked) std::copy(host, host + nsolves, seen);
     looked = true;
     grown = std::min(grown * 2, 32);
@@ -649,18 +653,19 @@ tg_status drive_cg_loop(tg_ctx* X, cudaStream_t st, IterFn iter, const CgScal* d
 // prof_iter tags), or INT_MIN to open one here
 template <class IterFn>
 tg_status drive_cg_on(tg_ctx* X, cudaStream_t st, IterFn iter, const CgScal* dev, int nsolves,
-                      int maxit, int prev, CgScal* host, long long queued = 0,
+                      int maxit, int prev, CgStart start, CgScal* host, long long queued = 0,
                       int slot = INT_MIN) {
   if (slot == INT_MIN) slot = prof_open_solve(X);
-  const tg_status s = drive_cg_loop(X, st, iter, dev, nsolves, maxit, prev, host, queued, slot);
+  const tg_status s = drive_cg_loop(X, st, iter, dev, nsolves, maxit, prev, start, host, queued,
+                                    slot);
   prof_close_solve(X, slot, host, nsolves);
   return s;
 }
 
 template <class IterFn>
 tg_status drive_cg(tg_ctx* X, IterFn iter, const CgScal* dev, int nsolves, int maxit, int prev,
-                   CgScal* host) {
-  return drive_cg_on(X, X->stream, iter, dev, nsolves, maxit, prev, host);
+                   CgStart start, CgScal* host) {
+  return drive_cg_on(X, X->stream, iter, dev, nsolves, maxit, prev, start, host);
 }
 
 // the single-species model (Eq. e:rd): c is carried in p, only it diffuses
@@ -765,7 +770,7 @@ tg_status cn_iterate(tg_ctx* X, const Cn3& C, CgScal host[3]) {
     return drive_cg(X, [&](int) {
       X->launches += 3;
       return launch_cn_iter(X->G, C, X->stream);
-    }, C.S, 3, X->prm.maxit_diff, X->prev_it_diff, host);
+    }, C.S, 3, X->prm.maxit_diff, X->prev_it_diff, CG_FROM_GUESS, host);
   if (small == SMALL_FAILED) return fail(X, TG_ERR_CUDA);
   CK(cudaMemcpyAsync(host, C.S, 3 * sizeof(CgScal), cudaMemcpyDeviceToHost, X->stream));
   CK(cudaStreamSynchronize(X->stream));
@@ -874,7 +879,7 @@ tg_status cn_solve3_mixed(tg_ctx* X, tg_stats* stats, int mask) {
     tg_status st = drive_cg(X, [&](int) {
       X->launches += 3;
       return launch_cn32_iter(X->G, I, X->stream, slot[0], slot[1], cap);
-    }, I.S, 3, X->prm.maxit_diff, X->prev_it_cn_inner[sw], host);
+    }, I.S, 3, X->prm.maxit_diff, X->prev_it_cn_inner[sw], CG_FROM_ZERO, host);
     if (st != TG_OK) return st;
     int itmax = 0;
     for (int r = 0; r < 3; ++r) {
@@ -989,8 +994,8 @@ tg_status ox_end(tg_ctx* X, tg_stats* stats) {
     return P.df ? launch_ox_iter(X->G, P.O, so) : launch_cn_iter(X->G, P.C, so);
   };
   CgScal host[3];
-  tg_status e = drive_cg_on(X, so, iter, P.dev, P.ns, X->prm.maxit_diff, X->prev_it_diff, host,
-                            X->ox_chunk, X->ox_slot);
+  tg_status e = drive_cg_on(X, so, iter, P.dev, P.ns, X->prm.maxit_diff, X->prev_it_diff,
+                            CG_FROM_GUESS, host, X->ox_chunk, X->ox_slot);
   if (e != TG_OK) return e;
   const CgScal& ho = P.df ? host[0] : host[1];
   if (P.df) {
@@ -1128,7 +1133,7 @@ tg_status elas_solve_mixed(tg_ctx* X, double* const u[3], double* const b_ext[3]
       if (e != cudaSuccess) return e;
       if (!spec) return launch_elas32_update(X->G, I, X->stream);
       return launch_spectral_update(V, I, X->z32, X->stream);
-    }, I.S, 1, X->prm.maxit_elas, X->prev_it_inner[slot], host);
+    }, I.S, 1, X->prm.maxit_elas, X->prev_it_inner[slot], CG_FROM_ZERO, host);
     if (s != TG_OK) return s;
     X->prev_it_inner[slot] = host[0].it;
     inner_total += host[0].it;
@@ -1200,7 +1205,7 @@ tg_status elas_solve(tg_ctx* X, double* const u[3], double* const b_ext[3], bool
       if (e == cudaSuccess) e = launch_spectral(V, r64, X->z64, E.S, X->stream);
       if (e == cudaSuccess) e = launch_elas_pupdate_spec(X->G, E, X->stream);
       return e;
-    }, E.S, 1, X->prm.maxit_elas, X->prev_it_elas, host);
+    }, E.S, 1, X->prm.maxit_elas, X->prev_it_elas, CG_FROM_GUESS, host);
   }
   if (s != TG_OK) return s;
   X->prev_it_elas = host[0].it;

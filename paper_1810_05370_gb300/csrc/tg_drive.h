@@ -28,10 +28,10 @@ inline int first_chunk(int prev) { return prev > 0 ? std::max(1, prev - prev / 8
 // they iterate; `grown` where a residual shows no rate).  Each read of the flags leaves the GPU
 // idle for some 10 us, so the queue is filled by an estimate and not by a growing guess: a solve
 // of 50 iterations takes two or three reads instead of four or five.  The residual is taken to
-// keep falling at its mean rate from |rhs|, which is where a refined solve starts.  A solve that
-// starts from a good guess starts lower, and that rate comes out too high: from the second read on
-// the rate since the first (first: the scalars read then, or null) counts too, for at most twice
-// the iterations that it was seen over, as a few iterations' rate may be off.
+// keep falling at its mean rate from |rhs|, which is where a solve from zero starts (a refined
+// one).  A solve from a good guess starts lower, and that rate comes out too high: from the second
+// read on the rate since the first (first: the scalars read then, else null) counts too, for at
+// most twice the iterations that it was seen over, as a few iterations' rate may be off.
 template <class S>
 int next_chunk(const S* host, const S* first, int nsolves, int running, int grown) {
   double need = 0.0;
