@@ -122,6 +122,7 @@ Geo make_geo(const tg_grid* g, int sms) {
   long long zc = (gx * gy * G.nz + target - 1) / target;
   zc = std::max(1LL, std::min(zc, (long long)G.nz));
   G.zc = (int)zc;
+  G.sms = sms;
   const long long gz = (G.nz + zc - 1) / zc;
   G.grid = dim3((unsigned)gx, (unsigned)gy, (unsigned)gz);
   G.nblocks = (int)(gx * gy * gz);
@@ -155,6 +156,7 @@ void spec_shape(const Geo& G, Spec<R>& V) {
   V.nx = G.nx;
   V.ny = G.ny;
   V.nz = G.nz;
+  V.sms = G.sms;
   V.nxh = G.nx / 2 + 1;
   V.nxp = (V.nxh + 15) / 16 * 16;
   V.pb = std::max(1, std::min(std::min(G.ny / 2, 16), floor_pow2(65536 / (2 * G.nx * cs))));

@@ -688,7 +688,7 @@ __global__ void __launch_bounds__(NT) k_cn_ir_correct(long long n, Cn3 C, Cn32 I
 
 int flat_blocks(const Geo& G) {   // never more blocks than the partial-sum buffer holds
   long long b = (G.nvox / 4 + NT - 1) / NT;
-  b = b < 8LL * 152 ? b : 8LL * 152;
+  b = b < 8LL * G.sms ? b : 8LL * G.sms;
   b = b < G.nblocks ? b : G.nblocks;
   return (int)(b > 0 ? b : 1);
 }

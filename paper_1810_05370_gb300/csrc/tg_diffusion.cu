@@ -7,8 +7,6 @@
 //   (A c)_j = c_j + sum_d [ a_d,j (c_j - c_{j+e_d}) + a_d,j-e_d (c_j - c_{j-e_d}) ].
 // The three right-hand sides share the coefficient reads: every kernel below streams the
 // six face values of a node once and applies them to all active solves.
-#include <algorithm>
-
 #include "tg_tiles.cuh"
 
 namespace tg {
@@ -271,13 +269,6 @@ __global__ void __launch_bounds__(NT) k_cn_pupdate(long long n, Cn3 C) {
     p[n - 1] = fma(beta, p[n - 1], di[n - 1] * r[n - 1]);
 }
 
-// (blocks over voxel pairs, solves), as the elasticity's flat updates
-dim3 cn_flat3(const Geo& G) {
-  const long long want = (G.nvox / 2 + NT - 1) / NT;
-  const long long most = std::min(304LL, (long long)G.nblocks);
-  return dim3((unsigned)std::max(1LL, std::min(want, most)), 3);
-}
-
 }  // namespace
 
 cudaError_t launch_diff_coef(const Geo& G, const DevParams& P, double dt, const double* g,
@@ -316,8 +307,8 @@ cudaError_t launch_cn_init(const Geo& G, const Cn3& C, cudaStream_t st, int mask
 
 cudaError_t launch_cn_iter(const Geo& G, const Cn3& C, cudaStream_t st) {
   TG_TIMED(K_CN_MATVEC, st, launch(k_cn_matvec, G.grid, dim3(BX, BY), 0, st, G, C));
-  TG_TIMED(K_CN_UPDATE, st, launch(k_cn_update, cn_flat3(G), NT, 0, st, G.nvox, C));
-  TG_TIMED(K_CN_PUPDATE, st, launch(k_cn_pupdate, cn_flat3(G), NT, 0, st, G.nvox, C));
+  TG_TIMED(K_CN_UPDATE, st, launch(k_cn_update, flat3(G), NT, 0, st, G.nvox, C));
+  TG_TIMED(K_CN_PUPDATE, st, launch(k_cn_pupdate, flat3(G), NT, 0, st, G.nvox, C));
   return cudaGetLastError();
 }
 

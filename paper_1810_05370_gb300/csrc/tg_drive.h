@@ -21,6 +21,27 @@ inline bool cg_small_fits(long long nvox, int sms, int sharers) {
   return nvox <= most && (sharers <= 1 || nvox * sharers <= 2 * most);
 }
 
+// Blocks of one component (solve) of the flat FP64 vector updates, `want` to have one voxel pair
+// per thread: two per SM, and never more than the partial-sum buffer holds (nine doubles for each
+// of the nblocks of the grid-shaped kernels; three components leave two each).
+inline long long flat_blocks(long long want, long long nblocks, int sms) {
+  return std::max(1LL, std::min(want, std::min(2LL * sms, nblocks)));
+}
+
+// a launch that leaves the SMs fewer than four blocks each
+inline bool few_blocks(long long blocks, int sms) { return blocks < 4LL * sms; }
+
+// Planes a block of the FP32 operator marches, zc those of a grid-shaped launch of nblocks.  A
+// block stages two planes more than it computes, so at one or a few planes per block (grids of
+// 64^3 to 128^3, where 16 blocks per SM leave no more) a third to two thirds of the staging is
+// halo: two chunks of planes per block where the launch still has four blocks per SM.  us a pass,
+// one -> two chunks: mixed 64^3 12937 -> 12352, 96^3 Jacobi 10136 -> 9257, 128^3 15503 -> 15217;
+// three or four chunks, or one wave of blocks, gain no more.  From nine planes a chunk on (256^3:
+// 27) the halo is small and the blocks' number counts: 70741 -> 70856.
+inline int op_planes(int zc, long long nblocks, int sms) {
+  return zc <= 8 && !few_blocks(nblocks, sms) ? 2 * zc : zc;
+}
+
 // Iterations queued before the first look at a solve's flags, prev those of the last such solve.
 inline int first_chunk(int prev) { return prev > 0 ? std::max(1, prev - prev / 8) : 4; }
 

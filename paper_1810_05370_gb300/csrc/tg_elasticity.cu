@@ -10,8 +10,6 @@
 // Per-step precomputation trades bytes for FP64 arithmetic: face coefficients already
 // divided by h_d^2 and the Jacobi diagonal are stored, so a matrix-vector product needs
 // 1 multiply and 6 fused multiply-adds per component for the face part.
-#include <algorithm>
-
 #include "tg_internal.cuh"
 
 namespace tg {
@@ -309,14 +307,6 @@ __global__ void __launch_bounds__(NT) k_elas_finish(Geo G, Elas E, double inv_dt
       }
     }
   }
-}
-
-// (blocks over voxel pairs, components): two blocks per SM and component, never more than the
-// partial-sum buffer holds (nine doubles per block of the grid-shaped kernels)
-dim3 flat3(const Geo& G) {
-  const long long want = (G.nvox / 2 + NT - 1) / NT;
-  const long long most = std::min(304LL, (long long)G.nblocks);
-  return dim3((unsigned)std::max(1LL, std::min(want, most)), 3);
 }
 
 }  // namespace

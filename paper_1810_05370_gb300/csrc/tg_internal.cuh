@@ -63,6 +63,7 @@ struct Geo {
   double inv2h[3];      // 1 / (2 h_d)
   double s_cross[3][3]; // 1 / (4 h_a h_d)
   int zc;               // z planes per block
+  int sms;              // SMs of the device
   dim3 grid;            // (ceil(nx/BX), ceil(ny/BY), ceil(nz/zc))
   int nblocks;
 };
@@ -400,6 +401,7 @@ struct Spec {
   double* partial;            // per-block partial sums (x inverse pass, means)
   unsigned int* counter;
   int nb_partial;             // capacity of partial, in doubles
+  int sms;                    // SMs of the device
   const void* zmap;           // host: TMA tensor map of W for the FP32 z pass (null: none)
 };
 
@@ -502,6 +504,11 @@ template <class... P, class... A>
 inline void launch(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
                    const A&... args) {
   launch_carved(PDL_CARVE_PERCENT, kernel, grid, block, smem, st, args...);
+}
+
+// the flat FP64 updates' grid: (blocks over voxel pairs, three components or solves)
+inline dim3 flat3(const Geo& G) {
+  return dim3((unsigned)flat_blocks((G.nvox / 2 + NT - 1) / NT, G.nblocks, G.sms), 3);
 }
 
 // ----------------------------------------------------------------------------- launches

@@ -380,16 +380,6 @@ int stream_blocks(long long n) {
   return (int)(b < 4096 ? (b > 0 ? b : 1) : 4096);
 }
 
-// Planes a block of the FP32 operator marches.  A block stages two planes more than it
-// computes, so at one or a few planes per block (grids of 64^3 to 128^3, where 16 blocks per SM
-// leave no more) a third to two thirds of the staging is halo: two chunks of planes per block
-// where the launch still has four blocks per SM.  us a pass, one -> two chunks: mixed 64^3
-// 12937 -> 12352, 96^3 Jacobi 10136 -> 9257, 100x84x60 7455 -> 7211, 128^3 15503 -> 15217; three
-// or four chunks, or one wave of blocks, gain no more (128^3: 15325, 15466; 100x84x60: 7260).
-// From nine planes a chunk on (256^3: 27) the halo is small and the blocks' number counts:
-// 70741 -> 70856.
-int op_planes(const Geo& G) { return G.zc <= 8 && G.nblocks >= 4 * 152 ? 2 * G.zc : G.zc; }
-
 dim3 op_grid(const Geo& G, int zb) {
   return dim3(G.grid.x, G.grid.y, (unsigned)((G.nz + zb - 1) / zb));
 }
@@ -432,7 +422,7 @@ cudaError_t launch_elas_ir_residual(const Geo& G, const Elas& E, const Elas32& I
 }
 
 cudaError_t launch_elas32_matvec(const Geo& G, const Elas32& I, cudaStream_t st) {
-  const int zb = op_planes(G);
+  const int zb = op_planes(G.zc, G.nblocks, G.sms);
   TG_TIMED(K_ELAS32_MATVEC, st,
            launch(k_elas32_matvec, op_grid(G, zb), dim3(BX, BY), 0, st, G, make_consts32(G), I, zb));
   return cudaGetLastError();
@@ -441,7 +431,7 @@ cudaError_t launch_elas32_matvec(const Geo& G, const Elas32& I, cudaStream_t st)
 // flat launches that reduce: never more blocks than the partial-sum buffer holds
 static int reduce_blocks(const Geo& G, long long items) {
   long long b = (items + NT - 1) / NT;
-  b = b < 8LL * 152 ? b : 8LL * 152;
+  b = b < 8LL * G.sms ? b : 8LL * G.sms;
   b = b < G.nblocks ? b : G.nblocks;
   return (int)(b > 0 ? b : 1);
 }
@@ -459,7 +449,7 @@ cudaError_t launch_elas32_scale_r(const Geo& G, const Elas32& I, cudaStream_t st
 }
 
 cudaError_t launch_elas32_matvec_spec(const Geo& G, const Elas32& I, cudaStream_t st) {
-  const int zb = op_planes(G);
+  const int zb = op_planes(G.zc, G.nblocks, G.sms);
   TG_TIMED(K_ELAS32_MATVEC_SPEC, st,
            launch(k_elas32_matvec_spec, op_grid(G, zb), dim3(BX, BY), 0, st, G, make_consts32(G), I,
                   zb));

@@ -1803,12 +1803,11 @@ cudaError_t launch_spec_mean(long long n, const double* mu, const double* lam,
   return cudaGetLastError();
 }
 
-// Narrow tiles while wide ones (16 columns at these nz) leave the SMs fewer than four blocks
-// each; their blocks' partial sums were counted in V.nb_partial.
+// Narrow tiles while wide ones (16 columns at these nz) leave the SMs few blocks; their blocks' partial sums were counted in V.nb_partial.
 bool spec_z_narrow(const Spec<float>& V) {
   const long long wide = (long long)((V.nxh + V.tz - 1) / V.tz) * V.ny;
   const long long narrow = (long long)((V.nxh + Z_NARROW - 1) / Z_NARROW) * V.ny;
-  return V.nz <= Z_NARROW_MAX && V.tz == 16 && wide < 4 * 152 && narrow <= V.nb_partial;
+  return V.nz <= Z_NARROW_MAX && V.tz == 16 && few_blocks(wide, V.sms) && narrow <= V.nb_partial;
 }
 
 // the z pass: for FP32 and nz = 128 or 256 in registers, from tiles staged by TMA when the

@@ -8,6 +8,12 @@ int tgd_small_fits(long long nvox, int sms, int sharers) {
   return tg::cg_small_fits(nvox, sms, sharers) ? 1 : 0;
 }
 
+long long tgd_flat_blocks(long long want, long long nblocks, int sms) {
+  return tg::flat_blocks(want, nblocks, sms);
+}
+
+int tgd_op_planes(int zc, long long nblocks, int sms) { return tg::op_planes(zc, nblocks, sms); }
+
 // a launch that returns `error`: the outcome, with *refused in and out and *launched counted up
 int tgd_run_small(int fits, int* refused, int error, int* launched) {
   bool r = *refused != 0;

@@ -67,6 +67,27 @@ def test_flags_are_read_few_times(lib, rr0, prev, total):
     assert reads <= most
 
 
+@pytest.mark.parametrize("sms", [1, 76, 148, 152])
+def test_launch_shapes_follow_the_device(lib, sms):
+    lib.tgd_flat_blocks.restype = ctypes.c_longlong
+
+    def flat(want, nblocks):
+        return lib.tgd_flat_blocks(ctypes.c_longlong(want), ctypes.c_longlong(nblocks), sms)
+
+    assert flat(0, 1) == 1 and flat(1 << 30, 1 << 30) == 2 * sms
+    for nblocks in (1, 5, sms, 4 * sms):
+        got = flat(1 << 30, nblocks)
+        assert got == min(nblocks, 2 * sms)
+        assert 3 * got * 2 <= 9 * nblocks              # two sums of three components each
+
+    def planes(zc, nblocks):
+        return lib.tgd_op_planes(zc, ctypes.c_longlong(nblocks), sms)
+
+    for zc in (1, 8):
+        assert planes(zc, 4 * sms) == 2 * zc and planes(zc, 4 * sms - 1) == zc
+    assert planes(9, 4 * sms) == 9
+
+
 TAKEN, QUEUE, FAILED = 0, 1, 2
 
 
