@@ -17,12 +17,6 @@
 namespace tg {
 namespace {
 
-__device__ __forceinline__ unsigned long long global_ns() {
-  unsigned long long t;
-  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-  return t;
-}
-
 __device__ bool grid_barrier(const BatchDev& B) {
   __shared__ int ok;
   __syncthreads();
@@ -38,13 +32,13 @@ __device__ bool grid_barrier(const BatchDev& B) {
       __threadfence();
       atomicAdd(B.bar + 1, 1u);
     } else {
-      const unsigned long long t0 = global_ns();
+      const unsigned long long t0 = wait_clock_ns();
       while (*gen == g) {
         if (*err) {
           good = 0;
           break;
         }
-        if (global_ns() - t0 > B.timeout_ns) {
+        if (wait_clock_ns() - t0 > B.timeout_ns) {
           atomicExch(B.err, 1);
           good = 0;
           break;

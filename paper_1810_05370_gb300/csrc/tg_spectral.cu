@@ -1240,18 +1240,13 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
       : "memory");
   return done != 0;
 }
-__device__ __forceinline__ uint64_t globaltimer_ns() {
-  uint64_t t;
-  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-  return t;
-}
 // true once the phase completed; false after limit_ns
 __device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t parity,
                                                   uint64_t limit_ns) {
-  const uint64_t t0 = globaltimer_ns();
+  const uint64_t t0 = wait_clock_ns();
   for (uint32_t it = 0;; ++it) {
     if (mbar_try_wait(bar, parity)) return true;
-    if ((it & 63) == 63 && globaltimer_ns() - t0 > limit_ns) return false;
+    if ((it & 63) == 63 && wait_clock_ns() - t0 > limit_ns) return false;
   }
 }
 __device__ __forceinline__ void tma_load_4d(void* dst, const CUtensorMap* map, int c0, int c1,
