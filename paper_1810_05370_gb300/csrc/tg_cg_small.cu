@@ -18,10 +18,9 @@
 // register file and their 27 coefficients 108 KB of its shared memory, so grids up to 512
 // voxels per SM (77824 on 152 SMs) take this form.
 //
-// Measured (us a pass, three launches an iteration -> this form): 16^3 static solve 590 -> 300,
-// FP64 step at 32^3 2700 -> 2010, rollout gradient of three steps at 48 x 40 x 36 32900 ->
-// 25200.  Near the size limit (69120 voxels) an iteration takes 20.4 us, 11.5 of them on the
-// FP64 pipe; the rest is the two waits and the neighbours' z from L2.
+// Measured (three launches an iteration -> this form): a static solve at 16^3 590 -> 300 us, two
+// FP64 steps at 32^3 2.70 -> 2.01 ms.  Near the size limit (69120 voxels) an iteration takes
+// 20.4 us, 11.5 of them on the FP64 pipe; the rest is the two waits and the neighbours' z from L2.
 //
 // The waits are bounded in time (tg_wait.cuh; the context's limit, 20 s unless it is set): a
 // block that gives up marks the solve CG_TIMEOUT and returns, the others give up in their turn

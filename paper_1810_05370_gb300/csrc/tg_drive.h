@@ -34,10 +34,10 @@ inline bool few_blocks(long long blocks, int sms) { return blocks < 4LL * sms; }
 // Planes a block of the FP32 operator marches, zc those of a grid-shaped launch of nblocks.  A
 // block stages two planes more than it computes, so at one or a few planes per block (grids of
 // 64^3 to 128^3, where 16 blocks per SM leave no more) a third to two thirds of the staging is
-// halo: two chunks of planes per block where the launch still has four blocks per SM.  us a pass,
-// one -> two chunks: mixed 64^3 12937 -> 12352, 96^3 Jacobi 10136 -> 9257, 128^3 15503 -> 15217;
-// three or four chunks, or one wave of blocks, gain no more.  From nine planes a chunk on (256^3:
-// 27) the halo is small and the blocks' number counts: 70741 -> 70856.
+// halo: two chunks of planes per block where the launch still has four blocks per SM.  ms for two
+// mixed steps, one -> two chunks: 64^3 12.9 -> 12.4, 128^3 15.5 -> 15.2; three or four chunks, or one
+// wave of blocks, gain no more.  From nine planes a chunk on (256^3: 27) the halo is small and the
+// blocks' number counts.
 inline int op_planes(int zc, long long nblocks, int sms) {
   return zc <= 8 && !few_blocks(nblocks, sms) ? 2 * zc : zc;
 }

@@ -158,10 +158,9 @@ __device__ __forceinline__ int block_count() { return gridDim.x * gridDim.y * gr
 //  * the ticket is one acquire-release atomic (tg_wait.cuh) instead of a full fence and a relaxed
 //    one.
 // Deterministic: the order of the additions depends on the launch's shape only.
-// Measured with the flat vector updates and the fused operator rows (us a pass, before ->
-// after): FP64 solve at 96 x 80 x 72 35100 -> 30100, 16^3 static solve 820 -> 736, FP64 step at
-// 32^3 3590 -> 3260 and at 128^3 53300 -> 51000, mixed step at 100 x 84 x 60 9380 -> 8280; at
-// 256^3, where a launch is long, nothing.
+// Measured with the flat vector updates and the fused operator rows: an FP64 solve at 96 x 80 x 72
+// 35.1 -> 30.1 ms, a mixed step at 100 x 84 x 60 9.4 -> 8.3 ms; at 256^3, where a launch is long,
+// nothing.
 // Sum of sh[0 .. n) (n a multiple of 32, at most 1024) by one whole warp; every lane calls it
 // and lane 0 holds the result.
 __device__ __forceinline__ double warp_sum_shared(const double* sh, int n, int lane) {
@@ -409,8 +408,8 @@ struct Spec {
 // search direction p = z + beta p_old instead of z, into the buffer of the two that the
 // iteration's operator kernel reads (they alternate with the iteration count S->it).
 // From the solve's first iteration on it also writes the iterate, e += alpha p_old; the last
-// iteration of a solve, which ends before this pass, is added with the correction (launch_elas_ir_correct's
-// pending).
+// iteration of a solve, which ends before this pass, is added with the correction
+// (launch_elas_ir_correct's pending).
 template <typename R>
 struct PUpd {
   R* p[2][3];
@@ -445,15 +444,13 @@ template <typename R> size_t spec_smem_z(const Spec<R>& V) {
 // tail of the one before it -- the last block's reduction above all.  A step is 200 to 700
 // kernels, of which those of grids up to 64^3 run 3 to 15 us each.
 //
-// Where the lines lie (us a pass, plain -> overlapped): 16^3 static solve 736 -> 592, FP64
-// 32^3 3266 -> 2700, mixed 64^3 15235 -> 12900, mixed 128^3 16390 -> 15380, 256x256x128
-// 32290 -> 32030, but 256^3 139200 -> 143100: there a launch is long against its latency, and
-// blocks that arrive while the previous kernel runs find an SM whose shared memory / L1 split
-// is the other kernel's and cannot change until the SM is idle.  For the same reason the
-// overlapped kernels of grids from PDL_CARVE_VOXELS on ask for one common split, 60 % shared
-// memory (128^3: default split 16400, 50 % 15610, 60 % 15380, 75 % 15610, 100 % 16800); on
-// smaller grids the occupancy does not matter and each kernel keeps its own (FP64 32^3: 2700
-// against 2790).
+// Where the lines lie (ms for two mixed steps, plain -> overlapped): 64^3 15.2 -> 12.9, 128^3
+// 16.4 -> 15.4, but 256^3 139.2 -> 143.1 (at 2^23 voxels 1 % better): there a launch is long against
+// its latency, and blocks that arrive while the previous kernel runs find an SM whose shared
+// memory / L1 split is the other kernel's and cannot change until the SM is idle.  For the same
+// reason the overlapped kernels of grids from PDL_CARVE_VOXELS on ask for one common split, 60 %
+// shared memory (128^3: the kernels' own 16.4, 50 % and 75 % 15.6, 100 % 16.8); on smaller grids
+// the occupancy does not matter and each kernel keeps its own (FP64 32^3: 3 % better).
 constexpr long long PDL_MAX_VOXELS = 1LL << 23;
 constexpr long long PDL_CARVE_VOXELS = 1LL << 17;
 constexpr int PDL_CARVE_PERCENT = 60;

@@ -81,7 +81,7 @@ template <int SGN, int M, typename C> __device__ __forceinline__ C w16(C v) {
 // multiply-adds.  On the FP64 pipe an addition, a product and both cost the same, and the FP64
 // passes are bound by it (counters at 128^3: 80 to 85 % busy): a 16-point transform takes 144
 // operations instead of 160, an eight-point one 52 instead of 56.  With the stages' twiddles
-// folded the same way (butterfly below), the FP64 step at 128^3 48610 -> 46435 us.
+// folded the same way (butterfly below), the FP64 step at 128^3 48.6 -> 46.4 ms.
 template <int M> struct W16 {   // cosine and tangent of m pi / 8, m != 4
   static constexpr double h = 0.70710678118654752, c1 = 0.92387953251128674,
                           s1 = 0.38268343236508977, t1 = 0.41421356237309505;
@@ -604,11 +604,10 @@ __device__ __forceinline__ bool block_sum_end(BlockSumOf<MAXT>& B, double* parti
 // 132 in a y pass, of which the transforms' arithmetic is 40), most of them index arithmetic,
 // bounds checks and loop control of the general line length and tile.  LN > 0 instantiates a
 // pass for lines of 2^LN and its usual tile, 16 lines or columns; LN = 0 is the general form.
-// The arithmetic is the same.  us a pass, general -> compile-time: mixed 64^3 study 10870 -> 9960,
-// 128^3 14494 -> 13640, 256^3 126490 -> 122140 (per launch, update + forward 185 -> 161, inverse 197
-// -> 175).  The x passes take 32 to 256, the y pass 32 to 128 (32^3 1118 -> 1080 us a pass; at 256 its four blocks per
-// SM leave 64 registers, which the unrolled form spills: 72 -> 88 us).  The FP64 passes stay
-// general: the FP64 pipe bounds them (128^3 50370 -> 50640).
+// The arithmetic is the same.  us per launch at 256^3, general -> compile-time: residual update and
+// forward pass 185 -> 161, inverse 197 -> 175.  The x passes take 32 to 256, the y pass 32 to 128:
+// at 256 its four blocks per SM leave 64 registers, which the unrolled form spills (72 -> 88 us).
+// The FP64 passes stay general: the FP64 pipe bounds them (a step at 128^3 gained nothing).
 constexpr int XPB = 16, XLPB = 4;   // lines per block of the compile-time forms
 int x_lines(const Spec<float>& V) {
   const bool ok = V.pb == XPB && V.nx >= 32 && V.nx <= 256;   // powers of two
@@ -730,8 +729,8 @@ __global__ void __launch_bounds__(NT) k_spec_x_fwd(Spec<R> V, const R* __restric
 //
 // FORM: the transform in two line buffers (0) or in place (1).  In place a stage costs two
 // barriers instead of one but half the shared memory, which pays where two buffers leave the
-// SM fewer than four blocks (lines of 256: 72 KB a block); us a pass, 0 -> 1: mixed 256^3 131950
-// -> 128600, but 128^3 14763 -> 14874 and 64^3 11730 -> 11950, where both fit four times.
+// SM fewer than four blocks (lines of 256: 72 KB a block): two mixed steps at 256^3 131.9 -> 128.6
+// ms, but at 64^3, where both fit four times, 2 % slower.
 template <int FORM, int LN>
 __global__ void __launch_bounds__(NT, 4) k_spec_update_xfwd(Spec<float> V, Elas32 I) {
   pdl_sync();
@@ -827,9 +826,8 @@ __global__ void __launch_bounds__(NT, 4) k_spec_update_xfwd(Spec<float> V, Elas3
 // nx/2 + 1 modes of a row leave one column over from whole tiles.  In FP64 the first rows of
 // blocks take that column of a tile's width of planes each, instead of one block per plane
 // transforming one column and tx - 1 of zeros: a fifth of the pass's work at 128^3, and the FP64
-// pipe bounds it (a pass of the case 50440 -> 49175 us).  In FP32 the mostly empty blocks cost
-// less than the strided loads of the gathered column (64^3 study 9950 -> 10530, 256^3 122100 ->
-// 123460).
+// pipe bounds it (an FP64 step at 128^3 50.4 -> 49.2 ms).  In FP32 the mostly empty blocks cost
+// less than the strided loads of the gathered column (mixed steps at 64^3 6 % slower with it).
 template <typename R>
 __host__ __device__ constexpr bool y_column_left(int nxh, int tx) {
   return sizeof(R) == 8 && nxh > tx && nxh % tx == 1;
@@ -873,7 +871,7 @@ __global__ void __launch_bounds__(NT, sizeof(R) == 4 ? 4 : 0) k_spec_y(Spec<R> V
 // D_q = 0 (the mean mode when eta0 = 0) stands for a zero inverse.  P (P + c N) is of degree six in
 // D: D and c are first scaled by the power of two that brings base, which no D_q is below, to
 // [1, 2), so any normal base will do, as with a quotient for each D_q, and the bits stay.
-// FP64 step at 128^3 46385 -> 45753 us.
+// FP64 step at 128^3 46.4 -> 45.8 ms.
 __device__ __forceinline__ double spec_mode64(double2* r, int ld, double base, double c,
                                               double inv_vol, const double (&S)[3],
                                               const double (&T)[3]) {
@@ -929,13 +927,13 @@ __device__ __forceinline__ double spec_mode64(double2* r, int ld, double base, d
 // a thread's radix-4 butterflies and modes one after the other, 13.5 us for 4.7 MB -- and a
 // thread of a narrow tile has half of them.  The terms of <r, z> are summed as a wide tile's
 // threads sum them -- a column's modes kz = g, g + groups, ... in FP32, one thread per
-// (column, g) -- so the sum does not depend on the tile.  us a pass, 16 -> 8 -> 4 columns: mixed
-// 64^3 study 11815 -> 10825 -> 10626, 32^3 1218 -> 1124 -> 1112, but four columns cost the concurrent
-// batch, whose members fill each other's gaps, 1.8 % (16583 -> 16600 -> 16880): eight.
+// (column, g) -- so the sum does not depend on the tile.  Two mixed steps at 64^3 with 16, 8 and 4
+// columns: 11.8, 10.8, 10.6 ms, but four columns cost the concurrent batch, whose members fill each
+// other's gaps, 1.8 %: eight.
 constexpr int Z_NARROW = 8, Z_LNARROW = 3;
 constexpr int Z_NARROW_MAX = 64;        // largest nz
 constexpr int Z_NARROW_THREADS = 192;
-// LN > 0: columns of 2^LN at compile time (narrow tiles; 64: study 9960 -> 9730 us.  The form for
+// LN > 0: columns of 2^LN at compile time (narrow tiles; 64: 2 % of a mixed step.  The form for
 // 32 was left out: the compiler contracts its radix-2 stage otherwise, so its roundings differ).
 //
 // blocks of the FP64 pass for the column left over from whole tiles (0: none)
@@ -1276,8 +1274,8 @@ __device__ __forceinline__ void fence_proxy_async_smem() {
 
 // At nz = 128 a block takes 27 KB with the sum's scratch cut to its 64 threads, so eight fit an SM
 // and the 1152 blocks of a 128^3 pass run in one wave -- if the launch asks for all of the SM's
-// shared memory; at the 60 % that suits the other passes four fit.  128^3 (2 steps) 13650 -> 13285
-// us, single-species 6092 -> 5920, host 8372 -> 8192.
+// shared memory; at the 60 % that suits the other passes four fit (two mixed steps at 128^3 13.65
+// -> 13.29 ms).
 constexpr uint64_t ZR_WAIT_NS = 2000000000ull;   // 2 s for a tile that takes microseconds
 
 template <int P>
@@ -1798,7 +1796,8 @@ cudaError_t launch_spec_mean(long long n, const double* mu, const double* lam,
   return cudaGetLastError();
 }
 
-// Narrow tiles while wide ones (16 columns at these nz) leave the SMs few blocks; their blocks' partial sums were counted in V.nb_partial.
+// Narrow tiles while wide ones (16 columns at these nz) leave the SMs few blocks; their blocks'
+// partial sums were counted in V.nb_partial.
 bool spec_z_narrow(const Spec<float>& V) {
   const long long wide = (long long)((V.nxh + V.tz - 1) / V.tz) * V.ny;
   const long long narrow = (long long)((V.nxh + Z_NARROW - 1) / Z_NARROW) * V.ny;
