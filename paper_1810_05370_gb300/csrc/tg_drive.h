@@ -7,7 +7,7 @@
 
 namespace tg {
 
-constexpr int CGS_MAX_THREADS = 512;   // voxels per SM of a solve that is one launch (tg_cg_small.cu)
+constexpr int CGS_MAX_THREADS = 512;   // most voxels per SM of a one-launch solve (tg_cg_small.cu)
 
 // Whether an FP64 Jacobi solve on nvox voxels runs as one cooperative launch.  It needs every SM's
 // registers for at most 512 voxels each.  sharers: the host threads that step simulations side
@@ -35,9 +35,9 @@ inline bool few_blocks(long long blocks, int sms) { return blocks < 4LL * sms; }
 // block stages two planes more than it computes, so at one or a few planes per block (grids of
 // 64^3 to 128^3, where 16 blocks per SM leave no more) a third to two thirds of the staging is
 // halo: two chunks of planes per block where the launch still has four blocks per SM.  ms for two
-// mixed steps, one -> two chunks: 64^3 12.9 -> 12.4, 128^3 15.5 -> 15.2; three or four chunks, or one
-// wave of blocks, gain no more.  From nine planes a chunk on (256^3: 27) the halo is small and the
-// blocks' number counts.
+// mixed steps, one -> two chunks: 64^3 12.9 -> 12.4, 128^3 15.5 -> 15.2; three or four chunks, or
+// one wave of blocks, gain no more.  From nine planes a chunk on (256^3: 27) the halo is small and
+// the blocks' number counts.
 inline int op_planes(int zc, long long nblocks, int sms) {
   return zc <= 8 && !few_blocks(nblocks, sms) ? 2 * zc : zc;
 }

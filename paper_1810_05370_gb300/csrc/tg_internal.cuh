@@ -445,10 +445,10 @@ template <typename R> size_t spec_smem_z(const Spec<R>& V) {
 // kernels, of which those of grids up to 64^3 run 3 to 15 us each.
 //
 // Where the lines lie (ms for two mixed steps, plain -> overlapped): 64^3 15.2 -> 12.9, 128^3
-// 16.4 -> 15.4, but 256^3 139.2 -> 143.1 (at 2^23 voxels 1 % better): there a launch is long against
-// its latency, and blocks that arrive while the previous kernel runs find an SM whose shared
-// memory / L1 split is the other kernel's and cannot change until the SM is idle.  For the same
-// reason the overlapped kernels of grids from PDL_CARVE_VOXELS on ask for one common split, 60 %
+// 16.4 -> 15.4, but 256^3 139.2 -> 143.1 (at 2^23 voxels 1 % better): there a launch is long
+// against its latency, and blocks that arrive while the previous kernel runs find an SM whose
+// shared memory / L1 split is the other kernel's and cannot change until the SM is idle.  For the
+// same reason the overlapped kernels of grids from PDL_CARVE_VOXELS on ask for one common split, 60 %
 // shared memory (128^3: the kernels' own 16.4, 50 % and 75 % 15.6, 100 % 16.8); on smaller grids
 // the occupancy does not matter and each kernel keeps its own (FP64 32^3: 3 % better).
 constexpr long long PDL_MAX_VOXELS = 1LL << 23;
