@@ -61,11 +61,11 @@ def mixed_kernel_bytes(n, precond):
         "k_sl32_pack": 120,          # v (3), 6 species in (FP64); 3 interleaved float4 out
         "k_lame_df": 116,            # p, i, n, g, w, f, bg in; mu, lam, eta (FP64 and FP32),
                                      # mu, lam and p + n pairs out
-        "k_df_pack3": 48,            # 3 FP64 in, 3 pairs out
+        "k_df_pack3": 32,            # i, l in; their pairs out (the third slot repeats i)
         "k_cn_ir_residual_df": 76,   # 3 face pairs, D^-1; per field (i, l): x pair, rhs pair, r, e
         "k_cn32_pupdate": 28,        # D^-1, r and p (2 fields) in, p out
         "k_cn32_matvec": 44,         # 3 FP32 faces, z, previous p (2 fields) in; p, q out
-        "k_cn32_update": 52,         # D^-1, e, r, p, q (2 fields) in, e, r out
+        "k_cn32_update": 48,         # e, r, p, q (2 fields) in, e, r out
         "k_cn_ir_correct": 56,       # x (FP64), e in; x, x pair out (2 fields)
         "k_cn32_neumann": 32,        # r (2 fields), 3 FP32 faces, D^-1 in; z (2 fields) out
         "k_diff_node_df": 40,        # g, w, f in; K pair, rho out
@@ -105,25 +105,25 @@ def mixed_kernel_bytes(n, precond):
 # of a single kernel, per voxel, with the hash of the source it was measured on: reported
 # only while the kernel's source (its .cu file and the shared headers) is unchanged.
 MEASURED_TRAFFIC = {   # 256^3 mixed step, profiles/launches_mixed_spectral_256.md
-    "k_spec_update_xfwd": {"bytes_per_voxel": 85.6, "sha": "d59493db2c07f8d9"},
-    "k_elas32_matvec_spec": {"bytes_per_voxel": 32.2, "sha": "7ec7d47f12615f35"},
-    "k_spec_x_inv_p": {"bytes_per_voxel": 42.6, "sha": "d59493db2c07f8d9"},
-    "k_spec_y_fwd": {"bytes_per_voxel": 19.9, "sha": "d59493db2c07f8d9"},
-    "k_spec_y_inv": {"bytes_per_voxel": 19.4, "sha": "d59493db2c07f8d9"},
-    "k_spec_zr": {"bytes_per_voxel": 20.4, "sha": "d59493db2c07f8d9"},
-    "k_cn32_neumann": {"bytes_per_voxel": 32.6, "sha": "7336241f68141960"},
-    "k_cn32_matvec": {"bytes_per_voxel": 40.4, "sha": "7336241f68141960"},
-    "k_cn32_update": {"bytes_per_voxel": 45.3, "sha": "7336241f68141960"},
-    "k_cn_ir_residual_df": {"bytes_per_voxel": 75.9, "sha": "7336241f68141960"},
-    "k_elas_ir_residual_df": {"bytes_per_voxel": 166.7, "sha": "7ec7d47f12615f35"},
-    "k_ox_matvec": {"bytes_per_voxel": 48.0, "sha": "63e5600d8107b556"},
-    "k_ox_update": {"bytes_per_voxel": 53.7, "sha": "63e5600d8107b556"},
-    "k_ox_pupdate": {"bytes_per_voxel": 28.8, "sha": "63e5600d8107b556"},
-    "k_sl32": {"bytes_per_voxel": 97.5, "sha": "7ec7d47f12615f35"},
-    "k_sl32_pack": {"bytes_per_voxel": 118.4, "sha": "7ec7d47f12615f35"},
-    "k_elas_coef_df": {"bytes_per_voxel": 126.4, "sha": "eb3281616b3713f0"},
-    "k_react": {"bytes_per_voxel": 125.2, "sha": "8ca213d5b6f3fcea"},
-    "k_lame_df": {"bytes_per_voxel": 113.0, "sha": "8ca213d5b6f3fcea"},
+    "k_spec_update_xfwd": {"bytes_per_voxel": 57.5, "sha": "513da5582dd5cb61"},
+    "k_elas32_matvec_spec": {"bytes_per_voxel": 35.1, "sha": "285798896f337e67"},
+    "k_spec_x_inv_p": {"bytes_per_voxel": 68.4, "sha": "513da5582dd5cb61"},
+    "k_spec_y_fwd": {"bytes_per_voxel": 22.4, "sha": "513da5582dd5cb61"},
+    "k_spec_y_inv": {"bytes_per_voxel": 22.4, "sha": "513da5582dd5cb61"},
+    "k_spec_zr": {"bytes_per_voxel": 22.9, "sha": "513da5582dd5cb61"},
+    "k_cn32_neumann": {"bytes_per_voxel": 32.6, "sha": "a89056ab9360318b"},
+    "k_cn32_matvec": {"bytes_per_voxel": 40.8, "sha": "a89056ab9360318b"},
+    "k_cn32_update": {"bytes_per_voxel": 45.2, "sha": "a89056ab9360318b"},
+    "k_cn_ir_residual_df": {"bytes_per_voxel": 75.7, "sha": "a89056ab9360318b"},
+    "k_elas_ir_residual_df": {"bytes_per_voxel": 162.2, "sha": "285798896f337e67"},
+    "k_ox_matvec": {"bytes_per_voxel": 48.0, "sha": "907d6a2460eed981"},
+    "k_ox_update": {"bytes_per_voxel": 53.7, "sha": "907d6a2460eed981"},
+    "k_ox_pupdate": {"bytes_per_voxel": 30.0, "sha": "907d6a2460eed981"},
+    "k_sl32": {"bytes_per_voxel": 97.5, "sha": "285798896f337e67"},
+    "k_sl32_pack": {"bytes_per_voxel": 118.7, "sha": "285798896f337e67"},
+    "k_elas_coef_df": {"bytes_per_voxel": 126.4, "sha": "e9d02f856bd68402"},
+    "k_react": {"bytes_per_voxel": 125.2, "sha": "2693642097585819"},
+    "k_lame_df": {"bytes_per_voxel": 113.0, "sha": "2693642097585819"},
 }
 KERNEL_SOURCE = {
     "k_spec_update_xfwd": "tg_spectral.cu", "k_elas32_matvec_spec": "tg_mixed.cu",
@@ -141,7 +141,8 @@ def kernel_source_sha(kernel):
     import hashlib
     csrc = os.path.join(ROOT, "paper_1810_05370_gb300", "csrc")
     h = hashlib.sha256()
-    for f in (KERNEL_SOURCE.get(kernel), "tg_internal.cuh", "tg_tiles.cuh", "tg_fpconv.cuh"):
+    for f in (KERNEL_SOURCE.get(kernel), "tg_internal.cuh", "tg_tiles.cuh", "tg_fpconv.cuh",
+              "tg_wait.cuh", "tg_drive.h"):
         if f is None:
             return None
         with open(os.path.join(csrc, f), "rb") as fh:

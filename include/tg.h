@@ -139,7 +139,9 @@ typedef struct {
   int64_t it_elas_total;
   int64_t launches;          /* CUDA kernels this call queued                                */
   double t_elas_matvec_ms;   /* with timing on: summed duration of the elasticity operator   */
-  int64_t n_elas_matvec;     /*   kernel over the launches that did work, and their count    */
+  int64_t n_elas_matvec;     /*   kernel over the launches that did work, and their count;   */
+                             /*   0 where an FP64 Jacobi solve of a small grid is one launch */
+                             /*   (k_elas_cg in tg_kernel_times)                             */
   double t_phase_ms[4];      /* with timing on: device time of S0-S1, S2, S3-S5 and S6-S7     */
                              /*   (event to event on the stream), summed over the call's steps */
   double t_spec_update_ms;   /* with timing on, TG_MIXED with a spectral preconditioner: summed */
